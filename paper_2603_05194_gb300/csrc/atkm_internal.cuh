@@ -12,15 +12,13 @@
 #include <vector>
 
 #include "../../include/atkm.h"
-#include "df32.cuh"
+#include "i64.cuh"
 
 namespace atkm {
 
 // ---------------------------------------------------------------- complex
 template <typename R> struct CT;
-template <> struct CT<double> { using c = double2; };
 template <> struct CT<float> { using c = float2; };
-template <> struct CT<df> { using c = cdf; };
 template <typename R> using cx = typename CT<R>::c;
 
 template <typename R> __host__ __device__ __forceinline__ cx<R> mk(R a, R b) {
@@ -66,35 +64,22 @@ template <> __device__ __forceinline__ float tor<float>(double v) { return d2f_b
 template <typename R> __device__ __forceinline__ double tod(R v);
 template <> __device__ __forceinline__ double tod<double>(double v) { return v; }
 template <> __device__ __forceinline__ double tod<float>(float v) { return f2d_bits(v); }
-// binary64 <-> double-word: the leading binary32 part from the bit layout, the
-// trailing part from the exact binary64 remainder (one binary64 subtraction).
-template <> __device__ __forceinline__ df tor<df>(double v) {
-  const float h = d2f_bits(v);
-  return df(h, d2f_bits(v - f2d_bits(h)));
-}
-template <> __device__ __forceinline__ double tod<df>(df v) { return f2d_bits(v.hi) + f2d_bits(v.lo); }
-
 template <typename R> __device__ __forceinline__ cx<R> add(cx<R> a, cx<R> b) {
-  if constexpr (std::is_same<R, df>::value) return df_cadd(a, b);
-  else return mk<R>(a.x + b.x, a.y + b.y);
+  return mk<R>(a.x + b.x, a.y + b.y);
 }
 template <typename R> __device__ __forceinline__ cx<R> sub(cx<R> a, cx<R> b) {
-  if constexpr (std::is_same<R, df>::value) return df_csub(a, b);
-  else return mk<R>(a.x - b.x, a.y - b.y);
+  return mk<R>(a.x - b.x, a.y - b.y);
 }
 template <typename R> __device__ __forceinline__ cx<R> scl(cx<R> a, R s) {
-  if constexpr (std::is_same<R, df>::value) return df_cscl(a, s);
-  else return mk<R>(a.x * s, a.y * s);
+  return mk<R>(a.x * s, a.y * s);
 }
 // a * b
 template <typename R> __device__ __forceinline__ cx<R> cmul(cx<R> a, cx<R> b) {
-  if constexpr (std::is_same<R, df>::value) return df_cmul(a, b, false);
-  else return mk<R>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  return mk<R>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 // a * conj(b)
 template <typename R> __device__ __forceinline__ cx<R> cmulc(cx<R> a, cx<R> b) {
-  if constexpr (std::is_same<R, df>::value) return df_cmul(a, b, true);
-  else return mk<R>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
+  return mk<R>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 // s * i * a  (s = +1 or -1)
 template <typename R, int S> __device__ __forceinline__ cx<R> mul_si(cx<R> a) {
@@ -130,38 +115,22 @@ inline int device_sm_count() {
 // read into registers before any is written (one shared buffer).
 constexpr int kThreads = 256;      // threads per FFT CTA
 constexpr int kMaxElems = 4096;    // complex elements per CTA tile (upper bound)
-// Tile size per arithmetic type: 8 complex doubles or 16 complex floats per
-// thread keep a stage's butterflies in registers without spilling.
+// 16 complex floats per thread keep a stage's butterflies in registers
+// without spilling.
 template <typename R> struct TileElems;
-template <> struct TileElems<double> { static constexpr int value = 2048; };
 template <> struct TileElems<float> { static constexpr int value = 4096; };
-template <> struct TileElems<df> { static constexpr int value = 2048; };
 constexpr int kMaxStages = 12;
-constexpr int kMaxLen = 2048;     // longest (padded) line; <= TileElems<double>
+constexpr int kMaxLen = 2048;     // longest (padded) line
 
 struct FftLen {
   int L;
   int nstages;
   int radix[kMaxStages];
-  const double2* tw64;  // e^{-2 pi i m / L}, m = 0..L-1
-  const float2* tw32;
-  const cdf* twdf;      // the binary64 table split into double-word
-  const double2* lf64;  // tw64 in multiply-add form (m, t), see lf_cform
+  const float2* tw32;  // e^{-2 pi i m / L}, m = 0..L-1
 };
 
-// Multiply-add form of the twiddle W_j = e^{-2 pi i j / L} = c + i s: with
-// |t| <= 1, W_j = m (1 + i t) (m = c, t = s / c) when |c| >= |s| (the
-// "c-form"), else W_j = m (t + i) (m = s, t = c / s).  The form follows from j
-// alone: |c| >= |s| exactly when q = j mod L/2 lies in [0, L/8] or [3L/8, L/2).
-__host__ __device__ __forceinline__ bool lf_cform(int j, int L) {
-  const int q = j % (L >> 1);
-  return 8 * q <= L || 8 * q >= 3 * L;
-}
-
 template <typename R> __host__ __device__ __forceinline__ const cx<R>* tw_table(const FftLen& f);
-template <> __host__ __device__ __forceinline__ const double2* tw_table<double>(const FftLen& f) { return f.tw64; }
 template <> __host__ __device__ __forceinline__ const float2* tw_table<float>(const FftLen& f) { return f.tw32; }
-template <> __host__ __device__ __forceinline__ const cdf* tw_table<df>(const FftLen& f) { return f.twdf; }
 template <typename R> inline const cx<R>* tw_table_host(const FftLen& f) { return tw_table<R>(f); }
 
 // Exact trigonometric constants of the small DFTs (closed forms in radicals).
@@ -380,6 +349,29 @@ __device__ __forceinline__ void block_reduce_store_f32(float (&acc)[NS], double*
   }
 }
 
+// A line length of the integer passes: its stages with the multiplicative
+// inverses of their divisors, and the stages' twiddles.  Stage s > 0 of radix R
+// after Ns = product of the earlier radices has (R - 1) Ns entries
+// e^{-2 pi i k r / (Ns R)} = (c.h, c.l, s.h, s.l) at w[off[s] + (r - 1) Ns + k]
+// in units 2^(stage_shift(R) - 64): a thread's R - 1 twiddles lie at fixed
+// distances, and those of neighbouring k next to each other.
+struct IntLen {
+  int L, nst, shift;  // shift: the exponent that a transform adds
+  int rad[kMaxStages], off[kMaxStages];
+  unsigned mns[kMaxStages], mnb[kMaxStages];
+  const int4* w;
+};
+
+// Per-axis tables of a plan (binary64, length N_a each): nu_k / N_a,
+// (nu_k^2 / 2) / N_a, nu_k^2 / 2, and half the square of the coordinate
+// -L_a + i h_a.
+struct AxT {
+  const double* nuN;
+  const double* kinN;
+  const double* hnu2;
+  const double* hxc2;
+};
+
 // ---------------------------------------------------------------- plan
 struct Geo {
   int Nx, Ny, Nz, Mx, My, Mz;
@@ -424,19 +416,21 @@ struct atkm_plan {
   double hvol;
   atkm::FftLen fN[3];  // unpadded lengths N_x, N_y, N_z
   atkm::FftLen fM[3];  // padded lengths 2N_x, 2N_y, 2N_z
-  double2* tw64;       // twiddle pool
-  float2* tw32;
-  double2* lf64;       // binary64 twiddles in multiply-add form
+  float2* tw32;        // twiddle pool
+  atkm::IntLen iN[3];  // the same lengths for the integer passes
+  atkm::IntLen iM[3];
+  int4* twi;           // integer twiddle pool
+  const int4* tw_x;    // e^{-2 pi i k / Mx}, k < Nx, in units 2^-61 (the real-data post-twist)
   double* U0;          // octant (Nz+1)(Ny+1)(Nx+1)
   float* U0f;          // FP32 copy of U0 (FP32 workspaces only)
-  double* Kz;          // z-pass multiplier K_sym / (Mx My Mz), [Mz][My][XS] half spectrum
-  double* axtab;       // per-axis tables (AxT): for a = x, y, z five arrays of N_a doubles
+  long long* Kz;       // z-pass multiplier K_sym / (2 Mx My Mz), [Mz][My][XS] half spectrum, integers
+  int k_midbits, k_midshift;  // scale of the z pass around that multiplier (k_multiplier_half)
+  double* axtab;       // per-axis tables (AxT): for a = x, y, z four arrays of N_a doubles
   double* Pw;          // [Nz][Ny][Nx] preconditioner weights, binary64 passes
-  atkm::df* Kzd;       // double-word copy of Kz (ATKM_PLAN_DF32 only)
-  atkm::cdf* twdf;     // double-word twiddle pool
-  double2* W1;         // [Nz][Ny][XS] half spectrum in x
-  double2* W2;         // [Nz][My][XS]
-  double2* T1;         // [Nz][Ny][Nx]
+  atkm::c64* W1;       // [Nz][Ny][XS] half spectrum in x
+  atkm::c64* W2;       // [Nz][My][XS]
+  atkm::c64* T1;       // [Nz][Ny][Nx]
+  int* ex[3];          // tile exponents of the integer arrays
   float2* W1f;
   float2* W2f;
   float2* T1f;
@@ -482,7 +476,7 @@ void prof_set_sink(atkm_plan* p, std::vector<ProfRec>* sink);
 // (call after the replay has completed).
 void prof_accumulate(atkm_plan* p, const std::vector<ProfRec>& recs);
 
-// Launchers (passes.cu).  All enqueue on `st`.
+// Launchers of the FP32 passes (passes_impl.cuh).  All enqueue on `st`.
 enum AtkmSrc { SRC_RHO = 0, SRC_PSI = 1, SRC_PAIR = 2 };
 template <typename R>
 cudaError_t launch_atkm(atkm_plan* p, int mode, const double* a, const double* b, double* phi,
@@ -496,7 +490,17 @@ template <typename R>
 cudaError_t launch_precond(atkm_plan* p, const Phys& ph, const double* alpha_dev, const double* r,
                            const double* phi, const double* Phi, double* Pr, cudaStream_t st);
 
-template <typename R> cudaError_t launch_cfft3(atkm_plan* p, cx<R>* buf, int sign, cudaStream_t st);
+
+// Launchers of the binary64 passes (ipasses_*.cu).  dw: called for the
+// double-word form (the same arithmetic; the profiler's and the tuner's name).
+cudaError_t launch_atkm64(atkm_plan* p, bool dw, int mode, const double* a, const double* b, double* phi,
+                          cudaStream_t st);
+cudaError_t launch_H64(atkm_plan* p, bool dw, const Phys& ph, const double* f, const double* phi, const double* Phi,
+                       double* Hf, int red_slot, cudaStream_t st);
+cudaError_t launch_precond64(atkm_plan* p, const Phys& ph, const double* alpha_dev, const double* r, const double* phi,
+                             const double* Phi, double* Pr, cudaStream_t st);
+// In-place unnormalised 3D complex FFT (sign S) of buf on the plan's grid.
+cudaError_t launch_cfft3(atkm_plan* p, double2* buf, int sign, cudaStream_t st);
 
 // Reductions (pcg.cu)
 cudaError_t launch_finalize(atkm_plan* p, int nslots, int nblocks, int dst_slot, cudaStream_t st);

@@ -1,0 +1,1185 @@
+// The binary64 passes of the spectral operators in 64-bit block floating
+// point (i64.cuh).  As in ops.cuh a pass is an op (load, spectral step, store,
+// fused sums) run by a line-FFT engine, with T adjacent lines per CTA:
+//   * k_ifast: power-of-two lengths 16 ... 1024, 8 elements a thread in
+//     registers, radix-8 stages (plus one radix-2/4 stage) exchanged through
+//     shared memory;
+//   * k_igen: every other {2,3,5}-smooth length up to 2048, radix-8/6/5/4/3/2
+//     stages between two shared-memory tiles.
+// A pass whose input is binary64 finds its tile's largest exponent and turns
+// the elements into integers; between passes the spectra stay integers in the
+// workspaces, each tile with its exponent in a small table, so only the first
+// and the last pass of an operator convert.  Between a forward and an inverse
+// transform the tile is scaled up again to its actual size.
+#pragma once
+
+#include <math.h>
+
+#include <atomic>
+#include <type_traits>
+
+#include "atkm_internal.cuh"
+#include "i64.cuh"
+
+namespace atkm {
+
+__device__ __forceinline__ int ikfreq(int m, int M) { return m < (M >> 1) ? m : m - M; }
+
+// p + i strides, the stride in bytes: one 32 x 32 -> 64 multiply-add
+template <typename T> __device__ __forceinline__ T* step(T* p, int i, int stride) {
+  return (T*)((const char*)p + (long long)i * stride);
+}
+
+// Exponents of an integer array written by one pass: element (row, col) of
+// the array belongs to the tile (row >> rs, col >> cs).
+struct ExpTab {
+  int* e;
+  int rs, cs, nc;
+  __device__ __forceinline__ int at(int row, int col) const { return __ldg(step(e + (col >> cs), row >> rs, nc * 4)); }
+};
+
+constexpr int kInBits = 59;  // components of a transform's input stay below 2^59
+
+enum ISrc { kSrcF64 = 0, kSrcInt = 1 };
+
+template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
+  static constexpr int kSign1 = S1;
+  static constexpr bool kSecond = SECOND;   // inverse transform after the spectral step
+  static constexpr int kRed = NRED;         // fused sums (binary64 per thread)
+  static constexpr bool kLM = LM;           // line-major (x) pass
+  static constexpr int kSrc = SRC;
+  static constexpr bool kMirror = false;    // post-processing needs the frequency L - k
+  static constexpr bool kTwin = false;      // the input is formed from the elements k and L - k
+  static constexpr bool kZeroUpper = false; // positions >= L/2 of the input are zero
+  static constexpr bool kHalfOut = false;   // only positions < L/2 of the output are used
+  static constexpr bool kNyqTail = false;   // column pass over columns 0..Nx (see ipass_line)
+  static constexpr bool kMul = false;       // the spectral step is mul_tile
+  static constexpr int kMinB = 3;           // CTAs per SM that the register engine is compiled for
+  static constexpr bool kPre = false;       // the spectral step's 8-byte table entries are prefetched (op.table)
+  double* part = nullptr;
+  int pstride = 0;
+  // bits the tile is scaled to before the spectral step, and the exponent
+  // that the step adds
+  __device__ __forceinline__ int midbits() const { return 62; }
+  __device__ __forceinline__ int midshift() const { return 0; }
+  struct Acc { int e; };
+  __device__ __forceinline__ c64 spectral(int, int, int, c64 v, Acc&, const long long*) const { return v; }
+  __device__ __forceinline__ double mult(int, int, int) const { return 1.0; }
+};
+
+// ------------------------------------------------------------ geometry
+// The line (o, x) and first position j of a thread: element r of a thread is
+// position j + P r of its line.
+struct Line {
+  int t, j, o, x;
+  bool ok, exit;
+};
+
+template <class Op> __device__ __forceinline__ Line ipass_line(const Op& op, int T, int P) {
+  Line l;
+  l.exit = false;
+  if (Op::kLM) {
+    l.t = threadIdx.x / P;
+    l.j = threadIdx.x - l.t * P;
+    l.o = blockIdx.x * T + l.t;
+    l.x = 0;
+    l.ok = op.valid(l.o, 0);
+    return l;
+  }
+  l.j = threadIdx.x / T;
+  l.t = threadIdx.x - l.j * T;
+  l.o = blockIdx.y;
+  l.x = blockIdx.x * T + l.t;
+  if constexpr (Op::kNyqTail) {
+    // Half-spectrum column passes (columns 0..Nx): when T divides Nx the last
+    // block column would carry column Nx alone; it takes column Nx of T
+    // consecutive rows instead, so that no CTA transforms idle columns.
+    if (blockIdx.x == gridDim.x - 1 && op.Nx % T == 0) {
+      if (blockIdx.y * T >= gridDim.y) {
+        l.exit = true;
+        return l;
+      }
+      l.x = op.Nx;
+      l.o = blockIdx.y * T + l.t;
+      l.ok = l.o < (int)gridDim.y && op.valid(l.o, l.x);
+      return l;
+    }
+  }
+  l.ok = op.valid(l.o, l.x);
+  return l;
+}
+
+// Scratch of the tile-wide reductions, one slot per use so that no barrier is
+// needed between a slot's readers and the next use.
+template <bool TWIN> struct TileRedT {
+  unsigned m[4][8];
+  int nan[128];
+};
+template <> struct TileRedT<true> : TileRedT<false> {
+  c64 last[128];  // element L of each line (load_twin)
+};
+using TileRed = TileRedT<false>;
+
+__device__ __forceinline__ unsigned tile_or(unsigned v, unsigned* slot) {
+  v = __reduce_or_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
+  __syncthreads();
+  const uint4 a = *reinterpret_cast<const uint4*>(slot), b = *reinterpret_cast<const uint4*>(slot + 4);
+  return a.x | a.y | a.z | a.w | b.x | b.y | b.z | b.w;
+}
+
+__device__ __forceinline__ unsigned tile_max(unsigned v, unsigned* slot) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
+  __syncthreads();
+  const uint4 a = *reinterpret_cast<const uint4*>(slot), b = *reinterpret_cast<const uint4*>(slot + 4);
+  return max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
+}
+__device__ __forceinline__ int tile_max_s(int v, unsigned* slot) {
+  return (int)(tile_max((unsigned)v ^ 0x80000000u, slot) ^ 0x80000000u);
+}
+
+__device__ __forceinline__ unsigned dmag(double2 z) {
+  return (unsigned)max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff);
+}
+
+// ------------------------------------------------------------ tile loads
+// State of a tile: its exponent, whether this thread's line holds a NaN or an
+// infinity (its values are then zero here), whether any line of the tile does.
+struct Tile {
+  int e;
+  bool bad, anybad;
+};
+
+// Loads a thread's E elements (guarded by pos < L) as integers of the tile's
+// common exponent, components below 2^59 (2^60 when the first stage sees a
+// zero upper half, unless the post-twist needs the room).
+template <int E, bool FULL, class Op>
+__device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], TileRed& tr) {
+  constexpr int EL = Op::kZeroUpper ? (E + 1) / 2 : E;  // elements that can lie below L/2 (P E >= L)
+  const int lim = Op::kZeroUpper ? L / 2 : L;
+  constexpr int B = (Op::kZeroUpper && !Op::kMirror) ? kInBits + 1 : kInBits;
+  if constexpr (Op::kSrc == kSrcF64) {
+    double2 d[EL];
+    unsigned m = 0;
+#pragma unroll
+    for (int r = 0; r < EL; ++r) {
+      const int pos = l.j + P * r;
+      d[r] = (l.ok && (FULL || pos < lim)) ? op.load(l.o, l.x, pos) : make_double2(0.0, 0.0);
+      m = max(m, dmag(d[r]));
+    }
+    unsigned M = tile_max(m, tr.m[0]);
+    bool bad = false, any = false;
+    if (M >= 0x7ff00000u) {  // a NaN or an infinity: the lines that hold one are left out of the tile's size
+      if (threadIdx.x < 128) tr.nan[threadIdx.x] = 0;
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < EL; ++r) bad |= dmag(d[r]) >= 0x7ff00000u;
+      if (bad) tr.nan[l.t] = 1;
+      __syncthreads();
+      bad = tr.nan[l.t] != 0;
+      any = true;
+      m = 0;
+#pragma unroll
+      for (int r = 0; r < EL; ++r) {
+        if (bad) d[r] = make_double2(0.0, 0.0);
+        m = max(m, dmag(d[r]));
+      }
+      M = tile_max(m, tr.m[1]);
+    }
+    const int ex = max((int)(M >> 20), 64);
+    const int base = 64 - B + ex;
+#pragma unroll
+    for (int r = 0; r < E; ++r) v[r] = r < EL ? c64{d2i(d[r < EL ? r : 0].x, base), d2i(d[r < EL ? r : 0].y, base)} : cz();
+    return Tile{ex - 1023 - (B - 1), bad, any};
+  } else {
+    int ee[EL];
+    int em = -0x40000000;
+#pragma unroll
+    for (int r = 0; r < EL; ++r) {
+      const int pos = l.j + P * r;
+      const bool in = l.ok && (FULL || pos < lim);
+      v[r] = in ? op.load(l.o, l.x, pos) : cz();
+      ee[r] = in ? op.lexp(l.o, l.x, pos) : -0x40000000;
+      em = max(em, ee[r]);
+    }
+    em = tile_max_s(em, tr.m[0]);
+    if (em >= kExpNaN / 2) {  // uniform in the CTA
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[r] = cz();
+      return Tile{kExpNaN, true, true};
+    }
+    unsigned m = 0;
+#pragma unroll
+    for (int r = 0; r < EL; ++r) {
+      const int d = min(em - ee[r], 64);
+      v[r].x = shr_clamp(v[r].x, d);
+      v[r].y = shr_clamp(v[r].y, d);
+      m |= mag(v[r]);
+    }
+    const int sh = B - mag_bits(tile_or(m, tr.m[1]));
+#pragma unroll
+    for (int r = 0; r < E; ++r) v[r] = r < EL ? cshift(v[r], sh) : cz();
+    return Tile{em - sh, false, false};
+  }
+}
+
+// The same for an op that forms its input from the elements k and L - k of
+// the stored half spectrum (op.combine): loads the elements, and element L
+// into *last for the threads of position 0, scaled to 60 bits.
+template <int E, bool FULL, class Op>
+__device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, int L, c64 (&v)[E], c64* last, TileRed& tr) {
+  int ev[E], el = -0x40000000;
+  *last = cz();
+  if (l.ok && l.j == 0) {
+    *last = op.load(l.o, L);
+    el = op.lexp(l.o, L);
+  }
+  int em = el;
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const int pos = l.j + P * r;
+    const bool in = l.ok && (FULL || pos < L);
+    v[r] = in ? op.load(l.o, pos) : cz();
+    ev[r] = in ? op.lexp(l.o, pos) : -0x40000000;
+    em = max(em, ev[r]);
+  }
+  em = tile_max_s(em, tr.m[0]);
+  if (em >= kExpNaN / 2) {
+#pragma unroll
+    for (int r = 0; r < E; ++r) v[r] = cz();
+    *last = cz();
+    return Tile{kExpNaN, true, true};
+  }
+  const int dl = min(em - el, 64);
+  *last = c64{shr_clamp(last->x, dl), shr_clamp(last->y, dl)};
+  unsigned m = mag(*last);
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const int d = min(em - ev[r], 64);
+    v[r] = c64{shr_clamp(v[r].x, d), shr_clamp(v[r].y, d)};
+    m |= mag(v[r]);
+  }
+  const int sh = 60 - mag_bits(tile_or(m, tr.m[1]));
+  *last = cshift(*last, sh);
+#pragma unroll
+  for (int r = 0; r < E; ++r) v[r] = cshift(v[r], sh);
+  return Tile{em - sh + 3, false, false};  // combine() divides by 8
+}
+
+// Scales the tile up to BITS = op.midbits() bits and applies the op's
+// spectral step to every element.
+template <int E, bool FULL, class Op>
+__device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], int* e,
+                                         typename Op::Acc& acc, unsigned* slot, const long long* pre) {
+  unsigned m = 0;
+#pragma unroll
+  for (int r = 0; r < E; ++r) m |= mag(v[r]);
+  const int sh = op.midbits() - mag_bits(tile_or(m, slot));
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const int pos = l.j + P * r;
+    if (l.ok && (FULL || pos < L)) v[r] = op.spectral(l.o, l.x, pos, cshift(v[r], sh), acc, FULL && Op::kPre ? pre + r * kThreads : nullptr);
+  }
+  *e -= sh;
+  acc.e = *e;
+  *e += op.midshift();
+}
+
+// The same for an op with real binary64 multipliers of any size
+// (op.mult(o, x, k), kMul): an element times the 53-bit mantissa of its
+// multiplier keeps the element's bits, and the products are then aligned to
+// the tile's largest one.  (With the multiplier in fixed point, nu^2 / 2 of
+// the low frequencies, 2^-18 of the largest at length 1024, would leave the
+// product 2^18 fewer units.)
+template <int E, bool FULL, class Op>
+__device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], Tile& tl,
+                                         typename Op::Acc& acc, TileRed& tr) {
+  unsigned m = 0;
+#pragma unroll
+  for (int r = 0; r < E; ++r) m |= mag(v[r]);
+  const int sh = 62 - mag_bits(tile_or(m, tr.m[2]));
+  acc.e = tl.e - sh;
+  int ex[E];
+  int eb = -0x40000000;
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const int pos = l.j + P * r;
+    ex[r] = 0;
+    if (l.ok && (FULL || pos < L)) {
+      const c64 u = cshift(v[r], sh);
+      const Limbs x = limbs(u.x), y = limbs(u.y);
+      op.tally(l.o, l.x, pos, x, y, acc);
+      const double d = op.mult(l.o, l.x, pos);
+      const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
+      ex[r] = (int)((dh >> 20) & 0x7ffu);
+      const long long mt = (long long)(((unsigned long long)((dh & 0xfffffu) | 0x100000u) << 32 | dl) << 9);  // [2^61, 2^62)
+      const Limbs w = limbs((int)dh < 0 ? -mt : mt);
+      v[r] = c64{mul64(x, w), mul64(y, w)};
+      eb = max(eb, 32 - __clz((int)mag(v[r])) + ex[r]);  // bits of the aligned product, less 32
+    }
+  }
+  const int M = tile_max_s(eb, tr.m[3]);
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const int s = kInBits - 32 - M + ex[r], lf = max(s, 0), rt = min(max(-s, 0), 64);
+    v[r].x = shr_clamp((long long)((unsigned long long)v[r].x << lf), rt);
+    v[r].y = shr_clamp((long long)((unsigned long long)v[r].y << lf), rt);
+  }
+  // an element of multiplier 2^(ex - 1023) f, f in [1, 2), held v f 2^61 / 2^64
+  tl.e += M - sh + 64 - 1084 - (kInBits - 32);
+  if (M >= 2040) {  // an infinite or NaN multiplier
+    tl.e = kExpNaN;
+    tl.bad = tl.anybad = true;
+  }
+}
+
+template <int NR> __device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* part, int pstride) {
+  block_reduce_store<NR>(acc, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
+}
+
+// ------------------------------------------------------------ k_ifast
+constexpr int kIElems = 2048;  // elements per CTA (256 threads x 8)
+
+template <int L> struct IFast {
+  static constexpr int TPL = L / 8;
+  static constexpr int T = kIElems / L;
+  static constexpr int A = (L >= 512) ? 3 : (L >= 64 ? 2 : 1);  // radix-8 stages
+  static constexpr int REM = L / (A == 3 ? 512 : (A == 2 ? 64 : 8));
+  static constexpr int SHIFT = 3 * (A - 1) + (REM > 1 ? 2 : 0);  // exponent gained by a transform
+  // Shared-memory index of element (t, pos): line-major tiles with one pad
+  // element every 8 positions, column tiles [pos][t] with a pad row every 8
+  // positions where a row is less than 128 bytes.  Both keep the 16-byte
+  // accesses of a quarter warp in distinct banks, and both are affine in the
+  // stage's inner index, so that an exchange computes two addresses.
+  template <bool LM> static constexpr bool kPad = LM || T < 8;
+  template <bool LM> static constexpr int kRow = LM ? 1 : T;  // index step of one position
+  template <bool LM> __device__ static __forceinline__ int at(int t, int pos) {
+    if (LM) return t * (L + L / 8) + pos + (pos >> 3);
+    return (kPad<LM> ? pos + (pos >> 3) : pos) * T + t;
+  }
+  // index step of n positions, n a multiple of 8 (or less than 8 within an aligned 8)
+  template <bool LM> static constexpr int span(int n) { return (kPad<LM> ? n + n / 8 : n) * kRow<LM>; }
+  template <bool LM> static constexpr size_t bytes() {
+    return (size_t)(kPad<LM> ? kIElems + kIElems / 8 : kIElems) * sizeof(c64);
+  }
+};
+
+// Transforms the register elements v[r] = line[j + TPL r] in place; on return
+// v[r] holds frequency j + TPL r.  The caller's last barrier frees b.  One
+// buffer and two barriers an exchange: with two buffers a CTA more per SM
+// would not fit.
+template <int L, int S, bool LM, bool ZU, bool LO>
+__device__ __forceinline__ void ifast_fft(c64 (&v)[8], c64* b, const int4* __restrict__ w, int t, int j) {
+  using C = IFast<L>;
+  int Ns = 1;
+#pragma unroll
+  for (int s = 0; s < C::A; ++s) {
+    const int k = j & (Ns - 1);
+    const bool last = (s == C::A - 1) && (C::REM == 1);
+    if (s > 0) {
+      const int4* wk = w + (s == 2 ? 56 : 0) + k;  // the tables of the stages before: 7 Ns entries each
+      v[0] = crsh<3>(v[0]);
+#pragma unroll
+      for (int r = 1; r < 8; ++r) v[r] = tmul<S>(v[r], __ldg(wk + (r - 1) * Ns));
+    }
+    if (ZU && s == 0) IDft<8, S>::template go<true, false>(v);
+    else if (LO && last) IDft<8, S>::template go<false, true>(v);
+    else IDft<8, S>::template go<false, false>(v);
+    if (!last) {
+      if (s > 0) __syncthreads();
+      c64* p = b + C::template at<LM>(t, (j - k) * 8 + k);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) p[C::template span<LM>(r * Ns)] = v[r];
+      __syncthreads();
+      if constexpr (C::TPL >= 8) {
+        const c64* q = b + C::template at<LM>(t, j);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = q[C::template span<LM>(C::TPL * r)];
+      } else {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = b[C::template at<LM>(t, j + C::TPL * r)];
+      }
+    }
+    Ns *= 8;
+  }
+  if constexpr (C::REM > 1) {
+    constexpr int Q = C::REM, M = 8 / C::REM, NsQ = L / Q;
+    const int4* wk = w + (C::A == 3 ? 504 : (C::A == 2 ? 56 : 0)) + j;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      c64 u[Q];
+      u[0] = crsh<2>(v[m]);
+#pragma unroll
+      for (int q = 1; q < Q; ++q) u[q] = tmul<S>(v[m + M * q], __ldg(wk + (q - 1) * NsQ + C::TPL * m));
+      IDft<Q, S>::template go<false, LO>(u);
+#pragma unroll
+      for (int q = 0; q < (LO ? Q / 2 : Q); ++q) v[m + M * q] = u[q];
+    }
+  }
+}
+
+__device__ __forceinline__ void icp_async8(void* smem_dst, const void* gsrc) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gsrc) : "memory");
+}
+
+template <int L, class Op>
+__global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4* __restrict__ w) {
+  using C = IFast<L>;
+  extern __shared__ __align__(16) unsigned char ism[];
+  __shared__ __align__(16) TileRedT<Op::kTwin> tr;
+  c64* b0 = reinterpret_cast<c64*>(ism);
+  // [r][thread]: this thread's table entries
+  long long* pre = reinterpret_cast<long long*>(ism + C::template bytes<Op::kLM>()) + threadIdx.x;
+  const Line l = ipass_line(op, C::T, C::TPL);
+  if (l.exit) return;  // the whole CTA
+  if constexpr (Op::kPre) {
+    if (l.ok) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) icp_async8(pre + r * kThreads, op.table(l.o, l.x, l.j + C::TPL * r));
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  c64 v[8];
+  Tile tl;
+  if constexpr (Op::kTwin) {
+    c64 last;
+    tl = load_twin<8, true>(op, l, C::TPL, L, v, &last, tr);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) b0[C::template at<Op::kLM>(l.t, l.j + C::TPL * r)] = v[r];
+    if (l.j == 0) tr.last[l.t] = last;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int pos = l.j + C::TPL * r;
+      v[r] = op.combine(pos, v[r], pos == 0 ? tr.last[l.t] : b0[C::template at<Op::kLM>(l.t, L - pos)]);
+    }
+    __syncthreads();
+  } else {
+    tl = load_tile<8, true>(op, l, C::TPL, L, v, tr);
+  }
+  typename Op::Acc acc{};
+  constexpr bool kLo1 = Op::kHalfOut && !Op::kSecond && !Op::kMirror;
+  ifast_fft<L, Op::kSign1, Op::kLM, Op::kZeroUpper, kLo1>(v, b0, w, l.t, l.j);
+  tl.e += C::SHIFT;
+  if constexpr (Op::kMirror) {
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 8; ++r) b0[C::template at<Op::kLM>(l.t, l.j + C::TPL * r)] = v[r];
+    __syncthreads();
+    if (l.ok) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int k = l.j + C::TPL * r;
+        op.post(l.o, k, v[r], b0[C::template at<Op::kLM>(l.t, (L - k) & (L - 1))]);
+      }
+    }
+  } else {
+    if constexpr (Op::kSecond) {
+      if constexpr (Op::kPre) asm volatile("cp.async.wait_all;\n" ::: "memory");
+      // its barrier also frees b0
+      if constexpr (Op::kMul) mul_tile<8, true>(op, l, C::TPL, L, v, tl, acc, tr);
+      else mid_tile<8, true>(op, l, C::TPL, L, v, &tl.e, acc, tr.m[2], pre);
+      ifast_fft<L, -Op::kSign1, Op::kLM, false, Op::kHalfOut>(v, b0, w, l.t, l.j);
+      tl.e += C::SHIFT;
+    }
+    if (l.ok) {
+#pragma unroll
+      for (int r = 0; r < (Op::kHalfOut ? 4 : 8); ++r) op.store(l.o, l.x, l.j + C::TPL * r, v[r], tl, acc);
+    }
+  }
+  op.put_exp(l, tl);
+  if constexpr (Op::kRed > 0) {
+    double a[Op::kRed];
+    op.sums(l, acc, tl, a);
+    ireduce_out<Op::kRed>(a, op.part, op.pstride);
+  }
+}
+
+// ------------------------------------------------------------ k_igen
+constexpr int kGenMax = 2560;  // elements per CTA at most (256 threads x 10)
+constexpr int kGenE = 10;
+
+__device__ __forceinline__ int fdiv(int n, unsigned magic, int d) { return d == 1 ? n : (int)__umulhi((unsigned)n, magic); }
+
+// Shared-memory index of element (t, pos): as in IFast, one pad element (a pad
+// row where a row is less than 128 bytes) every 8 positions.
+struct GenTile {
+  int T, tsh, ps, LP;
+  __device__ __forceinline__ GenTile(int T, int tsh, int L) : T(T), tsh(tsh), ps(tsh < 3 ? 3 : 31), LP(L + L / 8 + 1) {}
+  template <bool LM> __device__ __forceinline__ int at(int t, int pos) const {
+    return LM ? t * LP + pos + (pos >> 3) : ((pos + (pos >> ps)) << tsh) + t;
+  }
+};
+
+template <int RAD, int S, bool LM>
+__device__ __forceinline__ void igen_stage(const c64* __restrict__ src, c64* __restrict__ dst, const IntLen& f, int st,
+                                           int Ns, const GenTile& g) {
+  const int L = f.L, nb = L / RAD, total = nb * g.T;
+  const int4* __restrict__ w = f.w + f.off[st];
+  for (int b = threadIdx.x; b < total; b += kThreads) {
+    int t, j;
+    if (LM) {
+      t = fdiv(b, f.mnb[st], nb);
+      j = b - t * nb;
+    } else {
+      j = b >> g.tsh;
+      t = b - (j << g.tsh);
+    }
+    const int k = j - fdiv(j, f.mns[st], Ns) * Ns;
+    c64 v[RAD];
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) v[r] = src[g.template at<LM>(t, j + r * nb)];
+    if (Ns > 1) {
+      v[0] = crsh<stage_shift(RAD)>(v[0]);
+#pragma unroll
+      for (int r = 1; r < RAD; ++r) v[r] = tmul<S>(v[r], __ldg(w + k + (r - 1) * Ns));
+    }
+    IDft<RAD, S>::template go<false, false>(v);
+    const int base = (j - k) * RAD + k;
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) dst[g.template at<LM>(t, base + r * Ns)] = v[r];
+  }
+  __syncthreads();
+}
+
+// Transforms the tile in *a (filled, synchronised) through *b; the result is
+// in *a on return.
+template <int S, bool LM>
+__device__ __forceinline__ void igen_fft(c64** a, c64** b, const IntLen& f, const GenTile& g) {
+  int Ns = 1;
+  for (int s = 0; s < f.nst; ++s) {
+    const int rad = f.rad[s];
+    switch (rad) {
+      case 8: igen_stage<8, S, LM>(*a, *b, f, s, Ns, g); break;
+      case 6: igen_stage<6, S, LM>(*a, *b, f, s, Ns, g); break;
+      case 5: igen_stage<5, S, LM>(*a, *b, f, s, Ns, g); break;
+      case 4: igen_stage<4, S, LM>(*a, *b, f, s, Ns, g); break;
+      case 3: igen_stage<3, S, LM>(*a, *b, f, s, Ns, g); break;
+      default: igen_stage<2, S, LM>(*a, *b, f, s, Ns, g); break;
+    }
+    Ns *= rad;
+    c64* x = *a;
+    *a = *b;
+    *b = x;
+  }
+}
+
+template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op, IntLen f, int T, int tsh) {
+  extern __shared__ __align__(16) unsigned char ism[];
+  __shared__ __align__(16) TileRedT<Op::kTwin> tr;
+  const int L = f.L, P = kThreads >> tsh;
+  c64* a = reinterpret_cast<c64*>(ism);
+  const GenTile g(T, tsh, L);
+  c64* b = a + T * g.LP;
+  const Line l = ipass_line(op, T, P);
+  if (l.exit) return;  // the whole CTA
+  c64 v[kGenE];
+  Tile tl;
+  if constexpr (Op::kTwin) {
+    c64 last;
+    tl = load_twin<kGenE, false>(op, l, P, L, v, &last, tr);
+#pragma unroll
+    for (int r = 0; r < kGenE; ++r) {
+      const int pos = l.j + P * r;
+      if (pos < L) b[g.template at<Op::kLM>(l.t, pos)] = v[r];
+    }
+    if (l.j == 0) tr.last[l.t] = last;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kGenE; ++r) {
+      const int pos = l.j + P * r;
+      if (pos < L) v[r] = op.combine(pos, v[r], pos == 0 ? tr.last[l.t] : b[g.template at<Op::kLM>(l.t, L - pos)]);
+    }
+  } else {
+    tl = load_tile<kGenE, false>(op, l, P, L, v, tr);
+  }
+  typename Op::Acc acc{};
+#pragma unroll
+  for (int r = 0; r < kGenE; ++r) {
+    const int pos = l.j + P * r;
+    if (pos < L) a[g.template at<Op::kLM>(l.t, pos)] = v[r];
+  }
+  __syncthreads();
+  igen_fft<Op::kSign1, Op::kLM>(&a, &b, f, g);
+  tl.e += f.shift;
+  if constexpr (Op::kMirror) {
+    if (l.ok) {
+      for (int pos = l.j; pos < L; pos += P)
+        op.post(l.o, pos, a[g.template at<true>(l.t, pos)], a[g.template at<true>(l.t, pos == 0 ? 0 : L - pos)]);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < kGenE; ++r) {
+      const int pos = l.j + P * r;
+      v[r] = pos < L ? a[g.template at<Op::kLM>(l.t, pos)] : cz();
+    }
+    if constexpr (Op::kSecond) {
+      // its barrier also frees the tile
+      if constexpr (Op::kMul) mul_tile<kGenE, false>(op, l, P, L, v, tl, acc, tr);
+      else mid_tile<kGenE, false>(op, l, P, L, v, &tl.e, acc, tr.m[2], nullptr);
+#pragma unroll
+      for (int r = 0; r < kGenE; ++r) {
+        const int pos = l.j + P * r;
+        if (pos < L) a[g.template at<Op::kLM>(l.t, pos)] = v[r];
+      }
+      __syncthreads();
+      igen_fft<-Op::kSign1, Op::kLM>(&a, &b, f, g);
+      tl.e += f.shift;
+#pragma unroll
+      for (int r = 0; r < kGenE; ++r) {
+        const int pos = l.j + P * r;
+        v[r] = pos < L ? a[g.template at<Op::kLM>(l.t, pos)] : cz();
+      }
+    }
+    if (l.ok) {
+#pragma unroll
+      for (int r = 0; r < (Op::kHalfOut ? kGenE / 2 : kGenE); ++r) {
+        const int pos = l.j + P * r;
+        if (pos < (Op::kHalfOut ? L / 2 : L)) op.store(l.o, l.x, pos, v[r], tl, acc);
+      }
+    }
+  }
+  op.put_exp(l, tl);
+  if constexpr (Op::kRed > 0) {
+    double s[Op::kRed];
+    op.sums(l, acc, tl, s);
+    ireduce_out<Op::kRed>(s, op.part, op.pstride);
+  }
+}
+
+// ------------------------------------------------------------ dispatch
+struct IPassGrid {
+  dim3 grid;
+  int T, tsh;
+  bool fast;
+};
+
+inline int ilog2(int v) {
+  int s = 0;
+  while ((1 << (s + 1)) <= v) ++s;
+  return s;
+}
+
+// LM passes: `lines` lines; column passes: X columns x `outer` outer indices.
+// The tiles of the generic engine are powers of two, narrowed until the pass
+// has two CTAs per SM (a column tile not below 8, which keeps its accesses in
+// whole 128-byte lines).
+inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long lines, int X, int outer) {
+  IPassGrid pg;
+  pg.fast = L >= 16 && L <= 1024 && (L & (L - 1)) == 0;
+  if (pg.fast) {
+    pg.T = kIElems / L;
+  } else {
+    int T = 1 << ilog2(std::min(128, std::max(1, kGenMax / L)));
+    const long want = 2L * device_sm_count();
+    if (LM) {
+      while (T > 1 && (lines + T - 1) / T < want) T >>= 1;
+    } else {
+      while (T > 1 && T / 2 >= X) T >>= 1;
+      while (T > 8 && (long)((X + T - 1) / T) * outer < want) T >>= 1;
+    }
+    for (int i = 0; i < p->n_tune; ++i)
+      if (p->tune[i].r == r && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0)) T = std::max(T >> p->tune[i].shift, 1);
+    pg.T = T;
+  }
+  pg.tsh = ilog2(pg.T);
+  pg.grid = LM ? dim3((unsigned)((lines + pg.T - 1) / pg.T), 1, 1) : dim3((X + pg.T - 1) / pg.T, outer, 1);
+  return pg;
+}
+
+// Dynamic shared memory above the default is opted into once per kernel and
+// device; `done` holds one bit per device already prepared.
+template <typename K>
+inline cudaError_t iprepare(std::atomic<unsigned long long>& done, K kernel, size_t bytes) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
+  return e;
+}
+
+template <int L, class Op>
+inline cudaError_t launch_ifast(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
+  static std::atomic<unsigned long long> prepared{0};
+  constexpr size_t sm = IFast<L>::template bytes<Op::kLM>() + (Op::kPre ? (size_t)8 * 8 * kThreads : 0);
+  cudaError_t e = iprepare(prepared, k_ifast<L, Op>, sm);
+  if (e != cudaSuccess) return e;
+  k_ifast<L, Op><<<pg.grid, kThreads, sm, st>>>(op, f.w);
+  return cudaGetLastError();
+}
+
+template <class Op> inline cudaError_t irun(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
+  if (pg.fast) {
+    switch (f.L) {
+      case 16: return launch_ifast<16>(op, f, pg, st);
+      case 32: return launch_ifast<32>(op, f, pg, st);
+      case 64: return launch_ifast<64>(op, f, pg, st);
+      case 128: return launch_ifast<128>(op, f, pg, st);
+      case 256: return launch_ifast<256>(op, f, pg, st);
+      case 512: return launch_ifast<512>(op, f, pg, st);
+      case 1024: return launch_ifast<1024>(op, f, pg, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  static std::atomic<unsigned long long> prepared{0};
+  // T (L + L / 8 + 1) elements a buffer, T L <= kGenMax, T <= 128
+  constexpr size_t most = (size_t)2 * (kGenMax + kGenMax / 8 + 128) * sizeof(c64);
+  cudaError_t e = iprepare(prepared, k_igen<Op>, most);
+  if (e != cudaSuccess) return e;
+  k_igen<Op><<<pg.grid, kThreads, (size_t)2 * pg.T * (f.L + f.L / 8 + 1) * sizeof(c64), st>>>(op, f, pg.T, pg.tsh);
+  return cudaGetLastError();
+}
+
+// ================================================================ ops
+// Writes the tile's exponent (every line of the tile writes the same value).
+__device__ __forceinline__ void put_exp_at(const ExpTab& x, int row, int col, const Line& l, int e) {
+  if (l.j == 0 && l.ok) x.e[(row >> x.rs) * x.nc + (col >> x.cs)] = e;
+}
+
+__device__ __forceinline__ c64 ldc(const c64* p) {
+  const longlong2 t = *reinterpret_cast<const longlong2*>(p);
+  return c64{t.x, t.y};
+}
+__device__ __forceinline__ void stc(c64* p, c64 v) { *reinterpret_cast<longlong2*>(p) = make_longlong2(v.x, v.y); }
+
+// ---- ATKM (twofold-padded grid, real-data form).  The density is real, so
+// the x transform of each padded line (length Mx = 2 Nx, upper half zero) is
+// a complex FFT of length Nx of z_m = rho_{2m} + i rho_{2m+1} with the exact
+// post-twist X_k = (Z_k + conj Z_{Nx-k})/2 - (i/2) e^{-2 pi i k/Mx}
+// (Z_k - conj Z_{Nx-k}), k = 0..Nx (Hermitian symmetry gives the rest); the y
+// and z passes then run on the Nx + 1 half-spectrum columns only, and the
+// inverse x transform rebuilds the real output from that half.  With a real
+// density this equals the real part of the full complex convolution once K is
+// symmetrised on the padded Nyquist planes (k_multiplier_half).  W1:
+// [Nz][Ny][XS], W2: [Nz][My][XS], columns 0..Nx used; W1 and W2 hold 2 X
+// (the post-twist's 1/2 sits in the z pass's exponent).
+template <int MODE> struct IAtkmXF : IOpBase<-1, false, 0, true, kSrcF64> {
+  static constexpr bool kMirror = true;
+  static constexpr bool kZeroUpper = true;
+  const double* a;
+  const double* b;
+  c64* W1;
+  const int4* wM;
+  ExpTab ex;
+  int Nx, nl, XS;
+  __device__ __forceinline__ double dens(size_t i) const {
+    if (MODE == SRC_RHO) return a[i];
+    const double2 u = reinterpret_cast<const double2*>(a)[i];
+    const double2 w = MODE == SRC_PSI ? u : reinterpret_cast<const double2*>(b)[i];
+    return u.x * w.x + u.y * w.y;
+  }
+  __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
+  __device__ __forceinline__ double2 load(int o, int, int m) const {  // m < Nx / 2
+    const size_t i = (size_t)o * Nx + 2 * m;
+    return make_double2(dens(i), dens(i + 1));
+  }
+  // 2 X_k / 8 = (Z_k + conj Z_{Nx-k}) / 8 - i w (Z_k - conj Z_{Nx-k}) / 8.
+  // With the zero upper half the moduli stay below 2^61.5 here, so the sums fit.
+  __device__ __forceinline__ void post(int o, int k, c64 z, c64 m) const {
+    const c64 s = crsh<3>(c64{z.x + m.x, z.y - m.y});
+    const c64 d = tmul<-1>(c64{z.x - m.x, z.y + m.y}, __ldg(wM + k));
+    stc(W1 + (size_t)o * XS + k, c64{s.x + d.y, s.y - d.x});
+    if (k == 0) stc(W1 + (size_t)o * XS + Nx, c64{rsh<2>(z.x - z.y), 0});
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const {
+    put_exp_at(ex, l.o, 0, l, t.anybad ? kExpNaN : t.e + 3);
+  }
+};
+
+// y forward: o = z, x = kx in [0, Nx]; rows y < Ny of W1, zero beyond.
+struct IAtkmYF : IOpBase<-1, false, 0, false, kSrcInt> {
+  static constexpr bool kZeroUpper = true;
+  static constexpr bool kNyqTail = true;
+  const c64* W1;
+  c64* W2;
+  ExpTab in, ex;
+  int Nx, Ny, My, XS;
+  __device__ __forceinline__ bool valid(int, int x) const { return x <= Nx; }
+  __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(W1 + (size_t)o * Ny * XS + x, pos, XS * 16)); }
+  __device__ __forceinline__ int lexp(int o, int x, int pos) const { return in.at(o * Ny + pos, x); }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
+    stc(step(W2 + (size_t)o * My * XS + x, pos, XS * 16), v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, l.x, l, t.e); }
+};
+
+// z forward * K_sym * inverse: o = ky, x = kx in [0, Nx]; rows z < Nz.  The
+// multiplier is the plan's integer table in the layout of W2 (k_multiplier_half).
+struct IAtkmZ : IOpBase<-1, true, 0, false, kSrcInt> {
+  static constexpr bool kZeroUpper = true;
+  static constexpr bool kHalfOut = true;
+  static constexpr bool kNyqTail = true;
+  c64* W2;
+  const long long* K;
+  ExpTab in, ex;
+  int Nx, Nz, My, XS, mb, ms;
+  __device__ __forceinline__ int midbits() const { return mb; }
+  __device__ __forceinline__ int midshift() const { return ms; }
+  __device__ __forceinline__ bool valid(int, int x) const { return x <= Nx; }
+  __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(W2 + (size_t)o * XS + x, pos, My * XS * 16)); }
+  __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
+  static constexpr bool kPre = true;
+  __device__ __forceinline__ const long long* table(int o, int x, int k) const {
+    return step(K + (size_t)o * XS + x, k, My * XS * 8);
+  }
+  // pre: the prefetched entry (null in the generic engine)
+  __device__ __forceinline__ c64 spectral(int o, int x, int k, c64 v, Acc&, const long long* pre) const {
+    const Limbs m = limbs(pre ? *pre : __ldg(table(o, x, k)));
+    return c64{mul64(limbs(v.x), m), mul64(limbs(v.y), m)};
+  }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
+    stc(step(W2 + (size_t)o * XS + x, pos, My * XS * 16), v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, l.x, l, t.e); }
+};
+
+// y inverse: o = z, x = kx in [0, Nx]; output rows y < Ny into W1.
+struct IAtkmYI : IOpBase<1, false, 0, false, kSrcInt> {
+  static constexpr bool kHalfOut = true;
+  static constexpr bool kNyqTail = true;
+  const c64* W2;
+  c64* W1;
+  ExpTab in, ex;
+  int Nx, Ny, My, XS;
+  __device__ __forceinline__ bool valid(int, int x) const { return x <= Nx; }
+  __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(W2 + (size_t)o * My * XS + x, pos, XS * 16)); }
+  __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
+    stc(step(W1 + (size_t)o * Ny * XS + x, pos, XS * 16), v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, l.x, l, t.e); }
+};
+
+// x inverse: Z_k = (X_k + conj X_{Nx-k}) + i e^{2 pi i k/Mx} (X_k - conj
+// X_{Nx-k}), k < Nx, then an inverse FFT of length Nx gives z_m = Phi_{2m} +
+// i Phi_{2m+1}; kept for 2m < Nx (the crop).
+struct IAtkmXI : IOpBase<1, false, 0, true, kSrcInt> {
+  static constexpr bool kTwin = true;
+  static constexpr bool kHalfOut = true;
+  const c64* W1;
+  double* phi;
+  const int4* wM;
+  ExpTab in;
+  int Nx, Ny, nl, XS;
+  __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
+  __device__ __forceinline__ c64 load(int o, int k) const { return ldc(W1 + (size_t)o * XS + k); }
+  __device__ __forceinline__ int lexp(int o, int k) const { return in.at(o / Ny, k); }
+  __device__ __forceinline__ c64 combine(int k, c64 a, c64 b) const {  // Z_k / 8
+    const c64 s = crsh<3>(c64{a.x + b.x, a.y - b.y});
+    const c64 d = tmul<1>(c64{a.x - b.x, a.y + b.y}, __ldg(wM + k));
+    return c64{s.x - d.y, s.y + d.x};
+  }
+  __device__ __forceinline__ void store(int o, int, int m, c64 v, const Tile& t, Acc&) const {
+    double2 d;
+    if (i2d_ok(t.e)) d = make_double2(i2d(v.x, t.e + 1085), i2d(v.y, t.e + 1085));
+    else d = make_double2(i2d_any(v.x, t.e), i2d_any(v.y, t.e));
+    *reinterpret_cast<double2*>(phi + (size_t)o * Nx + 2 * m) = d;
+  }
+  __device__ __forceinline__ void put_exp(const Line&, const Tile&) const {}
+};
+
+// ---- H_phi f (unpadded grid).  A line's multiplier is (nu_k^2 / 2 + c nu_k) / N
+// with c = Omega y on x lines, -Omega x on y lines, from the axis's tables.
+// Sums of k^2 |v|^2 and k |v|^2 over a thread's elements, exact but for the
+// last step: |v|^2 / 2^64 = A + F 2^-31 (v below 2^62 a component; the 31
+// fraction bits matter because k^2 reaches 2^18 where |v|^2 is small), each
+// of A's two limbs and F multiplied by the integer k or k^2 and summed in 64
+// bits.
+struct KinAcc {
+  int e;  // exponent of v
+  long long h2, l2, f2, h1, l1, f1;
+  __device__ __forceinline__ void add(int k, Limbs x, Limbs y) {
+    const unsigned long long ll = (unsigned long long)mulw(x.l, x.l) + (unsigned long long)mulw(y.l, y.l);
+    const long long t = mulw(x.h, x.l) + mulw(y.h, y.l) + (long long)((unsigned)(ll >> 32) >> 1);
+    const Limbs a = limbs((t >> 31) + mulw(x.h, x.h) + mulw(y.h, y.h));
+    const int f = (int)t & 0x7fffffff, kk = k * k;
+    h2 += mulw(kk, a.h);
+    l2 += mulw(kk, a.l);
+    f2 += mulw(kk, f);
+    h1 += mulw(k, a.h);
+    l1 += mulw(k, a.l);
+    f1 += mulw(k, f);
+  }
+  // the sums of k^2 |v|^2 and k |v|^2 in binary64
+  __device__ __forceinline__ double2 get() const {
+    const double s = pow2d(2 * e + 64), q = 4.656612873077392578125e-10;  // 2^-31
+    return make_double2((fma((double)h2, 4294967296.0, (double)l2) + (double)f2 * q) * s,
+                        (fma((double)h1, 4294967296.0, (double)l1) + (double)f1 * q) * s);
+  }
+};
+
+// Marks an element of a line that holds a NaN or an infinity.
+constexpr long long kBadElem = (long long)0x8000000000000000ull;
+
+template <bool RED> struct IHX : IOpBase<-1, true, RED ? 2 : 0, true, kSrcF64> {
+  const double2* f;
+  c64* A;
+  ExpTab ex;
+  const double* kin;  // (nu_k^2 / 2) / N
+  const double* nu;   // nu_k / N
+  int Nx, Ny, nl;
+  double Om, Ly, hy;
+  double ck, cr;       // nu^2 / (2 N) = ck k'^2, Omega nu / N = cr k', k' the signed index
+  static constexpr bool kMul = true;
+  struct Acc : KinAcc {};
+  static constexpr int kMinB = 2;
+  __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
+  __device__ __forceinline__ double yc(int o) const { return -Ly + (double)(o % Ny) * hy; }
+  __device__ __forceinline__ double2 load(int o, int, int pos) const { return f[(size_t)o * Nx + pos]; }
+  __device__ __forceinline__ void tally(int, int, int k, Limbs x, Limbs y, Acc& a) const {
+    if (RED) a.add(ikfreq(k, Nx), x, y);
+  }
+  __device__ __forceinline__ double mult(int o, int, int k) const {
+    return fma(Om * yc(o), __ldg(nu + k), __ldg(kin + k));
+  }
+  __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile& t, Acc&) const {
+    if (t.bad) v.x = kBadElem;
+    stc(A + (size_t)o * Nx + pos, v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, 0, l, t.e); }
+  __device__ __forceinline__ void sums(const Line& l, const Acc& a, const Tile& t, double* s) const {
+    const double2 k = a.get();
+    s[0] = l.ok ? ck * k.x : 0.0;
+    s[1] = l.ok ? cr * yc(l.o) * k.y : 0.0;
+    if (t.bad) s[0] = s[1] = __longlong_as_double(0x7ff8000000000000ll);
+  }
+};
+
+template <bool RED> struct IHY : IOpBase<-1, true, RED ? 2 : 0, false, kSrcF64> {
+  const double2* f;
+  c64* A;
+  ExpTab ex;
+  const double* kin;
+  const double* nu;
+  int Nx, Ny;
+  double Om, Lx, hx;
+  double ck, cr;
+  static constexpr bool kMul = true;
+  struct Acc : KinAcc {};
+  static constexpr int kMinB = 2;
+  __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
+  __device__ __forceinline__ double xc(int x) const { return -Lx + (double)x * hx; }
+  __device__ __forceinline__ double2 load(int o, int x, int pos) const { return *step(f + (size_t)o * Ny * Nx + x, pos, Nx * 16); }
+  __device__ __forceinline__ void tally(int, int, int k, Limbs p, Limbs q, Acc& a) const {
+    if (RED) a.add(ikfreq(k, Ny), p, q);
+  }
+  __device__ __forceinline__ double mult(int, int x, int k) const {
+    return fma(-Om * xc(x), __ldg(nu + k), __ldg(kin + k));
+  }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc&) const {
+    if (t.bad) v.x = kBadElem;
+    stc(step(A + (size_t)o * Ny * Nx + x, pos, Nx * 16), v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, l.x, l, t.e); }
+  __device__ __forceinline__ void sums(const Line& l, const Acc& a, const Tile& t, double* s) const {
+    const double2 k = a.get();
+    s[0] = l.ok ? ck * k.x : 0.0;
+    s[1] = l.ok ? cr * xc(l.x) * k.y : 0.0;
+    if (t.bad) s[0] = s[1] = __longlong_as_double(0x7ff8000000000000ll);
+  }
+};
+
+// z: multiplier nu^2/2 on lines (o = y, x), then Hf = x part + y part + z part
+// + (V + beta |phi|^2 + lambda Phi) f, the last term in binary64.
+// Sums: kin_z, V|f|^2, |f|^4, Phi |f|^2, Re(Hf conj f), |f|^2.
+template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> {
+  const double2* f;
+  const double2* phi;
+  const double* Phi;
+  const c64* AX;
+  const c64* AY;
+  ExpTab ix, iy;
+  double2* Hf;
+  const double* kin;
+  int Nx, Ny, Nz;
+  const double* hx2;  // x_i^2 / 2 of each axis
+  const double* hy2;
+  const double* hz2;
+  double gx2, gy2, gz2, beta, lambda, ck;
+  bool same;  // f == phi: phi is not read a second time
+  static constexpr bool kMul = true;
+  struct Acc : KinAcc {
+    double s[5];
+  };
+  static constexpr int kMinB = 2;
+  __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
+  __device__ __forceinline__ double2 load(int o, int x, int pos) const { return *step(f + (size_t)o * Nx + x, pos, Ny * Nx * 16); }
+  __device__ __forceinline__ void tally(int, int, int k, Limbs p, Limbs q, Acc& a) const {
+    if (RED) a.add(ikfreq(k, Nz), p, q);
+  }
+  __device__ __forceinline__ double mult(int, int, int k) const { return __ldg(kin + k); }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc& a) const {
+    const size_t i0 = (size_t)o * Nx + x;
+    const int pl = Ny * Nx;
+    const double2 fv = __ldg(step(f + i0, pos, pl * 16));
+    const double Pd = __ldg(step(Phi + i0, pos, pl * 8));
+    const c64 u = ldc(step(AX + i0, pos, pl * 16)), w = ldc(step(AY + i0, pos, pl * 16));
+    const bool bad = t.bad || u.x == kBadElem || w.x == kBadElem;
+    const int eu = ix.at(pos * Ny + o, 0), ew = iy.at(pos, x);
+    const int e = max(t.e, max(eu, ew)) + 2;  // room for the sum of three
+    const int dv = min(e - t.e, 64), du = min(e - eu, 64), dw = min(e - ew, 64);
+    const long long sx = shr_clamp(v.x, dv) + shr_clamp(u.x, du) + shr_clamp(w.x, dw);
+    const long long sy = shr_clamp(v.y, dv) + shr_clamp(u.y, du) + shr_clamp(w.y, dw);
+    double2 kin;
+    if (bad) kin.x = kin.y = __longlong_as_double(0x7ff8000000000000ll);
+    else if (i2d_ok(e)) kin = make_double2(i2d(sx, e + 1085), i2d(sy, e + 1085));
+    else kin = make_double2(i2d_any(sx, e), i2d_any(sy, e));
+    const double V = gz2 * hz2[pos] + (gy2 * hy2[o] + gx2 * hx2[x]);
+    const double2 pv = same ? fv : __ldg(step(phi + i0, pos, pl * 16));
+    const double wt = V + beta * (pv.x * pv.x + pv.y * pv.y) + lambda * Pd;
+    const double ox = kin.x + wt * fv.x, oy = kin.y + wt * fv.y;
+    *step(Hf + i0, pos, pl * 16) = make_double2(ox, oy);
+    if (RED) {
+      const double f2 = fv.x * fv.x + fv.y * fv.y;
+      a.s[0] += V * f2;
+      a.s[1] += f2 * f2;
+      a.s[2] += Pd * f2;
+      a.s[3] += ox * fv.x + oy * fv.y;
+      a.s[4] += f2;
+    }
+  }
+  __device__ __forceinline__ void put_exp(const Line&, const Tile&) const {}
+  __device__ __forceinline__ void sums(const Line& l, const Acc& a, const Tile& t, double* s) const {
+    s[0] = l.ok ? ck * a.get().x : 0.0;
+    if (t.bad) s[0] = __longlong_as_double(0x7ff8000000000000ll);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) s[1 + i] = a.s[i];
+  }
+};
+
+// ---- preconditioner (unpadded grid); Wk: [Nz][Ny][Nx] workspace.  The weight
+// P_V^{-1/2} of each point is stored in Pw for the x inverse pass, which then
+// reads it instead of forming it again.
+struct IPXF : IOpBase<-1, false, 0, true, kSrcF64> {
+  const double2* r;
+  const double2* phi;
+  const double* Phi;
+  c64* Wk;
+  double* Pw;
+  ExpTab ex;
+  const double* hx2;
+  const double* hy2;
+  const double* hz2;
+  double gx2, gy2, gz2, beta, alam;
+  const double* alpha;
+  int Nx, Ny, nl;
+  __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
+  __device__ __forceinline__ double2 load(int o, int, int pos) const {
+    const size_t i = (size_t)o * Nx + pos;
+    const int y = o % Ny, z = o / Ny;
+    const double V = gx2 * hx2[pos] + (gy2 * hy2[y] + gz2 * hz2[z]);
+    const double2 pv = phi[i];
+    const double Pd = Phi[i];
+    const double den = *alpha + V + beta * (pv.x * pv.x + pv.y * pv.y) + alam * (Pd > 0.0 ? Pd : 0.0);
+    const double w = rsqrt(den);
+    Pw[i] = w;
+    const double2 rv = r[i];
+    return make_double2(rv.x * w, rv.y * w);
+  }
+  __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile&, Acc&) const {
+    stc(Wk + (size_t)o * Nx + pos, v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const {
+    put_exp_at(ex, l.o, 0, l, t.anybad ? kExpNaN : t.e);
+  }
+};
+
+// y transform of sign S in place: o = z.  LINES: the input's exponents are
+// indexed by the row z Ny + y (a line-major pass wrote them), else by y.
+template <int S, bool LINES> struct IPY : IOpBase<S, false, 0, false, kSrcInt> {
+  c64* Wk;
+  ExpTab in, ex;
+  int Nx, Ny;
+  __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
+  __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(Wk + (size_t)o * Ny * Nx + x, pos, Nx * 16)); }
+  __device__ __forceinline__ int lexp(int o, int x, int pos) const { return in.at(LINES ? o * Ny + pos : pos, x); }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, typename IPY::Acc&) const {
+    stc(step(Wk + (size_t)o * Ny * Nx + x, pos, Nx * 16), v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, l.x, l, t.e); }
+};
+
+// z forward * 1/((alpha + |nu|^2/2) N) * inverse on lines (o = y, x).
+struct IPZ : IOpBase<-1, true, 0, false, kSrcInt> {
+  c64* Wk;
+  ExpTab in, ex;
+  const double* alpha;
+  const double* nx2;  // nu^2 / 2 of each axis
+  const double* ny2;
+  const double* nz2;
+  double invN;
+  int Nx, Ny;
+  static constexpr bool kMul = true;
+  __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
+  __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16)); }
+  __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
+  __device__ __forceinline__ void tally(int, int, int, Limbs, Limbs, Acc&) const {}
+  __device__ __forceinline__ double mult(int o, int x, int k) const {
+    return invN / (*alpha + (nx2[x] + ny2[o]) + nz2[k]);
+  }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
+    stc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16), v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const { put_exp_at(ex, l.o, l.x, l, t.e); }
+};
+
+struct IPXI : IOpBase<1, false, 0, true, kSrcInt> {
+  const c64* Wk;
+  const double* Pw;
+  double2* Pr;
+  ExpTab in;
+  int Nx, Ny, nl;
+  __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
+  __device__ __forceinline__ c64 load(int o, int, int pos) const { return ldc(Wk + (size_t)o * Nx + pos); }
+  __device__ __forceinline__ int lexp(int o, int, int pos) const { return in.at(o / Ny, pos); }
+  __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile& t, Acc&) const {
+    const size_t i = (size_t)o * Nx + pos;
+    const double w = __ldg(Pw + i);
+    double2 d;
+    if (i2d_ok(t.e)) d = make_double2(i2d(v.x, t.e + 1085), i2d(v.y, t.e + 1085));
+    else d = make_double2(i2d_any(v.x, t.e), i2d_any(v.y, t.e));
+    Pr[i] = make_double2(w * d.x, w * d.y);
+  }
+  __device__ __forceinline__ void put_exp(const Line&, const Tile&) const {}
+};
+
+// ---- in-place 3D complex FFT on a plan's (unpadded) grid, sign S: binary64
+// in, integers between the passes (the y pass is IPY), binary64 out.
+template <int S> struct ICX : IOpBase<S, false, 0, true, kSrcF64> {
+  double2* buf;
+  ExpTab ex;
+  int Nx, nl;
+  __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
+  __device__ __forceinline__ double2 load(int o, int, int pos) const { return buf[(size_t)o * Nx + pos]; }
+  __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile&, typename ICX::Acc&) const {
+    stc(reinterpret_cast<c64*>(buf) + (size_t)o * Nx + pos, v);
+  }
+  __device__ __forceinline__ void put_exp(const Line& l, const Tile& t) const {
+    put_exp_at(ex, l.o, 0, l, t.anybad ? kExpNaN : t.e);
+  }
+};
+template <int S> struct ICZ : IOpBase<S, false, 0, false, kSrcInt> {
+  static constexpr int kMinB = 2;
+  double2* buf;
+  ExpTab in;
+  int Nx, Ny;
+  __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
+  __device__ __forceinline__ c64 load(int o, int x, int pos) const {
+    return ldc(reinterpret_cast<const c64*>(buf) + ((size_t)pos * Ny + o) * Nx + x);
+  }
+  __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
+  __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, typename ICZ::Acc&) const {
+    double2 d;
+    if (i2d_ok(t.e)) d = make_double2(i2d(v.x, t.e + 1085), i2d(v.y, t.e + 1085));
+    else d = make_double2(i2d_any(v.x, t.e), i2d_any(v.y, t.e));
+    buf[((size_t)pos * Ny + o) * Nx + x] = d;
+  }
+  __device__ __forceinline__ void put_exp(const Line&, const Tile&) const {}
+};
+
+}  // namespace atkm

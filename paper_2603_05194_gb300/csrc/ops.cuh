@@ -40,19 +40,6 @@ template <typename R> inline Cst<R> make_cst(const Geo& g) {
   return c;
 }
 
-// Per-axis tables of a plan (binary64, length N_a each), used by the binary64
-// H and preconditioner passes instead of forming the same values from integer
-// indices at every grid point (each index conversion and product is an
-// FP64-pipe instruction there): nu_k / N_a, (nu_k^2 / 2) / N_a, nu_k^2 / 2,
-// the coordinate -L_a + i h_a and half its square.
-struct AxT {
-  const double* nuN;
-  const double* kinN;
-  const double* hnu2;
-  const double* xc;
-  const double* hxc2;
-};
-
 template <typename R> struct PhysR {
   R gx2, gy2, gz2, beta, lambda, Omega;
 };
@@ -79,18 +66,18 @@ __device__ __forceinline__ int iabs(int a) { return a < 0 ? -a : a; }
 // integer pipe, to even in hardware).
 enum CvtMode { kCvtInt = 0, kCvtMixed = 1, kCvtHw = 2 };
 template <typename R, int CV = kCvtInt> __device__ __forceinline__ cx<R> from64(double2 z) {
-  if constexpr (std::is_same<R, float>::value && CV == kCvtHw) {
+  if constexpr (CV == kCvtHw) {
     return mk<R>(__double2float_rn(z.x), __double2float_rn(z.y));
-  } else if constexpr (std::is_same<R, float>::value && CV == kCvtMixed) {
+  } else if constexpr (CV == kCvtMixed) {
     return mk<R>(__double2float_rn(z.x), d2f_bits(z.y));
   } else {
     return mk<R>(tor<R>(z.x), tor<R>(z.y));
   }
 }
 template <typename R, int CV = kCvtInt> __device__ __forceinline__ double2 to64(R a, R b) {
-  if constexpr (std::is_same<R, float>::value && CV == kCvtHw) {
+  if constexpr (CV == kCvtHw) {
     return make_double2((double)a, (double)b);
-  } else if constexpr (std::is_same<R, float>::value && CV == kCvtMixed) {
+  } else if constexpr (CV == kCvtMixed) {
     return make_double2((double)a, f2d_bits(b));
   } else {
     return make_double2(tod<R>(a), tod<R>(b));
@@ -104,13 +91,6 @@ template <typename R, int CV = kCvtInt> __device__ __forceinline__ double2 to64(
 __device__ __forceinline__ double2 ldro(const double2* p) { return __ldg(p); }
 __device__ __forceinline__ float2 ldro(const float2* p) { return __ldg(p); }
 __device__ __forceinline__ double ldro(const double* p) { return __ldg(p); }
-__device__ __forceinline__ cdf ldro(const cdf* p) {  // (x.hi, x.lo, y.hi, y.lo), 16-byte aligned
-  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-  cdf r;
-  r.x = df(t.x, t.y);
-  r.y = df(t.z, t.w);
-  return r;
-}
 template <typename R> __device__ __forceinline__ cx<R> czero() { return mk<R>((R)0, (R)0); }
 
 // Asynchronous global -> shared copies (cp.async): an op that prefetches its
@@ -124,15 +104,11 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 template <typename R> __device__ __forceinline__ R rsq(R v);
-template <> __device__ __forceinline__ double rsq<double>(double v) { return rsqrt(v); }
 template <> __device__ __forceinline__ float rsq<float>(float v) { return rsqrtf(v); }
-template <> __device__ __forceinline__ df rsq<df>(df v) { return df_rsqrt(v); }
 
 // ------------------------------------------------------------- FastFft
 template <typename R> struct SmemShift;  // one pad element per 128 bytes
-template <> struct SmemShift<double> { static constexpr int value = 3; };
 template <> struct SmemShift<float> { static constexpr int value = 4; };
-template <> struct SmemShift<df> { static constexpr int value = 3; };
 
 constexpr int kFastElems = 2048;  // elements per CTA (256 threads x 8)
 
@@ -157,79 +133,6 @@ template <typename R, int L, bool LM> __device__ __forceinline__ int fsa(int t, 
   return lin + (lin >> SmemShift<R>::value);
 }
 
-// ---- binary64 twiddled butterflies in multiply-add form (Linzer and Feig's
-// modified FFT butterflies).  W = e^{S 2 pi i j / L} is read as (m, t) from
-// the multiply-add table of e^{-2 pi i j / L} (conjugated for S > 0), so that
-// W x = m y with y one FMA a component, and a +/- W x one FMA more a component:
-// 6 FP64 instructions a butterfly instead of 8 (complex product, then add and
-// subtract).  The form (lf_cform) is an integer test on j.  Nothing on the
-// FP64 pipe depends on it: it swaps operands with selects and flips the sign
-// of a scale factor with an integer XOR, and the remaining signs are the same
-// for every thread and fold into the FMAs.
-
-// a with its sign flipped when f (an integer operation on the high word).
-__device__ __forceinline__ double flip_sign(double a, bool f) {
-  return __hiloint2double(__double2hiint(a) ^ (f ? (int)0x80000000 : 0), __double2loint(a));
-}
-
-template <int L, int S, bool LO>
-__device__ __forceinline__ void lf_bfly(double2& a, double2& x, const double2* lf, int j) {
-  const double2 e = lf[j];
-  const bool sf = !lf_cform(j, L);
-  // W = m_e (1 + i t_e) or m_e (t_e + i): t_e = t and m_e = m for S < 0; for
-  // S > 0 (conjugate) t_e = -t, and m_e = -m in the s-form
-  const double t = (S > 0) ? -e.y : e.y;
-  const double mi = (S > 0) ? flip_sign(e.x, sf) : e.x;
-  const double mr = flip_sign(mi, sf);
-  // (P, Q) = (x.x, x.y) in the c-form, swapped in the s-form; then
-  // W x = (mr u, mi v) with u = P - t_e Q, v = Q + t_e P in both forms
-  const double P = sf ? x.y : x.x, Q = sf ? x.x : x.y;
-  const double u = fma(-t, Q, P), v = fma(t, P, Q);
-  if (!LO) x = make_double2(fma(-mr, u, a.x), fma(-mi, v, a.y));  // a - W x
-  a = make_double2(fma(mr, u, a.x), fma(mi, v, a.y));               // a + W x
-}
-
-// Twiddled radix-8 step: v[r] <- W^r v[r] (W = W_j), then the DFT of sign S,
-// as three layers of four multiply-add butterflies.  With r = 4 b2 + 2 b1 + b0
-// the layers apply W^4; W^2 and S i W^2 (= W_{2j + L/4}); and W, theta W,
-// theta^2 W, theta^3 W (theta = e^{S i pi / 4}, W_{j + qL/8}), where each odd
-// partial sum carries the common factor of its inputs so that one table
-// twiddle a butterfly suffices.  LO: only X_0..X_3 are formed.
-template <int L, int S, bool LO>
-__device__ __forceinline__ void lf_radix8(double2 (&v)[8], const double2* lf, int j) {
-  constexpr int L8 = L / 8, L4 = L / 4;
-  // v0 +/- W^4 v4, v2 +/- W^4 v6, v1 +/- W^4 v5, v3 +/- W^4 v7
-  lf_bfly<L, S, false>(v[0], v[4], lf, 4 * j);
-  lf_bfly<L, S, false>(v[2], v[6], lf, 4 * j);
-  lf_bfly<L, S, false>(v[1], v[5], lf, 4 * j);
-  lf_bfly<L, S, false>(v[3], v[7], lf, 4 * j);
-  // evens: E0, E2 in v0, v2; E1, E3 in v4, v6.  Odds / W: in v1, v3 and v5, v7
-  lf_bfly<L, S, false>(v[0], v[2], lf, 2 * j);
-  lf_bfly<L, S, false>(v[4], v[6], lf, 2 * j + L4);
-  lf_bfly<L, S, false>(v[1], v[3], lf, 2 * j);
-  lf_bfly<L, S, false>(v[5], v[7], lf, 2 * j + L4);
-  // X_q = E_q + theta^q O_q, X_{q+4} = E_q - theta^q O_q
-  lf_bfly<L, S, LO>(v[0], v[1], lf, j);           // X0, X4
-  lf_bfly<L, S, LO>(v[4], v[5], lf, j + L8);      // X1, X5
-  lf_bfly<L, S, LO>(v[2], v[3], lf, j + L4);      // X2, X6
-  lf_bfly<L, S, LO>(v[6], v[7], lf, j + 3 * L8);  // X3, X7
-  const double2 x1 = v[4], x3 = v[6], x4 = v[1], x6 = v[3];
-  v[1] = x1; v[3] = x3; v[4] = x4; v[6] = x6;
-}
-
-// Twiddled radix-4 step (W = W_b): v[q] <- W^q v[q], then the DFT of sign S:
-// v0 +/- W^2 v2, v1 +/- W^2 v3, then W and S i W (= W_{b + L/4}).  LO: only
-// X_0, X_1 are formed.
-template <int L, int S, bool LO>
-__device__ __forceinline__ void lf_radix4(double2 (&u)[4], const double2* lf, int b) {
-  lf_bfly<L, S, false>(u[0], u[2], lf, 2 * b);
-  lf_bfly<L, S, false>(u[1], u[3], lf, 2 * b);
-  lf_bfly<L, S, LO>(u[0], u[1], lf, b);           // X0, X2
-  lf_bfly<L, S, LO>(u[2], u[3], lf, b + L / 4);   // X1, X3
-  const double2 x1 = u[2], x2 = u[1];
-  u[1] = x1; u[2] = x2;
-}
-
 // Transforms the 8 register elements v[r] = line[j + TPL r] of line t in place
 // (sign S, unnormalised); on return v[r] holds frequency j + TPL r.  ZU: the
 // elements r >= 4 (positions >= L/2) are zero and not read.  LO: only the
@@ -238,34 +141,22 @@ template <typename R, int L, int S, bool LM, bool ZU = false, bool LO = false>
 __device__ __forceinline__ void fast_fft(cx<R> (&v)[8], cx<R>* b0, cx<R>* b1, const cx<R>* tw, int t, int j) {
   using C = FastCfg<L>;
   static_assert(!(ZU && LO && C::A == 1 && C::REM == 1), "ZU and LO in one radix-8 stage");
-  constexpr bool kLF = std::is_same<R, double>::value;  // tw is the multiply-add table
   int Ns = 1;
 #pragma unroll
   for (int s = 0; s < C::A; ++s) {
     const int k = j & (Ns - 1);
     const bool last = (s == C::A - 1) && (C::REM == 1);
-    if constexpr (kLF) {
-      if (s == 0) {
-        if (ZU) Dft<R, 8, S>::run_zu(v);
-        else Dft<R, 8, S>::run(v);
-      } else if (LO && last) {
-        lf_radix8<L, S, true>(v, tw, k * (L / (8 * Ns)));
-      } else {
-        lf_radix8<L, S, false>(v, tw, k * (L / (8 * Ns)));
-      }
-    } else {
-      if (s > 0) {
-        const int tws = L / (8 * Ns);
+    if (s > 0) {
+      const int tws = L / (8 * Ns);
 #pragma unroll
-        for (int r = 1; r < 8; ++r) {
-          const cx<R> w = tw[k * r * tws];
-          v[r] = (S < 0) ? cmul<R>(v[r], w) : cmulc<R>(v[r], w);
-        }
+      for (int r = 1; r < 8; ++r) {
+        const cx<R> w = tw[k * r * tws];
+        v[r] = (S < 0) ? cmul<R>(v[r], w) : cmulc<R>(v[r], w);
       }
-      if (ZU && s == 0) Dft<R, 8, S>::run_zu(v);
-      else if (LO && last) Dft<R, 8, S>::run_lo(v);
-      else Dft<R, 8, S>::run(v);
     }
+    if (ZU && s == 0) Dft<R, 8, S>::run_zu(v);
+    else if (LO && last) Dft<R, 8, S>::run_lo(v);
+    else Dft<R, 8, S>::run(v);
     if (!last) {
       cx<R>* b = (s & 1) ? b1 : b0;
       const int base = (j - k) * 8 + k;
@@ -285,19 +176,13 @@ __device__ __forceinline__ void fast_fft(cx<R> (&v)[8], cx<R>* b0, cx<R>* b1, co
       cx<R> u[Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) u[q] = v[m + M * q];
-      if constexpr (kLF && Q == 2) {
-        lf_bfly<L, S, LO>(u[0], u[1], tw, b);
-      } else if constexpr (kLF && Q == 4) {
-        lf_radix4<L, S, LO>(u, tw, b);
-      } else {
 #pragma unroll
-        for (int q = 1; q < Q; ++q) {
-          const cx<R> w = tw[b * q];
-          u[q] = (S < 0) ? cmul<R>(u[q], w) : cmulc<R>(u[q], w);
-        }
-        if (LO) Dft<R, Q, S>::run_lo(u);
-        else Dft<R, Q, S>::run(u);
+      for (int q = 1; q < Q; ++q) {
+        const cx<R> w = tw[b * q];
+        u[q] = (S < 0) ? cmul<R>(u[q], w) : cmulc<R>(u[q], w);
       }
+      if (LO) Dft<R, Q, S>::run_lo(u);
+      else Dft<R, Q, S>::run(u);
 #pragma unroll
       for (int q = 0; q < (LO ? Q / 2 : Q); ++q) v[m + M * q] = u[q];
     }
@@ -325,25 +210,15 @@ template <int S1, bool SECOND, int NRED, bool LM> struct OpBase {
 // ------------------------------------------------------------ kernels
 template <typename R, int NR>
 __device__ __forceinline__ void reduce_out(R (&acc)[NR], double* part, int pstride) {
-  if constexpr (sizeof(R) == 4) {
-    block_reduce_store_f32<NR>(acc, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
-  } else if constexpr (std::is_same<R, double>::value) {
-    block_reduce_store<NR>(acc, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
-  } else {  // double-word partials: widened per thread, FP64 beyond
-    double d[NR];
-#pragma unroll
-    for (int s = 0; s < NR; ++s) d[s] = tod<R>(acc[s]);
-    block_reduce_store<NR>(d, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
-  }
+  block_reduce_store_f32<NR>(acc, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
-// CTAs per SM the fast engine is compiled for: 4 in FP32 (64 registers); 3
+// CTAs per SM the fast engine is compiled for: 4 (64 registers); 3
 // (80 registers) with a prefetch buffer of 16 bytes an element, when two
 // exchange buffers already limit the shared memory to 3 CTAs, and for
-// L < 64, whose instances spill 8-88 bytes at 64 registers (L = 64: 4 bytes);
-// 2 otherwise (128 registers).
+// L < 64, whose instances spill 8-88 bytes at 64 registers (L = 64: 4 bytes).
 template <typename R, int L, class Op> constexpr int fast_min_blocks() {
-  return sizeof(R) == 4 ? (Op::kPre >= 16 && (FastSmem<R, L>::kTwoBufs || L < 64) ? 3 : 4) : 2;
+  return Op::kPre >= 16 && (FastSmem<R, L>::kTwoBufs || L < 64) ? 3 : 4;
 }
 
 template <typename R, int L, class Op>
@@ -393,14 +268,9 @@ __global__ void __launch_bounds__(kThreads, fast_min_blocks<R, L, Op>()) k_fast(
 #pragma unroll
     for (int r = 0; r < 8; ++r) vin[r] = v[r];
   }
-  // FP64 twiddles are staged in shared memory; FP32 twiddles are read through
-  // L1 from global memory, which avoids the bank conflicts of the strided
-  // table accesses (the FP32 passes are issue-bound, the FP64 ones ALU-bound).
+  // Twiddles are read through L1 from global memory, which avoids the bank
+  // conflicts of the strided table accesses (these passes are issue-bound).
   const cx<R>* twsrc = twg;
-  if (sizeof(R) == 8) {
-    for (int i = threadIdx.x; i < L; i += kThreads) tw[i] = twg[i];
-    twsrc = tw;
-  }
   __syncthreads();
   constexpr int NR = Op::kRed > 0 ? Op::kRed : 1;
   R acc[NR];
@@ -536,39 +406,23 @@ bool mix_len(int L);
 
 // LM passes: `lines` lines; strided passes: `X` columns x `outer` outer indices.
 // Engine: the power-of-two register engine, else the mixed-radix register
-// engine for 3 * 2^a (FP32 and binary64) and 5 * 2^a (FP32; in binary64 its
-// 20 complex doubles a thread make it slower than the generic engine,
-// measured), not with ATKM_PLAN_GENERIC_FFT, else the generic shared-memory
-// engine.
-template <typename R> constexpr int tune_r() {
-  return std::is_same<R, double>::value ? 0 : (std::is_same<R, float>::value ? 1 : 2);
-}
+// engine for 3 * 2^a and 5 * 2^a, not with ATKM_PLAN_GENERIC_FFT, else the
+// generic shared-memory engine.
 // An autotuned choice for (R, L, LM) of this plan, or null.
 template <typename R> inline const TuneEntry* tuned(const atkm_plan* p, int L, bool LM) {
   for (int i = 0; i < p->n_tune; ++i) {
     const TuneEntry& e = p->tune[i];
-    if (e.r == tune_r<R>() && e.L == L && e.lm == (LM ? 1 : 0)) return &e;
+    if (e.r == 1 && e.L == L && e.lm == (LM ? 1 : 0)) return &e;
   }
   return nullptr;
-}
-
-// Lengths the mixed-radix register engine is instantiated for in arithmetic
-// R (run_pass's switches): 3 * 2^a and 5 * 2^a in FP32, 3 * 2^a in binary64,
-// none in double-word.  Both the fixed rule and the autotuner go through this.
-template <typename R> inline bool mix_ok(int L) {
-  if (std::is_same<R, df>::value || !mix_len(L)) return false;
-  return !(std::is_same<R, double>::value && L % 5 == 0);
-}
-inline bool mix_ok_r(int r, int L) {
-  return r == 0 ? mix_ok<double>(L) : (r == 1 ? mix_ok<float>(L) : mix_ok<df>(L));
 }
 
 template <typename R> inline PassGrid pass_grid(const atkm_plan* p, int L, bool LM, long lines, int X, int outer) {
   PassGrid pg;
   pg.fast = fast_len(L);
-  pg.mix = !pg.fast && !(p->flags & ATKM_PLAN_GENERIC_FFT) && mix_ok<R>(L);
+  pg.mix = !pg.fast && !(p->flags & ATKM_PLAN_GENERIC_FFT) && mix_len(L);
   const TuneEntry* te = pg.fast ? nullptr : tuned<R>(p, L, LM);
-  if (te) pg.mix = te->mix != 0 && mix_ok<R>(L);
+  if (te) pg.mix = te->mix != 0 && mix_len(L);
   if (pg.fast) pg.T = kFastElems / L;
   else if (pg.mix) pg.T = kThreads / (L / (L % 3 == 0 ? 12 : 20));
   else {
@@ -605,9 +459,7 @@ inline cudaError_t launch_fast_L(const Op& op, const FftLen& f, const PassGrid& 
   const size_t sm = FastSmem<R, L>::bytes + (size_t)Op::kPre * 8 * kThreads;
   cudaError_t e = ensure_smem(prepared, k_fast<R, L, Op>, sm);
   if (e != cudaSuccess) return e;
-  // binary64 passes take the multiply-add form of the twiddles
-  const cx<R>* tw = std::is_same<R, double>::value ? reinterpret_cast<const cx<R>*>(f.lf64) : tw_table_host<R>(f);
-  k_fast<R, L, Op><<<pg.grid, kThreads, sm, st>>>(op, tw);
+  k_fast<R, L, Op><<<pg.grid, kThreads, sm, st>>>(op, tw_table_host<R>(f));
   return cudaGetLastError();
 }
 
@@ -617,7 +469,7 @@ namespace atkm {
 
 template <typename R, class Op>
 inline cudaError_t run_pass(const Op& op, const FftLen& f, const PassGrid& pg, cudaStream_t st) {
-  if constexpr (std::is_same<R, float>::value) {
+  {
     if (pg.mix) {
       switch (f.L) {
         case 20: return launch_mix_L<R, 20>(op, f, pg, st);
@@ -629,17 +481,6 @@ inline cudaError_t run_pass(const Op& op, const FftLen& f, const PassGrid& pg, c
         case 160: return launch_mix_L<R, 160>(op, f, pg, st);
         case 192: return launch_mix_L<R, 192>(op, f, pg, st);
         case 320: return launch_mix_L<R, 320>(op, f, pg, st);
-        case 384: return launch_mix_L<R, 384>(op, f, pg, st);
-        default: return cudaErrorInvalidValue;
-      }
-    }
-  } else if constexpr (std::is_same<R, double>::value) {
-    if (pg.mix) {
-      switch (f.L) {
-        case 24: return launch_mix_L<R, 24>(op, f, pg, st);
-        case 48: return launch_mix_L<R, 48>(op, f, pg, st);
-        case 96: return launch_mix_L<R, 96>(op, f, pg, st);
-        case 192: return launch_mix_L<R, 192>(op, f, pg, st);
         case 384: return launch_mix_L<R, 384>(op, f, pg, st);
         default: return cudaErrorInvalidValue;
       }
@@ -743,26 +584,21 @@ template <typename R> struct OpAtkmZ : OpBase<-1, true, 0, false> {
   static constexpr bool kZeroUpper = true;  // rows z >= Nz = L/2 are the padding
   static constexpr bool kHalfOut = true;    // only rows z < Nz are kept
   static constexpr bool kNyqTail = true;
-  static constexpr bool kTable = !std::is_same<R, float>::value;
-  cx<R>* W2; const R* K; const R* U0; Cst<R> c; R n0, n1, n2, invM; int XS;
+  cx<R>* W2; const R* U0; Cst<R> c; R n0, n1, n2, invM; int XS;
   __device__ bool valid(int, int x) const { return x <= c.Nx; }
   __device__ cx<R> load(int o, int x, int pos) const {
     return pos < c.Nz ? W2[((size_t)pos * c.My + o) * XS + x] : czero<R>();
   }
   __device__ void spectral(int o, int x, int k, cx<R>& v, R*) const {
-    if constexpr (kTable) {
-      v = scl<R>(v, K[((size_t)k * c.My + o) * XS + x]);
-    } else {
-      const int ky = kfreq(o, c.My), kz = kfreq(k, c.Mz);
-      const int kx = x == c.Nx ? -c.Nx : x;  // signed frequency of the half-spectrum column
-      const R tx = n0 * ((R)kx * c.pkx), ty = n1 * ((R)ky * c.pky), tz = n2 * ((R)kz * c.pkz);
-      R A = (R)0, B = (R)0;
-      if (x == c.Nx) B += tx; else A += tx;
-      if (o == c.Ny) B += ty; else A += ty;
-      if (k == c.Nz) B += tz; else A += tz;
-      const R u = U0[((size_t)iabs(kz) * (c.Ny + 1) + iabs(ky)) * (c.Nx + 1) + x];
-      v = scl<R>(v, ((R)3 * u * (A * A + B * B) - (R)1) * invM);
-    }
+    const int ky = kfreq(o, c.My), kz = kfreq(k, c.Mz);
+    const int kx = x == c.Nx ? -c.Nx : x;  // signed frequency of the half-spectrum column
+    const R tx = n0 * ((R)kx * c.pkx), ty = n1 * ((R)ky * c.pky), tz = n2 * ((R)kz * c.pkz);
+    R A = (R)0, B = (R)0;
+    if (x == c.Nx) B += tx; else A += tx;
+    if (o == c.Ny) B += ty; else A += ty;
+    if (k == c.Nz) B += tz; else A += tz;
+    const R u = U0[((size_t)iabs(kz) * (c.Ny + 1) + iabs(ky)) * (c.Nx + 1) + x];
+    v = scl<R>(v, ((R)3 * u * (A * A + B * B) - (R)1) * invM);
   }
   __device__ void store(int o, int x, int pos, cx<R> v, R*) const {
     if (pos < c.Nz) W2[((size_t)pos * c.My + o) * XS + x] = v;
@@ -810,20 +646,10 @@ template <typename R> struct OpAtkmXI : OpBase<1, false, 0, true> {
 // ---- H_phi f (unpadded grid); acc: [Nz][Ny][Nx] kinetic+rotation accumulator.
 // x: multiplier nu^2/2 + Omega y nu on lines o = z Ny + y.
 template <typename R, bool RED> struct OpHX : OpBase<-1, true, RED ? 2 : 0, true> {
-  const double2* f; cx<R>* acc; Cst<R> c; R Omega; AxT ax, ay;
+  const double2* f; cx<R>* acc; Cst<R> c; R Omega;
   __device__ bool valid(int o, int) const { return o < c.Nz * c.Ny; }
   __device__ cx<R> load(int o, int, int pos) const { return from64<R, kCvtMixed>(f[(size_t)o * c.Nx + pos]); }
   __device__ void spectral(int o, int, int k, cx<R>& v, R* a) const {
-    if constexpr (std::is_same<R, double>::value) {
-      const double kin = ax.kinN[k], rot = Omega * ay.xc[o % c.Ny] * ax.nuN[k];
-      if (RED) {
-        const double a2 = v.x * v.x + v.y * v.y;
-        a[0] += kin * a2;
-        a[1] += rot * a2;
-      }
-      v = scl<R>(v, kin + rot);
-      return;
-    }
     const R invL = (R)1 / (R)c.Nx;
     const R nu = (R)kfreq(k, c.Nx) * c.kx;
     const R y = -c.Ly + (R)(o % c.Ny) * c.hy;
@@ -840,20 +666,10 @@ template <typename R, bool RED> struct OpHX : OpBase<-1, true, RED ? 2 : 0, true
 
 // y: multiplier nu^2/2 - Omega x nu on lines (o = z, x); acc += result.
 template <typename R, bool RED> struct OpHY : OpBase<-1, true, RED ? 2 : 0, false> {
-  const double2* f; cx<R>* acc; Cst<R> c; R Omega; AxT ax, ay;
+  const double2* f; cx<R>* acc; Cst<R> c; R Omega;
   __device__ bool valid(int, int x) const { return x < c.Nx; }
   __device__ cx<R> load(int o, int x, int pos) const { return from64<R, kCvtHw>(f[((size_t)o * c.Ny + pos) * c.Nx + x]); }
   __device__ void spectral(int, int x, int k, cx<R>& v, R* a) const {
-    if constexpr (std::is_same<R, double>::value) {
-      const double kin = ay.kinN[k], rot = -Omega * ax.xc[x] * ay.nuN[k];
-      if (RED) {
-        const double a2 = v.x * v.x + v.y * v.y;
-        a[0] += kin * a2;
-        a[1] += rot * a2;
-      }
-      v = scl<R>(v, kin + rot);
-      return;
-    }
     const R invL = (R)1 / (R)c.Ny;
     const R nu = (R)kfreq(k, c.Ny) * c.ky;
     const R xc = -c.Lx + (R)x * c.hx;
@@ -870,7 +686,7 @@ template <typename R, bool RED> struct OpHY : OpBase<-1, true, RED ? 2 : 0, fals
     acc[idx] = add<R>(acc[idx], v);
   }
   // FP32: the accumulator (8 B a point) is prefetched into shared memory
-  static constexpr int kPre = std::is_same<R, float>::value ? 8 : 0;
+  static constexpr int kPre = 8;
   __device__ void prefetch(int o, int x, int pos, unsigned char* dst) const {
     cp_async8(dst, acc + ((size_t)o * c.Ny + pos) * c.Nx + x);
   }
@@ -884,17 +700,10 @@ template <typename R, bool RED> struct OpHY : OpBase<-1, true, RED ? 2 : 0, fals
 // Reductions: kin_z, sum V|f|^2, sum |f|^4, sum Phi |f|^2, sum Re(Hf conj f), sum |f|^2.
 template <typename R, bool RED> struct OpHZ : OpBase<-1, true, RED ? 6 : 0, false> {
   const double2* f; const double2* phi; const double* Phi; const cx<R>* acc; double2* Hf; Cst<R> c; PhysR<R> ph;
-  AxT ax, ay, az;
   bool same = false;  // f == phi (H phi): phi is not read a second time
   __device__ bool valid(int, int x) const { return x < c.Nx; }
   __device__ cx<R> load(int o, int x, int pos) const { return from64<R, kCvtMixed>(f[((size_t)pos * c.Ny + o) * c.Nx + x]); }
   __device__ void spectral(int, int, int k, cx<R>& v, R* a) const {
-    if constexpr (std::is_same<R, double>::value) {
-      const double m = az.kinN[k];
-      if (RED) a[0] += m * (v.x * v.x + v.y * v.y);
-      v = scl<R>(v, m);
-      return;
-    }
     const R invL = (R)1 / (R)c.Nz;
     const R nu = (R)kfreq(k, c.Nz) * c.kz;
     const R m = (R)0.5 * nu * nu;
@@ -907,13 +716,13 @@ template <typename R, bool RED> struct OpHZ : OpBase<-1, true, RED ? 6 : 0, fals
   }
   // FP32 and double-word: f at this point is the element the engine loaded
   // (the same conversion of the same value), kept in registers
-  static constexpr bool kKeepIn = !std::is_same<R, double>::value;
+  static constexpr bool kKeepIn = true;
   __device__ void store_k(int o, int x, int pos, cx<R> v, R* a, cx<R> fin) const {
     const size_t idx = ((size_t)pos * c.Ny + o) * c.Nx + x;
     finish(o, x, pos, idx, v, a, tor<R>(ldro(Phi + idx)), ldro(acc + idx), fin);
   }
   // FP32: Phi (8 B) and the accumulator (8 B) are prefetched into shared memory
-  static constexpr int kPre = std::is_same<R, float>::value ? 16 : 0;
+  static constexpr int kPre = 16;
   __device__ void prefetch(int o, int x, int pos, unsigned char* dst) const {
     const size_t idx = ((size_t)pos * c.Ny + o) * c.Nx + x;
     cp_async8(dst, Phi + idx);
@@ -932,12 +741,8 @@ template <typename R, bool RED> struct OpHZ : OpBase<-1, true, RED ? 6 : 0, fals
   __device__ __forceinline__ void finish(int o, int x, int pos, size_t idx, cx<R> v, R* a, R Pd, cx<R> accv,
                                          cx<R> fv) const {
     R V;
-    if constexpr (std::is_same<R, double>::value) {
-      V = ph.gz2 * az.hxc2[pos] + (ph.gy2 * ay.hxc2[o] + ph.gx2 * ax.hxc2[x]);
-    } else {
-      const R xc = -c.Lx + (R)x * c.hx, yc = -c.Ly + (R)o * c.hy, zc = -c.Lz + (R)pos * c.hz;
-      V = (R)0.5 * (ph.gx2 * xc * xc + ph.gy2 * yc * yc + ph.gz2 * zc * zc);
-    }
+    const R xc = -c.Lx + (R)x * c.hx, yc = -c.Ly + (R)o * c.hy, zc = -c.Lz + (R)pos * c.hz;
+    V = (R)0.5 * (ph.gx2 * xc * xc + ph.gy2 * yc * yc + ph.gz2 * zc * zc);
     const cx<R> pv = same ? fv : from64<R, kCvtMixed>(ldro(phi + idx));
     const R w = V + ph.beta * (pv.x * pv.x + pv.y * pv.y) + ph.lambda * Pd;
     const cx<R> kin = add<R>(accv, v);
@@ -970,20 +775,9 @@ __device__ __forceinline__ R pv_rsqrt(const Cst<R>& c, const PhysR<R>& ph, R alp
 // x inverse pass, which then reads it instead of forming it again.
 template <typename R> struct OpPXF : OpBase<-1, false, 0, true> {
   const double2* r; const double2* phi; const double* Phi; cx<R>* Wk; Cst<R> c; PhysR<R> ph; const double* alpha;
-  AxT ax, ay, az; double* Pw;
   __device__ bool valid(int o, int) const { return o < c.Nz * c.Ny; }
   __device__ cx<R> load(int o, int, int pos) const {
     const size_t idx = (size_t)o * c.Nx + pos;
-    if constexpr (std::is_same<R, double>::value) {
-      const int y = o % c.Ny, z = o / c.Ny;
-      const double V = ph.gx2 * ax.hxc2[pos] + (ph.gy2 * ay.hxc2[y] + ph.gz2 * az.hxc2[z]);
-      const double2 pv = phi[idx];
-      const double Pd = Phi[idx];
-      const double den = *alpha + V + ph.beta * (pv.x * pv.x + pv.y * pv.y) + fabs(ph.lambda) * (Pd > 0.0 ? Pd : 0.0);
-      const double w = rsqrt(den);
-      Pw[idx] = w;
-      return scl<R>(r[idx], w);
-    }
     const R w = pv_rsqrt<R>(c, ph, tor<R>(*alpha), pos, o % c.Ny, o / c.Ny, phi[idx], Phi[idx]);
     return scl<R>(from64<R, kCvtMixed>(r[idx]), w);
   }
@@ -1001,15 +795,10 @@ template <typename R, int S> struct OpPY : OpBase<S, false, 0, false> {
 
 // z forward * 1/((alpha + |nu|^2/2) N) * inverse on lines (o = y, x).
 template <typename R> struct OpPZ : OpBase<-1, true, 0, false> {
-  cx<R>* Wk; Cst<R> c; const double* alpha; AxT ax, ay, az;
+  cx<R>* Wk; Cst<R> c; const double* alpha;
   __device__ bool valid(int, int x) const { return x < c.Nx; }
   __device__ cx<R> load(int o, int x, int pos) const { return Wk[((size_t)pos * c.Ny + o) * c.Nx + x]; }
   __device__ void spectral(int o, int x, int k, cx<R>& v, R*) const {
-    if constexpr (std::is_same<R, double>::value) {
-      const double invN = 1.0 / ((double)c.Nx * (double)c.Ny * (double)c.Nz);
-      v = scl<R>(v, invN / (*alpha + (ax.hnu2[x] + ay.hnu2[o]) + az.hnu2[k]));
-      return;
-    }
     const R invN = (R)1 / ((R)c.Nx * (R)c.Ny * (R)c.Nz);
     const R nux = (R)kfreq(x, c.Nx) * c.kx, nuy = (R)kfreq(o, c.Ny) * c.ky, nuz = (R)kfreq(k, c.Nz) * c.kz;
     v = scl<R>(v, invN / (tor<R>(*alpha) + (R)0.5 * (nux * nux + nuy * nuy + nuz * nuz)));
@@ -1019,17 +808,11 @@ template <typename R> struct OpPZ : OpBase<-1, true, 0, false> {
 
 template <typename R> struct OpPXI : OpBase<1, false, 0, true> {
   const cx<R>* Wk; const double2* phi; const double* Phi; double2* Pr; Cst<R> c; PhysR<R> ph; const double* alpha;
-  const double* Pw;  // binary64: the weights the x forward pass stored
   __device__ bool valid(int o, int) const { return o < c.Nz * c.Ny; }
   __device__ cx<R> load(int o, int, int pos) const { return Wk[(size_t)o * c.Nx + pos]; }
   __device__ void spectral(int, int, int, cx<R>&, R*) const {}
   __device__ void store(int o, int, int pos, cx<R> v, R*) const {
     const size_t idx = (size_t)o * c.Nx + pos;
-    if constexpr (std::is_same<R, double>::value) {
-      const double w = ldro(Pw + idx);
-      Pr[idx] = make_double2(w * v.x, w * v.y);
-      return;
-    }
     const R w = pv_rsqrt<R>(c, ph, tor<R>(*alpha), pos, o % c.Ny, o / c.Ny, ldro(phi + idx), ldro(Phi + idx));
     Pr[idx] = to64<R, kCvtMixed>(w * v.x, w * v.y);
   }

@@ -850,7 +850,7 @@ struct Seq {
   void atkm(int mode, const double* a, const double* b, double* o, bool aux = false) {
     const bool use32 = f32 || (aux && aux32);
     chk(use32 ? launch_atkm<float>(p, mode, a, b, o, st())
-              : dw ? launch_atkm<df>(p, mode, a, b, o, st()) : launch_atkm<double>(p, mode, a, b, o, st()));
+              : launch_atkm64(p, dw, mode, a, b, o, st()));
   }
   void hop(const double2* f, double2* o, int red, bool aux = false) {
     const double* fp = reinterpret_cast<const double*>(f);
@@ -858,8 +858,7 @@ struct Seq {
     double* op = reinterpret_cast<double*>(o);
     const bool use32 = f32 || (aux && aux32);
     chk(use32 ? launch_H<float>(p, ph, fp, pp, B.Phi[q], op, red, st())
-              : dw ? launch_H<df>(p, ph, fp, pp, B.Phi[q], op, red, st())
-                   : launch_H<double>(p, ph, fp, pp, B.Phi[q], op, red, st()));
+              : launch_H64(p, dw, ph, fp, pp, B.Phi[q], op, red, st()));
   }
   template <typename K, typename... A> void ctl1(K kernel, A... args) {
     kernel<<<1, 1, 0, st()>>>(args...);
@@ -907,7 +906,7 @@ struct Seq {
     const double* phi = reinterpret_cast<const double*>(B.phi[q]);
     double* Pr = reinterpret_cast<double*>(B.Pr);
     return (f32 || aux32) ? launch_precond<float>(p, ph, &c()->alpha, r, phi, B.Phi[q], Pr, st())
-                          : launch_precond<double>(p, ph, &c()->alpha, r, phi, B.Phi[q], Pr, st());
+                          : launch_precond64(p, ph, &c()->alpha, r, phi, B.Phi[q], Pr, st());
   }
   // A whole iteration: Steps 2-4 up to the first trial.
   void iteration() {
@@ -1401,7 +1400,7 @@ struct Solver {
         Seq Z{plan, *B, ph, false, 0};
         const double* p0d = reinterpret_cast<const double*>(B->phi[0]);
         Z.atkm(SRC_PSI, p0d, nullptr, B->Phi1);
-        chk(launch_H<double>(plan, ph, p0d, p0d, B->Phi1, reinterpret_cast<double*>(B->Hp), -1, B->st));
+        chk(launch_H64(plan, false, ph, p0d, p0d, B->Phi1, reinterpret_cast<double*>(B->Hp), -1, B->st));
         chk(launch_H<float>(plan, ph, p0d, p0d, B->Phi[0], reinterpret_cast<double*>(B->Hphi), -1, B->st));
         Z.lincomb(B->Pr, B->Hp, Coef{nullptr, 1.0}, B->Hphi, Coef{nullptr, -1.0}, nullptr, Coef{nullptr, 0.0},
                   nullptr, S_Z, nullptr, false);
@@ -1645,7 +1644,7 @@ int atkm_energy_parts(atkm_plan* plan, const atkm_params* prm, const double* phi
   if (!plan || !prm || !phi || !Phi || !out) return fail(plan, ATKM_ERR_ARG, "atkm_energy_parts: NULL argument");
   cudaStream_t st = (cudaStream_t)stream;
   // W1 holds at least N complex values and is free outside the ATKM passes.
-  cudaError_t e = launch_H<double>(plan, make_phys(prm), phi, phi, Phi, reinterpret_cast<double*>(plan->W1), S_H, st);
+  cudaError_t e = launch_H64(plan, false, make_phys(prm), phi, phi, Phi, reinterpret_cast<double*>(plan->W1), S_H, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(plan->scal_host + S_H, plan->scal + S_H, 10 * sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1673,7 +1672,7 @@ int apply_preconditioner(atkm_plan* plan, const atkm_params* prm, double alpha, 
   k_set_scalar<<<1, 1, 0, st>>>(plan->scal + SC_ALPHA, alpha);
   count_launches(1);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_precond<double>(plan, make_phys(prm), plan->scal + SC_ALPHA, r, phi, Phi, Pr, st);
+  if (e == cudaSuccess) e = launch_precond64(plan, make_phys(prm), plan->scal + SC_ALPHA, r, phi, Phi, Pr, st);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(plan, e, "apply_preconditioner");
 }
 

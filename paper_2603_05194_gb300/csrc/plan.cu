@@ -106,20 +106,84 @@ struct GLNodes {
   double w[kGL];  // weights for (0, 1)
 };
 
-// Twiddles e^{-2 pi i m / L}, and the binary64 ones in multiply-add form
-// (lf_cform).
-__global__ void k_twiddles(double2* t64, float2* t32, cdf* tdf, double2* lf, int L) {
+// Unevaluated sums of two binary64 numbers (about 106 bits) for the integer
+// twiddles: Knuth's TwoSum, the FMA product error (Dekker; Ogita, Rump and
+// Oishi 2005).
+struct dd {
+  double h, l;
+};
+__device__ __forceinline__ dd dd_norm(double a, double b) {  // |a| >= |b|
+  const double s = a + b;
+  return dd{s, b - (s - a)};
+}
+__device__ __forceinline__ dd dd_add(dd a, dd b) {
+  const double s = a.h + b.h, t = s - a.h;
+  return dd_norm(s, (a.h - (s - t)) + (b.h - t) + a.l + b.l);
+}
+__device__ __forceinline__ dd dd_mul(dd a, dd b) {
+  const double p = a.h * b.h;
+  return dd_norm(p, fma(a.h, b.h, -p) + a.h * b.l + a.l * b.h);
+}
+__device__ __forceinline__ dd dd_div(dd a, double b) {
+  const double q = a.h / b;
+  return dd_norm(q, (fma(-q, b, a.h) + a.l) / b);
+}
+// cos or sin (odd = 1) of t in [0, pi/4] by its Taylor series (error < 2^-70)
+__device__ dd dd_taylor(dd t, int odd) {
+  const dd q = dd_mul(t, t);
+  dd sum = {0.0, 0.0}, term = odd ? t : dd{1.0, 0.0};
+  for (int n = odd + 1; n < 26; n += 2) {
+    sum = dd_add(sum, term);
+    term = dd_div(dd_mul(term, q), -(double)n * (double)(n + 1));
+  }
+  return sum;
+}
+// x 2^bits as two signed 32-bit limbs (the low one never -2^31)
+__device__ int2 dd_limbs(dd x, int bits) {
+  const long long v = __double2ll_rn(ldexp(x.h, bits)) + __double2ll_rn(ldexp(x.l, bits));
+  Limbs r = limbs(v);
+  if (r.l == (int)0x80000000) r.l += 1;
+  return make_int2(r.h, r.l);
+}
+
+// e^{-2 pi i m / L} as 64-bit integers in units 2^-bits, 0 <= m < L.
+__device__ int4 int_twiddle(int m, int L, int bits) {
+  // angle = (octant + rem / L) pi/4, reflected into the first octant
+  const int oct = 8 * m / L, rem = 8 * m - oct * L;
+  const dd pi4 = {0.78539816339744830962, 3.0616169978683829430651648306875e-17};
+  const dd t = dd_div(dd_mul(pi4, dd{(double)((oct & 1) ? L - rem : rem), 0.0}), (double)L);
+  const dd ct = dd_taylor(t, 0), sn = dd_taylor(t, 1);
+  const bool sw = ((oct + 1) >> 1) & 1;  // octants 1, 2, 5, 6: the roles swap
+  dd cc = sw ? sn : ct, ss = sw ? ct : sn;
+  if (oct >= 2 && oct < 6) cc = dd{-cc.h, -cc.l};
+  if (oct >= 4) ss = dd{-ss.h, -ss.l};
+  const int2 c = dd_limbs(cc, bits), s = dd_limbs(ss, bits);
+  return make_int4(c.x, c.y, s.x, s.y);
+}
+
+// Twiddles e^{-2 pi i m / L} in FP32, m < L.
+__global__ void k_twiddles(float2* t32, int L) {
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < L; m += gridDim.x * blockDim.x) {
     double s, c;
     sincospi(2.0 * (double)m / (double)L, &s, &c);
-    t64[m] = make_double2(c, -s);
     t32[m] = make_float2((float)c, (float)-s);
-    cdf w;
-    w.x = df(c);
-    w.y = df(-s);
-    tdf[m] = w;
-    lf[m] = lf_cform(m, L) ? make_double2(c, -s / c) : make_double2(-s, c / -s);
   }
+}
+// The stage tables of an integer length (IntLen) at w.
+__global__ void k_int_twiddles(int4* w, IntLen f) {
+  int Ns = f.rad[0];
+  for (int s = 1; s < f.nst; ++s) {
+    const int R = f.rad[s];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (R - 1) * Ns; i += gridDim.x * blockDim.x) {
+      const int r = i / Ns + 1, k = i - (r - 1) * Ns;
+      w[f.off[s] + i] = int_twiddle(k * r, Ns * R, 64 - stage_shift(R));
+    }
+    Ns *= R;
+  }
+}
+// e^{-2 pi i k / M}, k < M / 2.
+__global__ void k_post_twist(int4* w, int M) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M / 2; k += gridDim.x * blockDim.x) w[k] = int_twiddle(k, M, 61);
 }
 
 // table[q * (N + 1) + k] = I(s_q; nu_k), nu_k = pi k / a, k = 0..N.
@@ -211,18 +275,21 @@ __global__ void k_multiplier_full(double* __restrict__ K, const double* __restri
 // and B over those that are: the index of -k has the same Nyquist components
 // and the others negated, so the cross term 2AB cancels in the average (the
 // Nyquist index M_a / 2 stands for nu = -pi M_a / (4 L_a)).  Layout
-// [Mz][My][XS], columns x > Nx zero.
-__global__ void k_multiplier_half(double* __restrict__ Kh, const double* __restrict__ U0, Geo g, double n0,
-                                  double n1, double n2) {
+// [Mz][My][XS], columns x > Nx zero; integers K_sym mant 2^kq (mant the
+// fraction of 1 / (2 Mx My Mz) in [1/2, 1)).  With Kh null only the largest
+// |K_sym mant| is found (as the bits of a double, into *kmax).
+__global__ void k_multiplier_half(long long* __restrict__ Kh, unsigned long long* __restrict__ kmax,
+                                  const double* __restrict__ U0, Geo g, double n0, double n1, double n2, double mant,
+                                  double scale) {
   const size_t total = (size_t)g.Mz * g.My * g.XS;
   const double px = kPi / (2.0 * g.Lx), py = kPi / (2.0 * g.Ly), pz = kPi / (2.0 * g.Lz);
-  const double invM = 0.5 / ((double)g.Mx * g.My * g.Mz);
+  double most = 0.0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
     const int x = (int)(i % g.XS);
     const int o = (int)((i / g.XS) % g.My);
     const int k = (int)(i / ((size_t)g.XS * g.My));
     if (x > g.Nx) {
-      Kh[i] = 0.0;
+      if (Kh) Kh[i] = 0;
       continue;
     }
     const int kx = x == g.Nx ? -g.Nx : x;
@@ -233,18 +300,16 @@ __global__ void k_multiplier_half(double* __restrict__ Kh, const double* __restr
     if (o == g.Ny) B += ty; else A += ty;
     if (k == g.Nz) B += tz; else A += tz;
     const double u = U0[((size_t)abs(kz) * (g.Ny + 1) + abs(ky)) * (g.Nx + 1) + x];
-    Kh[i] = (3.0 * u * (A * A + B * B) - 1.0) * invM;
+    const double v = (3.0 * u * (A * A + B * B) - 1.0) * mant;
+    if (Kh) Kh[i] = __double2ll_rn(v * scale);
+    else most = fmax(most, fabs(v));
   }
+  if (!Kh) atomicMax(kmax, (unsigned long long)__double_as_longlong(most));
 }
 
 __global__ void k_to_f32(float* __restrict__ dst, const double* __restrict__ src, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = (float)src[i];
-}
-
-__global__ void k_to_df(df* __restrict__ dst, const double* __restrict__ src, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = df(src[i]);
 }
 
 // Fine spectrum <- coarse spectrum / Nc: fine frequency k (signed) takes the
@@ -288,9 +353,52 @@ bool make_fft_len(int L, FftLen& f) {
   return n == 1;
 }
 
+// The stages of an integer length: as few as possible, the large radices first
+// (the first stage has no twiddles); for the register engine's lengths radix 8
+// and one stage of radix 4 or 2.
+bool make_int_len(int L, IntLen& f) {
+  memset(&f, 0, sizeof(f));
+  f.L = L;
+  int n2 = 0, n3 = 0, n5 = 0, n = L;
+  while (n % 2 == 0) { n /= 2; ++n2; }
+  while (n % 3 == 0) { n /= 3; ++n3; }
+  while (n % 5 == 0) { n /= 5; ++n5; }
+  if (n != 1) return false;
+  // radix 6 takes a factor 2 with a 3 where the other twos then need fewer stages of 8, 4 and 2
+  int best = 0, n6 = 0;
+  for (int s = 0; s <= std::min(n2, n3); ++s) {
+    const int stages = s + (n3 - s) + (n2 - s + 2) / 3;
+    if (s == 0 || stages < best) { best = stages; n6 = s; }
+  }
+  n2 -= n6;
+  n3 -= n6;
+  std::vector<int> r;
+  const bool pow2 = n3 + n5 + n6 == 0;
+  while (n2 >= 3 && (pow2 || n2 != 4)) { r.push_back(8); n2 -= 3; }
+  for (int i = 0; i < n6; ++i) r.push_back(6);
+  for (int i = 0; i < n5; ++i) r.push_back(5);
+  while (n2 >= 2) { r.push_back(4); n2 -= 2; }
+  for (int i = 0; i < n3; ++i) r.push_back(3);
+  if (n2) r.push_back(2);
+  if ((int)r.size() > kMaxStages) return false;
+  auto magic = [](int d) { return d > 1 ? (unsigned)((0x100000000ull + d - 1) / d) : 0u; };
+  int Ns = 1, off = 0;
+  for (int q : r) {
+    f.rad[f.nst] = q;
+    f.off[f.nst] = off;
+    if (f.nst) off += (q - 1) * Ns;
+    f.mns[f.nst] = magic(Ns);
+    f.mnb[f.nst] = magic(L / q);
+    if (f.nst) f.shift += stage_shift(q);
+    Ns *= q;
+    ++f.nst;
+  }
+  return true;
+}
+
 void free_plan_memory(atkm_plan* p) {
-  void* ptrs[] = {p->tw64, p->tw32, p->twdf, p->lf64, p->axtab, p->Pw, p->U0, p->U0f, p->Kz, p->Kzd, p->W1, p->W2, p->T1, p->W1f, p->W2f, p->T1f,
-                  p->partials, p->scal};
+  void* ptrs[] = {p->tw32, p->twi, p->axtab, p->Pw, p->U0, p->U0f, p->Kz, p->W1, p->W2, p->T1,
+                  p->W1f, p->W2f, p->T1f, p->ex[0], p->ex[1], p->ex[2], p->partials, p->scal};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->scal_host) cudaFreeHost(p->scal_host);
@@ -445,10 +553,11 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   cudaStream_t st = (cudaStream_t)stream;
   atkm_plan* p = new atkm_plan();
   memset(&p->g, 0, sizeof(p->g));
-  p->tw64 = nullptr; p->tw32 = nullptr; p->twdf = nullptr; p->lf64 = nullptr; p->U0 = nullptr;
+  p->tw32 = nullptr; p->twi = nullptr; p->tw_x = nullptr; p->U0 = nullptr;
   p->axtab = nullptr; p->Pw = nullptr;
-  p->U0f = nullptr; p->Kz = nullptr; p->Kzd = nullptr;
+  p->U0f = nullptr; p->Kz = nullptr;
   p->W1 = p->W2 = p->T1 = nullptr;
+  p->ex[0] = p->ex[1] = p->ex[2] = nullptr;
   p->W1f = p->W2f = p->T1f = nullptr; p->partials = nullptr; p->scal = nullptr; p->scal_host = nullptr;
   p->pcg = nullptr; p->prof = nullptr; p->prof_stopped_ = nullptr; p->bytes = 0; p->flags = flags;
   p->n_tune = 0;
@@ -472,26 +581,27 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   const int lens[6] = {g.Nx, g.Ny, g.Nz, g.Mx, g.My, g.Mz};
   size_t twtot = 0;
   for (int i = 0; i < 6; ++i) twtot += lens[i];
-  if ((e = dev_alloc(p, (void**)&p->tw64, twtot * sizeof(double2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
   if ((e = dev_alloc(p, (void**)&p->tw32, twtot * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
-  if ((e = dev_alloc(p, (void**)&p->twdf, twtot * sizeof(cdf))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
-  if ((e = dev_alloc(p, (void**)&p->lf64, twtot * sizeof(double2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
+  // a length's stage tables take less than its length
+  if ((e = dev_alloc(p, (void**)&p->twi, (twtot + g.Nx) * sizeof(int4))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
   size_t off = 0;
   for (int i = 0; i < 6; ++i) {
     FftLen& f = (i < 3) ? p->fN[i] : p->fM[i - 3];
-    if (!make_fft_len(lens[i], f)) return bail(fail(nullptr, ATKM_ERR_UNSUPPORTED_SIZE, "plan: FFT factorisation"));
-    f.tw64 = p->tw64 + off;
+    IntLen& fi = (i < 3) ? p->iN[i] : p->iM[i - 3];
+    if (!make_fft_len(lens[i], f) || !make_int_len(lens[i], fi))
+      return bail(fail(nullptr, ATKM_ERR_UNSUPPORTED_SIZE, "plan: FFT factorisation"));
     f.tw32 = p->tw32 + off;
-    f.twdf = p->twdf + off;
-    f.lf64 = p->lf64 + off;
-    k_twiddles<<<(lens[i] + 255) / 256, 256, 0, st>>>(p->tw64 + off, p->tw32 + off, p->twdf + off, p->lf64 + off,
-                                                      lens[i]);
-    count_launches(1);
+    fi.w = p->twi + off;
+    k_twiddles<<<(lens[i] + 127) / 128, 128, 0, st>>>(p->tw32 + off, lens[i]);
+    k_int_twiddles<<<(lens[i] + 63) / 64, 64, 0, st>>>(p->twi + off, fi);
+    count_launches(2);
     off += lens[i];
   }
-  // ---- per-axis tables of the binary64 H and preconditioner passes (AxT):
-  // nu_k / N, (nu_k^2 / 2) / N, nu_k^2 / 2 with nu_k = k' pi / L (k' the signed
-  // index), and the coordinate x_i = -L + i h with x_i^2 / 2
+  p->tw_x = p->twi + off;
+  k_post_twist<<<(g.Nx + 63) / 64, 64, 0, st>>>(p->twi + off, g.Mx);
+  count_launches(1);
+  // ---- per-axis tables of the binary64 H and preconditioner passes (AxT)
+  // with nu_k = k' pi / L (k' the signed index)
   {
     const int Ns[3] = {g.Nx, g.Ny, g.Nz};
     const double Ls[3] = {g.Lx, g.Ly, g.Lz}, hs[3] = {g.hx, g.hy, g.hz};
@@ -499,17 +609,17 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
     for (int ax = 0; ax < 3; ++ax) {
       const int n = Ns[ax];
       const double kap = kPi / Ls[ax], invn = 1.0 / (double)n;
-      std::vector<double> nuN(n), kinN(n), hnu2(n), xc(n), hxc2(n);
+      std::vector<double> nuN(n), kinN(n), hnu2(n), hxc2(n);
       for (int k = 0; k < n; ++k) {
         const int kk = k < n / 2 ? k : k - n;
         const double nu = (double)kk * kap;
-        nuN[k] = nu * invn;
         hnu2[k] = 0.5 * nu * nu;
+        nuN[k] = nu * invn;
         kinN[k] = hnu2[k] * invn;
-        xc[k] = -Ls[ax] + (double)k * hs[ax];
-        hxc2[k] = 0.5 * xc[k] * xc[k];
+        const double xc = -Ls[ax] + (double)k * hs[ax];
+        hxc2[k] = 0.5 * xc * xc;
       }
-      for (auto* v : {&nuN, &kinN, &hnu2, &xc, &hxc2}) tab.insert(tab.end(), v->begin(), v->end());
+      for (auto* v : {&nuN, &kinN, &hnu2, &hxc2}) tab.insert(tab.end(), v->begin(), v->end());
     }
     if ((e = dev_alloc(p, (void**)&p->axtab, tab.size() * sizeof(double))) != cudaSuccess)
       return bail(cuda_fail(nullptr, e, "plan axis tables"));
@@ -566,19 +676,46 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   free_tmp();
   if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan U0 precompute"));
-  // ---- z-pass multiplier on the half spectrum (FP64; copies below)
+  // ---- z-pass multiplier on the half spectrum: its largest value first, then
+  // the integers |K mant| 2^kq < 2^62.  The pass scales its tile to k_midbits
+  // bits, so that products over 2^64 stay within a transform's input (2^59),
+  // and adds k_midshift to the exponent: 64 - kq for the product's scale, and
+  // the exponent of 1 / (2 Mx My Mz).
   const size_t n_kz = (size_t)g.Mz * g.My * g.XS;
-  if ((e = dev_alloc(p, (void**)&p->Kz, n_kz * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan Kz"));
-  k_multiplier_half<<<(int)std::min<size_t>((n_kz + 255) / 256, 4096), 256, 0, st>>>(p->Kz, p->U0, g, p->n[0], p->n[1],
-                                                                                     p->n[2]);
-  count_launches(1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan Kz"));
+  if ((e = dev_alloc(p, (void**)&p->Kz, n_kz * sizeof(long long))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan Kz"));
+  {
+    const int grid = (int)std::min<size_t>((n_kz + 255) / 256, 4096);
+    int mexp = 0, kexp = 0;
+    const double mant = frexp(0.5 / ((double)g.Mx * g.My * g.Mz), &mexp);
+    unsigned long long* d_max = reinterpret_cast<unsigned long long*>(p->Kz);  // before the table fills it
+    unsigned long long bits = 0;
+    e = cudaMemsetAsync(d_max, 0, sizeof(bits), st);
+    if (e == cudaSuccess) {
+      k_multiplier_half<<<grid, 256, 0, st>>>(nullptr, d_max, p->U0, g, p->n[0], p->n[1], p->n[2], mant, 0.0);
+      e = cudaMemcpyAsync(&bits, d_max, sizeof(bits), cudaMemcpyDeviceToHost, st);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan Kz"));
+    double kmax = 0.0;
+    memcpy(&kmax, &bits, sizeof(kmax));
+    frexp(std::max(kmax, 1.0), &kexp);  // |K mant| < 2^kexp, kexp >= 1
+    const int kq = 62 - kexp;
+    p->k_midbits = std::min(62, 123 - kq - kexp);
+    p->k_midshift = 64 - kq + mexp;
+    k_multiplier_half<<<grid, 256, 0, st>>>(p->Kz, nullptr, p->U0, g, p->n[0], p->n[1], p->n[2], mant, ldexp(1.0, kq));
+    count_launches(2);
+    if ((e = cudaGetLastError()) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan Kz"));
+  }
   // ---- workspaces
   const size_t Nt = (size_t)g.Nx * g.Ny * g.Nz;
   const size_t n_w1 = (size_t)g.Nz * g.Ny * g.XS, n_w2 = (size_t)g.Nz * g.My * g.XS;
-  if ((e = dev_alloc(p, (void**)&p->W1, n_w1 * sizeof(double2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
-  if ((e = dev_alloc(p, (void**)&p->W2, n_w2 * sizeof(double2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
-  if ((e = dev_alloc(p, (void**)&p->T1, Nt * sizeof(double2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
+  if ((e = dev_alloc(p, (void**)&p->W1, n_w1 * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
+  if ((e = dev_alloc(p, (void**)&p->W2, n_w2 * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
+  if ((e = dev_alloc(p, (void**)&p->T1, Nt * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
+  // tile exponents: at most one per x line, or one per outer index and column
+  const size_t n_ex = std::max((size_t)g.Nz * g.Ny, (size_t)std::max(g.My, std::max(g.Nz, g.Ny)) * g.Xh);
+  for (int** q : {&p->ex[0], &p->ex[1], &p->ex[2]})
+    if ((e = dev_alloc(p, (void**)q, n_ex * sizeof(int))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = dev_alloc(p, (void**)&p->Pw, Nt * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if (flags & ATKM_PLAN_F32) {
     if ((e = dev_alloc(p, (void**)&p->W1f, n_w1 * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
@@ -586,11 +723,6 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
     if ((e = dev_alloc(p, (void**)&p->T1f, Nt * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
     if ((e = dev_alloc(p, (void**)&p->U0f, n_oct * sizeof(float))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan U0f"));
     k_to_f32<<<(int)std::min<size_t>((n_oct + 255) / 256, 4096), 256, 0, st>>>(p->U0f, p->U0, n_oct);
-    count_launches(1);
-  }
-  if (flags & ATKM_PLAN_DF32) {
-    if ((e = dev_alloc(p, (void**)&p->Kzd, n_kz * sizeof(df))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan Kzd"));
-    k_to_df<<<(int)std::min<size_t>((n_kz + 255) / 256, 4096), 256, 0, st>>>(p->Kzd, p->Kz, n_kz);
     count_launches(1);
   }
   // reductions: the largest CTA count of a reducing pass, or the vector grid
@@ -634,19 +766,19 @@ int atkm_plan_copy_multiplier(const atkm_plan* plan, double* dst, void* stream) 
 int dipolar_potential(atkm_plan* plan, const double* rho, double* phi, void* stream) {
   if (!plan || !rho || !phi) return fail(plan, ATKM_ERR_ARG, "dipolar_potential: NULL argument");
   if (rho == phi) return fail(plan, ATKM_ERR_ARG, "dipolar_potential: phi must not alias rho");
-  cudaError_t e = launch_atkm<double>(plan, SRC_RHO, rho, nullptr, phi, (cudaStream_t)stream);
+  cudaError_t e = launch_atkm64(plan, false, SRC_RHO, rho, nullptr, phi, (cudaStream_t)stream);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(plan, e, "dipolar_potential");
 }
 
 int dipolar_potential_from_psi(atkm_plan* plan, const double* psi, double* phi, void* stream) {
   if (!plan || !psi || !phi) return fail(plan, ATKM_ERR_ARG, "dipolar_potential_from_psi: NULL argument");
-  cudaError_t e = launch_atkm<double>(plan, SRC_PSI, psi, nullptr, phi, (cudaStream_t)stream);
+  cudaError_t e = launch_atkm64(plan, false, SRC_PSI, psi, nullptr, phi, (cudaStream_t)stream);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(plan, e, "dipolar_potential_from_psi");
 }
 
 int dipolar_potential_from_pair(atkm_plan* plan, const double* a, const double* b, double* phi, void* stream) {
   if (!plan || !a || !b || !phi) return fail(plan, ATKM_ERR_ARG, "dipolar_potential_from_pair: NULL argument");
-  cudaError_t e = launch_atkm<double>(plan, SRC_PAIR, a, b, phi, (cudaStream_t)stream);
+  cudaError_t e = launch_atkm64(plan, false, SRC_PAIR, a, b, phi, (cudaStream_t)stream);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(plan, e, "dipolar_potential_from_pair");
 }
 
@@ -661,7 +793,7 @@ int dipolar_potential_from_psi_df32(atkm_plan* plan, const double* psi, double* 
   if (!plan || !psi || !phi) return fail(plan, ATKM_ERR_ARG, "dipolar_potential_from_psi_df32: NULL argument");
   if (!(plan->flags & ATKM_PLAN_DF32))
     return fail(plan, ATKM_ERR_ARG, "dipolar_potential_from_psi_df32: plan lacks ATKM_PLAN_DF32");
-  cudaError_t e = launch_atkm<df>(plan, SRC_PSI, psi, nullptr, phi, (cudaStream_t)stream);
+  cudaError_t e = launch_atkm64(plan, true, SRC_PSI, psi, nullptr, phi, (cudaStream_t)stream);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(plan, e, "dipolar_potential_from_psi_df32");
 }
 
@@ -669,7 +801,7 @@ int apply_H(atkm_plan* plan, const atkm_params* prm, const double* f, const doub
             double* Hf, void* stream) {
   if (!plan || !prm || !f || !phi || !Phi || !Hf) return fail(plan, ATKM_ERR_ARG, "apply_H: NULL argument");
   if (Hf == f || Hf == phi || Hf == Phi) return fail(plan, ATKM_ERR_ARG, "apply_H: output aliases an input");
-  cudaError_t e = launch_H<double>(plan, make_phys(prm), f, phi, Phi, Hf, -1, (cudaStream_t)stream);
+  cudaError_t e = launch_H64(plan, false, make_phys(prm), f, phi, Phi, Hf, -1, (cudaStream_t)stream);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(plan, e, "apply_H");
 }
 
@@ -758,14 +890,14 @@ int atkm_spectral_upsample(atkm_plan* coarse, atkm_plan* fine, const double* psi
   }
   cudaStream_t st = (cudaStream_t)stream;
   const size_t nc = (size_t)gc.Nx * gc.Ny * gc.Nz;
-  cudaError_t e = cudaMemcpyAsync(coarse->T1, psi_c, nc * sizeof(double2), cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess) e = launch_cfft3<double>(coarse, coarse->T1, -1, st);
+  cudaError_t e = cudaMemcpyAsync((void*)coarse->T1, psi_c, nc * sizeof(double2), cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess) e = launch_cfft3(coarse, reinterpret_cast<double2*>(coarse->T1), -1, st);
   if (e == cudaSuccess) {
-    k_embed_spectrum<<<1216, 256, 0, st>>>(coarse->T1, reinterpret_cast<double2*>(psi_f), gc, gf, 1.0 / (double)nc);
+    k_embed_spectrum<<<1216, 256, 0, st>>>(reinterpret_cast<const double2*>(coarse->T1), reinterpret_cast<double2*>(psi_f), gc, gf, 1.0 / (double)nc);
     count_launches(1);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = launch_cfft3<double>(fine, reinterpret_cast<double2*>(psi_f), 1, st);
+  if (e == cudaSuccess) e = launch_cfft3(fine, reinterpret_cast<double2*>(psi_f), 1, st);
   return e == cudaSuccess ? ATKM_OK : cuda_fail(fine, e, "atkm_spectral_upsample");
 }
 

@@ -1,17 +1,17 @@
 // FFT-tile autotuner.  Without it, a pass's engine and tile width follow a
 // fixed rule (ops.cuh, pass_grid): the power-of-two register engine where the
-// line length allows it, else the mixed-radix register engine (3 * 2^a, and
-// 5 * 2^a outside binary64), else the generic shared-memory engine at a tile
+// line length allows it, else (FP32) the mixed-radix register engine (3 * 2^a
+// and 5 * 2^a), else the generic shared-memory engine at a tile
 // width narrowed until the pass has two CTAs per SM.  The tuner replaces the
 // rule by measurement for every line length of the plan that is not a power
-// of two, per arithmetic the plan carries (binary64, and FP32 / double-word
-// with ATKM_PLAN_F32 / ATKM_PLAN_DF32) and per layout (the line-major x pass,
-// the strided y and z passes).  Candidates: the mixed-radix register engine
-// where run_pass instantiates it (3 * 2^a and 5 * 2^a up to 384 in FP32,
-// 3 * 2^a in binary64, none in double-word) and the
-// generic engine at its default tile width, half of it and a quarter of it.
+// of two, per arithmetic the plan carries (binary64, and FP32 / the
+// double-word form with ATKM_PLAN_F32 / ATKM_PLAN_DF32) and per layout (the
+// line-major x pass, the strided y and z passes).  Candidates: in FP32 the
+// mixed-radix register engine where run_pass instantiates it (3 * 2^a and
+// 5 * 2^a up to 384), and the generic engine of the arithmetic at its default
+// tile width, half of it and a quarter of it.
 // Each candidate is timed on the plan's own operators -- the ATKM of |psi|^2,
-// H psi and P r (no preconditioner in double-word) -- with CUDA events, the
+// H psi and P r (no preconditioner in the double-word form) -- with CUDA events, the
 // best of three runs after a warm-up, while every other length keeps its
 // current choice; lengths are tuned one after another in the order x, then
 // the padded and unpadded y and z lengths.  Timing and selection support of
@@ -45,16 +45,16 @@ struct Scratch {
 cudaError_t run_ops(atkm_plan* p, int r, const Phys& ph, const Scratch& s, cudaStream_t st) {
   cudaError_t e;
   if (r == 0) {
-    e = launch_atkm<double>(p, SRC_PSI, s.psi, nullptr, s.Phi, st);
-    if (e == cudaSuccess) e = launch_H<double>(p, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
-    if (e == cudaSuccess) e = launch_precond<double>(p, ph, s.alpha, s.psi, s.psi, s.Phi, s.out, st);
+    e = launch_atkm64(p, false, SRC_PSI, s.psi, nullptr, s.Phi, st);
+    if (e == cudaSuccess) e = launch_H64(p, false, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
+    if (e == cudaSuccess) e = launch_precond64(p, ph, s.alpha, s.psi, s.psi, s.Phi, s.out, st);
   } else if (r == 1) {
     e = launch_atkm<float>(p, SRC_PSI, s.psi, nullptr, s.Phi, st);
     if (e == cudaSuccess) e = launch_H<float>(p, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
     if (e == cudaSuccess) e = launch_precond<float>(p, ph, s.alpha, s.psi, s.psi, s.Phi, s.out, st);
   } else {
-    e = launch_atkm<df>(p, SRC_PSI, s.psi, nullptr, s.Phi, st);
-    if (e == cudaSuccess) e = launch_H<df>(p, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
+    e = launch_atkm64(p, true, SRC_PSI, s.psi, nullptr, s.Phi, st);
+    if (e == cudaSuccess) e = launch_H64(p, true, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
   }
   return e;
 }
@@ -78,7 +78,7 @@ cudaError_t time_ops(atkm_plan* p, int r, const Phys& ph, const Scratch& s, cuda
 }
 
 bool default_mix(const atkm_plan* p, int r, int L) {
-  return !(p->flags & ATKM_PLAN_GENERIC_FFT) && mix_ok_r(r, L);
+  return !(p->flags & ATKM_PLAN_GENERIC_FFT) && r == 1 && mix_len(L);
 }
 
 }  // namespace
@@ -126,7 +126,7 @@ int atkm_plan_autotune(atkm_plan* plan, void* stream) {
         seen = seen || (plan->tune[i].r == r && plan->tune[i].L == L && plan->tune[i].lm == lm);
       if (seen || plan->n_tune >= kMaxTune) continue;
       std::vector<std::pair<int, int>> cand;
-      if (!(plan->flags & ATKM_PLAN_GENERIC_FFT) && mix_ok_r(r, L)) cand.push_back({1, 0});
+      if (!(plan->flags & ATKM_PLAN_GENERIC_FFT) && r == 1 && mix_len(L)) cand.push_back({1, 0});
       for (int sh = 0; sh <= 2; ++sh) cand.push_back({0, sh});
       TuneEntry& te = plan->tune[plan->n_tune++];
       te.r = r;
