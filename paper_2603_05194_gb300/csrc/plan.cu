@@ -11,10 +11,12 @@
 // the evaluation below is this library's own:
 //   * s in [0, s_lo]: I_a(s) = I_a(0) + O(s^2) (head term s_lo prod I_a(0));
 //   * s in [s_lo, s_c], s_c = 7 / min_a a_a: composite 16-point Gauss-Legendre
-//     in tau = ln s; I_a by composite Gauss-Legendre in y, written as
-//     2 int_0^a expm1(-s^2 y^2) cos(nu y) dy + 2a [k = 0] so the small-s
-//     rounding floor scales with s^2, and with the cosine phase reduced
-//     exactly (integer part of k u taken mod 2) before cospi;
+//     in tau = ln s; I_a in closed form: with x = nu / (2 s), y = s a and
+//     sin(nu a) = 0, I_a = (sqrt(pi)/s) (e^{-x^2} - (-1)^k e^{-y^2} Re w(x + i y))
+//     (w the Faddeeva function, see re_w), so that I_a keeps its relative
+//     accuracy where it is small (a quadrature in y left an absolute error of
+//     about 1e-16 a there, which nu^2 raised to 2e-13 in K: ten times the
+//     rounding of a whole dipolar potential);
 //     if s a_a >= 7 the box edge is invisible to double precision and
 //     I_a = (sqrt(pi)/s) e^{-nu^2/(4 s^2)};
 //   * s >= s_c: every factor is Gaussian, the integral is closed form
@@ -101,11 +103,6 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w) {
   }
 }
 
-struct GLNodes {
-  double x[kGL];  // nodes mapped to (0, 1)
-  double w[kGL];  // weights for (0, 1)
-};
-
 // Unevaluated sums of two binary64 numbers (about 106 bits) for the integer
 // twiddles: Knuth's TwoSum, the FMA product error (Dekker; Ogita, Rump and
 // Oishi 2005).
@@ -186,40 +183,61 @@ __global__ void k_post_twist(int4* w, int M) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M / 2; k += gridDim.x * blockDim.x) w[k] = int_twiddle(k, M, 61);
 }
 
+// Re w(x + i y) of the Faddeeva function w(z) = (i/pi) int e^{-t^2}/(z - t) dt
+// for x >= 0, y > 0 with x y >= pi/2 (its use below: x y = pi k / 2).  |z| < 8:
+// the trapezoidal rule with step h = 1/2 and its pole correction (Chiarella
+// and Reichel 1968; Matta and Reichel 1971), error e^{-(pi/h)^2} = 7e-18; its
+// real part is a sum of positive terms.  Beyond: the asymptotic series
+// i/(sqrt(pi) z) sum_m (2m-1)!!/(2 z^2)^m, 22 terms.
+constexpr int kWNodes = 16;  // t = 0, h, ..., 15 h (7.5)
+struct WNodes {
+  double e[kWNodes];  // e^{-t^2}
+};
+__device__ double re_w(double x, double y, const WNodes& nd) {
+  const double r2 = x * x + y * y;
+  if (r2 >= 64.0) {
+    // q = 1 / (2 z^2) = (qr + i qi), Horner from the last term
+    const double f = 0.5 / (r2 * r2), qr = f * (x - y) * (x + y), qi = -2.0 * f * x * y;
+    double sr = 1.0, si = 0.0;
+    for (int m = 22; m >= 1; --m) {
+      const double c = 2.0 * m - 1.0;
+      const double tr = sr * qr - si * qi, ti = sr * qi + si * qr;
+      sr = 1.0 + c * tr;
+      si = c * ti;
+    }
+    return (y * sr - x * si) / (r2 * sqrt(kPi));  // Re (i S / (sqrt(pi) z))
+  }
+  const double h = 0.5, y2 = y * y;
+  double sum = nd.e[0] / r2;
+  for (int n = 1; n < kWNodes; ++n) {
+    const double t = h * n, u = x - t, v = x + t;
+    sum += nd.e[n] * (1.0 / (u * u + y2) + 1.0 / (v * v + y2));
+  }
+  double w = h * y / kPi * sum;
+  // Re (2 e^{-z^2} / (1 - e^{-2 pi i z / h}))
+  const double g = 2.0 * kPi * y / h;
+  if (g < 80.0) {
+    double sz, cz, sp, cp;
+    sincos(2.0 * x * y, &sz, &cz);         // e^{-z^2} = e^{y^2 - x^2} (cz - i sz)
+    sincospi(2.0 * x / h, &sp, &cp);       // e^{-2 pi i z / h} = e^g (cp - i sp)
+    const double eg = exp(g), dr = 1.0 - eg * cp, di = eg * sp;
+    w += 2.0 * exp((y - x) * (y + x)) * (cz * dr - sz * di) / (dr * dr + di * di);
+  }
+  return w;
+}
+
 // table[q * (N + 1) + k] = I(s_q; nu_k), nu_k = pi k / a, k = 0..N.
 __global__ void k_axis_table(double* __restrict__ table, const double* __restrict__ s_nodes, int Q, int N,
-                             double a, GLNodes gl) {
+                             double a, WNodes nd) {
   const int total = Q * (N + 1);
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < total; id += gridDim.x * blockDim.x) {
     const int q = id / (N + 1), k = id - q * (N + 1);
-    const double s = s_nodes[q];
+    const double s = s_nodes[q], y = s * a, x = kPi * k / (2.0 * a * s);
     double val;
-    if (s * a >= kEdge) {
-      const double nu = kPi * k / a;
-      val = sqrt(kPi) / s * exp(-nu * nu / (4.0 * s * s));
-    } else {
-      // 2 a int_0^1 expm1(-(s a u)^2) cospi(k u) du (+ 2a when k = 0),
-      // P panels of width 1/P; Neumaier-compensated sum.
-      const int P = k / 2 + 2;
-      const long twoP = 2L * P;
-      double sum = 0.0, comp = 0.0;
-      for (int pnl = 0; pnl < P; ++pnl) {
-        const double base = (double)(((long)k * pnl) % twoP) / (double)P;  // exact reduction
-        for (int i = 0; i < kGL; ++i) {
-          const double xi = gl.x[i];
-          const double u = (pnl + xi) / P;
-          const double su = s * a * u;
-          const double th = base + (double)k * xi / (double)P;
-          const double term = gl.w[i] * expm1(-su * su) * cospi(th);
-          const double tsum = sum + term;
-          comp += (fabs(sum) >= fabs(term)) ? (sum - tsum) + term : (term - tsum) + sum;
-          sum = tsum;
-        }
-      }
-      val = 2.0 * a * (sum + comp) / P;
-      if (k == 0) val += 2.0 * a;
-    }
-    table[id] = val;
+    if (k == 0) val = erf(y);
+    else if (y >= kEdge) val = exp(-x * x);
+    else val = exp(-x * x) - ((k & 1) ? -1.0 : 1.0) * exp(-y * y) * re_w(x, y, nd);
+    table[id] = sqrt(kPi) / s * val;
   }
 }
 
@@ -637,19 +655,20 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   const int Q = npan * kGL;
   std::vector<double> gx, gw;
   gauss_legendre(kGL, gx, gw);
-  GLNodes gl01;
-  for (int i = 0; i < kGL; ++i) {
-    gl01.x[i] = 0.5 * (gx[i] + 1.0);
-    gl01.w[i] = 0.5 * gw[i];
+  for (int i = 0; i < kGL; ++i) {  // onto (0, 1)
+    gx[i] = 0.5 * (gx[i] + 1.0);
+    gw[i] *= 0.5;
   }
+  WNodes nd;
+  for (int i = 0; i < kWNodes; ++i) nd.e[i] = exp(-0.25 * i * i);
   std::vector<double> s_nodes(Q), w_nodes(Q);
   const double wpan = (tau_c - tau_lo) / npan;
   for (int pnl = 0; pnl < npan; ++pnl)
     for (int i = 0; i < kGL; ++i) {
-      const double tau = tau_lo + wpan * (pnl + gl01.x[i]);
+      const double tau = tau_lo + wpan * (pnl + gx[i]);
       const double s = exp(tau);
       s_nodes[pnl * kGL + i] = s;
-      w_nodes[pnl * kGL + i] = wpan * gl01.w[i] * s;  // ds = s dtau
+      w_nodes[pnl * kGL + i] = wpan * gw[i] * s;  // ds = s dtau
     }
   const size_t n_oct = (size_t)(g.Nx + 1) * (g.Ny + 1) * (g.Nz + 1);
   if ((e = dev_alloc(p, (void**)&p->U0, n_oct * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan U0"));
@@ -666,7 +685,7 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   if (e == cudaSuccess) {
     for (int ax = 0; ax < 3; ++ax) {
       const int tot = Q * (N[ax] + 1);
-      k_axis_table<<<(tot + 127) / 128, 128, 0, st>>>(d_T[ax], d_s, Q, N[ax], a[ax], gl01);
+      k_axis_table<<<(tot + 127) / 128, 128, 0, st>>>(d_T[ax], d_s, Q, N[ax], a[ax], nd);
     }
     k_U0<<<(int)std::min<size_t>((n_oct + 255) / 256, 65535), 256, 0, st>>>(p->U0, d_T[0], d_T[1], d_T[2], d_w, Q,
                                                                           g.Nx, g.Ny, g.Nz, a[0], a[1], a[2], s_c);
