@@ -17,7 +17,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libatkm.so")
-SOURCES = ["plan.cu", "ipasses_a.cu", "ipasses_h.cu", "ipasses_p.cu", "passes_f32.cu", "passes_f32_a.cu", "passes_f32_h.cu",
+SOURCES = ["plan.cu", "ipasses_a.cu", "ipasses_ax.cu", "ipasses_ay.cu", "ipasses_az.cu", "ipasses_h.cu", "ipasses_hx.cu",
+           "ipasses_hy.cu", "ipasses_hz.cu", "ipasses_p.cu", "ipasses_px.cu", "ipasses_py.cu", "ipasses_pz.cu", "passes_f32.cu", "passes_f32_a.cu", "passes_f32_h.cu",
            "pcg.cu", "noalloc.cu", "guess_net.cu", "measure.cu", "tune.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr"]

@@ -355,11 +355,15 @@ __device__ __forceinline__ void block_reduce_store_f32(float (&acc)[NS], double*
 // e^{-2 pi i k r / (Ns R)} = (c.h, c.l, s.h, s.l) at w[off[s] + (r - 1) Ns + k]
 // in units 2^(stage_shift(R) - 64): a thread's R - 1 twiddles lie at fixed
 // distances, and those of neighbouring k next to each other.
+// wm, wr: the same tables for the orders of the engine k_imix (its list and the
+// reversed one), where the length is one of int_radices.
 struct IntLen {
   int L, nst, shift;  // shift: the exponent that a transform adds
   int rad[kMaxStages], off[kMaxStages];
   unsigned mns[kMaxStages], mnb[kMaxStages];
   const int4* w;
+  const int4* wm;
+  const int4* wr;
 };
 
 // Per-axis tables of a plan (binary64, length N_a each): nu_k / N_a,

@@ -184,6 +184,55 @@ template <int S> struct IDft<6, S> {
 // Scale (a power of two) that a stage of radix R applies with its twiddles.
 __host__ __device__ constexpr int stage_shift(int rad) { return rad > 4 ? 3 : 2; }
 
+// The composite lengths with an engine of their own (k_imix), radices in
+// ascending order; n = 0: none.
+#define ATKM_IMIX_LENGTHS(F) \
+  F(18) F(20) F(24) F(30) F(36) F(40) F(48) F(60) F(72) F(80) F(90) F(96) F(100) F(108) F(120) F(144) F(150) F(160) F(180) \
+  F(192) F(200) F(216) F(240) F(288) F(320) F(384)
+struct RadList {
+  int n;
+  int r[3];
+};
+__host__ __device__ constexpr RadList int_radices(int L) {
+  switch (L) {
+    case 18: return {2, {3, 6, 0}};
+    case 20: return {2, {4, 5, 0}};
+    case 24: return {2, {4, 6, 0}};
+    case 30: return {2, {5, 6, 0}};
+    case 36: return {2, {6, 6, 0}};
+    case 40: return {2, {5, 8, 0}};
+    case 48: return {2, {6, 8, 0}};
+    case 60: return {3, {3, 4, 5}};
+    case 72: return {3, {3, 4, 6}};
+    case 80: return {3, {4, 4, 5}};
+    case 90: return {3, {3, 5, 6}};
+    case 96: return {3, {4, 4, 6}};
+    case 100: return {3, {4, 5, 5}};
+    case 108: return {3, {3, 6, 6}};
+    case 120: return {3, {4, 5, 6}};
+    case 144: return {3, {4, 6, 6}};
+    case 150: return {3, {5, 5, 6}};
+    case 160: return {3, {4, 5, 8}};
+    case 180: return {3, {5, 6, 6}};
+    case 192: return {3, {4, 6, 8}};
+    case 200: return {3, {5, 5, 8}};
+    case 216: return {3, {6, 6, 6}};
+    case 240: return {3, {5, 6, 8}};
+    case 288: return {3, {6, 6, 8}};
+    case 320: return {3, {5, 8, 8}};
+    case 384: return {3, {6, 8, 8}};
+    default: return {0, {0, 0, 0}};
+  }
+}
+// Lines of a k_imix tile: a power of two (the tile exponents are found by
+// shifts), at least 8 (128-byte rows of a column tile), about 320 threads.
+__host__ __device__ constexpr int imix_tile(int L) {
+  const int M = L / int_radices(L).r[0];
+  int T = 8;
+  while (2 * T * M <= 320 && T < 64) T *= 2;
+  return T;
+}
+
 // ------------------------------------------------------------ conversions
 // |hi word| of a component: its largest over a tile gives the tile's size.
 __device__ __forceinline__ unsigned mag(long long v) {

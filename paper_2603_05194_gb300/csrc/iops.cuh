@@ -4,6 +4,8 @@
 //   * k_ifast: power-of-two lengths 16 ... 1024, 8 elements a thread in
 //     registers, radix-8 stages (plus one radix-2/4 stage) exchanged through
 //     shared memory;
+//   * k_imix: the composite lengths of int_radices, one butterfly a thread in
+//     every stage;
 //   * k_igen: every other {2,3,5}-smooth length up to 2048, radix-8/6/5/4/3/2
 //     stages between two shared-memory tiles.
 // A pass whose input is binary64 finds its tile's largest exponent and turns
@@ -52,7 +54,7 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   static constexpr bool kTwin = false;      // the input is formed from the elements k and L - k
   static constexpr bool kZeroUpper = false; // positions >= L/2 of the input are zero
   static constexpr bool kHalfOut = false;   // only positions < L/2 of the output are used
-  static constexpr bool kNyqTail = false;   // column pass over columns 0..Nx (see ipass_line)
+  static constexpr bool kNyqTail = false;   // column pass over columns 0..Nx (see ipass_place)
   static constexpr bool kMul = false;       // the spectral step is mul_tile
   static constexpr int kMinB = 3;           // CTAs per SM that the register engine is compiled for
   static constexpr bool kPre = false;       // the spectral step's 8-byte table entries are prefetched (op.table)
@@ -72,47 +74,48 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
 // position j + P r of its line.
 struct Line {
   int t, j, o, x;
-  bool ok, exit;
+  bool ok;
 };
 
-template <class Op> __device__ __forceinline__ Line ipass_line(const Op& op, int T, int P) {
-  Line l;
-  l.exit = false;
+// The line of a thread with l->t set; true: the CTA has none.
+template <class Op> __device__ __forceinline__ bool ipass_place(const Op& op, int T, Line* l) {
   if (Op::kLM) {
-    l.t = threadIdx.x / P;
-    l.j = threadIdx.x - l.t * P;
-    l.o = blockIdx.x * T + l.t;
-    l.x = 0;
-    l.ok = op.valid(l.o, 0);
-    return l;
+    l->o = blockIdx.x * T + l->t;
+    l->x = 0;
+    l->ok = op.valid(l->o, 0);
+    return false;
   }
-  l.j = threadIdx.x / T;
-  l.t = threadIdx.x - l.j * T;
-  l.o = blockIdx.y;
-  l.x = blockIdx.x * T + l.t;
+  l->o = blockIdx.y;
+  l->x = blockIdx.x * T + l->t;
   if constexpr (Op::kNyqTail) {
     // Half-spectrum column passes (columns 0..Nx): when T divides Nx the last
     // block column would carry column Nx alone; it takes column Nx of T
     // consecutive rows instead, so that no CTA transforms idle columns.
     if (blockIdx.x == gridDim.x - 1 && op.Nx % T == 0) {
-      if (blockIdx.y * T >= gridDim.y) {
-        l.exit = true;
-        return l;
-      }
-      l.x = op.Nx;
-      l.o = blockIdx.y * T + l.t;
-      l.ok = l.o < (int)gridDim.y && op.valid(l.o, l.x);
-      return l;
+      l->x = op.Nx;
+      l->o = blockIdx.y * T + l->t;
+      l->ok = l->o < (int)gridDim.y && op.valid(l->o, l->x);
+      return blockIdx.y * T >= gridDim.y;
     }
   }
-  l.ok = op.valid(l.o, l.x);
-  return l;
+  l->ok = op.valid(l->o, l->x);
+  return false;
+}
+template <class Op> __device__ __forceinline__ bool ipass_line(const Op& op, int T, int P, Line* l) {
+  if (Op::kLM) {
+    l->t = threadIdx.x / P;
+    l->j = threadIdx.x - l->t * P;
+  } else {
+    l->j = threadIdx.x / T;
+    l->t = threadIdx.x - l->j * T;
+  }
+  return ipass_place(op, T, l);
 }
 
 // Scratch of the tile-wide reductions, one slot per use so that no barrier is
 // needed between a slot's readers and the next use.
 template <bool TWIN> struct TileRedT {
-  unsigned m[4][8];
+  unsigned m[4][16];
   int nan[128];
 };
 template <> struct TileRedT<true> : TileRedT<false> {
@@ -120,23 +123,27 @@ template <> struct TileRedT<true> : TileRedT<false> {
 };
 using TileRed = TileRedT<false>;
 
-__device__ __forceinline__ unsigned tile_or(unsigned v, unsigned* slot) {
+// Over a CTA of NW warps.
+template <int NW> __device__ __forceinline__ unsigned tile_or(unsigned v, unsigned* slot) {
   v = __reduce_or_sync(0xffffffffu, v);
   if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
   __syncthreads();
-  const uint4 a = *reinterpret_cast<const uint4*>(slot), b = *reinterpret_cast<const uint4*>(slot + 4);
-  return a.x | a.y | a.z | a.w | b.x | b.y | b.z | b.w;
+  unsigned r = 0;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) r |= slot[i];
+  return r;
 }
-
-__device__ __forceinline__ unsigned tile_max(unsigned v, unsigned* slot) {
+template <int NW> __device__ __forceinline__ unsigned tile_max(unsigned v, unsigned* slot) {
   v = __reduce_max_sync(0xffffffffu, v);
   if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
   __syncthreads();
-  const uint4 a = *reinterpret_cast<const uint4*>(slot), b = *reinterpret_cast<const uint4*>(slot + 4);
-  return max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
+  unsigned r = 0;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) r = max(r, slot[i]);
+  return r;
 }
-__device__ __forceinline__ int tile_max_s(int v, unsigned* slot) {
-  return (int)(tile_max((unsigned)v ^ 0x80000000u, slot) ^ 0x80000000u);
+template <int NW> __device__ __forceinline__ int tile_max_s(int v, unsigned* slot) {
+  return (int)(tile_max<NW>((unsigned)v ^ 0x80000000u, slot) ^ 0x80000000u);
 }
 
 __device__ __forceinline__ unsigned dmag(double2 z) {
@@ -154,7 +161,7 @@ struct Tile {
 // Loads a thread's E elements (guarded by pos < L) as integers of the tile's
 // common exponent, components below 2^59 (2^60 when the first stage sees a
 // zero upper half, unless the post-twist needs the room).
-template <int E, bool FULL, class Op>
+template <int E, bool FULL, int NW, class Op>
 __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], TileRed& tr) {
   constexpr int EL = Op::kZeroUpper ? (E + 1) / 2 : E;  // elements that can lie below L/2 (P E >= L)
   const int lim = Op::kZeroUpper ? L / 2 : L;
@@ -168,7 +175,7 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
       d[r] = (l.ok && (FULL || pos < lim)) ? op.load(l.o, l.x, pos) : make_double2(0.0, 0.0);
       m = max(m, dmag(d[r]));
     }
-    unsigned M = tile_max(m, tr.m[0]);
+    unsigned M = tile_max<NW>(m, tr.m[0]);
     bool bad = false, any = false;
     if (M >= 0x7ff00000u) {  // a NaN or an infinity: the lines that hold one are left out of the tile's size
       if (threadIdx.x < 128) tr.nan[threadIdx.x] = 0;
@@ -185,7 +192,7 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
         if (bad) d[r] = make_double2(0.0, 0.0);
         m = max(m, dmag(d[r]));
       }
-      M = tile_max(m, tr.m[1]);
+      M = tile_max<NW>(m, tr.m[1]);
     }
     const int ex = max((int)(M >> 20), 64);
     const int base = 64 - B + ex;
@@ -203,7 +210,7 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
       ee[r] = in ? op.lexp(l.o, l.x, pos) : -0x40000000;
       em = max(em, ee[r]);
     }
-    em = tile_max_s(em, tr.m[0]);
+    em = tile_max_s<NW>(em, tr.m[0]);
     if (em >= kExpNaN / 2) {  // uniform in the CTA
 #pragma unroll
       for (int r = 0; r < E; ++r) v[r] = cz();
@@ -217,7 +224,7 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
       v[r].y = shr_clamp(v[r].y, d);
       m |= mag(v[r]);
     }
-    const int sh = B - mag_bits(tile_or(m, tr.m[1]));
+    const int sh = B - mag_bits(tile_or<NW>(m, tr.m[1]));
 #pragma unroll
     for (int r = 0; r < E; ++r) v[r] = r < EL ? cshift(v[r], sh) : cz();
     return Tile{em - sh, false, false};
@@ -227,7 +234,7 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
 // The same for an op that forms its input from the elements k and L - k of
 // the stored half spectrum (op.combine): loads the elements, and element L
 // into *last for the threads of position 0, scaled to 60 bits.
-template <int E, bool FULL, class Op>
+template <int E, bool FULL, int NW, class Op>
 __device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, int L, c64 (&v)[E], c64* last, TileRed& tr) {
   int ev[E], el = -0x40000000;
   *last = cz();
@@ -244,7 +251,7 @@ __device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, in
     ev[r] = in ? op.lexp(l.o, pos) : -0x40000000;
     em = max(em, ev[r]);
   }
-  em = tile_max_s(em, tr.m[0]);
+  em = tile_max_s<NW>(em, tr.m[0]);
   if (em >= kExpNaN / 2) {
 #pragma unroll
     for (int r = 0; r < E; ++r) v[r] = cz();
@@ -260,7 +267,7 @@ __device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, in
     v[r] = c64{shr_clamp(v[r].x, d), shr_clamp(v[r].y, d)};
     m |= mag(v[r]);
   }
-  const int sh = 60 - mag_bits(tile_or(m, tr.m[1]));
+  const int sh = 60 - mag_bits(tile_or<NW>(m, tr.m[1]));
   *last = cshift(*last, sh);
 #pragma unroll
   for (int r = 0; r < E; ++r) v[r] = cshift(v[r], sh);
@@ -269,17 +276,17 @@ __device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, in
 
 // Scales the tile up to BITS = op.midbits() bits and applies the op's
 // spectral step to every element.
-template <int E, bool FULL, class Op>
+template <int E, bool FULL, int NW, class Op>
 __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], int* e,
                                          typename Op::Acc& acc, unsigned* slot, const long long* pre) {
   unsigned m = 0;
 #pragma unroll
   for (int r = 0; r < E; ++r) m |= mag(v[r]);
-  const int sh = op.midbits() - mag_bits(tile_or(m, slot));
+  const int sh = op.midbits() - mag_bits(tile_or<NW>(m, slot));
 #pragma unroll
   for (int r = 0; r < E; ++r) {
     const int pos = l.j + P * r;
-    if (l.ok && (FULL || pos < L)) v[r] = op.spectral(l.o, l.x, pos, cshift(v[r], sh), acc, FULL && Op::kPre ? pre + r * kThreads : nullptr);
+    if (l.ok && (FULL || pos < L)) v[r] = op.spectral(l.o, l.x, pos, cshift(v[r], sh), acc, Op::kPre && pre ? pre + r * (NW * 32) : nullptr);
   }
   *e -= sh;
   acc.e = *e;
@@ -292,13 +299,13 @@ __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int
 // the tile's largest one.  (With the multiplier in fixed point, nu^2 / 2 of
 // the low frequencies, 2^-18 of the largest at length 1024, would leave the
 // product 2^18 fewer units.)
-template <int E, bool FULL, class Op>
+template <int E, bool FULL, int NW, class Op>
 __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], Tile& tl,
                                          typename Op::Acc& acc, TileRed& tr) {
   unsigned m = 0;
 #pragma unroll
   for (int r = 0; r < E; ++r) m |= mag(v[r]);
-  const int sh = 62 - mag_bits(tile_or(m, tr.m[2]));
+  const int sh = 62 - mag_bits(tile_or<NW>(m, tr.m[2]));
   acc.e = tl.e - sh;
   int ex[E];
   int eb = -0x40000000;
@@ -319,7 +326,7 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
       eb = max(eb, 32 - __clz((int)mag(v[r])) + ex[r]);  // bits of the aligned product, less 32
     }
   }
-  const int M = tile_max_s(eb, tr.m[3]);
+  const int M = tile_max_s<NW>(eb, tr.m[3]);
 #pragma unroll
   for (int r = 0; r < E; ++r) {
     const int s = kInBits - 32 - M + ex[r], lf = max(s, 0), rt = min(max(-s, 0), 64);
@@ -334,8 +341,22 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
   }
 }
 
-template <int NR> __device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* part, int pstride) {
-  block_reduce_store<NR>(acc, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
+// Block sums of the threads' NR values through shared memory (NR NW 256 bytes,
+// free of other use), one warp a value: each lane adds NW values and the warp
+// shuffles once, 12 binary64 additions a warp and value at 8 warps (a shuffle
+// tree in every warp took 40).
+template <int NR, int NW> __device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* sh, double* part, int pstride) {
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NR; ++i) sh[i * (NW * 32) + threadIdx.x] = acc[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < NR; i += NW) {
+    double v = sh[i * (NW * 32) + lane];
+    for (int w = 1; w < NW; ++w) v += sh[i * (NW * 32) + w * 32 + lane];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) part[i * pstride + blockIdx.y * gridDim.x + blockIdx.x] = v;
+  }
 }
 
 // ------------------------------------------------------------ k_ifast
@@ -432,8 +453,8 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
   c64* b0 = reinterpret_cast<c64*>(ism);
   // [r][thread]: this thread's table entries
   long long* pre = reinterpret_cast<long long*>(ism + C::template bytes<Op::kLM>()) + threadIdx.x;
-  const Line l = ipass_line(op, C::T, C::TPL);
-  if (l.exit) return;  // the whole CTA
+  Line l;
+  if (ipass_line(op, C::T, C::TPL, &l)) return;  // the whole CTA
   if constexpr (Op::kPre) {
     if (l.ok) {
 #pragma unroll
@@ -445,7 +466,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
   Tile tl;
   if constexpr (Op::kTwin) {
     c64 last;
-    tl = load_twin<8, true>(op, l, C::TPL, L, v, &last, tr);
+    tl = load_twin<8, true, 8>(op, l, C::TPL, L, v, &last, tr);
 #pragma unroll
     for (int r = 0; r < 8; ++r) b0[C::template at<Op::kLM>(l.t, l.j + C::TPL * r)] = v[r];
     if (l.j == 0) tr.last[l.t] = last;
@@ -457,7 +478,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
     }
     __syncthreads();
   } else {
-    tl = load_tile<8, true>(op, l, C::TPL, L, v, tr);
+    tl = load_tile<8, true, 8>(op, l, C::TPL, L, v, tr);
   }
   typename Op::Acc acc{};
   constexpr bool kLo1 = Op::kHalfOut && !Op::kSecond && !Op::kMirror;
@@ -479,8 +500,8 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
     if constexpr (Op::kSecond) {
       if constexpr (Op::kPre) asm volatile("cp.async.wait_all;\n" ::: "memory");
       // its barrier also frees b0
-      if constexpr (Op::kMul) mul_tile<8, true>(op, l, C::TPL, L, v, tl, acc, tr);
-      else mid_tile<8, true>(op, l, C::TPL, L, v, &tl.e, acc, tr.m[2], pre);
+      if constexpr (Op::kMul) mul_tile<8, true, 8>(op, l, C::TPL, L, v, tl, acc, tr);
+      else mid_tile<8, true, 8>(op, l, C::TPL, L, v, &tl.e, acc, tr.m[2], pre);
       ifast_fft<L, -Op::kSign1, Op::kLM, false, Op::kHalfOut>(v, b0, w, l.t, l.j);
       tl.e += C::SHIFT;
     }
@@ -493,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
   if constexpr (Op::kRed > 0) {
     double a[Op::kRed];
     op.sums(l, acc, tl, a);
-    ireduce_out<Op::kRed>(a, op.part, op.pstride);
+    ireduce_out<Op::kRed, 8>(a, reinterpret_cast<double*>(ism), op.part, op.pstride);
   }
 }
 
@@ -573,13 +594,13 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
   c64* a = reinterpret_cast<c64*>(ism);
   const GenTile g(T, tsh, L);
   c64* b = a + T * g.LP;
-  const Line l = ipass_line(op, T, P);
-  if (l.exit) return;  // the whole CTA
+  Line l;
+  if (ipass_line(op, T, P, &l)) return;  // the whole CTA
   c64 v[kGenE];
   Tile tl;
   if constexpr (Op::kTwin) {
     c64 last;
-    tl = load_twin<kGenE, false>(op, l, P, L, v, &last, tr);
+    tl = load_twin<kGenE, false, 8>(op, l, P, L, v, &last, tr);
 #pragma unroll
     for (int r = 0; r < kGenE; ++r) {
       const int pos = l.j + P * r;
@@ -593,7 +614,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
       if (pos < L) v[r] = op.combine(pos, v[r], pos == 0 ? tr.last[l.t] : b[g.template at<Op::kLM>(l.t, L - pos)]);
     }
   } else {
-    tl = load_tile<kGenE, false>(op, l, P, L, v, tr);
+    tl = load_tile<kGenE, false, 8>(op, l, P, L, v, tr);
   }
   typename Op::Acc acc{};
 #pragma unroll
@@ -617,8 +638,8 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
     }
     if constexpr (Op::kSecond) {
       // its barrier also frees the tile
-      if constexpr (Op::kMul) mul_tile<kGenE, false>(op, l, P, L, v, tl, acc, tr);
-      else mid_tile<kGenE, false>(op, l, P, L, v, &tl.e, acc, tr.m[2], nullptr);
+      if constexpr (Op::kMul) mul_tile<kGenE, false, 8>(op, l, P, L, v, tl, acc, tr);
+      else mid_tile<kGenE, false, 8>(op, l, P, L, v, &tl.e, acc, tr.m[2], nullptr);
 #pragma unroll
       for (int r = 0; r < kGenE; ++r) {
         const int pos = l.j + P * r;
@@ -645,7 +666,218 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
   if constexpr (Op::kRed > 0) {
     double s[Op::kRed];
     op.sums(l, acc, tl, s);
-    ireduce_out<Op::kRed>(s, op.part, op.pstride);
+    ireduce_out<Op::kRed, 8>(s, reinterpret_cast<double*>(ism), op.part, op.pstride);
+  }
+}
+
+// ------------------------------------------------------------ k_imix
+// Composite lengths known at compile time (int_radices): radices in ascending
+// order, one butterfly a thread in every stage.  A line has M = L / R0 threads;
+// in a stage of radix R the first L / R of them work (in a column tile whole
+// warps then idle; a line-major tile deals its butterflies out anew each
+// stage).  The inputs of the first stage and the outputs of the last one stay
+// in registers, and the inverse transform takes the radices in the opposite
+// order, so that its first stage finds its inputs in the registers where the
+// forward transform left them.
+template <int L> struct IMix {
+  static constexpr RadList R = int_radices(L);
+  static constexpr int n = R.n, R0 = R.r[0], RL = R.r[R.n - 1];
+  static constexpr int M = L / R0, ML = L / RL;
+  static constexpr int T = imix_tile(L);
+  static constexpr int NW = (T * M + 31) / 32;
+  static constexpr int LP = L + L / 8 + 1;
+  static constexpr int fshift() {
+    int v = 0;
+    for (int s = 1; s < n; ++s) v += stage_shift(R.r[s]);
+    return v;
+  }
+  static constexpr int rshift() {
+    int v = 0;
+    for (int s = 0; s < n - 1; ++s) v += stage_shift(R.r[s]);
+    return v;
+  }
+  // one pad element every 8 positions in a line-major tile; a column tile's
+  // rows have at least 128 bytes
+  template <bool LM> __device__ static __forceinline__ int at(int t, int pos) {
+    return LM ? t * LP + pos + (pos >> 3) : pos * T + t;
+  }
+  template <class Op> static constexpr size_t bytes() {
+    const size_t tile = (size_t)T * (Op::kLM ? LP : L) * sizeof(c64), red = (size_t)Op::kRed * NW * 32 * sizeof(double);
+    return tile > red ? tile : red;
+  }
+  // CTAs per SM: 768 threads at up to 85 registers, 512 at up to 128
+  template <class Op> static constexpr int minb() { return (Op::kMinB == 3 ? 768 : 512) / (NW * 32) > 0 ? (Op::kMinB == 3 ? 768 : 512) / (NW * 32) : 1; }
+};
+
+// The (t, j) of a thread in a stage with nb butterflies a line; false: none.
+template <int L, bool LM> __device__ __forceinline__ bool imix_map(int nb, int* t, int* j) {
+  constexpr int T = IMix<L>::T;
+  if (LM) {
+    *t = threadIdx.x / nb;
+    *j = threadIdx.x - *t * nb;
+  } else {
+    *j = threadIdx.x / T;
+    *t = threadIdx.x - *j * T;
+  }
+  return threadIdx.x < T * nb;
+}
+
+template <int L, int RAD, bool LM> __device__ __forceinline__ void imix_read(c64 (&v)[RAD], const c64* b, int t, int j) {
+  constexpr int nb = L / RAD;
+  if constexpr (!LM || nb % 8 == 0) {
+    const c64* p = b + IMix<L>::template at<LM>(t, j);
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) v[r] = p[LM ? r * (nb + nb / 8) : r * nb * IMix<L>::T];
+  } else {
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) v[r] = b[IMix<L>::template at<LM>(t, j + r * nb)];
+  }
+}
+template <int L, int RAD, int NS, bool LM> __device__ __forceinline__ void imix_write(const c64 (&v)[RAD], c64* b, int t, int j) {
+  const int k = j % NS, base = (j - k) * RAD + k;
+#pragma unroll
+  for (int r = 0; r < RAD; ++r) b[IMix<L>::template at<LM>(t, base + r * NS)] = v[r];
+}
+
+// Stage i > 0 of the order (REV: the opposite order) up to its DFT.
+template <int L, int S, bool LM, bool REV, int I> struct IStage {
+  using C = IMix<L>;
+  static constexpr int rad(int i) { return C::R.r[REV ? C::n - 1 - i : i]; }
+  static constexpr int ns(int i) {
+    int v = 1;
+    for (int q = 0; q < i; ++q) v *= rad(q);
+    return v;
+  }
+  static constexpr int off(int i) {  // of the stage's twiddles
+    int o = 0;
+    for (int q = 1; q < i; ++q) o += (rad(q) - 1) * ns(q);
+    return o;
+  }
+  static constexpr int RAD = rad(I), NS = ns(I);
+  template <bool LO> static __device__ __forceinline__ void go(c64 (&v)[RAD], const c64* b, const int4* __restrict__ w, int t, int j) {
+    imix_read<L, RAD, LM>(v, b, t, j);
+    const int4* wk = w + off(I) + j % NS;
+    v[0] = crsh<stage_shift(RAD)>(v[0]);
+#pragma unroll
+    for (int r = 1; r < RAD; ++r) v[r] = tmul<S>(v[r], __ldg(wk + (r - 1) * NS));
+    IDft<RAD, S>::template go<false, LO>(v);
+  }
+};
+// Stages 1 ... n - 2 in shared memory (entered and left synchronised).
+template <int L, int S, bool LM, bool REV, int I> __device__ __forceinline__ void imix_middle(c64* b, const int4* __restrict__ w) {
+  using C = IMix<L>;
+  if constexpr (I < C::n - 1) {
+    using St = IStage<L, S, LM, REV, I>;
+    c64 v[St::RAD];
+    int t, j;
+    const bool on = imix_map<L, LM>(L / St::RAD, &t, &j);
+    if (on) St::template go<false>(v, b, w, t, j);
+    __syncthreads();
+    if (on) imix_write<L, St::RAD, St::NS, LM>(v, b, t, j);
+    __syncthreads();
+    imix_middle<L, S, LM, REV, I + 1>(b, w);
+  }
+}
+
+template <int L, class Op>
+__global__ void __launch_bounds__(IMix<L>::NW * 32, IMix<L>::template minb<Op>())
+k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
+  using C = IMix<L>;
+  constexpr bool LM = Op::kLM;
+  extern __shared__ __align__(16) unsigned char ism[];
+  __shared__ __align__(16) TileRedT<Op::kTwin> tr;
+  c64* b = reinterpret_cast<c64*>(ism);
+  // la: this thread's line and elements j + M r; lb: those of the last stage, j + ML r
+  Line la, lb;
+  const bool ona = imix_map<L, LM>(C::M, &la.t, &la.j), onb = imix_map<L, LM>(C::ML, &lb.t, &lb.j);
+  if (ipass_place(op, C::T, &la)) return;  // the whole CTA
+  ipass_place(op, C::T, &lb);
+  la.ok = la.ok && ona;
+  lb.ok = lb.ok && onb;
+  if (!ona) la.t = 0, la.j = 1;
+  if (!onb) lb.t = 0, lb.j = 1;
+  c64 v[C::R0];
+  Tile tl;
+  if constexpr (Op::kTwin) {
+    c64 last;
+    tl = load_twin<C::R0, true, C::NW>(op, la, C::M, L, v, &last, tr);
+    if (ona) {
+#pragma unroll
+      for (int r = 0; r < C::R0; ++r) b[C::template at<LM>(la.t, la.j + C::M * r)] = v[r];
+      if (la.j == 0) tr.last[la.t] = last;
+    }
+    __syncthreads();
+    if (ona) {
+#pragma unroll
+      for (int r = 0; r < C::R0; ++r) {
+        const int pos = la.j + C::M * r;
+        v[r] = op.combine(pos, v[r], pos == 0 ? tr.last[la.t] : b[C::template at<LM>(la.t, L - pos)]);
+      }
+    }
+    __syncthreads();
+  } else {
+    // positions from L / 2 on are zero for kZeroUpper: with an odd radix they begin inside an element's range
+    tl = load_tile<C::R0, !Op::kZeroUpper || C::R0 % 2 == 0, C::NW>(op, la, C::M, L, v, tr);
+  }
+  typename Op::Acc acc{};
+  constexpr bool kZU = Op::kZeroUpper && (C::R0 == 4 || C::R0 == 8);
+  IDft<C::R0, Op::kSign1>::template go<kZU, false>(v);
+  if (ona) imix_write<L, C::R0, 1, LM>(v, b, la.t, la.j);
+  __syncthreads();
+  imix_middle<L, Op::kSign1, LM, false, 1>(b, wf);
+  c64 u[C::RL];
+  constexpr bool kLO = Op::kHalfOut && C::RL % 2 == 0;
+  if (onb) IStage<L, Op::kSign1, LM, false, C::n - 1>::template go<kLO && !Op::kSecond && !Op::kMirror>(u, b, wf, lb.t, lb.j);
+  tl.e += C::fshift();
+  if constexpr (Op::kMirror) {
+    __syncthreads();
+    if (onb) {
+#pragma unroll
+      for (int r = 0; r < C::RL; ++r) b[C::template at<LM>(lb.t, lb.j + C::ML * r)] = u[r];
+    }
+    __syncthreads();
+    if (lb.ok) {
+#pragma unroll
+      for (int r = 0; r < C::RL; ++r) {
+        const int k = lb.j + C::ML * r;
+        op.post(lb.o, k, u[r], b[C::template at<LM>(lb.t, k == 0 ? 0 : L - k)]);
+      }
+    }
+  } else if constexpr (Op::kSecond) {
+    if (!onb) {
+#pragma unroll
+      for (int r = 0; r < C::RL; ++r) u[r] = cz();
+    }
+    // its barriers also free the tile
+    if constexpr (Op::kMul) mul_tile<C::RL, true, C::NW>(op, lb, C::ML, L, u, tl, acc, tr);
+    else mid_tile<C::RL, true, C::NW>(op, lb, C::ML, L, u, &tl.e, acc, tr.m[2], nullptr);
+    IDft<C::RL, -Op::kSign1>::template go<false, false>(u);
+    if (onb) imix_write<L, C::RL, 1, LM>(u, b, lb.t, lb.j);
+    __syncthreads();
+    imix_middle<L, -Op::kSign1, LM, true, 1>(b, wr);
+    if (la.ok) {
+      IStage<L, -Op::kSign1, LM, true, C::n - 1>::template go<Op::kHalfOut && C::R0 % 2 == 0>(v, b, wr, la.t, la.j);
+      tl.e += C::rshift();
+#pragma unroll
+      for (int r = 0; r < (Op::kHalfOut ? (C::R0 + 1) / 2 : C::R0); ++r) {
+        const int pos = la.j + C::M * r;
+        if (!Op::kHalfOut || C::R0 % 2 == 0 || pos < L / 2) op.store(la.o, la.x, pos, v[r], tl, acc);
+      }
+    }
+  } else {
+    if (lb.ok) {
+#pragma unroll
+      for (int r = 0; r < (Op::kHalfOut ? (C::RL + 1) / 2 : C::RL); ++r) {
+        const int pos = lb.j + C::ML * r;
+        if (!Op::kHalfOut || C::RL % 2 == 0 || pos < L / 2) op.store(lb.o, lb.x, pos, u[r], tl, acc);
+      }
+    }
+  }
+  op.put_exp(la, tl);
+  if constexpr (Op::kRed > 0) {
+    double a[Op::kRed];
+    op.sums(lb, acc, tl, a);
+    ireduce_out<Op::kRed, C::NW>(a, reinterpret_cast<double*>(ism), op.part, op.pstride);
   }
 }
 
@@ -653,7 +885,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
 struct IPassGrid {
   dim3 grid;
   int T, tsh;
-  bool fast;
+  bool fast, mix;
 };
 
 inline int ilog2(int v) {
@@ -666,11 +898,16 @@ inline int ilog2(int v) {
 // The tiles of the generic engine are powers of two, narrowed until the pass
 // has two CTAs per SM (a column tile not below 8, which keeps its accesses in
 // whole 128-byte lines).
-inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long lines, int X, int outer) {
+inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long lines, int X, int outer, bool mix = true) {
   IPassGrid pg;
   pg.fast = L >= 16 && L <= 1024 && (L & (L - 1)) == 0;
+  pg.mix = mix && !pg.fast && int_radices(L).n > 0 && !(p->flags & ATKM_PLAN_GENERIC_FFT);
+  for (int i = 0; i < p->n_tune; ++i)
+    if (p->tune[i].r == r && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0) && p->tune[i].shift > 0) pg.mix = false;
   if (pg.fast) {
     pg.T = kIElems / L;
+  } else if (pg.mix) {
+    pg.T = imix_tile(L);
   } else {
     int T = 1 << ilog2(std::min(128, std::max(1, kGenMax / L)));
     const long want = 2L * device_sm_count();
@@ -713,7 +950,26 @@ inline cudaError_t launch_ifast(const Op& op, const IntLen& f, const IPassGrid& 
   return cudaGetLastError();
 }
 
-template <class Op> inline cudaError_t irun(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
+template <int L, class Op>
+inline cudaError_t launch_imix(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
+  static std::atomic<unsigned long long> prepared{0};
+  constexpr size_t sm = IMix<L>::template bytes<Op>();
+  cudaError_t e = iprepare(prepared, k_imix<L, Op>, sm);
+  if (e != cudaSuccess) return e;
+  k_imix<L, Op><<<pg.grid, IMix<L>::NW * 32, sm, st>>>(op, f.wm, f.wr);
+  return cudaGetLastError();
+}
+
+template <bool MIX, class Op> inline cudaError_t irun(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
+  if constexpr (MIX) {
+    if (pg.mix) switch (f.L) {
+#define ATKM_IMIX_CASE(L) \
+  case L: return launch_imix<L>(op, f, pg, st);
+      ATKM_IMIX_LENGTHS(ATKM_IMIX_CASE)
+#undef ATKM_IMIX_CASE
+      default: return cudaErrorInvalidValue;
+    }
+  }
   if (pg.fast) {
     switch (f.L) {
       case 16: return launch_ifast<16>(op, f, pg, st);
@@ -731,7 +987,8 @@ template <class Op> inline cudaError_t irun(const Op& op, const IntLen& f, const
   constexpr size_t most = (size_t)2 * (kGenMax + kGenMax / 8 + 128) * sizeof(c64);
   cudaError_t e = iprepare(prepared, k_igen<Op>, most);
   if (e != cudaSuccess) return e;
-  k_igen<Op><<<pg.grid, kThreads, (size_t)2 * pg.T * (f.L + f.L / 8 + 1) * sizeof(c64), st>>>(op, f, pg.T, pg.tsh);
+  const size_t sm = std::max((size_t)2 * pg.T * (f.L + f.L / 8 + 1) * sizeof(c64), (size_t)Op::kRed * kThreads * sizeof(double));
+  k_igen<Op><<<pg.grid, kThreads, sm, st>>>(op, f, pg.T, pg.tsh);
   return cudaGetLastError();
 }
 

@@ -600,8 +600,8 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   size_t twtot = 0;
   for (int i = 0; i < 6; ++i) twtot += lens[i];
   if ((e = dev_alloc(p, (void**)&p->tw32, twtot * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
-  // a length's stage tables take less than its length
-  if ((e = dev_alloc(p, (void**)&p->twi, (twtot + g.Nx) * sizeof(int4))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
+  // a length's stage tables take less than its length, for each order
+  if ((e = dev_alloc(p, (void**)&p->twi, (3 * twtot + g.Nx) * sizeof(int4))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
   size_t off = 0;
   for (int i = 0; i < 6; ++i) {
     FftLen& f = (i < 3) ? p->fN[i] : p->fM[i - 3];
@@ -609,14 +609,31 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
     if (!make_fft_len(lens[i], f) || !make_int_len(lens[i], fi))
       return bail(fail(nullptr, ATKM_ERR_UNSUPPORTED_SIZE, "plan: FFT factorisation"));
     f.tw32 = p->tw32 + off;
-    fi.w = p->twi + off;
+    int4* const tw = p->twi + 3 * off;
+    fi.w = tw;
+    fi.wm = tw + lens[i];
+    fi.wr = tw + 2 * lens[i];
     k_twiddles<<<(lens[i] + 127) / 128, 128, 0, st>>>(p->tw32 + off, lens[i]);
-    k_int_twiddles<<<(lens[i] + 63) / 64, 64, 0, st>>>(p->twi + off, fi);
+    k_int_twiddles<<<(lens[i] + 63) / 64, 64, 0, st>>>(tw, fi);
     count_launches(2);
+    if (const RadList rl = int_radices(lens[i]); rl.n > 0) {
+      for (int rev = 0; rev < 2; ++rev) {
+        IntLen o{};
+        o.nst = rl.n;
+        for (int s = 0, Ns = 1, at = 0; s < rl.n; ++s) {
+          o.rad[s] = rl.r[rev ? rl.n - 1 - s : s];
+          o.off[s] = at;
+          if (s) at += (o.rad[s] - 1) * Ns;
+          Ns *= o.rad[s];
+        }
+        k_int_twiddles<<<(lens[i] + 63) / 64, 64, 0, st>>>(tw + (1 + rev) * lens[i], o);
+        count_launches(1);
+      }
+    }
     off += lens[i];
   }
-  p->tw_x = p->twi + off;
-  k_post_twist<<<(g.Nx + 63) / 64, 64, 0, st>>>(p->twi + off, g.Mx);
+  p->tw_x = p->twi + 3 * off;
+  k_post_twist<<<(g.Nx + 63) / 64, 64, 0, st>>>(p->twi + 3 * off, g.Mx);
   count_launches(1);
   // ---- per-axis tables of the binary64 H and preconditioner passes (AxT)
   // with nu_k = k' pi / L (k' the signed index)
