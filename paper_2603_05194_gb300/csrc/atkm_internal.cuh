@@ -105,6 +105,35 @@ inline int device_sm_count() {
   return v;
 }
 
+// Programmatic dependent launch: a kernel started by launch_pdl may be resident
+// before its predecessor in the stream has ended, which hides the launch gap
+// (1 to 2 us, as long as a small pass itself).  It calls pdl_trigger() at its
+// start (its own successor may be placed as soon as all its CTAs are) and
+// pdl_wait() before its first access to memory that an earlier kernel reads or
+// writes: the wait ends when the predecessor has completed, which had itself
+// waited for its own.  Tables written at plan creation may be read before it.
+// Everything else is read by plain loads: a load through the read-only path
+// (__ldg, const __restrict__) may be moved ahead of the wait, or find a line
+// cached before it.  Kernels that read that way are launched in the ordinary
+// way (no wait needed) and may still trigger.  Both calls are without effect
+// in an ordinary launch.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ------------------------------------------------------------- FFT engine
 // A CTA transforms T lines of length L held in shared memory.  Stockham
 // auto-sort formulation (Govindaraju et al., "High performance discrete
@@ -349,6 +378,72 @@ __device__ __forceinline__ void block_reduce_store_f32(float (&acc)[NS], double*
   }
 }
 
+// The last block of a grid to arrive here (every thread of the block calls it;
+// `wrote`: the threads that wrote the block's partial results): true in that
+// block only, whose threads then see every block's partial results (read them
+// with __ldcg).  It leaves *cnt at zero for the next kernel of the stream.  A
+// reduction finished this way needs no second launch.  Only the writers fence:
+// the block's other stores need not have arrived.
+__device__ __forceinline__ bool last_block(unsigned* cnt, bool wrote) {
+  __shared__ int last;
+  if (wrote) __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned n = gridDim.x * gridDim.y;
+    last = atomicAdd(cnt, 1u) == n - 1u;
+    if (last) {
+      *cnt = 0u;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last != 0;
+}
+// Grid sums of the block sums part[s * nblocks + i], s < NS, by one block of
+// 256 threads in a fixed order: thread t adds i = t, t + 256, ..., then a tree
+// over the threads (pairs 128, 64, 32, ... apart).  All NS sums go through it
+// together (one after another they took about 2 us each).
+template <int NS> __device__ __forceinline__ void finalize_sums(const double* part, int nblocks, double* out) {
+  static_assert(NS <= 8, "one warp a sum");
+  __shared__ double fsh[NS][256];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  double acc[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) acc[s] = 0.0;
+#pragma unroll 2
+  for (int i = t; i < nblocks; i += 256) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) acc[s] += __ldcg(part + (size_t)s * nblocks + i);
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) fsh[s][t] = acc[s];
+  __syncthreads();
+#pragma unroll
+  for (int w = 128; w > 16; w >>= 1) {
+    if (t < w) {
+#pragma unroll
+      for (int s = 0; s < NS; ++s) fsh[s][t] += fsh[s][t + w];
+    }
+    __syncthreads();
+  }
+  if (warp < NS) {
+    double v = fsh[warp][lane];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) out[warp] = v;
+  }
+}
+// The same by a block of nw warps, one value a warp.
+__device__ __forceinline__ void finalize_sums_warps(const double* part, int nblocks, int ns, double* out, int nw) {
+  const int lane = threadIdx.x & 31;
+  for (int s = threadIdx.x >> 5; s < ns; s += nw) {
+    double acc = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < nblocks; i += 32) acc += __ldcg(part + (size_t)s * nblocks + i);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[s] = acc;
+  }
+}
+
 // A line length of the integer passes: its stages with the multiplicative
 // inverses of their divisors, and the stages' twiddles.  Stage s > 0 of radix R
 // after Ns = product of the earlier radices has (R - 1) Ns entries
@@ -441,6 +536,7 @@ struct atkm_plan {
   double* partials;    // reduction partials
   int partials_cap;    // doubles
   double* scal;        // device scalars
+  unsigned* cnt;       // arrival counter of last_block
   double* scal_host;   // pinned mirror
   atkm::PcgBuffers* pcg;
   atkm::TuneEntry tune[atkm::kMaxTune];  // autotuned engine choices (n_tune of them)
@@ -485,8 +581,7 @@ enum AtkmSrc { SRC_RHO = 0, SRC_PSI = 1, SRC_PAIR = 2 };
 template <typename R>
 cudaError_t launch_atkm(atkm_plan* p, int mode, const double* a, const double* b, double* phi,
                         cudaStream_t st);
-// H f; if red_slot >= 0 the per-pass energy reductions go to partials and are
-// finalised into scal[red_slot .. red_slot + 9].
+// H f; if red_slot >= 0 the energy sums go to scal[red_slot .. red_slot + 9].
 template <typename R>
 cudaError_t launch_H(atkm_plan* p, const Phys& ph, const double* f, const double* phi,
                      const double* Phi, double* Hf, int red_slot, cudaStream_t st);
@@ -505,9 +600,6 @@ cudaError_t launch_precond64(atkm_plan* p, const Phys& ph, const double* alpha_d
                              const double* Phi, double* Pr, cudaStream_t st);
 // In-place unnormalised 3D complex FFT (sign S) of buf on the plan's grid.
 cudaError_t launch_cfft3(atkm_plan* p, double2* buf, int sign, cudaStream_t st);
-
-// Reductions (pcg.cu)
-cudaError_t launch_finalize(atkm_plan* p, int nslots, int nblocks, int dst_slot, cudaStream_t st);
 
 Phys make_phys(const atkm_params* prm);
 

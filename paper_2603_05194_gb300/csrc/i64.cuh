@@ -184,10 +184,10 @@ template <int S> struct IDft<6, S> {
 // Scale (a power of two) that a stage of radix R applies with its twiddles.
 __host__ __device__ constexpr int stage_shift(int rad) { return rad > 4 ? 3 : 2; }
 
-// The composite lengths with an engine of their own (k_imix), radices in
-// ascending order; n = 0: none.
+// The lengths that the engine k_imix is built for, radices in ascending order;
+// n = 0: none.
 #define ATKM_IMIX_LENGTHS(F) \
-  F(18) F(20) F(24) F(30) F(36) F(40) F(48) F(60) F(72) F(80) F(90) F(96) F(100) F(108) F(120) F(144) F(150) F(160) F(180) \
+  F(16) F(32) F(64) F(128) F(256) F(18) F(20) F(24) F(30) F(36) F(40) F(48) F(60) F(72) F(80) F(90) F(96) F(100) F(108) F(120) F(144) F(150) F(160) F(180) \
   F(192) F(200) F(216) F(240) F(288) F(320) F(384)
 struct RadList {
   int n;
@@ -195,6 +195,11 @@ struct RadList {
 };
 __host__ __device__ constexpr RadList int_radices(int L) {
   switch (L) {
+    case 16: return {2, {4, 4, 0}};
+    case 32: return {2, {4, 8, 0}};
+    case 64: return {3, {4, 4, 4}};
+    case 128: return {3, {4, 4, 8}};
+    case 256: return {3, {4, 8, 8}};
     case 18: return {2, {3, 6, 0}};
     case 20: return {2, {4, 5, 0}};
     case 24: return {2, {4, 6, 0}};

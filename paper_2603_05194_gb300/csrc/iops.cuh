@@ -37,7 +37,7 @@ template <typename T> __device__ __forceinline__ T* step(T* p, int i, int stride
 struct ExpTab {
   int* e;
   int rs, cs, nc;
-  __device__ __forceinline__ int at(int row, int col) const { return __ldg(step(e + (col >> cs), row >> rs, nc * 4)); }
+  __device__ __forceinline__ int at(int row, int col) const { return *step(e + (col >> cs), row >> rs, nc * 4); }
 };
 
 constexpr int kInBits = 59;  // components of a transform's input stay below 2^59
@@ -60,6 +60,8 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   static constexpr bool kPre = false;       // the spectral step's 8-byte table entries are prefetched (op.table)
   double* part = nullptr;
   int pstride = 0;
+  double* sums_out = nullptr;  // where the last block leaves the grid sums
+  unsigned* cnt = nullptr;
   // bits the tile is scaled to before the spectral step, and the exponent
   // that the step adds
   __device__ __forceinline__ int midbits() const { return 62; }
@@ -345,7 +347,9 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
 // free of other use), one warp a value: each lane adds NW values and the warp
 // shuffles once, 12 binary64 additions a warp and value at 8 warps (a shuffle
 // tree in every warp took 40).
-template <int NR, int NW> __device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* sh, double* part, int pstride) {
+template <int NR, int NW>
+__device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* sh, double* part, int pstride, double* out,
+                                            unsigned* cnt) {
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < NR; ++i) sh[i * (NW * 32) + threadIdx.x] = acc[i];
@@ -357,6 +361,7 @@ template <int NR, int NW> __device__ __forceinline__ void ireduce_out(double (&a
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if (lane == 0) part[i * pstride + blockIdx.y * gridDim.x + blockIdx.x] = v;
   }
+  if (last_block(cnt, lane == 0)) finalize_sums_warps(part, pstride, NR, out, NW);
 }
 
 // ------------------------------------------------------------ k_ifast
@@ -454,6 +459,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
   // [r][thread]: this thread's table entries
   long long* pre = reinterpret_cast<long long*>(ism + C::template bytes<Op::kLM>()) + threadIdx.x;
   Line l;
+  pdl_trigger();
   if (ipass_line(op, C::T, C::TPL, &l)) return;  // the whole CTA
   if constexpr (Op::kPre) {
     if (l.ok) {
@@ -462,6 +468,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   }
+  pdl_wait();
   c64 v[8];
   Tile tl;
   if constexpr (Op::kTwin) {
@@ -514,7 +521,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
   if constexpr (Op::kRed > 0) {
     double a[Op::kRed];
     op.sums(l, acc, tl, a);
-    ireduce_out<Op::kRed, 8>(a, reinterpret_cast<double*>(ism), op.part, op.pstride);
+    ireduce_out<Op::kRed, 8>(a, reinterpret_cast<double*>(ism), op.part, op.pstride, op.sums_out, op.cnt);
   }
 }
 
@@ -595,7 +602,9 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
   const GenTile g(T, tsh, L);
   c64* b = a + T * g.LP;
   Line l;
+  pdl_trigger();
   if (ipass_line(op, T, P, &l)) return;  // the whole CTA
+  pdl_wait();
   c64 v[kGenE];
   Tile tl;
   if constexpr (Op::kTwin) {
@@ -666,7 +675,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
   if constexpr (Op::kRed > 0) {
     double s[Op::kRed];
     op.sums(l, acc, tl, s);
-    ireduce_out<Op::kRed, 8>(s, reinterpret_cast<double*>(ism), op.part, op.pstride);
+    ireduce_out<Op::kRed, 8>(s, reinterpret_cast<double*>(ism), op.part, op.pstride, op.sums_out, op.cnt);
   }
 }
 
@@ -790,12 +799,14 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   // la: this thread's line and elements j + M r; lb: those of the last stage, j + ML r
   Line la, lb;
   const bool ona = imix_map<L, LM>(C::M, &la.t, &la.j), onb = imix_map<L, LM>(C::ML, &lb.t, &lb.j);
+  pdl_trigger();
   if (ipass_place(op, C::T, &la)) return;  // the whole CTA
   ipass_place(op, C::T, &lb);
   la.ok = la.ok && ona;
   lb.ok = lb.ok && onb;
   if (!ona) la.t = 0, la.j = 1;
   if (!onb) lb.t = 0, lb.j = 1;
+  pdl_wait();
   c64 v[C::R0];
   Tile tl;
   if constexpr (Op::kTwin) {
@@ -877,7 +888,7 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   if constexpr (Op::kRed > 0) {
     double a[Op::kRed];
     op.sums(lb, acc, tl, a);
-    ireduce_out<Op::kRed, C::NW>(a, reinterpret_cast<double*>(ism), op.part, op.pstride);
+    ireduce_out<Op::kRed, C::NW>(a, reinterpret_cast<double*>(ism), op.part, op.pstride, op.sums_out, op.cnt);
   }
 }
 
@@ -904,6 +915,17 @@ inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long line
   pg.mix = mix && !pg.fast && int_radices(L).n > 0 && !(p->flags & ATKM_PLAN_GENERIC_FFT);
   for (int i = 0; i < p->n_tune; ++i)
     if (p->tune[i].r == r && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0) && p->tune[i].shift > 0) pg.mix = false;
+  // Power-of-two lengths up to 256 where the register engine's CTAs (2048
+  // elements, 8 a thread) would not give every SM one: k_imix has half the
+  // elements a thread and a CTA, so twice the warps share the work.
+  if (pg.fast && mix && int_radices(L).n > 0) {
+    const int T = kIElems / L;
+    const long ctas = LM ? (lines + T - 1) / T : (long)std::max(X / T, 1) * outer;
+    if (ctas < (long)device_sm_count()) {
+      pg.fast = false;
+      pg.mix = true;
+    }
+  }
   if (pg.fast) {
     pg.T = kIElems / L;
   } else if (pg.mix) {
@@ -946,8 +968,7 @@ inline cudaError_t launch_ifast(const Op& op, const IntLen& f, const IPassGrid& 
   constexpr size_t sm = IFast<L>::template bytes<Op::kLM>() + (Op::kPre ? (size_t)8 * 8 * kThreads : 0);
   cudaError_t e = iprepare(prepared, k_ifast<L, Op>, sm);
   if (e != cudaSuccess) return e;
-  k_ifast<L, Op><<<pg.grid, kThreads, sm, st>>>(op, f.w);
-  return cudaGetLastError();
+  return launch_pdl(k_ifast<L, Op>, pg.grid, kThreads, sm, st, op, f.w);
 }
 
 template <int L, class Op>
@@ -956,8 +977,7 @@ inline cudaError_t launch_imix(const Op& op, const IntLen& f, const IPassGrid& p
   constexpr size_t sm = IMix<L>::template bytes<Op>();
   cudaError_t e = iprepare(prepared, k_imix<L, Op>, sm);
   if (e != cudaSuccess) return e;
-  k_imix<L, Op><<<pg.grid, IMix<L>::NW * 32, sm, st>>>(op, f.wm, f.wr);
-  return cudaGetLastError();
+  return launch_pdl(k_imix<L, Op>, pg.grid, IMix<L>::NW * 32, sm, st, op, f.wm, f.wr);
 }
 
 template <bool MIX, class Op> inline cudaError_t irun(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
@@ -988,8 +1008,7 @@ template <bool MIX, class Op> inline cudaError_t irun(const Op& op, const IntLen
   cudaError_t e = iprepare(prepared, k_igen<Op>, most);
   if (e != cudaSuccess) return e;
   const size_t sm = std::max((size_t)2 * pg.T * (f.L + f.L / 8 + 1) * sizeof(c64), (size_t)Op::kRed * kThreads * sizeof(double));
-  k_igen<Op><<<pg.grid, kThreads, sm, st>>>(op, f, pg.T, pg.tsh);
-  return cudaGetLastError();
+  return launch_pdl(k_igen<Op>, pg.grid, kThreads, sm, st, op, f, pg.T, pg.tsh);
 }
 
 // ================================================================ ops
@@ -1273,8 +1292,8 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc& a) const {
     const size_t i0 = (size_t)o * Nx + x;
     const int pl = Ny * Nx;
-    const double2 fv = __ldg(step(f + i0, pos, pl * 16));
-    const double Pd = __ldg(step(Phi + i0, pos, pl * 8));
+    const double2 fv = *step(f + i0, pos, pl * 16);
+    const double Pd = *step(Phi + i0, pos, pl * 8);
     const c64 u = ldc(step(AX + i0, pos, pl * 16)), w = ldc(step(AY + i0, pos, pl * 16));
     const bool bad = t.bad || u.x == kBadElem || w.x == kBadElem;
     const int eu = ix.at(pos * Ny + o, 0), ew = iy.at(pos, x);
@@ -1287,7 +1306,7 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
     else if (i2d_ok(e)) kin = make_double2(i2d(sx, e + 1085), i2d(sy, e + 1085));
     else kin = make_double2(i2d_any(sx, e), i2d_any(sy, e));
     const double V = gz2 * hz2[pos] + (gy2 * hy2[o] + gx2 * hx2[x]);
-    const double2 pv = same ? fv : __ldg(step(phi + i0, pos, pl * 16));
+    const double2 pv = same ? fv : *step(phi + i0, pos, pl * 16);
     const double wt = V + beta * (pv.x * pv.x + pv.y * pv.y) + lambda * Pd;
     const double ox = kin.x + wt * fv.x, oy = kin.y + wt * fv.y;
     *step(Hf + i0, pos, pl * 16) = make_double2(ox, oy);
@@ -1396,7 +1415,7 @@ struct IPXI : IOpBase<1, false, 0, true, kSrcInt> {
   __device__ __forceinline__ int lexp(int o, int, int pos) const { return in.at(o / Ny, pos); }
   __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile& t, Acc&) const {
     const size_t i = (size_t)o * Nx + pos;
-    const double w = __ldg(Pw + i);
+    const double w = Pw[i];
     double2 d;
     if (i2d_ok(t.e)) d = make_double2(i2d(v.x, t.e + 1085), i2d(v.y, t.e + 1085));
     else d = make_double2(i2d_any(v.x, t.e), i2d_any(v.y, t.e));

@@ -13,14 +13,12 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   const double N = (double)g.Nx * g.Ny * g.Nz;
   const double pi = 3.14159265358979323846264338327950288, ky = pi / g.Ly;
   const double2* fin = reinterpret_cast<const double2*>(h.f);
-  cudaError_t e;
   IHY<RED> op;
   op.f = fin; op.A = p->W2; op.ex = exp_cols(p->ex[1], gy); op.Nx = g.Nx; op.Ny = g.Ny;
   op.ck = 0.5 * ky * ky / g.Ny; op.cr = -ph.Omega * ky / g.Ny;
   op.kin = iaxt(p, 1).kinN; op.nu = iaxt(p, 1).nuN; op.Om = ph.Omega; op.Lx = g.Lx; op.hx = g.hx;
-  op.part = p->partials; op.pstride = gy.grid.x * gy.grid.y;
+  op.part = p->partials; op.pstride = gy.grid.x * gy.grid.y; op.sums_out = p->scal + red_slot + 2; op.cnt = p->cnt;
   ATKM_IRUN(dw ? "H_y_df" : "H_y_f64", 32 * N, 2.0 * g.Nz * g.Nx * ifftflops(g.Ny), op, p->iN[1], gy);
-  if (RED && (e = launch_finalize(p, 2, op.pstride, red_slot + 2, st)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 }  // namespace

@@ -13,7 +13,6 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   const double N = (double)g.Nx * g.Ny * g.Nz;
   const double pi = 3.14159265358979323846264338327950288, kz = pi / g.Lz;
   const double2* fin = reinterpret_cast<const double2*>(h.f);
-  cudaError_t e;
   IHZ<RED> op;
   op.f = fin; op.phi = reinterpret_cast<const double2*>(h.phi); op.Phi = h.Phi; op.AX = p->T1; op.AY = p->W2;
   op.ix = exp_lines(p->ex[0], gx); op.iy = exp_cols(p->ex[1], gy);
@@ -21,9 +20,8 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   op.hx2 = iaxt(p, 0).hxc2; op.hy2 = iaxt(p, 1).hxc2; op.hz2 = iaxt(p, 2).hxc2;
   op.gx2 = ph.gx2; op.gy2 = ph.gy2; op.gz2 = ph.gz2; op.beta = ph.beta; op.lambda = ph.lambda;
   op.ck = 0.5 * kz * kz / g.Nz; op.same = h.f == h.phi;
-  op.part = p->partials; op.pstride = gz.grid.x * gz.grid.y;
+  op.part = p->partials; op.pstride = gz.grid.x * gz.grid.y; op.sums_out = p->scal + red_slot + 4; op.cnt = p->cnt;
   ATKM_IRUN(dw ? "H_z_df" : "H_z_f64", (op.same ? 72 : 88) * N, 2.0 * g.Ny * g.Nx * ifftflops(g.Nz), op, p->iN[2], gz);
-  if (RED && (e = launch_finalize(p, 6, op.pstride, red_slot + 4, st)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 }  // namespace

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mix(Op op, const cx<R>* __restr
       for (int e = 0; e < EH; ++e) op.store(o, x, j + C::TPL * e, v[e], acc);
     }
   }
-  if (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride);
+  if constexpr (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride, op.sums, op.cnt);
 }
 
 template <typename R, int L, class Op>

@@ -205,12 +205,15 @@ template <int S1, bool SECOND, int NRED, bool LM> struct OpBase {
   static constexpr bool kKeepIn = false;
   double* part = nullptr;                  // reduction partials [slot][block]
   int pstride = 0;
+  double* sums = nullptr;                  // where the last block leaves the grid sums
+  unsigned* cnt = nullptr;
 };
 
 // ------------------------------------------------------------ kernels
 template <typename R, int NR>
-__device__ __forceinline__ void reduce_out(R (&acc)[NR], double* part, int pstride) {
+__device__ __forceinline__ void reduce_out(R (&acc)[NR], double* part, int pstride, double* sums, unsigned* cnt) {
   block_reduce_store_f32<NR>(acc, part, pstride, blockIdx.y * gridDim.x + blockIdx.x);
+  if (last_block(cnt, threadIdx.x == 0)) finalize_sums<NR>(part, pstride, sums);
 }
 
 // CTAs per SM the fast engine is compiled for: 4 (64 registers); 3
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, fast_min_blocks<R, L, Op>()) k_fast(
       }
     }
   }
-  if (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride);
+  if constexpr (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride, op.sums, op.cnt);
 }
 
 template <typename R, class Op>
@@ -350,7 +353,7 @@ __global__ void __launch_bounds__(kThreads) k_generic(Op op, FftLen f, int T) {
       const int pm = pos == 0 ? 0 : L - pos;
       if (op.valid(o, x)) op.post(o, x, pos, tile[e], tile[tix<Op::kLM>(t, pm, T, L)], acc);
     }
-    if (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride);
+    if constexpr (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride, op.sums, op.cnt);
     return;
   }
   for (int e = threadIdx.x; e < T * L; e += kThreads) {
@@ -369,7 +372,7 @@ __global__ void __launch_bounds__(kThreads) k_generic(Op op, FftLen f, int T) {
     const int x = Op::kLM ? 0 : blockIdx.x * T + t;
     if (op.valid(o, x)) op.store(o, x, pos, tile[e], acc);
   }
-  if (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride);
+  if constexpr (Op::kRed > 0) reduce_out<R, NR>(acc, op.part, op.pstride, op.sums, op.cnt);
 }
 
 // ------------------------------------------------------------ dispatch

@@ -155,8 +155,7 @@ cudaError_t h_pass_x(atkm_plan* p, const Phys& ph, const double* f, const double
   double2* out = reinterpret_cast<double2*>(Hf);
   const double N = (double)g.Nx * g.Ny * g.Nz, s = (double)sizeof(cx<R>);
   const long nl = (long)g.Nz * g.Ny;
-  cudaError_t e;
-  (void)pin; (void)out; (void)nl; (void)pr; (void)e;
+  (void)pin; (void)out; (void)nl; (void)pr;
   // x
   {
     const PassGrid pg = pass_grid<R>(p, g.Nx, true, nl, 0, 0);
@@ -165,8 +164,8 @@ cudaError_t h_pass_x(atkm_plan* p, const Phys& ph, const double* f, const double
     if (red) {
       OpHX<R, true> op; op.f = fin; op.acc = acc; op.c = c; op.Omega = pr.Omega;
       op.part = p->partials; op.pstride = pg.grid.x * pg.grid.y;
+      op.sums = p->scal + red_slot + 0; op.cnt = p->cnt;
       ATKM_RUN(n, 16 * N + N * s, fl, op, p->fN[0], pg);
-      if ((e = launch_finalize(p, 2, pg.grid.x * pg.grid.y, red_slot + 0, st)) != cudaSuccess) return e;
     } else {
       OpHX<R, false> op; op.f = fin; op.acc = acc; op.c = c; op.Omega = pr.Omega;
       ATKM_RUN(n, 16 * N + N * s, fl, op, p->fN[0], pg);
@@ -189,8 +188,7 @@ cudaError_t h_pass_y(atkm_plan* p, const Phys& ph, const double* f, const double
   double2* out = reinterpret_cast<double2*>(Hf);
   const double N = (double)g.Nx * g.Ny * g.Nz, s = (double)sizeof(cx<R>);
   const long nl = (long)g.Nz * g.Ny;
-  cudaError_t e;
-  (void)pin; (void)out; (void)nl; (void)pr; (void)e;
+  (void)pin; (void)out; (void)nl; (void)pr;
   // y
   {
     const PassGrid pg = pass_grid<R>(p, g.Ny, false, 0, g.Nx, g.Nz);
@@ -199,8 +197,8 @@ cudaError_t h_pass_y(atkm_plan* p, const Phys& ph, const double* f, const double
     if (red) {
       OpHY<R, true> op; op.f = fin; op.acc = acc; op.c = c; op.Omega = pr.Omega;
       op.part = p->partials; op.pstride = pg.grid.x * pg.grid.y;
+      op.sums = p->scal + red_slot + 2; op.cnt = p->cnt;
       ATKM_RUN(n, 16 * N + 2 * N * s, fl, op, p->fN[1], pg);
-      if ((e = launch_finalize(p, 2, pg.grid.x * pg.grid.y, red_slot + 2, st)) != cudaSuccess) return e;
     } else {
       OpHY<R, false> op; op.f = fin; op.acc = acc; op.c = c; op.Omega = pr.Omega;
       ATKM_RUN(n, 16 * N + 2 * N * s, fl, op, p->fN[1], pg);
@@ -223,8 +221,7 @@ cudaError_t h_pass_z(atkm_plan* p, const Phys& ph, const double* f, const double
   double2* out = reinterpret_cast<double2*>(Hf);
   const double N = (double)g.Nx * g.Ny * g.Nz, s = (double)sizeof(cx<R>);
   const long nl = (long)g.Nz * g.Ny;
-  cudaError_t e;
-  (void)pin; (void)out; (void)nl; (void)pr; (void)e;
+  (void)pin; (void)out; (void)nl; (void)pr;
   // z + pointwise
   {
     const PassGrid pg = pass_grid<R>(p, g.Nz, false, 0, g.Nx, g.Ny);
@@ -235,8 +232,8 @@ cudaError_t h_pass_z(atkm_plan* p, const Phys& ph, const double* f, const double
      
       op.same = fin == pin;
       op.part = p->partials; op.pstride = pg.grid.x * pg.grid.y;
+      op.sums = p->scal + red_slot + 4; op.cnt = p->cnt;
       ATKM_RUN(n, (op.same ? 40 : 56) * N + N * s, fl, op, p->fN[2], pg);
-      if ((e = launch_finalize(p, 6, pg.grid.x * pg.grid.y, red_slot + 4, st)) != cudaSuccess) return e;
     } else {
       OpHZ<R, false> op; op.f = fin; op.phi = pin; op.Phi = Phi; op.acc = acc; op.Hf = out; op.c = c; op.ph = pr;
      

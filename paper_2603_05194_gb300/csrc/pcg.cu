@@ -68,38 +68,6 @@ struct Ctl {
   atkm_iter_log* log;  // device array of log_cap entries
 };
 
-// ------------------------------------------------------------ reductions
-__global__ void k_finalize(const double* __restrict__ part, int nblocks, double* __restrict__ out,
-                           const int* __restrict__ pred) {
-  if (pred && !*pred) return;
-  __shared__ double sh[kRedThreads];
-  const int s = blockIdx.x;
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nblocks; i += kRedThreads) acc += part[(size_t)s * nblocks + i];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[s] = sh[0];
-}
-
-// Grid maximum of the block maxima; out = its square root (the partials hold
-// squared distances).
-__global__ void k_finalize_max(const double* __restrict__ part, int nblocks, double* __restrict__ out) {
-  __shared__ double sh[kRedThreads];
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nblocks; i += kRedThreads) acc = fmax(acc, part[i]);
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[0] = sqrt(sh[0]);
-}
-
 // Vector kernels of the driver.  Vectors are FP64 in memory.  T is the type
 // of the per-element arithmetic: double in the FP64 phase; float in the FP32
 // phase of the precision form, where every operand carries FP32-level
@@ -168,135 +136,6 @@ template <typename T, int NS> struct Sums {
 #define ATKM_GRID_LOOP(j, N) \
   for (size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x; j < (N); j += (size_t)gridDim.x * blockDim.x)
 
-// sum_j Re(u_j conj(v_j)) (FP64).
-__global__ void __launch_bounds__(kRedThreads) k_dot(const double2* __restrict__ u, const double2* __restrict__ v,
-                                                     size_t N, double* __restrict__ part) {
-  Sums<double, 1> acc;
-  ATKM_GRID_LOOP(j, N) {
-    const double2 a = u[j], b = v[j];
-    acc.mac(0, a.x, b.x);
-    acc.mac(0, a.y, b.y);
-  }
-  acc.store(part);
-}
-
-// The seven sums of the direction step from one read of its five vectors:
-// <Pr,phi>, <r,Pr>, <r,phi>, <r_prev,Pr>, <r_prev,phi>, <p_prev,phi>, <phi,phi>.
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
-k_dir_dots(const double2* __restrict__ Pr, const double2* __restrict__ phi, const double2* __restrict__ r,
-           const double2* __restrict__ rp, const double2* __restrict__ pp, size_t N, double* __restrict__ part) {
-  Sums<T, 7> acc;
-  ATKM_GRID_LOOP(j, N) {
-    const V2<T> P = ld2<T>(Pr[j]), f = ld2<T>(phi[j]), a = ld2<T>(r[j]), b = ld2<T>(rp[j]), c = ld2<T>(pp[j]);
-    acc.dot(0, P, f);
-    acc.dot(1, a, P);
-    acc.dot(2, a, f);
-    acc.dot(3, b, P);
-    acc.dot(4, b, f);
-    acc.dot(5, c, f);
-    acc.dot(6, f, f);
-    acc.next();
-  }
-  acc.store(part);
-}
-
-// A coefficient m * (*p) (p may be null: then m).
-struct Coef {
-  const double* p;
-  double m;
-};
-__device__ __forceinline__ double cval(const Coef& c) { return c.p ? c.m * *c.p : c.m; }
-
-// out = c0 v0 + c1 v1 + c2 v2 (null vectors skipped); sums |out|^2 and
-// Re(w conj(out)) when w is given.  Skipped entirely when *pred == 0.
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
-k_lincomb(double2* __restrict__ out, const double2* __restrict__ v0, Coef c0, const double2* __restrict__ v1,
-          Coef c1, const double2* __restrict__ v2, Coef c2, const double2* __restrict__ w, size_t N,
-          double* __restrict__ part, const int* __restrict__ pred) {
-  if (pred && !*pred) return;
-  const T a0 = tor<T>(cval(c0)), a1 = tor<T>(cval(c1)), a2 = tor<T>(cval(c2));
-  Sums<T, 2> acc;
-  ATKM_GRID_LOOP(j, N) {
-    V2<T> o{(T)0, (T)0};
-    if (v0) { const V2<T> a = ld2<T>(v0[j]); o.x += a0 * a.x; o.y += a0 * a.y; }
-    if (v1) { const V2<T> a = ld2<T>(v1[j]); o.x += a1 * a.x; o.y += a1 * a.y; }
-    if (v2) { const V2<T> a = ld2<T>(v2[j]); o.x += a2 * a.x; o.y += a2 * a.y; }
-    out[j] = make_double2(tod<T>(o.x), tod<T>(o.y));
-    acc.dot(0, o, o);
-    if (w) acc.dot(1, ld2<T>(w[j]), o);
-    acc.next();
-  }
-  acc.store(part);
-}
-
-// phi+ *= *inv (FP64: the renormalisation); block max of |phi+ - phi|^2, the
-// difference taken in T (FP32 in the FP32 phase, where it is only logged).
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
-k_scale_linf(double2* __restrict__ phin, const double2* __restrict__ phi, const double* __restrict__ invp, size_t N,
-             double* __restrict__ part) {
-  __shared__ T sh[kRedThreads];
-  const double inv = *invp;
-  T m = (T)0;
-  ATKM_GRID_LOOP(j, N) {
-    double2 a = phin[j];
-    a.x *= inv; a.y *= inv;
-    phin[j] = a;
-    const V2<T> x = ld2<T>(a), y = ld2<T>(phi[j]);
-    const T dx = x.x - y.x, dy = x.y - y.y;
-    m = fmax(m, dx * dx + dy * dy);
-  }
-  sh[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = tod<T>(sh[0]);
-}
-
-// Sums for the curvature of the quadratic model:
-//   [0] <Hp, p>
-//   [1] sum rho'(beta rho' + lambda Phi'),  rho' = Re(conj(phi) p)
-//   [2] sum (beta|phi|^2 + lambda Phi) Re(phi conj(p))
-//   [3] sum (beta|phi|^2 + lambda Phi) |p|^2
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
-k_curv_sums(const double2* __restrict__ Hp, const double2* __restrict__ phi, const double2* __restrict__ p,
-            const double* __restrict__ Phi, const double* __restrict__ Phi1, double beta, double lambda, size_t N,
-            double* __restrict__ part) {
-  const T bt = tor<T>(beta), lm = tor<T>(lambda);
-  Sums<T, 4> acc;
-  ATKM_GRID_LOOP(j, N) {
-    const V2<T> a = ld2<T>(phi[j]), b = ld2<T>(p[j]), h = ld2<T>(Hp[j]);
-    const T rp = dotr(a, b);
-    const T w = bt * dotr(a, a) + lm * ld1<T>(Phi[j]);
-    acc.dot(0, h, b);
-    acc.mac(1, rp, bt * rp + lm * ld1<T>(Phi1[j]));
-    acc.mac(2, w, rp);
-    acc.mac(3, w, dotr(b, b));
-    acc.next();
-  }
-  acc.store(part);
-}
-
-// [0] sum |phi|^4, [1] sum Phi |phi|^2
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
-k_quartic_sums(const double2* __restrict__ phi, const double* __restrict__ Phi, size_t N, double* __restrict__ part) {
-  Sums<T, 2> acc;
-  ATKM_GRID_LOOP(j, N) {
-    const V2<T> a = ld2<T>(phi[j]);
-    const T r = dotr(a, a);
-    acc.mac(0, r, r);
-    acc.mac(1, ld1<T>(Phi[j]), r);
-    acc.next();
-  }
-  acc.store(part);
-}
-
 __global__ void k_set_scalar(double* dst, double v) { *dst = v; }
 
 int red_grid(size_t N) {
@@ -348,10 +187,12 @@ enum {
   S_Z = SC_RED + 32      // |H phi_0 in FP32 - H phi_0 in FP64|^2 (+ unused)
 };
 
-// ------------------------------------------------------------ control kernels
+// ------------------------------------------------------------ control steps
+// Each runs in one thread: at the end of the reduction whose sums it reads
+// (Fin), or in a kernel of its own.
 __device__ __forceinline__ bool fin(double v) { return isfinite(v); }
 
-__global__ void k_c_init(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_init(Ctl* c, const double* s) {
   const double n0 = sqrt(c->hv * s[S_N]);
   c->nan = !(n0 > 0.0) || !fin(n0);
   c->inv0 = c->nan ? 0.0 : 1.0 / n0;
@@ -359,10 +200,10 @@ __global__ void k_c_init(Ctl* c, const double* s) {
 
 // the FP32 arithmetic's noise in the residual at phi_0: ||H_32 phi_0 - H_64 phi_0||
 // (each with its own Phi), in the residual's norm
-__global__ void k_c_noise(Ctl* c, const double* s) { c->noise = sqrt(c->hv * s[S_Z]); }
+__device__ __forceinline__ void c_noise(Ctl* c, const double* s) { c->noise = sqrt(c->hv * s[S_Z]); }
 
 // loop top: energy terms of phi, mu, alpha (Step 2 and the shift of §2.3)
-__global__ void k_c_parts(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_parts(Ctl* c, const double* s) {
   const double hv = c->hv;
   c->kin = hv * (s[S_H + 0] + s[S_H + 2] + s[S_H + 4]);
   c->rot = hv * (s[S_H + 1] + s[S_H + 3]);
@@ -378,13 +219,13 @@ __global__ void k_c_parts(Ctl* c, const double* s) {
   c->alpha = c->kin + c->pot + c->beta * c->f4 + fabs(c->lam * c->dip);
 }
 
-__global__ void k_c_res(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_res(Ctl* c, const double* s) {
   c->res = sqrt(c->hv * s[S_R]);
   c->nan = !fin(c->E) || !fin(c->res) || !fin(c->mu);
 }
 
 // Step 3: PR+ coefficients, p = cp0 P r + cp1 p_prev + cp2 phi
-__global__ void k_c_dir(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_dir(Ctl* c, const double* s) {
   const double hv = c->hv;
   const double b = hv * s[S_D + 0], rPr = hv * s[S_D + 1], rphi = hv * s[S_D + 2];
   const double rpPr = hv * s[S_D + 3], a = hv * s[S_D + 4], cc = hv * s[S_D + 5], nphi = hv * s[S_D + 6];
@@ -404,7 +245,7 @@ __global__ void k_c_dir(Ctl* c, const double* s) {
 }
 
 // Step 4 (i): keep p if <H phi, p> < 0, otherwise re-form it as J(-P r)
-__global__ void k_c_reset(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_reset(Ctl* c, const double* s) {
   c->pn2 = c->hv * s[S_P];
   c->d1 = c->hv * s[S_P + 1];
   c->redo = 0;
@@ -418,14 +259,14 @@ __global__ void k_c_reset(Ctl* c, const double* s) {
   }
 }
 
-__global__ void k_c_reset2(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_reset2(Ctl* c, const double* s) {
   if (!c->redo) return;
   c->pn2 = c->hv * s[S_P];
   c->d1 = c->hv * s[S_P + 1];
 }
 
 // Step 4 (ii): quadratic model, initial t, first retraction coefficients
-__global__ void k_c_step(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_step(Ctl* c, const double* s) {
   const double hv = c->hv;
   c->Hpp = hv * s[S_C]; c->S1 = hv * s[S_C + 1]; c->S2 = hv * s[S_C + 2]; c->S3 = hv * s[S_C + 3];
   c->curv = c->Hpp + 2.0 * c->S1 - c->mu * c->pn2;
@@ -444,13 +285,13 @@ __global__ void k_c_step(Ctl* c, const double* s) {
   c->sr = sin(c->t * c->pn) / c->pn;
 }
 
-__global__ void k_c_norm(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_norm(Ctl* c, const double* s) {
   c->nrm2 = c->hv * s[S_T];
   c->inv = 1.0 / sqrt(c->nrm2);
 }
 
 // Step 4 (iii): trial energy and the acceptance test
-__global__ void k_c_accept(Ctl* c, const double* s) {
+__device__ __forceinline__ void c_accept(Ctl* c, const double* s) {
   const double quad = (c->cr * c->cr * c->Aphiphi + 2.0 * c->cr * c->sr * c->Aphip + c->sr * c->sr * c->App) / c->nrm2;
   c->En = quad + 0.5 * c->beta * c->hv * s[S_Q] + 0.5 * c->lam * c->hv * s[S_Q + 1];
   c->linf = s[S_L];
@@ -473,12 +314,20 @@ __device__ __forceinline__ void halve_body(Ctl* c, int mode) {
   c->cr = cos(c->t * c->pn);
   c->sr = sin(c->t * c->pn) / c->pn;
 }
-__global__ void k_c_halve(Ctl* c, int mode) { halve_body(c, mode); }
+__global__ void k_c_halve(Ctl* c, int mode) {
+  pdl_trigger();
+  pdl_wait();
+  halve_body(c, mode); }
 // The same with the mode taken on the device: halve while halvings remain.
-__global__ void k_c_halve_auto(Ctl* c) { halve_body(c, c->nh < c->max_halv ? 0 : 1); }
+__global__ void k_c_halve_auto(Ctl* c) {
+  pdl_trigger();
+  pdl_wait();
+  halve_body(c, c->nh < c->max_halv ? 0 : 1); }
 
 // End of an iteration: the trial becomes phi_{n+1}.
 __global__ void k_c_end(Ctl* c) {
+  pdl_trigger();
+  pdl_wait();
   c->den_prev = c->den;
   c->have_prev = 1;
   c->E = c->En;
@@ -487,6 +336,8 @@ __global__ void k_c_end(Ctl* c) {
 
 // Host-driven state changes (precision hand-over, start of a solve).
 __global__ void k_c_reset_state(Ctl* c, int have_E, int force_sd, int clear_prev) {
+  pdl_trigger();
+  pdl_wait();
   c->have_E = have_E;
   c->force_sd = force_sd;
   if (clear_prev) c->have_prev = 0;
@@ -528,6 +379,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 __global__ void k_d_setup(Ctl* c, LoopInit L) {
+  pdl_trigger();
+  pdl_wait();
   c->n = c->n_start = L.n;
   c->max_iter = L.max_iter;
   c->max_halv = L.max_halv;
@@ -555,7 +408,7 @@ __global__ void k_d_setup(Ctl* c, LoopInit L) {
 }
 
 // After Step 2 (loop top): log entry, stop rule, hand-over test.
-__global__ void k_d_check(Ctl* c, cudaGraphConditionalHandle h_rest, int nodes) {
+__device__ void d_check(Ctl* c, cudaGraphConditionalHandle h_rest, int nodes) {
   c->launches += nodes;
   if (c->final_top) {  // the residual of the final state after a stagnated run
     c->final_top = 0;
@@ -602,7 +455,7 @@ __global__ void k_d_check(Ctl* c, cudaGraphConditionalHandle h_rest, int nodes) 
 }
 
 // After each trial of Step 4 (iii): another halving (or the forced trial)?
-__global__ void k_d_after_trial(Ctl* c, cudaGraphConditionalHandle h_halve, int nodes) {
+__device__ void d_after_trial(Ctl* c, cudaGraphConditionalHandle h_halve, int nodes) {
   c->launches += nodes;
   int more;
   if (c->forced) {
@@ -624,6 +477,8 @@ __global__ void k_d_after_trial(Ctl* c, cudaGraphConditionalHandle h_halve, int 
 
 // End of an iteration: the trial becomes phi_{n+1} (k_c_end), bookkeeping.
 __global__ void k_d_end(Ctl* c, int nodes) {
+  pdl_trigger();
+  pdl_wait();
   c->launches += nodes;
   if (c->done) return;
   const int acc = c->accepted && !c->forced;
@@ -650,12 +505,16 @@ __global__ void k_d_end(Ctl* c, int nodes) {
 
 // Between the two iterations of a loop body: run the second one?
 __global__ void k_d_gate(Ctl* c, cudaGraphConditionalHandle h_go1, int nodes) {
+  pdl_trigger();
+  pdl_wait();
   c->launches += nodes;
   cudaGraphSetConditional(h_go1, !c->done || c->final_top);
 }
 
 // End of a loop body (two iterations): run again?
 __global__ void k_d_loop(Ctl* c, cudaGraphConditionalHandle h_run, cudaGraphConditionalHandle h_go0, int nodes) {
+  pdl_trigger();
+  pdl_wait();
   c->launches += nodes;
   int run = !c->done || c->final_top;
   if (run && ++c->guard > c->guard_max) {
@@ -670,6 +529,8 @@ __global__ void k_d_loop(Ctl* c, cudaGraphConditionalHandle h_run, cudaGraphCond
 
 // After the FP32 loop: hand over at the parity where it stopped.
 __global__ void k_d_phase(Ctl* c, cudaGraphConditionalHandle h0, cudaGraphConditionalHandle h1, int nodes) {
+  pdl_trigger();
+  pdl_wait();
   c->launches += nodes;
   const int ho = c->handover;
   cudaGraphSetConditional(h0, ho && c->q == 0);
@@ -678,6 +539,8 @@ __global__ void k_d_phase(Ctl* c, cudaGraphConditionalHandle h0, cudaGraphCondit
 
 // The hand-over's state change (after the FP64 ATKM of phi): FP64 from here.
 __global__ void k_d_handover(Ctl* c, double tolE_eps, int nodes) {
+  pdl_trigger();
+  pdl_wait();
   c->launches += nodes;
   c->f32 = 0;
   c->caps = 0;
@@ -688,13 +551,210 @@ __global__ void k_d_handover(Ctl* c, double tolE_eps, int nodes) {
   c->tolE_eps = tolE_eps;
 }
 
-}  // namespace
-
-cudaError_t launch_finalize(atkm_plan* p, int nslots, int nblocks, int dst_slot, cudaStream_t st) {
-  k_finalize<<<nslots, kRedThreads, 0, st>>>(p->partials, nblocks, p->scal + dst_slot, nullptr);
-  count_launches(1);
-  return cudaGetLastError();
+// What the last block of a reducing vector kernel does: the grid sums (in the
+// fixed order of finalize_sums) into out, then the control step that reads
+// them.  s is the plan's scalar block.
+enum Then {
+  kThenNone, kThenInit, kThenNoise, kThenTop, kThenTopCheck, kThenDir, kThenReset, kThenReset2, kThenStep, kThenNorm,
+  kThenAccept, kThenAcceptLoop
+};
+struct Fin {
+  double* part;
+  double* out;
+  unsigned* cnt;
+  const double* s;
+  Ctl* c;
+  int then, nodes;
+  cudaGraphConditionalHandle h;
+};
+__device__ __forceinline__ void run_then(const Fin& f) {
+  Ctl* c = f.c;
+  switch (f.then) {
+    case kThenInit: c_init(c, f.s); break;
+    case kThenNoise: c_noise(c, f.s); break;
+    case kThenTop:
+    case kThenTopCheck:
+      c_parts(c, f.s);
+      c_res(c, f.s);
+      if (f.then == kThenTopCheck) d_check(c, f.h, f.nodes);
+      break;
+    case kThenDir: c_dir(c, f.s); break;
+    case kThenReset: c_reset(c, f.s); break;
+    case kThenReset2: c_reset2(c, f.s); break;
+    case kThenStep: c_step(c, f.s); break;
+    case kThenNorm: c_norm(c, f.s); break;
+    case kThenAccept:
+    case kThenAcceptLoop:
+      c_accept(c, f.s);
+      if (f.then == kThenAcceptLoop) d_after_trial(c, f.h, f.nodes);
+      break;
+    default: break;
+  }
 }
+template <int NS> __device__ __forceinline__ void finish(const Fin& f) {
+  if (!last_block(f.cnt, threadIdx.x == 0)) return;
+  finalize_sums<NS>(f.part, gridDim.x, f.out);
+  __syncthreads();
+  if (threadIdx.x == 0) run_then(f);
+}
+// Grid maximum of the block maxima; out = its square root (the partials hold
+// squared distances).
+__device__ __forceinline__ void finish_max(const Fin& f) {
+  __shared__ double sh[kRedThreads];
+  if (!last_block(f.cnt, threadIdx.x == 0)) return;
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedThreads) acc = fmax(acc, __ldcg(f.part + i));
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) f.out[0] = sqrt(sh[0]);
+}
+
+// sum_j Re(u_j conj(v_j)) (FP64).
+__global__ void __launch_bounds__(kRedThreads) k_dot(const double2* __restrict__ u, const double2* __restrict__ v,
+                                                     size_t N, Fin f) {
+  pdl_trigger();
+  Sums<double, 1> acc;
+  ATKM_GRID_LOOP(j, N) {
+    const double2 a = u[j], b = v[j];
+    acc.mac(0, a.x, b.x);
+    acc.mac(0, a.y, b.y);
+  }
+  acc.store(f.part);
+  finish<1>(f);
+}
+
+// The seven sums of the direction step from one read of its five vectors:
+// <Pr,phi>, <r,Pr>, <r,phi>, <r_prev,Pr>, <r_prev,phi>, <p_prev,phi>, <phi,phi>.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+k_dir_dots(const double2* __restrict__ Pr, const double2* __restrict__ phi, const double2* __restrict__ r,
+           const double2* __restrict__ rp, const double2* __restrict__ pp, size_t N, Fin f) {
+  pdl_trigger();
+  Sums<T, 7> acc;
+  ATKM_GRID_LOOP(j, N) {
+    const V2<T> P = ld2<T>(Pr[j]), g = ld2<T>(phi[j]), a = ld2<T>(r[j]), b = ld2<T>(rp[j]), c = ld2<T>(pp[j]);
+    acc.dot(0, P, g);
+    acc.dot(1, a, P);
+    acc.dot(2, a, g);
+    acc.dot(3, b, P);
+    acc.dot(4, b, g);
+    acc.dot(5, c, g);
+    acc.dot(6, g, g);
+    acc.next();
+  }
+  acc.store(f.part);
+  finish<7>(f);
+}
+
+// A coefficient m * (*p) (p may be null: then m).
+struct Coef {
+  const double* p;
+  double m;
+};
+__device__ __forceinline__ double cval(const Coef& c) { return c.p ? c.m * *c.p : c.m; }
+
+// out = c0 v0 + c1 v1 + c2 v2 (null vectors skipped); sums |out|^2 and
+// Re(w conj(out)) when w is given.  Skipped entirely when *pred == 0.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+k_lincomb(double2* __restrict__ out, const double2* __restrict__ v0, Coef c0, const double2* __restrict__ v1,
+          Coef c1, const double2* __restrict__ v2, Coef c2, const double2* __restrict__ w, size_t N,
+          Fin f, const int* __restrict__ pred) {
+  pdl_trigger();
+  if (pred && !*pred) return;
+  const T a0 = tor<T>(cval(c0)), a1 = tor<T>(cval(c1)), a2 = tor<T>(cval(c2));
+  Sums<T, 2> acc;
+  ATKM_GRID_LOOP(j, N) {
+    V2<T> o{(T)0, (T)0};
+    if (v0) { const V2<T> a = ld2<T>(v0[j]); o.x += a0 * a.x; o.y += a0 * a.y; }
+    if (v1) { const V2<T> a = ld2<T>(v1[j]); o.x += a1 * a.x; o.y += a1 * a.y; }
+    if (v2) { const V2<T> a = ld2<T>(v2[j]); o.x += a2 * a.x; o.y += a2 * a.y; }
+    out[j] = make_double2(tod<T>(o.x), tod<T>(o.y));
+    acc.dot(0, o, o);
+    if (w) acc.dot(1, ld2<T>(w[j]), o);
+    acc.next();
+  }
+  acc.store(f.part);
+  finish<2>(f);
+}
+
+// phi+ *= *inv (FP64: the renormalisation); block max of |phi+ - phi|^2, the
+// difference taken in T (FP32 in the FP32 phase, where it is only logged).
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+k_scale_linf(double2* __restrict__ phin, const double2* __restrict__ phi, const double* __restrict__ invp, size_t N,
+             Fin f) {
+  __shared__ T sh[kRedThreads];
+  pdl_trigger();
+  const double inv = *invp;
+  T m = (T)0;
+  ATKM_GRID_LOOP(j, N) {
+    double2 a = phin[j];
+    a.x *= inv; a.y *= inv;
+    phin[j] = a;
+    const V2<T> x = ld2<T>(a), y = ld2<T>(phi[j]);
+    const T dx = x.x - y.x, dy = x.y - y.y;
+    m = fmax(m, dx * dx + dy * dy);
+  }
+  sh[threadIdx.x] = m;
+  __syncthreads();
+  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) f.part[blockIdx.x] = tod<T>(sh[0]);
+  finish_max(f);
+}
+
+// Sums for the curvature of the quadratic model:
+//   [0] <Hp, p>
+//   [1] sum rho'(beta rho' + lambda Phi'),  rho' = Re(conj(phi) p)
+//   [2] sum (beta|phi|^2 + lambda Phi) Re(phi conj(p))
+//   [3] sum (beta|phi|^2 + lambda Phi) |p|^2
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+k_curv_sums(const double2* __restrict__ Hp, const double2* __restrict__ phi, const double2* __restrict__ p,
+            const double* __restrict__ Phi, const double* __restrict__ Phi1, double beta, double lambda, size_t N,
+            Fin f) {
+  pdl_trigger();
+  const T bt = tor<T>(beta), lm = tor<T>(lambda);
+  Sums<T, 4> acc;
+  ATKM_GRID_LOOP(j, N) {
+    const V2<T> a = ld2<T>(phi[j]), b = ld2<T>(p[j]), h = ld2<T>(Hp[j]);
+    const T rp = dotr(a, b);
+    const T w = bt * dotr(a, a) + lm * ld1<T>(Phi[j]);
+    acc.dot(0, h, b);
+    acc.mac(1, rp, bt * rp + lm * ld1<T>(Phi1[j]));
+    acc.mac(2, w, rp);
+    acc.mac(3, w, dotr(b, b));
+    acc.next();
+  }
+  acc.store(f.part);
+  finish<4>(f);
+}
+
+// [0] sum |phi|^4, [1] sum Phi |phi|^2
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+k_quartic_sums(const double2* __restrict__ phi, const double* __restrict__ Phi, size_t N, Fin f) {
+  pdl_trigger();
+  Sums<T, 2> acc;
+  ATKM_GRID_LOOP(j, N) {
+    const V2<T> a = ld2<T>(phi[j]);
+    const T r = dotr(a, a);
+    acc.mac(0, r, r);
+    acc.mac(1, ld1<T>(Phi[j]), r);
+    acc.next();
+  }
+  acc.store(f.part);
+  finish<2>(f);
+}
+
+}  // namespace
 
 // ------------------------------------------------------------- PCG state
 struct PcgBuffers {
@@ -822,29 +882,30 @@ struct Seq {
   cudaStream_t st() const { return B.st; }
   void chk(cudaError_t e) { if (err == cudaSuccess && e != cudaSuccess) err = e; }
 
-  void dot(const double2* u, const double2* v, int dst) {
+  Fin fin(int dst, int then, int nodes = 0, cudaGraphConditionalHandle h = 0) const {
+    return Fin{p->partials, p->scal + dst, p->cnt, p->scal, B.ctl, then, nodes, h};
+  }
+  void dot(const double2* u, const double2* v, int dst, int then) {
     prof_begin(p, "vec_dots", 32.0 * B.N, 0.0, st());
     const int g = wave_grid((const void*)k_dot, B.N);
-    k_dot<<<g, kRedThreads, 0, st()>>>(u, v, B.N, p->partials);
+    k_dot<<<g, kRedThreads, 0, st()>>>(u, v, B.N, fin(dst, then));
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
-    chk(launch_finalize(p, 1, g, dst, st()));
   }
   // FP64 arithmetic unless this is the FP32 phase and `phase_type` allows it.
   void lincomb(double2* out, const double2* v0, Coef c0, const double2* v1, Coef c1, const double2* v2, Coef c2,
-               const double2* w, int dst, const int* pred = nullptr, bool phase_type = true) {
+               const double2* w, const Fin& f, const int* pred = nullptr, bool phase_type = true) {
     const double nv = (v0 ? 1 : 0) + (v1 ? 1 : 0) + (v2 ? 1 : 0) + (w ? 1 : 0) + 1;
     prof_begin(p, "vec_lincomb", 16.0 * nv * B.N, 0.0, st());
     const bool fl = f32 && phase_type;
     const int g = fl ? wave_grid((const void*)k_lincomb<float>, B.N) : wave_grid((const void*)k_lincomb<double>, B.N);
     if (fl)
-      k_lincomb<float><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, p->partials, pred);
+      k_lincomb<float><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
     else
-      k_lincomb<double><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, p->partials, pred);
+      k_lincomb<double><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
     prof_end(p, st());
-    k_finalize<<<2, kRedThreads, 0, st()>>>(p->partials, g, p->scal + dst, pred);
-    count_launches(2);
+    count_launches(1);
     chk(cudaGetLastError());
   }
   void atkm(int mode, const double* a, const double* b, double* o, bool aux = false) {
@@ -861,46 +922,45 @@ struct Seq {
               : launch_H64(p, dw, ph, fp, pp, B.Phi[q], op, red, st()));
   }
   template <typename K, typename... A> void ctl1(K kernel, A... args) {
-    kernel<<<1, 1, 0, st()>>>(args...);
+    chk(launch_pdl(kernel, 1, 1, 0, st(), args...));
     count_launches(1);
-    chk(cudaGetLastError());
   }
 
-  // Step 2 only (loop top): H phi, parts, r, ||r||.
-  void top() {
+  // Step 2 only (loop top): H phi, parts, r, ||r||; in the device-driven loop
+  // then its check (sofar: the kernels launched in this segment so far).
+  template <class F> void top(bool loop, cudaGraphConditionalHandle h, F sofar) {
     hop(B.phi[q], B.Hphi, S_H);
-    ctl1(k_c_parts, c(), s());
-    lincomb(B.r[q], B.Hphi, Coef{nullptr, 1.0}, B.phi[q], Coef{&c()->mu, -1.0}, nullptr, Coef{nullptr, 0.0}, nullptr,
-            S_R);
-    ctl1(k_c_res, c(), s());
+    // mu = hvol <H phi, phi> read from the sums themselves (c->mu is set by the
+    // control step that ends this kernel)
+    lincomb(B.r[q], B.Hphi, Coef{nullptr, 1.0}, B.phi[q], Coef{s() + S_H + 8, -p->hvol}, nullptr, Coef{nullptr, 0.0},
+            nullptr, fin(S_R, loop ? kThenTopCheck : kThenTop, loop ? sofar() + 1 : 0, h));
   }
+  void top() { top(false, 0, [] { return 0; }); }
   // One trial of Step 4 (iii) with the current retraction coefficients.
-  void trial() {
+  template <class F> void trial(bool loop, cudaGraphConditionalHandle h, F sofar) {
     double2* phin = B.phi[q ^ 1];
     lincomb(phin, B.phi[q], Coef{&c()->cr, 1.0}, B.p[q], Coef{&c()->sr, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr,
-            S_T, nullptr, false);  // the retraction stays FP64
-    ctl1(k_c_norm, c(), s());
+            fin(S_T, kThenNorm), nullptr, false);  // the retraction stays FP64
     prof_begin(p, "vec_scale_linf", 48.0 * B.N, 0.0, st());
     const int gs = f32 ? wave_grid((const void*)k_scale_linf<float>, B.N)
                        : wave_grid((const void*)k_scale_linf<double>, B.N);
-    if (f32) k_scale_linf<float><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, p->partials);
-    else k_scale_linf<double><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, p->partials);
+    if (f32) k_scale_linf<float><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L, kThenNone));
+    else k_scale_linf<double><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L, kThenNone));
     prof_end(p, st());
-    k_finalize_max<<<1, kRedThreads, 0, st()>>>(p->partials, gs, p->scal + S_L);
-    count_launches(2);
+    count_launches(1);
     chk(cudaGetLastError());
     atkm(SRC_PSI, reinterpret_cast<const double*>(phin), nullptr, B.Phi[q ^ 1]);
     prof_begin(p, "vec_quartic", 24.0 * B.N, 0.0, st());
     const int gq = f32 ? wave_grid((const void*)k_quartic_sums<float>, B.N)
                        : wave_grid((const void*)k_quartic_sums<double>, B.N);
-    if (f32) k_quartic_sums<float><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, p->partials);
-    else k_quartic_sums<double><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, p->partials);
+    const Fin f = fin(S_Q, loop ? kThenAcceptLoop : kThenAccept, loop ? sofar() + 1 : 0, h);
+    if (f32) k_quartic_sums<float><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
+    else k_quartic_sums<double><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
-    chk(launch_finalize(p, 2, gq, S_Q, st()));
-    ctl1(k_c_accept, c(), s());
   }
+  void trial() { trial(false, 0, [] { return 0; }); }
   cudaError_t precond() {
     const double* r = reinterpret_cast<const double*>(B.r[q]);
     const double* phi = reinterpret_cast<const double*>(B.phi[q]);
@@ -914,46 +974,41 @@ struct Seq {
     rest();
   }
   // Steps 3-4 up to the first trial (after top()).
-  void rest() {
+  template <class F> void rest(bool loop, cudaGraphConditionalHandle h, F sofar) {
     chk(precond());
     prof_begin(p, "vec_dir_dots", 80.0 * B.N, 0.0, st());
     const int gd = f32 ? wave_grid((const void*)k_dir_dots<float>, B.N)
                        : wave_grid((const void*)k_dir_dots<double>, B.N);
+    const Fin fd = fin(S_D, kThenDir);
     if (f32)
-      k_dir_dots<float><<<gd, kRedThreads, 0, st()>>>(B.Pr, B.phi[q], B.r[q], B.r[q ^ 1], B.p[q ^ 1], B.N,
-                                                      p->partials);
+      k_dir_dots<float><<<gd, kRedThreads, 0, st()>>>(B.Pr, B.phi[q], B.r[q], B.r[q ^ 1], B.p[q ^ 1], B.N, fd);
     else
-      k_dir_dots<double><<<gd, kRedThreads, 0, st()>>>(B.Pr, B.phi[q], B.r[q], B.r[q ^ 1], B.p[q ^ 1], B.N,
-                                                       p->partials);
+      k_dir_dots<double><<<gd, kRedThreads, 0, st()>>>(B.Pr, B.phi[q], B.r[q], B.r[q ^ 1], B.p[q ^ 1], B.N, fd);
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
-    chk(launch_finalize(p, 7, gd, S_D, st()));
-    ctl1(k_c_dir, c(), s());
     lincomb(B.p[q], B.Pr, Coef{&c()->cp0, 1.0}, B.p[q ^ 1], Coef{&c()->cp1, 1.0}, B.phi[q], Coef{&c()->cp2, 1.0},
-            B.Hphi, S_P);
-    ctl1(k_c_reset, c(), s());
-    lincomb(B.p[q], B.Pr, Coef{nullptr, -1.0}, B.phi[q], Coef{&c()->b, 1.0}, nullptr, Coef{nullptr, 0.0}, B.Hphi, S_P,
-            &c()->redo);
-    ctl1(k_c_reset2, c(), s());
+            B.Hphi, fin(S_P, kThenReset));
+    lincomb(B.p[q], B.Pr, Coef{nullptr, -1.0}, B.phi[q], Coef{&c()->b, 1.0}, nullptr, Coef{nullptr, 0.0}, B.Hphi,
+            fin(S_P, kThenReset2), &c()->redo);
     hop(B.p[q], B.Hp, -1, true);
     atkm(SRC_PAIR, reinterpret_cast<const double*>(B.phi[q]), reinterpret_cast<const double*>(B.p[q]), B.Phi1, true);
     prof_begin(p, "vec_curv_sums", 64.0 * B.N, 0.0, st());
     const int gc = f32 ? wave_grid((const void*)k_curv_sums<float>, B.N)
                        : wave_grid((const void*)k_curv_sums<double>, B.N);
+    const Fin fc = fin(S_C, kThenStep);
     if (f32)
       k_curv_sums<float><<<gc, kRedThreads, 0, st()>>>(B.Hp, B.phi[q], B.p[q], B.Phi[q], B.Phi1, ph.beta, ph.lambda,
-                                                       B.N, p->partials);
+                                                       B.N, fc);
     else
       k_curv_sums<double><<<gc, kRedThreads, 0, st()>>>(B.Hp, B.phi[q], B.p[q], B.Phi[q], B.Phi1, ph.beta,
-                                                        ph.lambda, B.N, p->partials);
+                                                        ph.lambda, B.N, fc);
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
-    chk(launch_finalize(p, 4, gc, S_C, st()));
-    ctl1(k_c_step, c(), s());
-    trial();
+    trial(loop, h, sofar);
   }
+  void rest() { rest(false, 0, [] { return 0; }); }
   void run(int kind) {
     if (kind == 0) {
       iteration();
@@ -1101,23 +1156,20 @@ struct GraphBuild {
     Ctl* c = B.ctl;
     cudaGraphNode_t d = nullptr;
     capture(g, &d, [&](auto sofar) {
-      S.top();
-      S.ctl1(k_d_check, c, h_rest, sofar() + 1);
+      S.top(true, h_rest, sofar);
     });
     cudaGraph_t rb = cond(g, &d, h_rest, cudaGraphCondTypeIf);
     if (err != cudaSuccess) return;
     cudaGraphNode_t r = nullptr;
     capture(rb, &r, [&](auto sofar) {
-      S.rest();
-      S.ctl1(k_d_after_trial, c, h_halve, sofar() + 1);
+      S.rest(true, h_halve, sofar);
     });
     cudaGraph_t hb = cond(rb, &r, h_halve, cudaGraphCondTypeWhile);
     if (err != cudaSuccess) return;
     cudaGraphNode_t h = nullptr;
     capture(hb, &h, [&](auto sofar) {
       S.ctl1(k_c_halve_auto, c);
-      S.trial();
-      S.ctl1(k_d_after_trial, c, h_halve, sofar() + 1);
+      S.trial(true, h_halve, sofar);
     });
     capture(rb, &r, [&](auto) { S.ctl1(k_d_end, c, 1); });
   }
@@ -1385,12 +1437,11 @@ struct Solver {
       q = 0;
       Seq S = seq(f32);
       const double2* p0 = reinterpret_cast<const double2*>(psi);
-      S.dot(p0, p0, S_N);
-      S.ctl1(k_c_init, B->ctl, (const double*)plan->scal);
+      S.dot(p0, p0, S_N, kThenInit);
       // the normalisation stays FP64 in every precision form (as the
       // renormalisation after each retraction does)
       S.lincomb(B->phi[0], p0, Coef{&B->ctl->inv0, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr, Coef{nullptr, 0.0},
-                nullptr, S_T, nullptr, false);
+                nullptr, S.fin(S_T, kThenNone), nullptr, false);
       S.atkm(SRC_PSI, reinterpret_cast<const double*>(B->phi[0]), nullptr, B->Phi[0]);
       S.ctl1(k_c_reset_state, B->ctl, 0, 1, 1);
       chk(S.err);
@@ -1403,8 +1454,7 @@ struct Solver {
         chk(launch_H64(plan, false, ph, p0d, p0d, B->Phi1, reinterpret_cast<double*>(B->Hp), -1, B->st));
         chk(launch_H<float>(plan, ph, p0d, p0d, B->Phi[0], reinterpret_cast<double*>(B->Hphi), -1, B->st));
         Z.lincomb(B->Pr, B->Hp, Coef{nullptr, 1.0}, B->Hphi, Coef{nullptr, -1.0}, nullptr, Coef{nullptr, 0.0},
-                  nullptr, S_Z, nullptr, false);
-        Z.ctl1(k_c_noise, B->ctl, (const double*)plan->scal);
+                  nullptr, Z.fin(S_Z, kThenNoise), nullptr, false);
         chk(Z.err);
       }
       fetch_async();

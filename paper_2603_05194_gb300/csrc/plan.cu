@@ -416,7 +416,7 @@ bool make_int_len(int L, IntLen& f) {
 
 void free_plan_memory(atkm_plan* p) {
   void* ptrs[] = {p->tw32, p->twi, p->axtab, p->Pw, p->U0, p->U0f, p->Kz, p->W1, p->W2, p->T1,
-                  p->W1f, p->W2f, p->T1f, p->ex[0], p->ex[1], p->ex[2], p->partials, p->scal};
+                  p->W1f, p->W2f, p->T1f, p->ex[0], p->ex[1], p->ex[2], p->partials, p->scal, p->cnt};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->scal_host) cudaFreeHost(p->scal_host);
@@ -576,7 +576,7 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   p->U0f = nullptr; p->Kz = nullptr;
   p->W1 = p->W2 = p->T1 = nullptr;
   p->ex[0] = p->ex[1] = p->ex[2] = nullptr;
-  p->W1f = p->W2f = p->T1f = nullptr; p->partials = nullptr; p->scal = nullptr; p->scal_host = nullptr;
+  p->W1f = p->W2f = p->T1f = nullptr; p->partials = nullptr; p->scal = nullptr; p->cnt = nullptr; p->scal_host = nullptr;
   p->pcg = nullptr; p->prof = nullptr; p->prof_stopped_ = nullptr; p->bytes = 0; p->flags = flags;
   p->n_tune = 0;
   Geo& g = p->g;
@@ -770,6 +770,8 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   if ((e = dev_alloc(p, (void**)&p->partials, (size_t)p->partials_cap * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan partials"));
   if ((e = dev_alloc(p, (void**)&p->scal, SC_COUNT * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = cudaMallocHost((void**)&p->scal_host, SC_COUNT * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
+  if ((e = dev_alloc(p, (void**)&p->cnt, sizeof(unsigned))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
+  if ((e = cudaMemsetAsync(p->cnt, 0, sizeof(unsigned), st)) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = cudaMemsetAsync(p->scal, 0, SC_COUNT * sizeof(double), st)) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan create"));
   if (flags & ATKM_PLAN_AUTOTUNE) {
