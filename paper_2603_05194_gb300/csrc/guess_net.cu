@@ -155,13 +155,27 @@ __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__floa
 
 constexpr int kRowsThreads = 256;
 
+// What a row product does to its outputs before storing them: nothing, add
+// bias[n % cb] (and, with relu, clamp at zero), or zero them where the forward
+// output `mask` (laid out like C) was not positive.  Each is one pass over the
+// activations less than a kernel of its own (at batch 32: 8.3 and 5.1 us a
+// layer for the last two transposed convolutions), with the same rounding.
+struct RowsEpi {
+  const float* bias = nullptr;
+  int cb = 1, relu = 0;
+  const float* mask = nullptr;
+};
+
 // C[M x N] = A[M x K] B[K x N] with A's rows contiguous and 16-byte aligned
 // (A(m,k) = A[m*sam + k], sam and K multiples of 4) and C's rows too (ldc a
-// multiple of 4): each thread forms NT consecutive outputs of one row from
-// float4 loads of the row; B (K x N, any strides) is staged in shared memory.
+// multiple of 4): each thread forms NT outputs of one row, NT / 4 groups of four
+// columns 4 N / NT apart (neighbouring threads then read neighbouring 16 bytes
+// of B: with NT consecutive columns a thread, its reads met 4-way bank
+// conflicts), from float4 loads of the row; B (K x N, any strides) is staged in
+// shared memory.
 template <int NT>
 __device__ __forceinline__ void gemm_rows(const float* __restrict__ A, long sam, const float* __restrict__ Bm, long sbk,
-                                          long sbn, float* __restrict__ C, int ldc, int M, int N, int K) {
+                                          long sbn, float* __restrict__ C, int ldc, int M, int N, int K, const RowsEpi& ep) {
   extern __shared__ __align__(16) float bsm[];  // [K][N]
   for (int i = threadIdx.x; i < K * N; i += kRowsThreads) {
     const int k = i / N, n = i - k * N;
@@ -183,10 +197,10 @@ __device__ __forceinline__ void gemm_rows(const float* __restrict__ A, long sam,
     const float ak[4] = {bf16r(av.x), bf16r(av.y), bf16r(av.z), bf16r(av.w)};
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-      const float4* b4 = reinterpret_cast<const float4*>(bsm + (4 * k4 + kk) * N + c * NT);
+      const float4* b4 = reinterpret_cast<const float4*>(bsm + (4 * k4 + kk) * N) + c;
 #pragma unroll
       for (int q = 0; q < NT / 4; ++q) {
-        const float4 bv = b4[q];
+        const float4 bv = b4[q * chunks];
         acc[4 * q] = fmaf(ak[kk], bv.x, acc[4 * q]);
         acc[4 * q + 1] = fmaf(ak[kk], bv.y, acc[4 * q + 1]);
         acc[4 * q + 2] = fmaf(ak[kk], bv.z, acc[4 * q + 2]);
@@ -194,19 +208,33 @@ __device__ __forceinline__ void gemm_rows(const float* __restrict__ A, long sam,
       }
     }
   }
-  float4* out = reinterpret_cast<float4*>(C + row * ldc + c * NT);
+  if (ep.bias) {
 #pragma unroll
-  for (int q = 0; q < NT / 4; ++q) out[q] = make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+    for (int n = 0; n < NT; ++n) {
+      const float v = acc[n] + __ldg(ep.bias + ((n / 4 * chunks + c) * 4 + n % 4) % ep.cb);
+      acc[n] = (ep.relu && v < 0.f) ? 0.f : v;
+    }
+  }
+  if (ep.mask) {
+    const float4* my = reinterpret_cast<const float4*>(ep.mask + row * ldc) + c;
+#pragma unroll
+    for (int q = 0; q < NT / 4; ++q) {
+      const float4 y = __ldg(my + q * chunks);
+      if (!(y.x > 0.f)) acc[4 * q] = 0.f;
+      if (!(y.y > 0.f)) acc[4 * q + 1] = 0.f;
+      if (!(y.z > 0.f)) acc[4 * q + 2] = 0.f;
+      if (!(y.w > 0.f)) acc[4 * q + 3] = 0.f;
+    }
+  }
+  float4* out = reinterpret_cast<float4*>(C + row * ldc) + c;
+#pragma unroll
+  for (int q = 0; q < NT / 4; ++q) out[q * chunks] = make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
 }
+template <int NT>
 __global__ void __launch_bounds__(kRowsThreads)
-k_gemm_rows8(const float* __restrict__ A, long sam, const float* __restrict__ Bm, long sbk, long sbn,
-             float* __restrict__ C, int ldc, int M, int N, int K) {
-  gemm_rows<8>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K);
-}
-__global__ void __launch_bounds__(kRowsThreads)
-k_gemm_rows16(const float* __restrict__ A, long sam, const float* __restrict__ Bm, long sbk, long sbn,
-              float* __restrict__ C, int ldc, int M, int N, int K) {
-  gemm_rows<16>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K);
+k_gemm_rows(const float* __restrict__ A, long sam, const float* __restrict__ Bm, long sbk, long sbn,
+            float* __restrict__ C, int ldc, int M, int N, int K, RowsEpi ep) {
+  gemm_rows<NT>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K, ep);
 }
 
 // C[M x N] += X^T Y summed over the K rows of X (K x M, rows ldx apart) and
@@ -215,11 +243,14 @@ k_gemm_rows16(const float* __restrict__ A, long sam, const float* __restrict__ B
 // thread % tiles) and sums the rows of its phase (ph = thread / tiles: rows
 // k0 + ph, k0 + ph + P, ... of the CTA's range, P = 256 / tiles), from
 // float4 loads; the phases are then summed through shared memory and each
-// CTA adds its sums into C (zeroed by the caller) atomically.
+// CTA adds its sums into C (zeroed by the caller) atomically.  With db, the
+// column sums of Y (of the unrounded values) are added to db[n % cb]: the bias
+// gradient, formed by the tiles of the first rows from values they hold anyway
+// (a pass of its own over the layer's gradient took 24 us).
 constexpr int kTnTM = 4, kTnTN = 8, kTnPad = kTnTM * kTnTN + 1;
 __global__ void __launch_bounds__(kRowsThreads)
 k_gemm_tn(const float* __restrict__ X, long ldx, const float* __restrict__ Y, long ldy, float* __restrict__ C,
-          int ldc, int M, int N, long K, long rows_per_cta) {
+          int ldc, int M, int N, long K, long rows_per_cta, float* __restrict__ db, int cb) {
   __shared__ float red[kRowsThreads * kTnPad];
   const int tn = N / kTnTN, tiles = (M / kTnTM) * tn;
   const int P = kRowsThreads / tiles;
@@ -230,6 +261,9 @@ k_gemm_tn(const float* __restrict__ X, long ldx, const float* __restrict__ Y, lo
   for (int i = 0; i < kTnTM; ++i)
 #pragma unroll
     for (int j = 0; j < kTnTN; ++j) acc[i][j] = 0.f;
+  float ysum[kTnTN];
+#pragma unroll
+  for (int j = 0; j < kTnTN; ++j) ysum[j] = 0.f;
   const long k0 = (long)blockIdx.x * rows_per_cta, k1 = k0 + rows_per_cta < K ? k0 + rows_per_cta : K;
   if (ph < P) {
 #pragma unroll 2
@@ -237,6 +271,8 @@ k_gemm_tn(const float* __restrict__ X, long ldx, const float* __restrict__ Y, lo
       const float4 xa = __ldg(reinterpret_cast<const float4*>(X + r * ldx + m0));
       const float4 ya = __ldg(reinterpret_cast<const float4*>(Y + r * ldy + n0));
       const float4 yb = __ldg(reinterpret_cast<const float4*>(Y + r * ldy + n0 + 4));
+      ysum[0] += ya.x; ysum[1] += ya.y; ysum[2] += ya.z; ysum[3] += ya.w;
+      ysum[4] += yb.x; ysum[5] += yb.y; ysum[6] += yb.z; ysum[7] += yb.w;
       const float xv[kTnTM] = {bf16r(xa.x), bf16r(xa.y), bf16r(xa.z), bf16r(xa.w)};
       const float yv[kTnTN] = {bf16r(ya.x), bf16r(ya.y), bf16r(ya.z), bf16r(ya.w),
                                bf16r(yb.x), bf16r(yb.y), bf16r(yb.z), bf16r(yb.w)};
@@ -250,7 +286,27 @@ k_gemm_tn(const float* __restrict__ X, long ldx, const float* __restrict__ Y, lo
   for (int i = 0; i < kTnTM; ++i)
 #pragma unroll
     for (int j = 0; j < kTnTN; ++j) red[threadIdx.x * kTnPad + i * kTnTN + j] = acc[i][j];
+  __shared__ float dbs[kC1];
+  if (db) {
+    if (threadIdx.x < cb) dbs[threadIdx.x] = 0.f;
+  }
   __syncthreads();
+  if (db) {
+    // the tiles of the first rows hold every column once; a warp adds up its
+    // lanes' columns of one channel group of 8 (n0 is a multiple of 8, so
+    // column j of a tile is channel (n0 + j) % cb)
+    for (int grp = 0; grp < cb; grp += kTnTN) {
+      const bool mine = ph < P && m0 == 0 && (cb <= kTnTN || n0 % cb == grp);
+#pragma unroll
+      for (int j = 0; j < kTnTN; ++j) {
+        float v = mine ? ysum[j] : 0.f;
+        for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+        if ((threadIdx.x & 31) == 0 && v != 0.f) atomicAdd(&dbs[(grp + j) % cb], v);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < cb) atomicAdd(db + threadIdx.x, dbs[threadIdx.x]);
+  }
   // output o = (m, n): G = 256 / MN thread groups (at least 1) share its phases
   const int MN = M * N;
   const int G = MN >= kRowsThreads ? 1 : kRowsThreads / MN;
@@ -281,8 +337,21 @@ __global__ void k_relu_back(float* __restrict__ dx, const float* __restrict__ y,
     if (!(y[i] > 0.f)) dx[i] = 0.f;
 }
 
-// db[c] += sum over rows and over the column groups of dy[.., g*cb + c]
-__global__ void k_bias_grad(const float* __restrict__ dy, float* __restrict__ db, long rows, int cols, int cb) {
+// db[c] = sum over the rows of dy[.., c]: one thread a column, neighbouring
+// threads on neighbouring columns (a CTA a column took 31 us for the 8192
+// columns of the MLP's second layer).
+__global__ void k_bias_grad(const float* __restrict__ dy, float* __restrict__ db, int rows, int cols) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= cols) return;
+  float acc = 0.f;
+#pragma unroll 8
+  for (int r = 0; r < rows; ++r) acc += dy[(long)r * cols + c];
+  db[c] = acc;
+}
+
+// db[c] += sum over rows and over the column groups of dy[.., g*cb + c], for
+// small batches, whose weight gradients do not go through k_gemm_tn.
+__global__ void k_bias_grad_groups(const float* __restrict__ dy, float* __restrict__ db, long rows, int cols, int cb) {
   __shared__ float sh[256];
   const int c = blockIdx.x;  // output channel
   float acc = 0.f;
@@ -338,69 +407,98 @@ __global__ void k_out_to_psi(const float* __restrict__ o, double* __restrict__ p
   }
 }
 
-// Per-sample sums for the loss: s = <u, t> (complex), uu = |u|^2, tt = |t|^2.
-// One block per sample; u is read from the L3 output, t from FP64 targets.
-__global__ void k_loss_sums(const float* __restrict__ o, const double* __restrict__ t, double* __restrict__ sums) {
+// Per-sample sums for the loss: s = <u, t> (complex), uu = |u|^2, tt = |t|^2,
+// u read from the L3 output, t from FP64 targets.  kLossChunks CTAs a sample,
+// each leaving its four sums in sums[b][chunk][4] (with one CTA a sample, 32
+// of the 152 SMs worked, 278 us at batch 32; these 32 x 16 take 40).  Bound by
+// the FP64 pipe: 8 operations a point.
+constexpr int kLossChunks = 16;
+__global__ void __launch_bounds__(256)
+k_loss_sums(const float* __restrict__ o, const double* __restrict__ t, double* __restrict__ sums) {
   __shared__ double sh[4][256];
   const int b = blockIdx.x;
   double a[4] = {0, 0, 0, 0};
   const long base = (long)b * kOutN * 2;
-  for (long i = threadIdx.x; i < (long)kOutN; i += blockDim.x) {
+  constexpr int per = kOutN / kLossChunks;
+  const int i0 = blockIdx.y * per;
+#pragma unroll 4
+  for (int i = i0 + threadIdx.x; i < i0 + per; i += 256) {
     // iterate over grid points via output rows: element pairs (ch 0, ch 1)
     const long e = base + 2 * i;             // index into o of (row, 2*s3)
-    const long row = e / kN3;
-    const int col = (int)(e % kN3);
     int bb, z, y, x, ch;
-    out_pos(row, col, bb, z, y, x, ch);
-    const double ur = o[e], ui = o[e + 1];
-    const long ti = (((long)b * kOutZ + z) * kOutY + y) * kOutX + x;
-    const double tr = t[2 * ti], tim = t[2 * ti + 1];
-    a[0] += ur * tr + ui * tim;   // Re <u,t> = Re sum u conj(t)
-    a[1] += ui * tr - ur * tim;   // Im
-    a[2] += ur * ur + ui * ui;
-    a[3] += tr * tr + tim * tim;
+    out_pos(e / kN3, (int)(e % kN3), bb, z, y, x, ch);
+    const float2 u = *reinterpret_cast<const float2*>(o + e);
+    const double2 tv = *reinterpret_cast<const double2*>(t + 2 * ((((long)b * kOutZ + z) * kOutY + y) * kOutX + x));
+    const double ur = f2d_bits(u.x), ui = f2d_bits(u.y);
+    a[0] = fma(ur, tv.x, fma(ui, tv.y, a[0]));     // Re <u,t> = Re sum u conj(t)
+    a[1] = fma(ui, tv.x, fma(-ur, tv.y, a[1]));    // Im
+    a[2] = fma(ur, ur, fma(ui, ui, a[2]));
+    a[3] = fma(tv.x, tv.x, fma(tv.y, tv.y, a[3]));
   }
+  // one warp a sum: 12 additions a lane instead of a tree over 256 threads
   for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] = a[k];
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-      for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
-    __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < 4) {
+    double v = sh[w][lane];
+    for (int q = 1; q < 8; ++q) v += sh[w][q * 32 + lane];
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+    if (lane == 0) sums[((long)b * kLossChunks + blockIdx.y) * 4 + w] = v;
   }
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 4; ++k) sums[b * 4 + k] = sh[k][0];
+}
+
+// A sample's four sums from its chunks.
+__device__ __forceinline__ void loss_total(const double* __restrict__ sums, int b, double (&v)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = 0.0;
+  for (int c = 0; c < kLossChunks; ++c) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += sums[((long)b * kLossChunks + c) * 4 + k];
+  }
 }
 
 // Loss (mean over the batch) and dL/d(Re u, Im u) in the L3 output layout:
-// g = -2 (s t / (uu tt) - |s|^2 u / (uu^2 tt)) / B.
-__global__ void k_loss_grad(const float* __restrict__ o, const double* __restrict__ t, const double* __restrict__ sums,
-                            float* __restrict__ dO, float* __restrict__ loss, int B) {
-  const long total = (long)B * kOutN;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const long e = 2 * i;
-    const long row = e / kN3;
-    const int col = (int)(e % kN3);
-    int b, z, y, x, ch;
-    out_pos(row, col, b, z, y, x, ch);
-    const double sr = sums[b * 4 + 0], si = sums[b * 4 + 1], uu = sums[b * 4 + 2], tt = sums[b * 4 + 3];
-    const double s2 = sr * sr + si * si;
-    const long ti = (((long)b * kOutZ + z) * kOutY + y) * kOutX + x;
-    const double tr = t[2 * ti], tim = t[2 * ti + 1];
-    const double ur = o[e], ui = o[e + 1];
-    // s t = (sr + i si)(tr + i tim)
-    const double str = sr * tr - si * tim, sti = sr * tim + si * tr;
-    const double c1 = 1.0 / (uu * tt), c2 = s2 / (uu * uu * tt);
-    const double scale = -2.0 / B;
-    dO[e] = (float)(scale * (c1 * str - c2 * ur));
-    dO[e + 1] = (float)(scale * (c1 * sti - c2 * ui));
+// g = -2 (s t / (uu tt) - |s|^2 u / (uu^2 tt)) / B = A t - C u.  A CTA works on
+// one sample and forms its coefficients once (per point they cost two
+// divisions); 6 FP64 operations a point remain (139 -> 36 us at batch 32).
+__global__ void __launch_bounds__(256)
+k_loss_grad(const float* __restrict__ o, const double* __restrict__ t, const double* __restrict__ sums,
+            float* __restrict__ dO, float* __restrict__ loss, int B) {
+  __shared__ double co[3];
+  const int b = blockIdx.x;
+  if (threadIdx.x == 0) {
+    double v[4];
+    loss_total(sums, b, v);
+    const double scale = -2.0 / B, c1 = 1.0 / (v[2] * v[3]);
+    co[0] = scale * c1 * v[0];
+    co[1] = scale * c1 * v[1];
+    co[2] = scale * ((v[0] * v[0] + v[1] * v[1]) / (v[2] * v[2] * v[3]));
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  __syncthreads();
+  const double ar = co[0], ai = co[1], c = co[2];
+  const long base = (long)b * kOutN * 2;
+  constexpr int per = kOutN / kLossChunks;
+  const int i0 = blockIdx.y * per;
+#pragma unroll 4
+  for (int i = i0 + threadIdx.x; i < i0 + per; i += 256) {
+    const long e = base + 2 * i;
+    int bb, z, y, x, ch;
+    out_pos(e / kN3, (int)(e % kN3), bb, z, y, x, ch);
+    const float2 u = *reinterpret_cast<const float2*>(o + e);
+    const double2 tv = *reinterpret_cast<const double2*>(t + 2 * ((((long)b * kOutZ + z) * kOutY + y) * kOutX + x));
+    const double ur = f2d_bits(u.x), ui = f2d_bits(u.y);
+    const double gr = fma(ar, tv.x, fma(-ai, tv.y, -c * ur)), gi = fma(ar, tv.y, fma(ai, tv.x, -c * ui));
+    *reinterpret_cast<float2*>(dO + e) = make_float2(d2f_bits(gr), d2f_bits(gi));
+  }
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
     double acc = 0.0;
-    for (int b = 0; b < B; ++b) {
-      const double sr = sums[b * 4], si = sums[b * 4 + 1], uu = sums[b * 4 + 2], tt = sums[b * 4 + 3];
-      acc += 1.0 - (sr * sr + si * si) / (uu * tt);
+    for (int q = threadIdx.x; q < B; q += 32) {
+      double v[4];
+      loss_total(sums, q, v);
+      acc += 1.0 - (v[0] * v[0] + v[1] * v[1]) / (v[2] * v[3]);
     }
-    *loss = (float)(acc / B);
+    for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+    if (threadIdx.x == 0) *loss = (float)(acc / B);
   }
 }
 
@@ -488,7 +586,7 @@ cudaError_t net_ensure(atkm_guess_net* n, int B) {
   al(&n->dy1, (size_t)B * kV0 * kN1);
   al(&n->dy2, (size_t)B * kV0 * 8 * kN2);
   al(&n->dO, (size_t)B * kV0 * 64 * kN3);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&n->sums, (size_t)B * 4 * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&n->sums, (size_t)B * kLossChunks * 4 * sizeof(double));
   if (e != cudaSuccess) {
     net_free_acts(n);
     return e;
@@ -577,17 +675,27 @@ cudaError_t gemm_tc(const float* A, long sam, long sak, const float* Bm, long sb
   return launch_tc<128>(grid, Ap, asm_, ask, Bp, bsk, bsn, C, scm, scn, Mm, Nn, K, kchunk, st);
 }
 
+// What a product may do besides: an epilogue (RowsEpi), or the column sums of
+// its second operand.  `done` tells whether the kernel chosen did it; if not,
+// the caller runs the separate kernel.
+struct GemmExtra {
+  RowsEpi epi;
+  float* db = nullptr;
+  int cb = 1;
+  bool done = false;
+};
+
 cudaError_t gemm_launch(const float* A, long sam, long sak, const float* Bm, long sbk, long sbn, float* C, int ldc,
-                        int M, int N, int K, cudaStream_t st, bool split_k);
+                        int M, int N, int K, cudaStream_t st, bool split_k, GemmExtra* x);
 
 cudaError_t gemm(const float* A, long sam, long sak, const float* Bm, long sbk, long sbn, float* C, int ldc, int M, int N,
-                 int K, cudaStream_t st, bool split_k) {
-  if (!g_gemm_timer) return gemm_launch(A, sam, sak, Bm, sbk, sbn, C, ldc, M, N, K, st, split_k);
+                 int K, cudaStream_t st, bool split_k, GemmExtra* x = nullptr) {
+  if (!g_gemm_timer) return gemm_launch(A, sam, sak, Bm, sbk, sbn, C, ldc, M, N, K, st, split_k, x);
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   if (e == cudaSuccess) e = cudaEventRecord(a, st);
-  if (e == cudaSuccess) e = gemm_launch(A, sam, sak, Bm, sbk, sbn, C, ldc, M, N, K, st, split_k);
+  if (e == cudaSuccess) e = gemm_launch(A, sam, sak, Bm, sbk, sbn, C, ldc, M, N, K, st, split_k, x);
   if (e == cudaSuccess) e = cudaEventRecord(b, st);
   if (a && b) g_gemm_timer->ev.emplace_back(a, b);
   else {
@@ -598,19 +706,23 @@ cudaError_t gemm(const float* A, long sam, long sak, const float* Bm, long sbk, 
 }
 
 cudaError_t gemm_launch(const float* A, long sam, long sak, const float* Bm, long sbk, long sbn, float* C, int ldc,
-                        int M, int N, int K, cudaStream_t st, bool split_k) {
+                        int M, int N, int K, cudaStream_t st, bool split_k, GemmExtra* x) {
   // row-local products: the output rows need only K x N <= 4096 weights
   const bool a16 = ((uintptr_t)A & 15) == 0 && ((uintptr_t)C & 15) == 0;
   if (sak == 1 && (long)K * N <= 4096 && N % 8 == 0 && M >= 1024 && K % 4 == 0 && sam % 4 == 0 && ldc % 4 == 0 &&
       a16) {
-    const int nt = N % 16 == 0 ? 16 : 8;
+    // as many outputs a thread as leave two CTAs per SM
+    const long want = 2L * std::max(device_sm_count(), 1) * kRowsThreads;
+    int nt = N % 16 == 0 ? 16 : 8;
+    while (nt > 4 && (long)M * (N / nt) < want) nt >>= 1;
     const long threads = (long)M * (N / nt);
     const int blocks = (int)((threads + kRowsThreads - 1) / kRowsThreads);
     const size_t sm = (size_t)K * N * sizeof(float);
-    if (nt == 16)
-      k_gemm_rows16<<<blocks, kRowsThreads, sm, st>>>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K);
-    else
-      k_gemm_rows8<<<blocks, kRowsThreads, sm, st>>>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K);
+    const RowsEpi ep = x ? x->epi : RowsEpi{};
+    if (x) x->done = true;
+    if (nt == 16) k_gemm_rows<16><<<blocks, kRowsThreads, sm, st>>>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K, ep);
+    else if (nt == 8) k_gemm_rows<8><<<blocks, kRowsThreads, sm, st>>>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K, ep);
+    else k_gemm_rows<4><<<blocks, kRowsThreads, sm, st>>>(A, sam, Bm, sbk, sbn, C, ldc, M, N, K, ep);
     count_launches(1);
     return cudaGetLastError();
   }
@@ -625,7 +737,10 @@ cudaError_t gemm_launch(const float* A, long sam, long sak, const float* Bm, lon
     long ctas = std::min<long>((long)nsm * 2, std::max<long>(1, (long)K / (P * 16)));
     const long rows = ((long)K + ctas - 1) / ctas;
     ctas = ((long)K + rows - 1) / rows;
-    k_gemm_tn<<<(int)ctas, kRowsThreads, 0, st>>>(A, sak, Bm, sbk, C, ldc, M, N, (long)K, rows);
+    const bool with_db = x && x->db && x->cb <= kC1;
+    if (with_db) x->done = true;
+    k_gemm_tn<<<(int)ctas, kRowsThreads, 0, st>>>(A, sak, Bm, sbk, C, ldc, M, N, (long)K, rows, with_db ? x->db : nullptr,
+                                                  with_db ? x->cb : 1);
     count_launches(1);
     return cudaGetLastError();
   }
@@ -662,13 +777,23 @@ cudaError_t net_forward(atkm_guess_net* n, int B, cudaStream_t st) {
   k_bias_act<<<ew_grid((long)B * kH), 256, 0, st>>>(n->h1, w + kL.b1, B, kH, kH, 1);
   if ((e = gemm(n->h1, kH, 1, w + kL.W2, kZ, 1, n->z, kZ, B, kZ, kH, st, false))) return e;
   k_bias_act<<<ew_grid((long)B * kZ), 256, 0, st>>>(n->z, w + kL.b2, B, kZ, kZ, 0);
-  if ((e = gemm(n->z, kC0, 1, w + kL.W3, kN1, 1, n->y1, kN1, (int)r1, kN1, kC0, st, false))) return e;
-  k_bias_act<<<ew_grid(r1 * kN1), 256, 0, st>>>(n->y1, w + kL.b3, r1, kN1, kC1, 1);
-  if ((e = gemm(n->y1, kC1, 1, w + kL.W4, kN2, 1, n->y2, kN2, (int)r2, kN2, kC1, st, false))) return e;
-  k_bias_act<<<ew_grid(r2 * kN2), 256, 0, st>>>(n->y2, w + kL.b4, r2, kN2, kC2, 1);
-  if ((e = gemm(n->y2, kC2, 1, w + kL.W5, kN3, 1, n->o, kN3, (int)r3, kN3, kC2, st, false))) return e;
-  k_bias_act<<<ew_grid(r3 * kN3), 256, 0, st>>>(n->o, w + kL.b5, r3, kN3, kC3, 0);
-  count_launches(5);
+  // the transposed convolutions: bias and activation in the product's epilogue
+  auto conv = [&](const float* in, int k, size_t W, size_t b, float* out, int nout, int cb, long rows, int relu) {
+    GemmExtra x;
+    x.epi.bias = w + b;
+    x.epi.cb = cb;
+    x.epi.relu = relu;
+    cudaError_t r = gemm(in, k, 1, w + W, nout, 1, out, nout, (int)rows, nout, k, st, false, &x);
+    if (r == cudaSuccess && !x.done) {
+      k_bias_act<<<ew_grid(rows * nout), 256, 0, st>>>(out, w + b, rows, nout, cb, relu);
+      count_launches(1);
+    }
+    return r;
+  };
+  if ((e = conv(n->z, kC0, kL.W3, kL.b3, n->y1, kN1, kC1, r1, 1))) return e;
+  if ((e = conv(n->y1, kC1, kL.W4, kL.b4, n->y2, kN2, kC2, r2, 1))) return e;
+  if ((e = conv(n->y2, kC2, kL.W5, kL.b5, n->o, kN3, kC3, r3, 0))) return e;
+  count_launches(2);
   return cudaGetLastError();
 }
 
@@ -678,32 +803,43 @@ cudaError_t net_backward(atkm_guess_net* n, int B, const double* targets, float*
   float* g = n->g;
   cudaError_t e;
   const long r1 = (long)B * kV0, r2 = r1 * 8, r3 = r2 * 8;
-  k_loss_sums<<<B, 256, 0, st>>>(n->o, targets, n->sums);
-  k_loss_grad<<<ew_grid((long)B * kOutN), 256, 0, st>>>(n->o, targets, n->sums, n->dO, loss_dev, B);
+  k_loss_sums<<<dim3(B, kLossChunks), 256, 0, st>>>(n->o, targets, n->sums);
+  k_loss_grad<<<dim3(B, kLossChunks), 256, 0, st>>>(n->o, targets, n->sums, n->dO, loss_dev, B);
   if ((e = cudaMemsetAsync(g, 0, kL.total * sizeof(float), st))) return e;
-  // L3
-  if ((e = gemm(n->y2, 1, kC2, n->dO, kN3, 1, g + kL.W5, kN3, kC2, kN3, (int)r3, st, true))) return e;
-  k_bias_grad<<<dim3(kC3, 64), 256, 0, st>>>(n->dO, g + kL.b5, r3, kN3, kC3);
-  if ((e = gemm(n->dO, kN3, 1, w + kL.W5, 1, kN3, n->dy2, kC2, (int)r3, kC2, kN3, st, false))) return e;
-  k_relu_back<<<ew_grid(r2 * kN2), 256, 0, st>>>(n->dy2, n->y2, r2 * kN2);
-  // L2
-  if ((e = gemm(n->y1, 1, kC1, n->dy2, kN2, 1, g + kL.W4, kN2, kC1, kN2, (int)r2, st, true))) return e;
-  k_bias_grad<<<dim3(kC2, 64), 256, 0, st>>>(n->dy2, g + kL.b4, r2, kN2, kC2);
-  if ((e = gemm(n->dy2, kN2, 1, w + kL.W4, 1, kN2, n->dy1, kC1, (int)r2, kC1, kN2, st, false))) return e;
-  k_relu_back<<<ew_grid(r1 * kN1), 256, 0, st>>>(n->dy1, n->y1, r1 * kN1);
-  // L1
-  if ((e = gemm(n->z, 1, kC0, n->dy1, kN1, 1, g + kL.W3, kN1, kC0, kN1, (int)r1, st, true))) return e;
-  k_bias_grad<<<dim3(kC1, 64), 256, 0, st>>>(n->dy1, g + kL.b3, r1, kN1, kC1);
-  if ((e = gemm(n->dy1, kN1, 1, w + kL.W3, 1, kN1, n->dz, kC0, (int)r1, kC0, kN1, st, false))) return e;
+  // A transposed convolution's gradients: weights and biases from its input x
+  // (cin channels) and the gradient dy of its output (nout wide, cb channels),
+  // then dx = dy W^T, zero where the input's activation was not positive.
+  auto back = [&](const float* x, int cin, const float* dy, int nout, int cb, size_t W, size_t b, float* dx, long rows,
+                  const float* mask) {
+    GemmExtra gw, gx;
+    gw.db = g + b;
+    gw.cb = cb;
+    cudaError_t r = gemm(x, 1, cin, dy, nout, 1, g + W, nout, cin, nout, (int)rows, st, true, &gw);
+    if (r != cudaSuccess) return r;
+    if (!gw.done) {
+      k_bias_grad_groups<<<dim3(cb, 64), 256, 0, st>>>(dy, g + b, rows, nout, cb);
+      count_launches(1);
+    }
+    gx.epi.mask = mask;
+    r = gemm(dy, nout, 1, w + W, 1, nout, dx, cin, (int)rows, cin, nout, st, false, &gx);
+    if (r == cudaSuccess && mask && !gx.done) {
+      k_relu_back<<<ew_grid(rows * cin), 256, 0, st>>>(dx, mask, rows * cin);
+      count_launches(1);
+    }
+    return r;
+  };
+  if ((e = back(n->y2, kC2, n->dO, kN3, kC3, kL.W5, kL.b5, n->dy2, r3, n->y2))) return e;
+  if ((e = back(n->y1, kC1, n->dy2, kN2, kC2, kL.W4, kL.b4, n->dy1, r2, n->y1))) return e;
+  if ((e = back(n->z, kC0, n->dy1, kN1, kC1, kL.W3, kL.b3, n->dz, r1, nullptr))) return e;
   // MLP2 (no activation on z)
   if ((e = gemm(n->h1, 1, kH, n->dz, kZ, 1, g + kL.W2, kZ, kH, kZ, B, st, true))) return e;
-  k_bias_grad<<<dim3(kZ, 1), 256, 0, st>>>(n->dz, g + kL.b2, B, kZ, kZ);
+  k_bias_grad<<<kZ / 64, 64, 0, st>>>(n->dz, g + kL.b2, B, kZ);
   if ((e = gemm(n->dz, kZ, 1, w + kL.W2, 1, kZ, n->dh1, kH, B, kH, kZ, st, true))) return e;
   k_relu_back<<<ew_grid((long)B * kH), 256, 0, st>>>(n->dh1, n->h1, (long)B * kH);
   // MLP1
   if ((e = gemm(n->fpad, 1, kFpad, n->dh1, kH, 1, g + kL.W1, kH, kFpad, kH, B, st, true))) return e;
-  k_bias_grad<<<dim3(kH, 1), 256, 0, st>>>(n->dh1, g + kL.b1, B, kH, kH);
-  count_launches(11);
+  k_bias_grad<<<kH / 64, 64, 0, st>>>(n->dh1, g + kL.b1, B, kH);
+  count_launches(5);
   return cudaGetLastError();
 }
 
