@@ -105,6 +105,11 @@ inline int device_sm_count() {
   return v;
 }
 
+// p + i strides, the stride in bytes: one 32 x 32 -> 64 multiply-add
+template <typename T> __device__ __forceinline__ T* step(T* p, int i, int stride) {
+  return (T*)((const char*)p + (long long)i * stride);
+}
+
 // Programmatic dependent launch: a kernel started by launch_pdl may be resident
 // before its predecessor in the stream has ended, which hides the launch gap
 // (1 to 2 us, as long as a small pass itself).  It calls pdl_trigger() at its
@@ -156,6 +161,7 @@ struct FftLen {
   int nstages;
   int radix[kMaxStages];
   const float2* tw32;  // e^{-2 pi i m / L}, m = 0..L-1
+  const float2* tws;   // the same by stage, for the power-of-two register engine (k_fast_twiddles)
 };
 
 template <typename R> __host__ __device__ __forceinline__ const cx<R>* tw_table(const FftLen& f);
@@ -515,7 +521,7 @@ struct atkm_plan {
   double hvol;
   atkm::FftLen fN[3];  // unpadded lengths N_x, N_y, N_z
   atkm::FftLen fM[3];  // padded lengths 2N_x, 2N_y, 2N_z
-  float2* tw32;        // twiddle pool
+  float2* tw32;        // twiddle pool (by index, then by stage)
   atkm::IntLen iN[3];  // the same lengths for the integer passes
   atkm::IntLen iM[3];
   int4* twi;           // integer twiddle pool

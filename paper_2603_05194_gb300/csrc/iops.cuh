@@ -27,11 +27,6 @@ namespace atkm {
 
 __device__ __forceinline__ int ikfreq(int m, int M) { return m < (M >> 1) ? m : m - M; }
 
-// p + i strides, the stride in bytes: one 32 x 32 -> 64 multiply-add
-template <typename T> __device__ __forceinline__ T* step(T* p, int i, int stride) {
-  return (T*)((const char*)p + (long long)i * stride);
-}
-
 // Exponents of an integer array written by one pass: element (row, col) of
 // the array belongs to the tile (row >> rs, col >> cs).
 struct ExpTab {

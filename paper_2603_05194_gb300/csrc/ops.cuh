@@ -117,21 +117,31 @@ template <int L> struct FastCfg {
   static constexpr int T = kFastElems / L;      // lines per CTA
   static constexpr int A = (L >= 512) ? 3 : (L >= 64 ? 2 : 1);  // radix-8 stages
   static constexpr int REM = L / (A == 3 ? 512 : (A == 2 ? 64 : 8));  // 1, 2 or 4
+  // Shared-memory index of element (t, pos): line-major tiles with one pad
+  // element every 8 positions, column tiles [pos][t] with a pad row every 8
+  // positions where a row is less than 128 bytes.  The 8-byte accesses of a
+  // half warp fall into distinct banks, and the index is affine in the stage's
+  // inner index, so that an exchange computes two addresses (a pad after every
+  // 16 elements of the linear index took two instructions an access more).
+  template <bool LM> static constexpr bool kPad = LM || T < 16;
+  template <bool LM> __device__ static __forceinline__ int at(int t, int pos) {
+    if (LM) return t * (L + L / 8) + pos + (pos >> 3);
+    return (kPad<LM> ? pos + (pos >> 3) : pos) * T + t;
+  }
+  // index step of n positions, n a multiple of 8 (or less than 8 within an aligned 8)
+  template <bool LM> static constexpr int span(int n) { return (kPad<LM> ? n + n / 8 : n) * (LM ? 1 : T); }
+  template <bool LM> static constexpr int buf() { return kPad<LM> ? kFastElems + kFastElems / 8 : kFastElems; }
 };
 
 template <typename R, int L> struct FastSmem {
-  static constexpr int buf = kFastElems + (kFastElems >> SmemShift<R>::value) + 1;
   // stage s exchanges through b0 (s even) or b1 (s odd) unless it is the last
   // stage; with one or two radix-8 stages and nothing after them (L <= 64)
   // only b0 is used, so b1 takes no shared memory
   static constexpr bool kTwoBufs = FastCfg<L>::A == 3 || (FastCfg<L>::A == 2 && FastCfg<L>::REM > 1);
-  static constexpr size_t bytes = (size_t)(L + (kTwoBufs ? 2 : 1) * buf) * sizeof(cx<R>);
+  template <bool LM> static constexpr size_t bytes() {
+    return (size_t)((kTwoBufs ? 2 : 1) * FastCfg<L>::template buf<LM>()) * sizeof(cx<R>);
+  }
 };
-
-template <typename R, int L, bool LM> __device__ __forceinline__ int fsa(int t, int pos) {
-  const int lin = LM ? t * L + pos : pos * FastCfg<L>::T + t;
-  return lin + (lin >> SmemShift<R>::value);
-}
 
 // Transforms the 8 register elements v[r] = line[j + TPL r] of line t in place
 // (sign S, unnormalised); on return v[r] holds frequency j + TPL r.  ZU: the
@@ -147,10 +157,10 @@ __device__ __forceinline__ void fast_fft(cx<R> (&v)[8], cx<R>* b0, cx<R>* b1, co
     const int k = j & (Ns - 1);
     const bool last = (s == C::A - 1) && (C::REM == 1);
     if (s > 0) {
-      const int tws = L / (8 * Ns);
+      const cx<R>* wk = tw + (s == 2 ? 56 : 0) + k;  // the tables of the stages before: 7 Ns entries each
 #pragma unroll
       for (int r = 1; r < 8; ++r) {
-        const cx<R> w = tw[k * r * tws];
+        const cx<R> w = __ldg(wk + (r - 1) * Ns);
         v[r] = (S < 0) ? cmul<R>(v[r], w) : cmulc<R>(v[r], w);
       }
     }
@@ -159,26 +169,32 @@ __device__ __forceinline__ void fast_fft(cx<R> (&v)[8], cx<R>* b0, cx<R>* b1, co
     else Dft<R, 8, S>::run(v);
     if (!last) {
       cx<R>* b = (s & 1) ? b1 : b0;
-      const int base = (j - k) * 8 + k;
+      cx<R>* wp = b + C::template at<LM>(t, (j - k) * 8 + k);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) b[fsa<R, L, LM>(t, base + r * Ns)] = v[r];
+      for (int r = 0; r < 8; ++r) wp[C::template span<LM>(r * Ns)] = v[r];
       __syncthreads();
+      if constexpr (C::TPL >= 8) {
+        const cx<R>* rp = b + C::template at<LM>(t, j);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = b[fsa<R, L, LM>(t, j + C::TPL * r)];
+        for (int r = 0; r < 8; ++r) v[r] = rp[C::template span<LM>(C::TPL * r)];
+      } else {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = b[C::template at<LM>(t, j + C::TPL * r)];
+      }
     }
     Ns *= 8;
   }
   if constexpr (C::REM > 1) {
-    constexpr int Q = C::REM, M = 8 / C::REM;  // M butterflies of radix Q per thread
+    constexpr int Q = C::REM, M = 8 / C::REM, NsQ = L / Q;  // M butterflies of radix Q per thread
+    const cx<R>* wk = tw + (C::A == 3 ? 504 : (C::A == 2 ? 56 : 0)) + j;
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-      const int b = j + C::TPL * m;  // butterfly index = its twiddle exponent base (Ns = L/Q)
       cx<R> u[Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) u[q] = v[m + M * q];
 #pragma unroll
       for (int q = 1; q < Q; ++q) {
-        const cx<R> w = tw[b * q];
+        const cx<R> w = __ldg(wk + (q - 1) * NsQ + C::TPL * m);
         u[q] = (S < 0) ? cmul<R>(u[q], w) : cmulc<R>(u[q], w);
       }
       if (LO) Dft<R, Q, S>::run_lo(u);
@@ -228,9 +244,8 @@ template <typename R, int L, class Op>
 __global__ void __launch_bounds__(kThreads, fast_min_blocks<R, L, Op>()) k_fast(Op op, const cx<R>* __restrict__ twg) {
   using C = FastCfg<L>;
   extern __shared__ __align__(16) unsigned char fast_smem[];
-  cx<R>* tw = reinterpret_cast<cx<R>*>(fast_smem);
-  cx<R>* b0 = tw + L;
-  cx<R>* b1 = b0 + FastSmem<R, L>::buf;
+  cx<R>* b0 = reinterpret_cast<cx<R>*>(fast_smem);
+  cx<R>* b1 = b0 + C::template buf<Op::kLM>();
   int t, j;
   if (Op::kLM) { t = threadIdx.x / C::TPL; j = threadIdx.x % C::TPL; }
   else { j = threadIdx.x / C::T; t = threadIdx.x % C::T; }
@@ -254,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, fast_min_blocks<R, L, Op>()) k_fast(
     ok = op.valid(o, x);
   }
   // epilogue inputs of this thread's elements, [r][thread] (ops with kPre > 0)
-  unsigned char* pre = fast_smem + FastSmem<R, L>::bytes;
+  unsigned char* pre = fast_smem + FastSmem<R, L>::template bytes<Op::kLM>();
   if constexpr (Op::kPre > 0) {
     if (ok) {
 #pragma unroll
@@ -271,27 +286,25 @@ __global__ void __launch_bounds__(kThreads, fast_min_blocks<R, L, Op>()) k_fast(
 #pragma unroll
     for (int r = 0; r < 8; ++r) vin[r] = v[r];
   }
-  // Twiddles are read through L1 from global memory, which avoids the bank
-  // conflicts of the strided table accesses (these passes are issue-bound).
-  const cx<R>* twsrc = twg;
+  // twiddles are read through L1 from the stage tables in global memory
   __syncthreads();
   constexpr int NR = Op::kRed > 0 ? Op::kRed : 1;
   R acc[NR];
 #pragma unroll
   for (int s = 0; s < NR; ++s) acc[s] = (R)0;
   constexpr bool kLo1 = Op::kHalfOut && !Op::kSecond && !Op::kMirror;
-  fast_fft<R, L, Op::kSign1, Op::kLM, Op::kZeroUpper, kLo1>(v, b0, b1, twsrc, t, j);
+  fast_fft<R, L, Op::kSign1, Op::kLM, Op::kZeroUpper, kLo1>(v, b0, b1, twg, t, j);
   if constexpr (Op::kMirror) {
     // exchange so every thread sees the frequency L - k of each of its k
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < 8; ++r) b0[fsa<R, L, Op::kLM>(t, j + C::TPL * r)] = v[r];
+    for (int r = 0; r < 8; ++r) b0[C::template at<Op::kLM>(t, j + C::TPL * r)] = v[r];
     __syncthreads();
     if (ok) {
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
         const int k = j + C::TPL * r;
-        op.post(o, x, k, v[r], b0[fsa<R, L, Op::kLM>(t, (L - k) & (L - 1))], acc);
+        op.post(o, x, k, v[r], b0[C::template at<Op::kLM>(t, (L - k) & (L - 1))], acc);
       }
     }
   } else {
@@ -301,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, fast_min_blocks<R, L, Op>()) k_fast(
     }
     if (Op::kSecond) {
       __syncthreads();
-      fast_fft<R, L, -Op::kSign1, Op::kLM, false, Op::kHalfOut>(v, b0, b1, twsrc, t, j);
+      fast_fft<R, L, -Op::kSign1, Op::kLM, false, Op::kHalfOut>(v, b0, b1, twg, t, j);
     }
     if constexpr (Op::kPre > 0) {
       cp_async_wait_all();
@@ -459,10 +472,10 @@ inline cudaError_t ensure_smem(std::atomic<unsigned long long>& done, K kernel, 
 template <typename R, int L, class Op>
 inline cudaError_t launch_fast_L(const Op& op, const FftLen& f, const PassGrid& pg, cudaStream_t st) {
   static std::atomic<unsigned long long> prepared{0};
-  const size_t sm = FastSmem<R, L>::bytes + (size_t)Op::kPre * 8 * kThreads;
+  const size_t sm = FastSmem<R, L>::template bytes<Op::kLM>() + (size_t)Op::kPre * 8 * kThreads;
   cudaError_t e = ensure_smem(prepared, k_fast<R, L, Op>, sm);
   if (e != cudaSuccess) return e;
-  k_fast<R, L, Op><<<pg.grid, kThreads, sm, st>>>(op, tw_table_host<R>(f));
+  k_fast<R, L, Op><<<pg.grid, kThreads, sm, st>>>(op, f.tws);
   return cudaGetLastError();
 }
 
@@ -568,21 +581,20 @@ template <typename R> struct OpAtkmYF : OpBase<-1, false, 0, false> {
   const cx<R>* W1; cx<R>* W2; Cst<R> c; int XS;
   __device__ bool valid(int, int x) const { return x <= c.Nx; }
   __device__ cx<R> load(int o, int x, int pos) const {
-    return pos < c.Ny ? W1[((size_t)o * c.Ny + pos) * XS + x] : czero<R>();
+    return pos < c.Ny ? *step(W1 + (size_t)o * c.Ny * XS + x, pos, XS * (int)sizeof(cx<R>)) : czero<R>();
   }
   __device__ void spectral(int, int, int, cx<R>&, R*) const {}
-  __device__ void store(int o, int x, int pos, cx<R> v, R*) const { W2[((size_t)o * c.My + pos) * XS + x] = v; }
+  __device__ void store(int o, int x, int pos, cx<R> v, R*) const {
+    *step(W2 + (size_t)o * c.My * XS + x, pos, XS * (int)sizeof(cx<R>)) = v;
+  }
 };
 
 // z forward * K_sym / (2 Mx My Mz) * inverse: o = ky, x = kx in [0, Nx]; rows z < Nz
 // (the 2 undoes the doubled half spectrum that OpAtkmXF stores).
 // K_sym = (K(k) + K(-k))/2 = -1 + 3 U0 (A^2 + B^2), A = sum of n_a nu_a over
 // axes whose index is not the padded Nyquist index, B over those that are.
-// FP64 and double-word passes are bound by arithmetic: they read K_sym, pre-
-// scaled, from the plan's table in the layout of W2 (k_multiplier_half; 8 B a
-// point, about 9 FP64 instructions fewer).  FP32 passes are bound by issue and
-// bandwidth: they form it from the U0 octant (mostly L2-resident), which
-// costs less than the table's extra 4 B a point.
+// It is formed from the U0 octant (mostly L2-resident), which costs less than
+// a table's extra 4 B a point.
 template <typename R> struct OpAtkmZ : OpBase<-1, true, 0, false> {
   static constexpr bool kZeroUpper = true;  // rows z >= Nz = L/2 are the padding
   static constexpr bool kHalfOut = true;    // only rows z < Nz are kept
@@ -590,7 +602,7 @@ template <typename R> struct OpAtkmZ : OpBase<-1, true, 0, false> {
   cx<R>* W2; const R* U0; Cst<R> c; R n0, n1, n2, invM; int XS;
   __device__ bool valid(int, int x) const { return x <= c.Nx; }
   __device__ cx<R> load(int o, int x, int pos) const {
-    return pos < c.Nz ? W2[((size_t)pos * c.My + o) * XS + x] : czero<R>();
+    return pos < c.Nz ? *step(W2 + (size_t)o * XS + x, pos, c.My * XS * (int)sizeof(cx<R>)) : czero<R>();
   }
   __device__ void spectral(int o, int x, int k, cx<R>& v, R*) const {
     const int ky = kfreq(o, c.My), kz = kfreq(k, c.Mz);
@@ -600,11 +612,11 @@ template <typename R> struct OpAtkmZ : OpBase<-1, true, 0, false> {
     if (x == c.Nx) B += tx; else A += tx;
     if (o == c.Ny) B += ty; else A += ty;
     if (k == c.Nz) B += tz; else A += tz;
-    const R u = U0[((size_t)iabs(kz) * (c.Ny + 1) + iabs(ky)) * (c.Nx + 1) + x];
+    const R u = *step(U0 + (size_t)iabs(ky) * (c.Nx + 1) + x, iabs(kz), (c.Ny + 1) * (c.Nx + 1) * (int)sizeof(R));
     v = scl<R>(v, ((R)3 * u * (A * A + B * B) - (R)1) * invM);
   }
   __device__ void store(int o, int x, int pos, cx<R> v, R*) const {
-    if (pos < c.Nz) W2[((size_t)pos * c.My + o) * XS + x] = v;
+    if (pos < c.Nz) *step(W2 + (size_t)o * XS + x, pos, c.My * XS * (int)sizeof(cx<R>)) = v;
   }
 };
 
@@ -614,10 +626,10 @@ template <typename R> struct OpAtkmYI : OpBase<1, false, 0, false> {
   static constexpr bool kNyqTail = true;
   const cx<R>* W2; cx<R>* W1; Cst<R> c; int XS;
   __device__ bool valid(int, int x) const { return x <= c.Nx; }
-  __device__ cx<R> load(int o, int x, int pos) const { return W2[((size_t)o * c.My + pos) * XS + x]; }
+  __device__ cx<R> load(int o, int x, int pos) const { return *step(W2 + (size_t)o * c.My * XS + x, pos, XS * (int)sizeof(cx<R>)); }
   __device__ void spectral(int, int, int, cx<R>&, R*) const {}
   __device__ void store(int o, int x, int pos, cx<R> v, R*) const {
-    if (pos < c.Ny) W1[((size_t)o * c.Ny + pos) * XS + x] = v;
+    if (pos < c.Ny) *step(W1 + (size_t)o * c.Ny * XS + x, pos, XS * (int)sizeof(cx<R>)) = v;
   }
 };
 
@@ -671,7 +683,7 @@ template <typename R, bool RED> struct OpHX : OpBase<-1, true, RED ? 2 : 0, true
 template <typename R, bool RED> struct OpHY : OpBase<-1, true, RED ? 2 : 0, false> {
   const double2* f; cx<R>* acc; Cst<R> c; R Omega;
   __device__ bool valid(int, int x) const { return x < c.Nx; }
-  __device__ cx<R> load(int o, int x, int pos) const { return from64<R, kCvtHw>(f[((size_t)o * c.Ny + pos) * c.Nx + x]); }
+  __device__ cx<R> load(int o, int x, int pos) const { return from64<R, kCvtHw>(*step(f + (size_t)o * c.Ny * c.Nx + x, pos, c.Nx * 16)); }
   __device__ void spectral(int, int x, int k, cx<R>& v, R* a) const {
     const R invL = (R)1 / (R)c.Ny;
     const R nu = (R)kfreq(k, c.Ny) * c.ky;
@@ -691,10 +703,10 @@ template <typename R, bool RED> struct OpHY : OpBase<-1, true, RED ? 2 : 0, fals
   // FP32: the accumulator (8 B a point) is prefetched into shared memory
   static constexpr int kPre = 8;
   __device__ void prefetch(int o, int x, int pos, unsigned char* dst) const {
-    cp_async8(dst, acc + ((size_t)o * c.Ny + pos) * c.Nx + x);
+    cp_async8(dst, step(acc + (size_t)o * c.Ny * c.Nx + x, pos, c.Nx * 8));
   }
   __device__ void store_pre(int o, int x, int pos, cx<R> v, R*, const unsigned char* src) const {
-    acc[((size_t)o * c.Ny + pos) * c.Nx + x] = add<R>(*reinterpret_cast<const cx<R>*>(src), v);
+    *step(acc + (size_t)o * c.Ny * c.Nx + x, pos, c.Nx * 8) = add<R>(*reinterpret_cast<const cx<R>*>(src), v);
   }
 };
 
@@ -705,7 +717,7 @@ template <typename R, bool RED> struct OpHZ : OpBase<-1, true, RED ? 6 : 0, fals
   const double2* f; const double2* phi; const double* Phi; const cx<R>* acc; double2* Hf; Cst<R> c; PhysR<R> ph;
   bool same = false;  // f == phi (H phi): phi is not read a second time
   __device__ bool valid(int, int x) const { return x < c.Nx; }
-  __device__ cx<R> load(int o, int x, int pos) const { return from64<R, kCvtMixed>(f[((size_t)pos * c.Ny + o) * c.Nx + x]); }
+  __device__ cx<R> load(int o, int x, int pos) const { return from64<R, kCvtMixed>(*step(f + (size_t)o * c.Nx + x, pos, c.Ny * c.Nx * 16)); }
   __device__ void spectral(int, int, int k, cx<R>& v, R* a) const {
     const R invL = (R)1 / (R)c.Nz;
     const R nu = (R)kfreq(k, c.Nz) * c.kz;
@@ -727,9 +739,9 @@ template <typename R, bool RED> struct OpHZ : OpBase<-1, true, RED ? 6 : 0, fals
   // FP32: Phi (8 B) and the accumulator (8 B) are prefetched into shared memory
   static constexpr int kPre = 16;
   __device__ void prefetch(int o, int x, int pos, unsigned char* dst) const {
-    const size_t idx = ((size_t)pos * c.Ny + o) * c.Nx + x;
-    cp_async8(dst, Phi + idx);
-    cp_async8(dst + 8, acc + idx);
+    const size_t i0 = (size_t)o * c.Nx + x;
+    cp_async8(dst, step(Phi + i0, pos, c.Ny * c.Nx * 8));
+    cp_async8(dst + 8, step(acc + i0, pos, c.Ny * c.Nx * 8));
   }
   __device__ void store_pre(int o, int x, int pos, cx<R> v, R* a, const unsigned char* src) const {
     const size_t idx = ((size_t)pos * c.Ny + o) * c.Nx + x;
@@ -791,22 +803,26 @@ template <typename R> struct OpPXF : OpBase<-1, false, 0, true> {
 template <typename R, int S> struct OpPY : OpBase<S, false, 0, false> {
   cx<R>* Wk; Cst<R> c;
   __device__ bool valid(int, int x) const { return x < c.Nx; }
-  __device__ cx<R> load(int o, int x, int pos) const { return Wk[((size_t)o * c.Ny + pos) * c.Nx + x]; }
+  __device__ cx<R> load(int o, int x, int pos) const { return *step(Wk + (size_t)o * c.Ny * c.Nx + x, pos, c.Nx * (int)sizeof(cx<R>)); }
   __device__ void spectral(int, int, int, cx<R>&, R*) const {}
-  __device__ void store(int o, int x, int pos, cx<R> v, R*) const { Wk[((size_t)o * c.Ny + pos) * c.Nx + x] = v; }
+  __device__ void store(int o, int x, int pos, cx<R> v, R*) const {
+    *step(Wk + (size_t)o * c.Ny * c.Nx + x, pos, c.Nx * (int)sizeof(cx<R>)) = v;
+  }
 };
 
 // z forward * 1/((alpha + |nu|^2/2) N) * inverse on lines (o = y, x).
 template <typename R> struct OpPZ : OpBase<-1, true, 0, false> {
   cx<R>* Wk; Cst<R> c; const double* alpha;
   __device__ bool valid(int, int x) const { return x < c.Nx; }
-  __device__ cx<R> load(int o, int x, int pos) const { return Wk[((size_t)pos * c.Ny + o) * c.Nx + x]; }
+  __device__ cx<R> load(int o, int x, int pos) const { return *step(Wk + (size_t)o * c.Nx + x, pos, c.Ny * c.Nx * (int)sizeof(cx<R>)); }
   __device__ void spectral(int o, int x, int k, cx<R>& v, R*) const {
     const R invN = (R)1 / ((R)c.Nx * (R)c.Ny * (R)c.Nz);
     const R nux = (R)kfreq(x, c.Nx) * c.kx, nuy = (R)kfreq(o, c.Ny) * c.ky, nuz = (R)kfreq(k, c.Nz) * c.kz;
     v = scl<R>(v, invN / (tor<R>(*alpha) + (R)0.5 * (nux * nux + nuy * nuy + nuz * nuz)));
   }
-  __device__ void store(int o, int x, int pos, cx<R> v, R*) const { Wk[((size_t)pos * c.Ny + o) * c.Nx + x] = v; }
+  __device__ void store(int o, int x, int pos, cx<R> v, R*) const {
+    *step(Wk + (size_t)o * c.Nx + x, pos, c.Ny * c.Nx * (int)sizeof(cx<R>)) = v;
+  }
 };
 
 template <typename R> struct OpPXI : OpBase<1, false, 0, true> {
@@ -819,22 +835,6 @@ template <typename R> struct OpPXI : OpBase<1, false, 0, true> {
     const R w = pv_rsqrt<R>(c, ph, tor<R>(*alpha), pos, o % c.Ny, o / c.Ny, ldro(phi + idx), ldro(Phi + idx));
     Pr[idx] = to64<R, kCvtMixed>(w * v.x, w * v.y);
   }
-};
-
-// ---- in-place 3D complex FFT on a plan's (unpadded) grid, sign S.
-template <typename R, int S> struct OpCX : OpBase<S, false, 0, true> {
-  cx<R>* buf; Cst<R> c;
-  __device__ bool valid(int o, int) const { return o < c.Nz * c.Ny; }
-  __device__ cx<R> load(int o, int, int pos) const { return buf[(size_t)o * c.Nx + pos]; }
-  __device__ void spectral(int, int, int, cx<R>&, R*) const {}
-  __device__ void store(int o, int, int pos, cx<R> v, R*) const { buf[(size_t)o * c.Nx + pos] = v; }
-};
-template <typename R, int S> struct OpCZ : OpBase<S, false, 0, false> {
-  cx<R>* buf; Cst<R> c;
-  __device__ bool valid(int, int x) const { return x < c.Nx; }
-  __device__ cx<R> load(int o, int x, int pos) const { return buf[((size_t)pos * c.Ny + o) * c.Nx + x]; }
-  __device__ void spectral(int, int, int, cx<R>&, R*) const {}
-  __device__ void store(int o, int x, int pos, cx<R> v, R*) const { buf[((size_t)pos * c.Ny + o) * c.Nx + x] = v; }
 };
 
 }  // namespace atkm

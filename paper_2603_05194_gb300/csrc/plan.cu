@@ -166,6 +166,24 @@ __global__ void k_twiddles(float2* t32, int L) {
     t32[m] = make_float2((float)c, (float)-s);
   }
 }
+// The stage tables of the FP32 register engine, L a power of two: for each
+// stage after the first (radix R after Ns = 8 or 64, then the last radix 2 or
+// 4) the (R - 1) Ns values e^{-2 pi i k r / (Ns R)} at [(r - 1) Ns + k], from
+// the same expression as the table by index.
+__global__ void k_fast_twiddles(float2* w, int L) {
+  int Ns = 8, at = 0;
+  while (Ns < L) {
+    const int R = L / Ns >= 8 ? 8 : L / Ns;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (R - 1) * Ns; i += gridDim.x * blockDim.x) {
+      const int r = i / Ns + 1, k = i - (r - 1) * Ns;
+      double s, c;
+      sincospi(2.0 * (double)(k * r * (L / (Ns * R))) / (double)L, &s, &c);
+      w[at + i] = make_float2((float)c, (float)-s);
+    }
+    at += (R - 1) * Ns;
+    Ns *= R;
+  }
+}
 // The stage tables of an integer length (IntLen) at w.
 __global__ void k_int_twiddles(int4* w, IntLen f) {
   int Ns = f.rad[0];
@@ -599,7 +617,7 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   const int lens[6] = {g.Nx, g.Ny, g.Nz, g.Mx, g.My, g.Mz};
   size_t twtot = 0;
   for (int i = 0; i < 6; ++i) twtot += lens[i];
-  if ((e = dev_alloc(p, (void**)&p->tw32, twtot * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
+  if ((e = dev_alloc(p, (void**)&p->tw32, 2 * twtot * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
   // a length's stage tables take less than its length, for each order
   if ((e = dev_alloc(p, (void**)&p->twi, (3 * twtot + g.Nx) * sizeof(int4))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan twiddles"));
   size_t off = 0;
@@ -614,6 +632,11 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
     fi.wm = tw + lens[i];
     fi.wr = tw + 2 * lens[i];
     k_twiddles<<<(lens[i] + 127) / 128, 128, 0, st>>>(p->tw32 + off, lens[i]);
+    f.tws = p->tw32 + twtot + off;
+    if (lens[i] >= 16 && (lens[i] & (lens[i] - 1)) == 0) {
+      k_fast_twiddles<<<(lens[i] + 127) / 128, 128, 0, st>>>(p->tw32 + twtot + off, lens[i]);
+      count_launches(1);
+    }
     k_int_twiddles<<<(lens[i] + 63) / 64, 64, 0, st>>>(tw, fi);
     count_launches(2);
     if (const RadList rl = int_radices(lens[i]); rl.n > 0) {
