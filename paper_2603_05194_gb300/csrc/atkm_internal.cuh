@@ -535,7 +535,8 @@ struct atkm_plan {
   atkm::c64* W1;       // [Nz][Ny][XS] half spectrum in x
   atkm::c64* W2;       // [Nz][My][XS]
   atkm::c64* T1;       // [Nz][Ny][Nx]
-  int* ex[3];          // tile exponents of the integer arrays
+  atkm::c64* T2;       // [Nz][Ny][Nx], the y part of H
+  int* ex[5];          // tile exponents of the integer arrays (ATKM and P: 0..2, H: 3, 4)
   float2* W1f;
   float2* W2f;
   float2* T1f;

@@ -32,6 +32,7 @@ __device__ __forceinline__ int ikfreq(int m, int M) { return m < (M >> 1) ? m : 
 struct ExpTab {
   int* e;
   int rs, cs, nc;
+  __device__ __forceinline__ int at_ro(int row, int col) const { return __ldg(step(e + (col >> cs), row >> rs, nc * 4)); }
   __device__ __forceinline__ int at(int row, int col) const { return *step(e + (col >> cs), row >> rs, nc * 4); }
 };
 
@@ -51,6 +52,9 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   static constexpr bool kHalfOut = false;   // only positions < L/2 of the output are used
   static constexpr bool kNyqTail = false;   // column pass over columns 0..Nx (see ipass_place)
   static constexpr bool kMul = false;       // the spectral step is mul_tile
+  // launched by launch_pdl, inputs read by plain loads; an op whose loads should
+  // be moved ahead of its own stores reads by __ldg and is launched normally
+  static constexpr bool kPdl = true;
   static constexpr int kMinB = 3;           // CTAs per SM that the register engine is compiled for
   static constexpr bool kPre = false;       // the spectral step's 8-byte table entries are prefetched (op.table)
   double* part = nullptr;
@@ -463,7 +467,7 @@ __global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   }
-  pdl_wait();
+  if constexpr (Op::kPdl) pdl_wait();
   c64 v[8];
   Tile tl;
   if constexpr (Op::kTwin) {
@@ -599,7 +603,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
   Line l;
   pdl_trigger();
   if (ipass_line(op, T, P, &l)) return;  // the whole CTA
-  pdl_wait();
+  if constexpr (Op::kPdl) pdl_wait();
   c64 v[kGenE];
   Tile tl;
   if constexpr (Op::kTwin) {
@@ -801,7 +805,7 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   lb.ok = lb.ok && onb;
   if (!ona) la.t = 0, la.j = 1;
   if (!onb) lb.t = 0, lb.j = 1;
-  pdl_wait();
+  if constexpr (Op::kPdl) pdl_wait();
   c64 v[C::R0];
   Tile tl;
   if constexpr (Op::kTwin) {
@@ -963,7 +967,9 @@ inline cudaError_t launch_ifast(const Op& op, const IntLen& f, const IPassGrid& 
   constexpr size_t sm = IFast<L>::template bytes<Op::kLM>() + (Op::kPre ? (size_t)8 * 8 * kThreads : 0);
   cudaError_t e = iprepare(prepared, k_ifast<L, Op>, sm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_ifast<L, Op>, pg.grid, kThreads, sm, st, op, f.w);
+  if constexpr (Op::kPdl) return launch_pdl(k_ifast<L, Op>, pg.grid, kThreads, sm, st, op, f.w);
+  k_ifast<L, Op><<<pg.grid, kThreads, sm, st>>>(op, f.w);
+  return cudaGetLastError();
 }
 
 template <int L, class Op>
@@ -972,7 +978,9 @@ inline cudaError_t launch_imix(const Op& op, const IntLen& f, const IPassGrid& p
   constexpr size_t sm = IMix<L>::template bytes<Op>();
   cudaError_t e = iprepare(prepared, k_imix<L, Op>, sm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_imix<L, Op>, pg.grid, IMix<L>::NW * 32, sm, st, op, f.wm, f.wr);
+  if constexpr (Op::kPdl) return launch_pdl(k_imix<L, Op>, pg.grid, IMix<L>::NW * 32, sm, st, op, f.wm, f.wr);
+  k_imix<L, Op><<<pg.grid, IMix<L>::NW * 32, sm, st>>>(op, f.wm, f.wr);
+  return cudaGetLastError();
 }
 
 template <bool MIX, class Op> inline cudaError_t irun(const Op& op, const IntLen& f, const IPassGrid& pg, cudaStream_t st) {
@@ -1003,7 +1011,9 @@ template <bool MIX, class Op> inline cudaError_t irun(const Op& op, const IntLen
   cudaError_t e = iprepare(prepared, k_igen<Op>, most);
   if (e != cudaSuccess) return e;
   const size_t sm = std::max((size_t)2 * pg.T * (f.L + f.L / 8 + 1) * sizeof(c64), (size_t)Op::kRed * kThreads * sizeof(double));
-  return launch_pdl(k_igen<Op>, pg.grid, kThreads, sm, st, op, f, pg.T, pg.tsh);
+  if constexpr (Op::kPdl) return launch_pdl(k_igen<Op>, pg.grid, kThreads, sm, st, op, f, pg.T, pg.tsh);
+  k_igen<Op><<<pg.grid, kThreads, sm, st>>>(op, f, pg.T, pg.tsh);
+  return cudaGetLastError();
 }
 
 // ================================================================ ops
@@ -1014,6 +1024,10 @@ __device__ __forceinline__ void put_exp_at(const ExpTab& x, int row, int col, co
 
 __device__ __forceinline__ c64 ldc(const c64* p) {
   const longlong2 t = *reinterpret_cast<const longlong2*>(p);
+  return c64{t.x, t.y};
+}
+__device__ __forceinline__ c64 ldc_ro(const c64* p) {
+  const longlong2 t = __ldg(reinterpret_cast<const longlong2*>(p));
   return c64{t.x, t.y};
 }
 __device__ __forceinline__ void stc(c64* p, c64 v) { *reinterpret_cast<longlong2*>(p) = make_longlong2(v.x, v.y); }
@@ -1274,6 +1288,7 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   double gx2, gy2, gz2, beta, lambda, ck;
   bool same;  // f == phi: phi is not read a second time
   static constexpr bool kMul = true;
+  static constexpr bool kPdl = false;
   struct Acc : KinAcc {
     double s[5];
   };
@@ -1287,11 +1302,11 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc& a) const {
     const size_t i0 = (size_t)o * Nx + x;
     const int pl = Ny * Nx;
-    const double2 fv = *step(f + i0, pos, pl * 16);
-    const double Pd = *step(Phi + i0, pos, pl * 8);
-    const c64 u = ldc(step(AX + i0, pos, pl * 16)), w = ldc(step(AY + i0, pos, pl * 16));
+    const double2 fv = __ldg(step(f + i0, pos, pl * 16));
+    const double Pd = __ldg(step(Phi + i0, pos, pl * 8));
+    const c64 u = ldc_ro(step(AX + i0, pos, pl * 16)), w = ldc_ro(step(AY + i0, pos, pl * 16));
     const bool bad = t.bad || u.x == kBadElem || w.x == kBadElem;
-    const int eu = ix.at(pos * Ny + o, 0), ew = iy.at(pos, x);
+    const int eu = ix.at_ro(pos * Ny + o, 0), ew = iy.at_ro(pos, x);
     const int e = max(t.e, max(eu, ew)) + 2;  // room for the sum of three
     const int dv = min(e - t.e, 64), du = min(e - eu, 64), dw = min(e - ew, 64);
     const long long sx = shr_clamp(v.x, dv) + shr_clamp(u.x, du) + shr_clamp(w.x, dw);
@@ -1301,7 +1316,7 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
     else if (i2d_ok(e)) kin = make_double2(i2d(sx, e + 1085), i2d(sy, e + 1085));
     else kin = make_double2(i2d_any(sx, e), i2d_any(sy, e));
     const double V = gz2 * hz2[pos] + (gy2 * hy2[o] + gx2 * hx2[x]);
-    const double2 pv = same ? fv : *step(phi + i0, pos, pl * 16);
+    const double2 pv = same ? fv : __ldg(step(phi + i0, pos, pl * 16));
     const double wt = V + beta * (pv.x * pv.x + pv.y * pv.y) + lambda * Pd;
     const double ox = kin.x + wt * fv.x, oy = kin.y + wt * fv.y;
     *step(Hf + i0, pos, pl * 16) = make_double2(ox, oy);
@@ -1323,10 +1338,36 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   }
 };
 
+// 1 / sqrt(v) from the binary32 estimate y by one step of third order,
+// y + y e (1/2 + 3/8 e) with e = 1 - v y^2 (|e| < 2^-20, so 5/16 e^3 < 2^-61): 5
+// FP64 operations; 1 / v likewise by two Newton steps, 4.  Outside the range
+// of the estimate the library's functions.
+__device__ __forceinline__ bool f32_range(double v) {
+  return (unsigned)(__double2hiint(v) - 0x39000000) < 0x0e000000u;  // 2^-111 <= v < 2^113
+}
+__device__ __forceinline__ double rsqrt_fast(double v) {
+  if (!f32_range(v)) return rsqrt(v);
+  const double y = f2d_bits(rsqrtf(d2f_bits(v)));
+  const double e = fma(-(v * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double rcp_fast(double v) {
+  if (!f32_range(v)) return 1.0 / v;
+  double y = f2d_bits(__frcp_rn(d2f_bits(v)));
+  y = fma(y, fma(-v, y, 1.0), y);
+  return fma(y, fma(-v, y, 1.0), y);
+}
+// max(v, 0), 0 for a NaN, off the FP64 pipe
+__device__ __forceinline__ double pos_part(double v) {
+  const unsigned h = (unsigned)__double2hiint(v);
+  return h < 0x7ff00000u || (h == 0x7ff00000u && __double2loint(v) == 0) ? v : 0.0;
+}
+
 // ---- preconditioner (unpadded grid); Wk: [Nz][Ny][Nx] workspace.  The weight
 // P_V^{-1/2} of each point is stored in Pw for the x inverse pass, which then
 // reads it instead of forming it again.
 struct IPXF : IOpBase<-1, false, 0, true, kSrcF64> {
+  static constexpr bool kPdl = false;
   const double2* r;
   const double2* phi;
   const double* Phi;
@@ -1343,13 +1384,13 @@ struct IPXF : IOpBase<-1, false, 0, true, kSrcF64> {
   __device__ __forceinline__ double2 load(int o, int, int pos) const {
     const size_t i = (size_t)o * Nx + pos;
     const int y = o % Ny, z = o / Ny;
-    const double V = gx2 * hx2[pos] + (gy2 * hy2[y] + gz2 * hz2[z]);
-    const double2 pv = phi[i];
-    const double Pd = Phi[i];
-    const double den = *alpha + V + beta * (pv.x * pv.x + pv.y * pv.y) + alam * (Pd > 0.0 ? Pd : 0.0);
-    const double w = rsqrt(den);
+    const double2 pv = __ldg(phi + i);
+    // alpha and the terms of y and z are the line's
+    const double V = fma(gx2, hx2[pos], *alpha + (gy2 * hy2[y] + gz2 * hz2[z]));
+    const double den = fma(alam, pos_part(__ldg(Phi + i)), fma(beta, fma(pv.x, pv.x, pv.y * pv.y), V));
+    const double w = rsqrt_fast(den);
     Pw[i] = w;
-    const double2 rv = r[i];
+    const double2 rv = __ldg(r + i);
     return make_double2(rv.x * w, rv.y * w);
   }
   __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile&, Acc&) const {
@@ -1383,7 +1424,7 @@ struct IPZ : IOpBase<-1, true, 0, false, kSrcInt> {
   const double* nx2;  // nu^2 / 2 of each axis
   const double* ny2;
   const double* nz2;
-  double invN;
+  double Nt;  // grid points
   int Nx, Ny;
   static constexpr bool kMul = true;
   __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
@@ -1391,7 +1432,7 @@ struct IPZ : IOpBase<-1, true, 0, false, kSrcInt> {
   __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
   __device__ __forceinline__ void tally(int, int, int, Limbs, Limbs, Acc&) const {}
   __device__ __forceinline__ double mult(int o, int x, int k) const {
-    return invN / (*alpha + (nx2[x] + ny2[o]) + nz2[k]);
+    return rcp_fast(fma(Nt, nz2[k], Nt * (*alpha + (nx2[x] + ny2[o]))));
   }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
     stc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16), v);
@@ -1400,6 +1441,7 @@ struct IPZ : IOpBase<-1, true, 0, false, kSrcInt> {
 };
 
 struct IPXI : IOpBase<1, false, 0, true, kSrcInt> {
+  static constexpr bool kPdl = false;
   const c64* Wk;
   const double* Pw;
   double2* Pr;
@@ -1410,7 +1452,7 @@ struct IPXI : IOpBase<1, false, 0, true, kSrcInt> {
   __device__ __forceinline__ int lexp(int o, int, int pos) const { return in.at(o / Ny, pos); }
   __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile& t, Acc&) const {
     const size_t i = (size_t)o * Nx + pos;
-    const double w = Pw[i];
+    const double w = __ldg(Pw + i);
     double2 d;
     if (i2d_ok(t.e)) d = make_double2(i2d(v.x, t.e + 1085), i2d(v.y, t.e + 1085));
     else d = make_double2(i2d_any(v.x, t.e), i2d_any(v.y, t.e));

@@ -1,6 +1,6 @@
 // The binary64 H_phi f: three integer passes (iops.cuh).  The x and y passes
-// leave their parts in T1 and W2 (free outside the ATKM passes, and at least
-// as large as the grid), the z pass adds them up.
+// leave their parts in T1 and T2, the z pass adds them up.  Nothing here is
+// shared with the ATKM passes, so that the two may run side by side.
 #include "ipasses_impl.cuh"
 
 namespace atkm {

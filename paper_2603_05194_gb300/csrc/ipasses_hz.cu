@@ -14,8 +14,8 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   const double pi = 3.14159265358979323846264338327950288, kz = pi / g.Lz;
   const double2* fin = reinterpret_cast<const double2*>(h.f);
   IHZ<RED> op;
-  op.f = fin; op.phi = reinterpret_cast<const double2*>(h.phi); op.Phi = h.Phi; op.AX = p->T1; op.AY = p->W2;
-  op.ix = exp_lines(p->ex[0], gx); op.iy = exp_cols(p->ex[1], gy);
+  op.f = fin; op.phi = reinterpret_cast<const double2*>(h.phi); op.Phi = h.Phi; op.AX = p->T1; op.AY = p->T2;
+  op.ix = exp_lines(p->ex[3], gx); op.iy = exp_cols(p->ex[4], gy);
   op.Hf = reinterpret_cast<double2*>(h.Hf); op.kin = iaxt(p, 2).kinN; op.Nx = g.Nx; op.Ny = g.Ny; op.Nz = g.Nz;
   op.hx2 = iaxt(p, 0).hxc2; op.hy2 = iaxt(p, 1).hxc2; op.hz2 = iaxt(p, 2).hxc2;
   op.gx2 = ph.gx2; op.gy2 = ph.gy2; op.gz2 = ph.gz2; op.beta = ph.beta; op.lambda = ph.lambda;

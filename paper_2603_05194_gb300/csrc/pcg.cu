@@ -53,6 +53,7 @@ struct Ctl {
   // step
   double Hpp, S1, S2, S3, curv, t0, t, pn, Aphiphi, Aphip, App, tolE;
   double cr, sr, nrm2, inv, En, linf, bestE, best_t;
+  double nphi, fp, ca, cb;  // <phi, phi>, <phi, p>; cr inv and sr inv of the binary64 phase
   int accepted, nh, forced, pad1;
   double inv0;   // normalisation of psi_0
   double noise;  // FP32 noise of the residual at phi_0 (automatic hand-over)
@@ -127,8 +128,23 @@ template <typename T, int NS> struct Sums {
 #pragma unroll
       for (int s = 0; s < NS; ++s) v[s] = tor<float>(d[s]);
       block_reduce_store_f32<NS>(v, part, gridDim.x, blockIdx.x);
-    } else {
+    } else if constexpr (NS <= 2) {
       block_reduce_store<NS>(d, part, gridDim.x, blockIdx.x);
+    } else {
+      // one warp a sum: its lanes add 8 values each and shuffle once, 12
+      // binary64 additions a warp and sum (a shuffle tree in every warp: 40)
+      __shared__ double sh[NS][kRedThreads];
+#pragma unroll
+      for (int s = 0; s < NS; ++s) sh[s][threadIdx.x] = d[s];
+      __syncthreads();
+      const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      if (w < NS) {
+        double v = sh[w][lane];
+#pragma unroll
+        for (int q = 1; q < kRedThreads / 32; ++q) v += sh[w][q * 32 + lane];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) part[w * gridDim.x + blockIdx.x] = v;
+      }
     }
   }
 };
@@ -138,8 +154,12 @@ template <typename T, int NS> struct Sums {
 
 __global__ void k_set_scalar(double* dst, double v) { *dst = v; }
 
-int red_grid(size_t N) {
-  size_t b = (N + kRedThreads * 4 - 1) / (kRedThreads * 4);
+// per: elements a thread has at least.  The FP32-phase kernels take 4; the
+// binary64 ones, bound by their SM's FP64 pipe, 1, so that a small grid's work
+// reaches every SM (65536 points: 64 CTAs of 152 SMs before); those that both
+// phases run take 4 in both.
+int red_grid(size_t N, int per) {
+  size_t b = (N + kRedThreads * per - 1) / (kRedThreads * per);
   if (b < 1) b = 1;
   if (b > (size_t)kRedGrid) b = kRedGrid;
   return (int)b;
@@ -147,8 +167,8 @@ int red_grid(size_t N) {
 
 // Grid of a grid-stride vector kernel: whole waves (SMs x resident blocks of
 // that kernel, from the occupancy calculator, cached per kernel), at most
-// red_grid(N) -- a partial last wave would leave SMs idle at the end.
-int wave_grid(const void* kernel, size_t N) {
+// red_grid(N, per) -- a partial last wave would leave SMs idle at the end.
+int wave_grid(const void* kernel, size_t N, int per) {
   static std::mutex mu;
   static std::vector<std::pair<const void*, int>> cache;
   const int nsm = device_sm_count();
@@ -166,7 +186,7 @@ int wave_grid(const void* kernel, size_t N) {
       cache.emplace_back(kernel, per_sm);
     }
   }
-  const size_t cap = (size_t)red_grid(N);
+  const size_t cap = (size_t)red_grid(N, per);
   if (nsm <= 0) return (int)cap;  // SM count unknown: the size-based grid
   const size_t full = (size_t)nsm * per_sm;
   if (cap < full) return (int)cap;
@@ -242,6 +262,8 @@ __device__ __forceinline__ void c_dir(Ctl* c, const double* s) {
     c->beta_cg = 0.0;
     c->cp0 = -1.0; c->cp1 = 0.0; c->cp2 = b;
   }
+  c->nphi = nphi;
+  c->fp = c->cp0 * b + c->cp1 * cc + c->cp2 * nphi;
 }
 
 // Step 4 (i): keep p if <H phi, p> < 0, otherwise re-form it as J(-P r)
@@ -254,6 +276,7 @@ __device__ __forceinline__ void c_reset(Ctl* c, const double* s) {
     c->beta_cg = 0.0;
     if (c->use_cg) {
       c->cp0 = -1.0; c->cp1 = 0.0; c->cp2 = c->b;
+      c->fp = -c->b + c->b * c->nphi;
       c->redo = 1;
     }
   }
@@ -263,6 +286,20 @@ __device__ __forceinline__ void c_reset2(Ctl* c, const double* s) {
   if (!c->redo) return;
   c->pn2 = c->hv * s[S_P];
   c->d1 = c->hv * s[S_P + 1];
+}
+
+// Retraction coefficients of the step t.  The norm of phi+ = cr phi + sr p
+// follows from <phi, phi>, <phi, p> and <p, p>; the binary64 phase scales by it
+// while it forms phi+ (ca, cb).  The FP32 phase measures it afterwards (c_norm).
+__device__ __forceinline__ void retract(Ctl* c) {
+  double sn, cs;
+  sincos(c->t * c->pn, &sn, &cs);
+  c->cr = cs;
+  c->sr = sn / c->pn;
+  c->nrm2 = c->cr * c->cr * c->nphi + 2.0 * c->cr * c->sr * c->fp + c->sr * c->sr * c->pn2;
+  c->inv = 1.0 / sqrt(c->nrm2);
+  c->ca = c->cr * c->inv;
+  c->cb = c->sr * c->inv;
 }
 
 // Step 4 (ii): quadratic model, initial t, first retraction coefficients
@@ -281,8 +318,7 @@ __device__ __forceinline__ void c_step(Ctl* c, const double* s) {
   c->forced = 0;
   c->bestE = INFINITY;
   c->best_t = c->t;
-  c->cr = cos(c->t * c->pn);
-  c->sr = sin(c->t * c->pn) / c->pn;
+  retract(c);
 }
 
 __device__ __forceinline__ void c_norm(Ctl* c, const double* s) {
@@ -311,8 +347,7 @@ __device__ __forceinline__ void halve_body(Ctl* c, int mode) {
     c->t = c->best_t;
     c->forced = 1;
   }
-  c->cr = cos(c->t * c->pn);
-  c->sr = sin(c->t * c->pn) / c->pn;
+  retract(c);
 }
 __global__ void k_c_halve(Ctl* c, int mode) {
   pdl_trigger();
@@ -592,7 +627,7 @@ __device__ __forceinline__ void run_then(const Fin& f) {
   }
 }
 template <int NS> __device__ __forceinline__ void finish(const Fin& f) {
-  if (!last_block(f.cnt, threadIdx.x == 0)) return;
+  if (!last_block(f.cnt, (threadIdx.x & 31) == 0)) return;
   finalize_sums<NS>(f.part, gridDim.x, f.out);
   __syncthreads();
   if (threadIdx.x == 0) run_then(f);
@@ -710,6 +745,36 @@ k_scale_linf(double2* __restrict__ phin, const double2* __restrict__ phi, const 
   finish_max(f);
 }
 
+// phi+ = *ca phi + *cb p (the retraction, normalised), and the block maximum of
+// |phi+ - phi|^2: 48 bytes and 8 FP64 operations a point in one kernel, in place
+// of the combination with its norm and a scaling pass (128 bytes, 141 -> 72 us
+// at 256x256x64).  The maximum is taken on the bit patterns, which order
+// nonnegative binary64 values like the values and stay off the FP64 pipe.
+__global__ void __launch_bounds__(kRedThreads)
+k_trial(double2* __restrict__ phin, const double2* __restrict__ phi, const double2* __restrict__ p,
+        const double* __restrict__ ca, const double* __restrict__ cb, size_t N, Fin f) {
+  __shared__ double sh[kRedThreads];
+  pdl_trigger();
+  const double a = *ca, b = *cb;
+  long long m = 0;
+  ATKM_GRID_LOOP(j, N) {
+    const double2 u = phi[j], v = p[j];
+    const double2 o = make_double2(a * u.x + b * v.x, a * u.y + b * v.y);
+    phin[j] = o;
+    const double dx = o.x - u.x, dy = o.y - u.y;
+    const long long q = __double_as_longlong(dx * dx + dy * dy);
+    m = q > m ? q : m;
+  }
+  sh[threadIdx.x] = __longlong_as_double(m);
+  __syncthreads();
+  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) f.part[blockIdx.x] = sh[0];
+  finish_max(f);
+}
+
 // Sums for the curvature of the quadratic model:
 //   [0] <Hp, p>
 //   [1] sum rho'(beta rho' + lambda Phi'),  rho' = Re(conj(phi) p)
@@ -769,6 +834,8 @@ struct PcgBuffers {
   Ctl* ctl_h = nullptr;      // pinned host mirror
   cudaStream_t st = nullptr; // plan-owned stream (capturable)
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  cudaStream_t side = nullptr;  // second branch of captured graphs
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // graphs: [f32][parity][kind: 0 iteration, 1 halve+trial, 2 best+trial]
   // captured graphs per [form: FP64, FP32, FP64 with FP32 auxiliaries][parity][kind]
   cudaGraphExec_t gx[4][2][3] = {};
@@ -831,6 +898,9 @@ void pcg_free(atkm_plan* p) {
   if (b->st) cudaStreamDestroy(b->st);
   if (b->ev_in) cudaEventDestroy(b->ev_in);
   if (b->ev_out) cudaEventDestroy(b->ev_out);
+  if (b->side) cudaStreamDestroy(b->side);
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+  if (b->ev_join) cudaEventDestroy(b->ev_join);
   delete b;
   p->pcg = nullptr;
 }
@@ -853,6 +923,9 @@ static cudaError_t pcg_alloc(atkm_plan* p) {
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->st, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming);
   // previous-iteration vectors are read (and ignored) before the first step
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
     e = cudaMemset(b->r[i], 0, N * sizeof(double2));
@@ -874,6 +947,9 @@ struct Seq {
   // FP64 phase of the split form: the operators that only shape the search
   // direction and the step-size model (P r, H p, the pair ATKM) run in FP32.
   bool aux32 = false;
+  // In a captured graph the operators of a step that do not depend on each
+  // other (H p and the ATKM of Re(conj(phi) p)) become parallel branches.
+  bool fork = false;
   // Double-word form of that phase: H phi and the trial-energy ATKM run in
   // double-FP32 arithmetic instead of binary64.
   bool dw = false;
@@ -887,7 +963,7 @@ struct Seq {
   }
   void dot(const double2* u, const double2* v, int dst, int then) {
     prof_begin(p, "vec_dots", 32.0 * B.N, 0.0, st());
-    const int g = wave_grid((const void*)k_dot, B.N);
+    const int g = wave_grid((const void*)k_dot, B.N, 4);
     k_dot<<<g, kRedThreads, 0, st()>>>(u, v, B.N, fin(dst, then));
     prof_end(p, st());
     count_launches(1);
@@ -899,7 +975,7 @@ struct Seq {
     const double nv = (v0 ? 1 : 0) + (v1 ? 1 : 0) + (v2 ? 1 : 0) + (w ? 1 : 0) + 1;
     prof_begin(p, "vec_lincomb", 16.0 * nv * B.N, 0.0, st());
     const bool fl = f32 && phase_type;
-    const int g = fl ? wave_grid((const void*)k_lincomb<float>, B.N) : wave_grid((const void*)k_lincomb<double>, B.N);
+    const int g = fl ? wave_grid((const void*)k_lincomb<float>, B.N, 4) : wave_grid((const void*)k_lincomb<double>, B.N, f32 ? 4 : 1);
     if (fl)
       k_lincomb<float><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
     else
@@ -908,10 +984,10 @@ struct Seq {
     count_launches(1);
     chk(cudaGetLastError());
   }
-  void atkm(int mode, const double* a, const double* b, double* o, bool aux = false) {
+  void atkm(int mode, const double* a, const double* b, double* o, bool aux = false, cudaStream_t on = nullptr) {
     const bool use32 = f32 || (aux && aux32);
-    chk(use32 ? launch_atkm<float>(p, mode, a, b, o, st())
-              : launch_atkm64(p, dw, mode, a, b, o, st()));
+    const cudaStream_t to = on ? on : st();
+    chk(use32 ? launch_atkm<float>(p, mode, a, b, o, to) : launch_atkm64(p, dw, mode, a, b, o, to));
   }
   void hop(const double2* f, double2* o, int red, bool aux = false) {
     const double* fp = reinterpret_cast<const double*>(f);
@@ -939,20 +1015,24 @@ struct Seq {
   // One trial of Step 4 (iii) with the current retraction coefficients.
   template <class F> void trial(bool loop, cudaGraphConditionalHandle h, F sofar) {
     double2* phin = B.phi[q ^ 1];
-    lincomb(phin, B.phi[q], Coef{&c()->cr, 1.0}, B.p[q], Coef{&c()->sr, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr,
-            fin(S_T, kThenNorm), nullptr, false);  // the retraction stays FP64
-    prof_begin(p, "vec_scale_linf", 48.0 * B.N, 0.0, st());
-    const int gs = f32 ? wave_grid((const void*)k_scale_linf<float>, B.N)
-                       : wave_grid((const void*)k_scale_linf<double>, B.N);
-    if (f32) k_scale_linf<float><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L, kThenNone));
-    else k_scale_linf<double><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L, kThenNone));
+    if (f32) {
+      lincomb(phin, B.phi[q], Coef{&c()->cr, 1.0}, B.p[q], Coef{&c()->sr, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr,
+              fin(S_T, kThenNorm), nullptr, false);  // the retraction stays FP64
+      prof_begin(p, "vec_scale_linf", 48.0 * B.N, 0.0, st());
+      const int gs = wave_grid((const void*)k_scale_linf<float>, B.N, 4);
+      k_scale_linf<float><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L, kThenNone));
+    } else {
+      prof_begin(p, "vec_trial", 48.0 * B.N, 0.0, st());
+      const int gs = wave_grid((const void*)k_trial, B.N, 1);
+      k_trial<<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], B.p[q], &c()->ca, &c()->cb, B.N, fin(S_L, kThenNone));
+    }
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
     atkm(SRC_PSI, reinterpret_cast<const double*>(phin), nullptr, B.Phi[q ^ 1]);
     prof_begin(p, "vec_quartic", 24.0 * B.N, 0.0, st());
-    const int gq = f32 ? wave_grid((const void*)k_quartic_sums<float>, B.N)
-                       : wave_grid((const void*)k_quartic_sums<double>, B.N);
+    const int gq = f32 ? wave_grid((const void*)k_quartic_sums<float>, B.N, 4)
+                       : wave_grid((const void*)k_quartic_sums<double>, B.N, 1);
     const Fin f = fin(S_Q, loop ? kThenAcceptLoop : kThenAccept, loop ? sofar() + 1 : 0, h);
     if (f32) k_quartic_sums<float><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
     else k_quartic_sums<double><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
@@ -977,8 +1057,8 @@ struct Seq {
   template <class F> void rest(bool loop, cudaGraphConditionalHandle h, F sofar) {
     chk(precond());
     prof_begin(p, "vec_dir_dots", 80.0 * B.N, 0.0, st());
-    const int gd = f32 ? wave_grid((const void*)k_dir_dots<float>, B.N)
-                       : wave_grid((const void*)k_dir_dots<double>, B.N);
+    const int gd = f32 ? wave_grid((const void*)k_dir_dots<float>, B.N, 4)
+                       : wave_grid((const void*)k_dir_dots<double>, B.N, 1);
     const Fin fd = fin(S_D, kThenDir);
     if (f32)
       k_dir_dots<float><<<gd, kRedThreads, 0, st()>>>(B.Pr, B.phi[q], B.r[q], B.r[q ^ 1], B.p[q ^ 1], B.N, fd);
@@ -991,11 +1071,22 @@ struct Seq {
             B.Hphi, fin(S_P, kThenReset));
     lincomb(B.p[q], B.Pr, Coef{nullptr, -1.0}, B.phi[q], Coef{&c()->b, 1.0}, nullptr, Coef{nullptr, 0.0}, B.Hphi,
             fin(S_P, kThenReset2), &c()->redo);
+    // H p and Phi' write different buffers and share no workspace (H: T1, T2,
+    // ex[3], ex[4]; ATKM: W1, W2, ex[0..2])
+    if (fork) {
+      chk(cudaEventRecord(B.ev_fork, st()));
+      chk(cudaStreamWaitEvent(B.side, B.ev_fork, 0));
+    }
+    atkm(SRC_PAIR, reinterpret_cast<const double*>(B.phi[q]), reinterpret_cast<const double*>(B.p[q]), B.Phi1, true,
+         fork ? B.side : nullptr);
     hop(B.p[q], B.Hp, -1, true);
-    atkm(SRC_PAIR, reinterpret_cast<const double*>(B.phi[q]), reinterpret_cast<const double*>(B.p[q]), B.Phi1, true);
+    if (fork) {
+      chk(cudaEventRecord(B.ev_join, B.side));
+      chk(cudaStreamWaitEvent(st(), B.ev_join, 0));
+    }
     prof_begin(p, "vec_curv_sums", 64.0 * B.N, 0.0, st());
-    const int gc = f32 ? wave_grid((const void*)k_curv_sums<float>, B.N)
-                       : wave_grid((const void*)k_curv_sums<double>, B.N);
+    const int gc = f32 ? wave_grid((const void*)k_curv_sums<float>, B.N, 4)
+                       : wave_grid((const void*)k_curv_sums<double>, B.N, 1);
     const Fin fc = fin(S_C, kThenStep);
     if (f32)
       k_curv_sums<float><<<gc, kRedThreads, 0, st()>>>(B.Hp, B.phi[q], B.p[q], B.Phi[q], B.Phi1, ph.beta, ph.lambda,
@@ -1263,6 +1354,7 @@ struct Solver {
     Seq S{plan, *B, ph, is32, qq};
     S.aux32 = (split || dwm) && !is32;
     S.dw = dwm && !is32;
+    S.fork = true;  // seq_q's kernels are captured into the solve graph
     return S;
   }
   int log_room() const { return (logbuf && opts->log_capacity > logc) ? opts->log_capacity - logc : 0; }

@@ -433,8 +433,8 @@ bool make_int_len(int L, IntLen& f) {
 }
 
 void free_plan_memory(atkm_plan* p) {
-  void* ptrs[] = {p->tw32, p->twi, p->axtab, p->Pw, p->U0, p->U0f, p->Kz, p->W1, p->W2, p->T1,
-                  p->W1f, p->W2f, p->T1f, p->ex[0], p->ex[1], p->ex[2], p->partials, p->scal, p->cnt};
+  void* ptrs[] = {p->tw32, p->twi, p->axtab, p->Pw, p->U0, p->U0f, p->Kz, p->W1, p->W2, p->T1, p->T2,
+                  p->W1f, p->W2f, p->T1f, p->ex[0], p->ex[1], p->ex[2], p->ex[3], p->ex[4], p->partials, p->scal, p->cnt};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->scal_host) cudaFreeHost(p->scal_host);
@@ -592,8 +592,8 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   p->tw32 = nullptr; p->twi = nullptr; p->tw_x = nullptr; p->U0 = nullptr;
   p->axtab = nullptr; p->Pw = nullptr;
   p->U0f = nullptr; p->Kz = nullptr;
-  p->W1 = p->W2 = p->T1 = nullptr;
-  p->ex[0] = p->ex[1] = p->ex[2] = nullptr;
+  p->W1 = p->W2 = p->T1 = p->T2 = nullptr;
+  for (int*& q : p->ex) q = nullptr;
   p->W1f = p->W2f = p->T1f = nullptr; p->partials = nullptr; p->scal = nullptr; p->cnt = nullptr; p->scal_host = nullptr;
   p->pcg = nullptr; p->prof = nullptr; p->prof_stopped_ = nullptr; p->bytes = 0; p->flags = flags;
   p->n_tune = 0;
@@ -771,10 +771,11 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   if ((e = dev_alloc(p, (void**)&p->W1, n_w1 * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = dev_alloc(p, (void**)&p->W2, n_w2 * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = dev_alloc(p, (void**)&p->T1, Nt * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
+  if ((e = dev_alloc(p, (void**)&p->T2, Nt * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   // tile exponents: at most one per x line, or one per outer index and column
   const size_t n_ex = std::max((size_t)g.Nz * g.Ny, (size_t)std::max(g.My, std::max(g.Nz, g.Ny)) * g.Xh);
-  for (int** q : {&p->ex[0], &p->ex[1], &p->ex[2]})
-    if ((e = dev_alloc(p, (void**)q, n_ex * sizeof(int))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
+  for (int*& q : p->ex)
+    if ((e = dev_alloc(p, (void**)&q, n_ex * sizeof(int))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = dev_alloc(p, (void**)&p->Pw, Nt * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if (flags & ATKM_PLAN_F32) {
     if ((e = dev_alloc(p, (void**)&p->W1f, n_w1 * sizeof(float2))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
