@@ -38,6 +38,18 @@ struct ExpTab {
 
 constexpr int kInBits = 59;  // components of a transform's input stay below 2^59
 
+// A real multiplier m 2^(ex - 1084): |m| in [2^61, 2^62), to within 2^-22 of it
+// at either end; ex = 0 stands for 0, ex >= 2040 for infinity and NaN.
+struct Mult {
+  long long m;
+  int ex;
+};
+__device__ __forceinline__ Mult mult_of(double d) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  const long long m = (long long)(((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | l) << 9);
+  return Mult{(int)h < 0 ? -m : m, (int)((h >> 20) & 0x7ffu)};
+}
+
 enum ISrc { kSrcF64 = 0, kSrcInt = 1 };
 
 template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
@@ -55,7 +67,6 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   // launched by launch_pdl, inputs read by plain loads; an op whose loads should
   // be moved ahead of its own stores reads by __ldg and is launched normally
   static constexpr bool kPdl = true;
-  static constexpr int kMinB = 3;           // CTAs per SM that the register engine is compiled for
   static constexpr bool kPre = false;       // the spectral step's 8-byte table entries are prefetched (op.table)
   double* part = nullptr;
   int pstride = 0;
@@ -67,7 +78,7 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   __device__ __forceinline__ int midshift() const { return 0; }
   struct Acc { int e; };
   __device__ __forceinline__ c64 spectral(int, int, int, c64 v, Acc&, const long long*) const { return v; }
-  __device__ __forceinline__ double mult(int, int, int) const { return 1.0; }
+  __device__ __forceinline__ Mult mult(int, int, int) const { return Mult{1ll << 61, 1023}; }
 };
 
 // ------------------------------------------------------------ geometry
@@ -294,9 +305,8 @@ __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int
   *e += op.midshift();
 }
 
-// The same for an op with real binary64 multipliers of any size
-// (op.mult(o, x, k), kMul): an element times the 53-bit mantissa of its
-// multiplier keeps the element's bits, and the products are then aligned to
+// The same for an op with real multipliers of any size (op.mult(o, x, k),
+// kMul): an element times the mantissa of its multiplier keeps the element's bits, and the products are then aligned to
 // the tile's largest one.  (With the multiplier in fixed point, nu^2 / 2 of
 // the low frequencies, 2^-18 of the largest at length 1024, would leave the
 // product 2^18 fewer units.)
@@ -318,11 +328,9 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
       const c64 u = cshift(v[r], sh);
       const Limbs x = limbs(u.x), y = limbs(u.y);
       op.tally(l.o, l.x, pos, x, y, acc);
-      const double d = op.mult(l.o, l.x, pos);
-      const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
-      ex[r] = (int)((dh >> 20) & 0x7ffu);
-      const long long mt = (long long)(((unsigned long long)((dh & 0xfffffu) | 0x100000u) << 32 | dl) << 9);  // [2^61, 2^62)
-      const Limbs w = limbs((int)dh < 0 ? -mt : mt);
+      const Mult d = op.mult(l.o, l.x, pos);
+      ex[r] = d.ex;
+      const Limbs w = limbs(d.m);
       v[r] = c64{mul64(x, w), mul64(y, w)};
       eb = max(eb, 32 - __clz((int)mag(v[r])) + ex[r]);  // bits of the aligned product, less 32
     }
@@ -450,7 +458,7 @@ __device__ __forceinline__ void icp_async8(void* smem_dst, const void* gsrc) {
 }
 
 template <int L, class Op>
-__global__ void __launch_bounds__(kThreads, Op::kMinB) k_ifast(Op op, const int4* __restrict__ w) {
+__global__ void __launch_bounds__(kThreads, 3) k_ifast(Op op, const int4* __restrict__ w) {
   using C = IFast<L>;
   extern __shared__ __align__(16) unsigned char ism[];
   __shared__ __align__(16) TileRedT<Op::kTwin> tr;
@@ -713,8 +721,8 @@ template <int L> struct IMix {
     const size_t tile = (size_t)T * (Op::kLM ? LP : L) * sizeof(c64), red = (size_t)Op::kRed * NW * 32 * sizeof(double);
     return tile > red ? tile : red;
   }
-  // CTAs per SM: 768 threads at up to 85 registers, 512 at up to 128
-  template <class Op> static constexpr int minb() { return (Op::kMinB == 3 ? 768 : 512) / (NW * 32) > 0 ? (Op::kMinB == 3 ? 768 : 512) / (NW * 32) : 1; }
+  // CTAs per SM: 768 threads at up to 85 registers
+  static constexpr int kMinB = 768 / (NW * 32) > 0 ? 768 / (NW * 32) : 1;
 };
 
 // The (t, j) of a thread in a stage with nb butterflies a line; false: none.
@@ -788,7 +796,7 @@ template <int L, int S, bool LM, bool REV, int I> __device__ __forceinline__ voi
 }
 
 template <int L, class Op>
-__global__ void __launch_bounds__(IMix<L>::NW * 32, IMix<L>::template minb<Op>())
+__global__ void __launch_bounds__(IMix<L>::NW * 32, IMix<L>::kMinB)
 k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   using C = IMix<L>;
   constexpr bool LM = Op::kLM;
@@ -1212,15 +1220,14 @@ template <bool RED> struct IHX : IOpBase<-1, true, RED ? 2 : 0, true, kSrcF64> {
   double ck, cr;       // nu^2 / (2 N) = ck k'^2, Omega nu / N = cr k', k' the signed index
   static constexpr bool kMul = true;
   struct Acc : KinAcc {};
-  static constexpr int kMinB = 2;
   __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
   __device__ __forceinline__ double yc(int o) const { return -Ly + (double)(o % Ny) * hy; }
   __device__ __forceinline__ double2 load(int o, int, int pos) const { return f[(size_t)o * Nx + pos]; }
   __device__ __forceinline__ void tally(int, int, int k, Limbs x, Limbs y, Acc& a) const {
     if (RED) a.add(ikfreq(k, Nx), x, y);
   }
-  __device__ __forceinline__ double mult(int o, int, int k) const {
-    return fma(Om * yc(o), __ldg(nu + k), __ldg(kin + k));
+  __device__ __forceinline__ Mult mult(int o, int, int k) const {
+    return mult_of(fma(Om * yc(o), __ldg(nu + k), __ldg(kin + k)));
   }
   __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile& t, Acc&) const {
     if (t.bad) v.x = kBadElem;
@@ -1246,15 +1253,14 @@ template <bool RED> struct IHY : IOpBase<-1, true, RED ? 2 : 0, false, kSrcF64> 
   double ck, cr;
   static constexpr bool kMul = true;
   struct Acc : KinAcc {};
-  static constexpr int kMinB = 2;
   __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
   __device__ __forceinline__ double xc(int x) const { return -Lx + (double)x * hx; }
   __device__ __forceinline__ double2 load(int o, int x, int pos) const { return *step(f + (size_t)o * Ny * Nx + x, pos, Nx * 16); }
   __device__ __forceinline__ void tally(int, int, int k, Limbs p, Limbs q, Acc& a) const {
     if (RED) a.add(ikfreq(k, Ny), p, q);
   }
-  __device__ __forceinline__ double mult(int, int x, int k) const {
-    return fma(-Om * xc(x), __ldg(nu + k), __ldg(kin + k));
+  __device__ __forceinline__ Mult mult(int, int x, int k) const {
+    return mult_of(fma(-Om * xc(x), __ldg(nu + k), __ldg(kin + k)));
   }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc&) const {
     if (t.bad) v.x = kBadElem;
@@ -1271,7 +1277,10 @@ template <bool RED> struct IHY : IOpBase<-1, true, RED ? 2 : 0, false, kSrcF64> 
 
 // z: multiplier nu^2/2 on lines (o = y, x), then Hf = x part + y part + z part
 // + (V + beta |phi|^2 + lambda Phi) f, the last term in binary64.
-// Sums: kin_z, V|f|^2, |f|^4, Phi |f|^2, Re(Hf conj f), |f|^2.
+// RED (f = phi) sums: kin_z, V|f|^2, |f|^4, Phi |f|^2, Re(Hf conj f), |f|^2; the
+// fifth is the sum of all kinetic and rotation sums, the second, beta times the
+// third and lambda times the fourth, which spares two of the 13 binary64 operations
+// a point that bound this pass.
 template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> {
   const double2* f;
   const double2* phi;
@@ -1290,15 +1299,14 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   static constexpr bool kMul = true;
   static constexpr bool kPdl = false;
   struct Acc : KinAcc {
-    double s[5];
+    double s[4];
   };
-  static constexpr int kMinB = 2;
   __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
   __device__ __forceinline__ double2 load(int o, int x, int pos) const { return *step(f + (size_t)o * Nx + x, pos, Ny * Nx * 16); }
   __device__ __forceinline__ void tally(int, int, int k, Limbs p, Limbs q, Acc& a) const {
     if (RED) a.add(ikfreq(k, Nz), p, q);
   }
-  __device__ __forceinline__ double mult(int, int, int k) const { return __ldg(kin + k); }
+  __device__ __forceinline__ Mult mult(int, int, int k) const { return mult_of(__ldg(kin + k)); }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc& a) const {
     const size_t i0 = (size_t)o * Nx + x;
     const int pl = Ny * Nx;
@@ -1316,17 +1324,16 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
     else if (i2d_ok(e)) kin = make_double2(i2d(sx, e + 1085), i2d(sy, e + 1085));
     else kin = make_double2(i2d_any(sx, e), i2d_any(sy, e));
     const double V = gz2 * hz2[pos] + (gy2 * hy2[o] + gx2 * hx2[x]);
-    const double2 pv = same ? fv : __ldg(step(phi + i0, pos, pl * 16));
-    const double wt = V + beta * (pv.x * pv.x + pv.y * pv.y) + lambda * Pd;
+    const double2 pv = RED || same ? fv : __ldg(step(phi + i0, pos, pl * 16));
+    const double f2 = pv.x * pv.x + pv.y * pv.y;
+    const double wt = V + beta * f2 + lambda * Pd;
     const double ox = kin.x + wt * fv.x, oy = kin.y + wt * fv.y;
     *step(Hf + i0, pos, pl * 16) = make_double2(ox, oy);
     if (RED) {
-      const double f2 = fv.x * fv.x + fv.y * fv.y;
       a.s[0] += V * f2;
       a.s[1] += f2 * f2;
       a.s[2] += Pd * f2;
-      a.s[3] += ox * fv.x + oy * fv.y;
-      a.s[4] += f2;
+      a.s[3] += f2;
     }
   }
   __device__ __forceinline__ void put_exp(const Line&, const Tile&) const {}
@@ -1334,28 +1341,55 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
     s[0] = l.ok ? ck * a.get().x : 0.0;
     if (t.bad) s[0] = __longlong_as_double(0x7ff8000000000000ll);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) s[1 + i] = a.s[i];
+    for (int i = 0; i < 3; ++i) s[1 + i] = a.s[i];
+    s[4] = s[0] + fma(lambda, a.s[2], fma(beta, a.s[1], a.s[0]));
+    // the sums of the x and y passes lie before this pass's
+    if (blockIdx.x + blockIdx.y + threadIdx.x == 0)
+      s[4] += (this->sums_out[-4] + this->sums_out[-2]) + (this->sums_out[-3] + this->sums_out[-1]);
+    s[5] = a.s[3];
   }
 };
 
-// 1 / sqrt(v) from the binary32 estimate y by one step of third order,
-// y + y e (1/2 + 3/8 e) with e = 1 - v y^2 (|e| < 2^-20, so 5/16 e^3 < 2^-61): 5
-// FP64 operations; 1 / v likewise by two Newton steps, 4.  Outside the range
-// of the estimate the library's functions.
+// 1 / v and 1 / sqrt(v) as mantissa and exponent: the binary32 estimate y and one
+// correction step in integers, off the FP64 pipe (2 operations a clock and SM
+// against 64 integer products; the binary64 steps took 4 and 5 operations).  The
+// residual e = 1 - v y (|e| < 2^-22), 1 - v y^2 (|e| < 2^-20) is exact to 2^-62,
+// so the results are good to 2^-55.  Outside the estimate's range the library's.
 __device__ __forceinline__ bool f32_range(double v) {
   return (unsigned)(__double2hiint(v) - 0x39000000) < 0x0e000000u;  // 2^-111 <= v < 2^113
 }
+// y (1 + f 2^-56), y's mantissa my in [2^23, 2^24), its biased exponent ey
+__device__ __forceinline__ Mult mult_corr(unsigned my, int ey, long long f) {
+  return Mult{(long long)((unsigned long long)my << 38) + (((long long)my * f) >> 18), ey - 127 + 1023};
+}
+__device__ __forceinline__ unsigned long long mantissa53(double v) {  // of a normal v
+  return (unsigned long long)(((unsigned)__double2hiint(v) & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(v);
+}
+// To binary64, rounded.
+__device__ __forceinline__ double mult_double(Mult w) {
+  // the correction may have moved the mantissa a little out of [2^61, 2^62)
+  const int h = (int)(w.m >> 32), d = (h >= 0x40000000 ? 1 : 0) - (h < 0x20000000 ? 1 : 0);
+  return __longlong_as_double(((w.m + (128ll << (1 + d))) >> (9 + d)) + ((long long)(w.ex - 1 + d) << 52));
+}
+__device__ __forceinline__ Mult mult_rcp(double v) {
+  if (!f32_range(v)) return mult_of(1.0 / v);
+  const unsigned yb = __float_as_uint(__frcp_rn(d2f_bits(v))), my = (yb & 0x7fffffu) | 0x800000u;
+  const int ey = (int)(yb >> 23);
+  const int s = 1150 - ey - (__double2hiint(v) >> 20);  // 0 or 1
+  const long long E = (long long)(0ull - (mantissa53(v) << 9) * my) << (1 - s);  // e 2^85; 2^(84 + s) is 0 modulo 2^64
+  const int eh = (int)(E >> 32);                                                 // e 2^53
+  return mult_corr(my, ey, (E >> 29) + (mulw(eh, eh) >> 50));
+}
 __device__ __forceinline__ double rsqrt_fast(double v) {
   if (!f32_range(v)) return rsqrt(v);
-  const double y = f2d_bits(rsqrtf(d2f_bits(v)));
-  const double e = fma(-(v * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-__device__ __forceinline__ double rcp_fast(double v) {
-  if (!f32_range(v)) return 1.0 / v;
-  double y = f2d_bits(__frcp_rn(d2f_bits(v)));
-  y = fma(y, fma(-v, y, 1.0), y);
-  return fma(y, fma(-v, y, 1.0), y);
+  const unsigned yb = __float_as_uint(rsqrtf(d2f_bits(v))), my = (yb & 0x7fffffu) | 0x800000u;
+  const int ey = (int)(yb >> 23);
+  const int s = 1277 - 2 * ey - (__double2hiint(v) >> 20);  // 0 ... 3
+  // v y^2 is 2^(60 + s) here; E = e 2^63
+  const long long E = (long long)((1ull << (60 + s)) - __umul64hi(mantissa53(v) << 10, ((unsigned long long)my * my) << 16)) << (3 - s);
+  const int eh = (int)(E >> 12);  // e 2^51
+  // e / 2 + 3/8 e^2 in units 2^-56
+  return mult_double(mult_corr(my, ey, (E + 3 * (mulw(eh, eh) >> 41)) >> 8));
 }
 // max(v, 0), 0 for a NaN, off the FP64 pipe
 __device__ __forceinline__ double pos_part(double v) {
@@ -1431,8 +1465,8 @@ struct IPZ : IOpBase<-1, true, 0, false, kSrcInt> {
   __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16)); }
   __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
   __device__ __forceinline__ void tally(int, int, int, Limbs, Limbs, Acc&) const {}
-  __device__ __forceinline__ double mult(int o, int x, int k) const {
-    return rcp_fast(fma(Nt, nz2[k], Nt * (*alpha + (nx2[x] + ny2[o]))));
+  __device__ __forceinline__ Mult mult(int o, int x, int k) const {
+    return mult_rcp(fma(Nt, nz2[k], Nt * (*alpha + (nx2[x] + ny2[o]))));
   }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
     stc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16), v);
@@ -1477,7 +1511,6 @@ template <int S> struct ICX : IOpBase<S, false, 0, true, kSrcF64> {
   }
 };
 template <int S> struct ICZ : IOpBase<S, false, 0, false, kSrcInt> {
-  static constexpr int kMinB = 2;
   double2* buf;
   ExpTab in;
   int Nx, Ny;

@@ -8,6 +8,7 @@ namespace {
 template <bool RED>
 cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_t st) {
   const Geo& g = p->g;
+  if (RED && h.f != h.phi) return cudaErrorInvalidValue;  // the sums are those of phi
   const Phys& ph = *h.ph;
   const IPassGrid &gx = h.gx, &gy = h.gy, &gz = h.gz;
   const double N = (double)g.Nx * g.Ny * g.Nz;

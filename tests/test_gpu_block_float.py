@@ -4,6 +4,8 @@ whose scale lies far from one or varies over hundreds of orders of magnitude,
 zeros, and NaNs.  Bars: relative 2-norm 1e-13 against the oracle (its own
 rounding is below 1e-15 here; the integer passes carry 58 bits), bitwise where
 the arithmetic is exact under a power of two."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -54,6 +56,38 @@ def test_operators_on_edge_lengths(lib, N):
     assert rel2(host(plan.apply_H(prm, dev(f), dev(phi), dev(Phi))), O.apply_H(oplan, oprm, f, phi, Phi)) <= 1e-13
     got = host(plan.apply_preconditioner(prm, 7.0, dev(f), dev(phi), dev(Phi)))
     assert rel2(got, O.apply_precond(oplan, oprm, f, phi, Phi, 7.0)) <= 1e-13
+
+
+def precond_at_rest(N, L, gamma, alpha, f, fused):
+    """P f for phi = Phi = 0 by numpy's transforms.  The middle of the grid has
+    V = 0 up to the rounding of its coordinates -L + i h, which differs with a
+    fused multiply-add (the library's tables are formed on the host, which may
+    have one): both forms."""
+    def coord(a):
+        h = 2.0 * L[a] / N[a]
+        if fused:
+            return np.array([float(Fraction(i) * Fraction(h) - Fraction(L[a])) for i in range(N[a])])
+        return -L[a] + np.arange(N[a]) * h
+    view = [(None, None, slice(None)), (None, slice(None), None), (slice(None), None, None)]
+    den = alpha + sum(
+        (gamma[a] * gamma[a] * (0.5 * coord(a) * coord(a)))[view[a]] for a in (2, 1, 0))
+    k2 = sum((0.5 * (np.pi / L[a] * N[a] * np.fft.fftfreq(N[a])) ** 2)[view[a]] for a in range(3))
+    w = 1.0 / np.sqrt(den)
+    return w * np.fft.ifftn(np.fft.fftn(w * f) / (alpha + k2))
+
+
+@pytest.mark.parametrize("N", [(32, 64, 16), (36, 20, 18)])
+@pytest.mark.parametrize("alpha", [1e-40, 2.0 ** -20, 2.0 ** 40, 1e40])
+def test_preconditioner_weights_at_range_edges(lib, N, alpha):
+    """The integer square roots and reciprocals of the weights: arguments next
+    to powers of two, and beyond the binary32 range on either side (the bar of
+    this file; phi = Phi = 0, so that the weights range from 1 / sqrt(alpha))."""
+    L, n = (3.0, 2.5, 2.0), (0.6, 0.0, 0.8)
+    plan, prm = lib.Plan(N, L, n), lib.make_params(GAMMA, BETA, LAM, OM)
+    shape = (N[2], N[1], N[0])
+    f, z, zr = W.random_field(shape, 14), np.zeros(shape, complex), np.zeros(shape)
+    got = host(plan.apply_preconditioner(prm, alpha, dev(f), dev(z), dev(zr)))
+    assert min(rel2(got, precond_at_rest(N, L, GAMMA, alpha, f, fused)) for fused in (False, True)) <= 1e-13
 
 
 @pytest.mark.parametrize("N", [(32, 64, 16), (36, 20, 18)])
