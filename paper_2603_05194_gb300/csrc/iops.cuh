@@ -78,7 +78,8 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   __device__ __forceinline__ int midshift() const { return 0; }
   struct Acc { int e; };
   __device__ __forceinline__ c64 spectral(int, int, int, c64 v, Acc&, const long long*) const { return v; }
-  __device__ __forceinline__ Mult mult(int, int, int) const { return Mult{1ll << 61, 1023}; }
+  __device__ __forceinline__ double mline(int, int) const { return 0.0; }
+  __device__ __forceinline__ Mult mult(double, int) const { return Mult{1ll << 61, 1023}; }
 };
 
 // ------------------------------------------------------------ geometry
@@ -305,8 +306,10 @@ __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int
   *e += op.midshift();
 }
 
-// The same for an op with real multipliers of any size (op.mult(o, x, k),
-// kMul): an element times the mantissa of its multiplier keeps the element's bits, and the products are then aligned to
+// The same for an op with real multipliers of any size (kMul; op.mult(c, k), c =
+// op.mline(o, x) the line's part, formed once a thread: left to the compiler, H x
+// formed it at every element, 3 of its 4 binary64 operations, 86 against 77 us at
+// 256x256x64): an element times the mantissa of its multiplier keeps the element's bits, and the products are then aligned to
 // the tile's largest one.  (With the multiplier in fixed point, nu^2 / 2 of
 // the low frequencies, 2^-18 of the largest at length 1024, would leave the
 // product 2^18 fewer units.)
@@ -318,6 +321,7 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
   for (int r = 0; r < E; ++r) m |= mag(v[r]);
   const int sh = 62 - mag_bits(tile_or<NW>(m, tr.m[2]));
   acc.e = tl.e - sh;
+  const double c = op.mline(l.o, l.x);
   int ex[E];
   int eb = -0x40000000;
 #pragma unroll
@@ -328,7 +332,7 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
       const c64 u = cshift(v[r], sh);
       const Limbs x = limbs(u.x), y = limbs(u.y);
       op.tally(l.o, l.x, pos, x, y, acc);
-      const Mult d = op.mult(l.o, l.x, pos);
+      const Mult d = op.mult(c, pos);
       ex[r] = d.ex;
       const Limbs w = limbs(d.m);
       v[r] = c64{mul64(x, w), mul64(y, w)};
@@ -372,6 +376,13 @@ __device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* sh, doubl
 }
 
 // ------------------------------------------------------------ k_ifast
+// Bound by instruction issue (52-62% of the slots; ALU and integer multiplier
+// half busy each; DRAM a quarter or less).  Three CTAs an SM at 80 registers: two
+// cost 10-15% (H 318 against 276 us at 256x256x64), four, at 64, gained 2% in the
+// forward passes and lost 7% in the inverse ones.  At 256x256x64, against radix-8
+// transforms in FP64 instructions (FP64 pipe 88-93% busy): ATKM x, y, z, y, x 246,
+// 336, 1063, 357, 238 -> 51, 72, 231, 76, 59 us; H x, y, z 351, 369, 344 -> 77, 80,
+// 110; P x, y, z, y, x 298, 168, 336, 168, 183 -> 107, 43, 70, 43, 61.
 constexpr int kIElems = 2048;  // elements per CTA (256 threads x 8)
 
 template <int L> struct IFast {
@@ -694,7 +705,9 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
 // stage).  The inputs of the first stage and the outputs of the last one stay
 // in registers, and the inverse transform takes the radices in the opposite
 // order, so that its first stage finds its inputs in the registers where the
-// forward transform left them.
+// forward transform left them.  All passes of an ATKM, an H and a P against
+// k_igen: 550 -> 348 us at 144x144x36, 648 -> 475 at 160x160x40, 231 -> 152 at
+// 96x96x24.  Bound by instruction issue, as k_ifast.
 template <int L> struct IMix {
   static constexpr RadList R = int_radices(L);
   static constexpr int n = R.n, R0 = R.r[0], RL = R.r[R.n - 1];
@@ -924,7 +937,9 @@ inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long line
     if (p->tune[i].r == r && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0) && p->tune[i].shift > 0) pg.mix = false;
   // Power-of-two lengths up to 256 where the register engine's CTAs (2048
   // elements, 8 a thread) would not give every SM one: k_imix has half the
-  // elements a thread and a CTA, so twice the warps share the work.
+  // elements a thread and a CTA, so twice the warps share the work.  All passes
+  // of an ATKM, an H and a P: 148 -> 124 us at 64x64x16, 139 -> 119 at 32x32x16;
+  // at two CTAs per SM the line would cost 226 -> 243 us at 128x128x32.
   if (pg.fast && mix && int_radices(L).n > 0) {
     const int T = kIElems / L;
     const long ctas = LM ? (lines + T - 1) / T : (long)std::max(X / T, 1) * outer;
@@ -1226,9 +1241,8 @@ template <bool RED> struct IHX : IOpBase<-1, true, RED ? 2 : 0, true, kSrcF64> {
   __device__ __forceinline__ void tally(int, int, int k, Limbs x, Limbs y, Acc& a) const {
     if (RED) a.add(ikfreq(k, Nx), x, y);
   }
-  __device__ __forceinline__ Mult mult(int o, int, int k) const {
-    return mult_of(fma(Om * yc(o), __ldg(nu + k), __ldg(kin + k)));
-  }
+  __device__ __forceinline__ double mline(int o, int) const { return Om * yc(o); }
+  __device__ __forceinline__ Mult mult(double c, int k) const { return mult_of(fma(c, __ldg(nu + k), __ldg(kin + k))); }
   __device__ __forceinline__ void store(int o, int, int pos, c64 v, const Tile& t, Acc&) const {
     if (t.bad) v.x = kBadElem;
     stc(A + (size_t)o * Nx + pos, v);
@@ -1259,9 +1273,8 @@ template <bool RED> struct IHY : IOpBase<-1, true, RED ? 2 : 0, false, kSrcF64> 
   __device__ __forceinline__ void tally(int, int, int k, Limbs p, Limbs q, Acc& a) const {
     if (RED) a.add(ikfreq(k, Ny), p, q);
   }
-  __device__ __forceinline__ Mult mult(int, int x, int k) const {
-    return mult_of(fma(-Om * xc(x), __ldg(nu + k), __ldg(kin + k)));
-  }
+  __device__ __forceinline__ double mline(int, int x) const { return -Om * xc(x); }
+  __device__ __forceinline__ Mult mult(double c, int k) const { return mult_of(fma(c, __ldg(nu + k), __ldg(kin + k))); }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc&) const {
     if (t.bad) v.x = kBadElem;
     stc(step(A + (size_t)o * Ny * Nx + x, pos, Nx * 16), v);
@@ -1306,7 +1319,7 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   __device__ __forceinline__ void tally(int, int, int k, Limbs p, Limbs q, Acc& a) const {
     if (RED) a.add(ikfreq(k, Nz), p, q);
   }
-  __device__ __forceinline__ Mult mult(int, int, int k) const { return mult_of(__ldg(kin + k)); }
+  __device__ __forceinline__ Mult mult(double, int k) const { return mult_of(__ldg(kin + k)); }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile& t, Acc& a) const {
     const size_t i0 = (size_t)o * Nx + x;
     const int pl = Ny * Nx;
@@ -1465,9 +1478,9 @@ struct IPZ : IOpBase<-1, true, 0, false, kSrcInt> {
   __device__ __forceinline__ c64 load(int o, int x, int pos) const { return ldc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16)); }
   __device__ __forceinline__ int lexp(int, int x, int pos) const { return in.at(pos, x); }
   __device__ __forceinline__ void tally(int, int, int, Limbs, Limbs, Acc&) const {}
-  __device__ __forceinline__ Mult mult(int o, int x, int k) const {
-    return mult_rcp(fma(Nt, nz2[k], Nt * (*alpha + (nx2[x] + ny2[o]))));
-  }
+  // x may lie beyond the grid for the lines that a tile's last CTA leaves idle
+  __device__ __forceinline__ double mline(int o, int x) const { return valid(o, x) ? Nt * (*alpha + (nx2[x] + ny2[o])) : 1.0; }
+  __device__ __forceinline__ Mult mult(double c, int k) const { return mult_rcp(fma(Nt, nz2[k], c)); }
   __device__ __forceinline__ void store(int o, int x, int pos, c64 v, const Tile&, Acc&) const {
     stc(step(Wk + (size_t)o * Nx + x, pos, Ny * Nx * 16), v);
   }
