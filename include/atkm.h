@@ -51,7 +51,7 @@ typedef struct atkm_plan atkm_plan;
 /* Plan flags (bit set). */
 #define ATKM_PLAN_F64 0u   /* FP64 workspaces (always present)                  */
 #define ATKM_PLAN_F32 1u   /* also allocate complex64 workspaces for the _f32 calls */
-#define ATKM_PLAN_DF32 2u  /* also keep a double-word copy of U0 for the _df32 calls  */
+#define ATKM_PLAN_DF32 2u  /* allows the _df32 call and ATKM_PRECISION_DF32_SPLIT     */
 #define ATKM_PLAN_GENERIC_FFT 4u  /* lengths that are not powers of two run on the generic
                                      shared-memory FFT engine also where the mixed-radix
                                      register engine covers them (3 * 2^a and 5 * 2^a,
@@ -72,8 +72,8 @@ typedef struct atkm_plan atkm_plan;
  * the nonnegative frequency octant of the twofold-padded grid (Eq. (FUk)),
  * and from it the dipolar multiplier K = -1 + 3 (n.nu)^2 U0, symmetrised on the
  * padded Nyquist planes, on the half spectrum kept by the real-data transform
- * (FP64, and a double-word copy with ATKM_PLAN_DF32; FP32 passes form it from
- * an FP32 copy of U0).  Also holds the twiddle tables, per-axis frequency and
+ * (64-bit integers with one exponent; FP32 passes form it from an FP32 copy of
+ * U0).  Also holds the twiddle tables, per-axis frequency and
  * coordinate tables and the workspaces (atkm_plan_device_bytes gives the
  * total: about 0.5 GB for an FP64 plan at 256 x 256 x 64, more once a solve
  * has allocated its vectors).  Synchronises `stream` before
@@ -114,9 +114,9 @@ typedef struct atkm_kernel_stat {
 unsigned long long atkm_launch_count(void);
 
 /*
- * atkm_measure_fp64_fma -- peak binary64 FMA rate of the current device, the
- * denominator of the roofline of the binary64 FFT passes (bound by that
- * pipe on this GPU).  Launches blocks_per_sm x (SM count) CTAs of 256
+ * atkm_measure_fp64_fma -- peak binary64 FMA rate of the current device, which
+ * bounds the binary64 vector kernels and pointwise work (the FFT passes run in
+ * integer arithmetic).  Launches blocks_per_sm x (SM count) CTAs of 256
  * threads, each thread running 8 independent FMA chains of `iters` steps;
  * times `repeats` launches (after one warm-up) with CUDA events on `stream`
  * and writes the best rate in GFLOP/s (2 flops per FMA) to *gflops (host).
@@ -128,11 +128,11 @@ int atkm_measure_fp64_fma(int blocks_per_sm, int iters, int repeats, double* gfl
 /*
  * atkm_plan_autotune -- FFT-tile autotuner: for every line length of the
  * plan's passes that is not a power of two, per arithmetic the plan carries
- * (binary64; FP32 with ATKM_PLAN_F32; double-word with ATKM_PLAN_DF32) and per
- * layout (line-major x pass, strided y / z pass), times the candidates -- the
- * mixed-radix register engine (FP32: lengths 3 * 2^a and 5 * 2^a <= 384;
- * binary64: 3 * 2^a <= 384; not double-word; not with ATKM_PLAN_GENERIC_FFT)
- * and the generic shared-memory engine
+ * (binary64; FP32 with ATKM_PLAN_F32; the DF32 form with ATKM_PLAN_DF32) and
+ * per layout (line-major x pass, strided y / z pass), times the candidates --
+ * in FP32 the mixed-radix register engine (lengths 3 * 2^a and 5 * 2^a <= 384;
+ * not with ATKM_PLAN_GENERIC_FFT), in the others the engine that the fixed rule
+ * takes, and the generic shared-memory engine
  * at its default tile width, 1/2 and 1/4 of it -- on the plan's own ATKM of
  * |psi|^2, H psi and P r (CUDA events on `stream`, best of 3 after a warm-up)
  * and keeps the fastest; every later pass of that length and layout uses it.
@@ -145,7 +145,7 @@ int atkm_measure_fp64_fma(int blocks_per_sm, int iters, int repeats, double* gfl
 int atkm_plan_autotune(atkm_plan* plan, void* stream);
 
 typedef struct atkm_tune_info {
-  int precision;   /* 0 binary64, 1 FP32, 2 double-word                        */
+  int precision;   /* 0 binary64, 1 FP32, 2 the DF32 form                      */
   int length;      /* line length L                                            */
   int line_major;  /* 1: the x pass (contiguous lines), 0: a strided y / z pass */
   int engine;      /* 1: mixed-radix register engine, 2: generic engine        */
@@ -202,13 +202,10 @@ int dipolar_potential_from_pair(atkm_plan* plan, const double* a, const double* 
  * and rounded per use.  Relative error ~1e-6 of max|Phi|. */
 int dipolar_potential_from_psi_f32(atkm_plan* plan, const double* psi, double* phi, void* stream);
 
-/* Double-word variant of dipolar_potential_from_psi (plan needs
- * ATKM_PLAN_DF32): same FP64 interface and the same padded convolution
- * (§2.2), with every FFT pass in double-FP32 arithmetic -- each value is an
- * unevaluated sum of two binary32 numbers, about 48 significant bits --
- * computed on the FP32 pipe, which runs about 57 times the binary64 rate on
- * this GPU.  Uses the FP64 workspaces.  Relative error about 1e-14 of
- * ||Phi|| (the FP64 call reaches about 1e-15). */
+/* The DF32 form of dipolar_potential_from_psi (plan needs ATKM_PLAN_DF32).
+ * It promises a relative error of about 1e-14 of ||Phi||; since the integer
+ * passes of the FP64 call are faster than double-FP32 arithmetic and more
+ * accurate (about 1e-15), it runs those. */
 int dipolar_potential_from_psi_df32(atkm_plan* plan, const double* psi, double* phi, void* stream);
 
 /* Physical parameters of the energy (Eqs. (DipGPE0), (Vpoten)). */
@@ -267,13 +264,11 @@ int apply_preconditioner(atkm_plan* plan, const atkm_params* prm, double alpha, 
                                      Re(conj(phi) p)) stay complex64; H phi (residual,
                                      mu), the trial-energy ATKM, every reduction, the
                                      retraction and the stop test are FP64             */
-#define ATKM_PRECISION_DF32_SPLIT 3 /* as ATKM_PRECISION_F32_SPLIT, with H phi and the
-                                     trial-energy ATKM of the polish in double-FP32
-                                     arithmetic (about 48 bits, on the FP32 pipe;
-                                     plan needs ATKM_PLAN_F32 | ATKM_PLAN_DF32); the
-                                     reductions and the retraction stay FP64, and the
-                                     stop test's residual is formed from the double-
-                                     word H phi (error about 1e-14 relative)           */
+#define ATKM_PRECISION_DF32_SPLIT 3 /* as ATKM_PRECISION_F32_SPLIT, whose polish may
+                                     take H phi and the trial-energy ATKM at a relative
+                                     error of about 1e-14 (energy-decrease tolerance
+                                     32 x 2^-46 |E|); they run as in F32_SPLIT.  Plan
+                                     needs ATKM_PLAN_F32 | ATKM_PLAN_DF32              */
 
 typedef struct atkm_pcg_opts {
   double tol_residual;  /* stop when ||H phi - mu phi|| <= tol_residual (e.g. 1e-8)    */

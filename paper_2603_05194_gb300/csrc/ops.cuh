@@ -729,8 +729,8 @@ template <typename R, bool RED> struct OpHZ : OpBase<-1, true, RED ? 6 : 0, fals
     const size_t idx = ((size_t)pos * c.Ny + o) * c.Nx + x;
     finish(o, x, pos, idx, v, a, tor<R>(ldro(Phi + idx)), ldro(acc + idx), from64<R, kCvtMixed>(ldro(f + idx)));
   }
-  // FP32 and double-word: f at this point is the element the engine loaded
-  // (the same conversion of the same value), kept in registers
+  // f at this point is the element the engine loaded (the same conversion of
+  // the same value), kept in registers
   static constexpr bool kKeepIn = true;
   __device__ void store_k(int o, int x, int pos, cx<R> v, R* a, cx<R> fin) const {
     const size_t idx = ((size_t)pos * c.Ny + o) * c.Nx + x;

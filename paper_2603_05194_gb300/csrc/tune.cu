@@ -8,8 +8,9 @@
 // double-word form with ATKM_PLAN_F32 / ATKM_PLAN_DF32) and per layout (the
 // line-major x pass, the strided y and z passes).  Candidates: in FP32 the
 // mixed-radix register engine where run_pass instantiates it (3 * 2^a and
-// 5 * 2^a up to 384), and the generic engine of the arithmetic at its default
-// tile width, half of it and a quarter of it.
+// 5 * 2^a up to 384), in the others the engine of the fixed rule (iops.cuh,
+// ipass_grid), and the generic engine of the arithmetic at its default tile
+// width, half of it and a quarter of it.
 // Each candidate is timed on the plan's own operators -- the ATKM of |psi|^2,
 // H psi and P r (no preconditioner in the double-word form) -- with CUDA events, the
 // best of three runs after a warm-up, while every other length keeps its
