@@ -747,7 +747,7 @@ k_scale_linf(double2* __restrict__ phin, const double2* __restrict__ phi, const 
 
 // phi+ = *ca phi + *cb p (the retraction, normalised), and the block maximum of
 // |phi+ - phi|^2: 48 bytes and 8 FP64 operations a point in one kernel, in place
-// of the combination with its norm and a scaling pass (128 bytes, 141 -> 72 us
+// of the combination with its norm and a scaling pass (128 bytes, 141 -> 78 us
 // at 256x256x64).  The maximum is taken on the bit patterns, which order
 // nonnegative binary64 values like the values and stay off the FP64 pipe.
 __global__ void __launch_bounds__(kRedThreads)
