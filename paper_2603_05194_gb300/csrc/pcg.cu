@@ -165,27 +165,19 @@ int red_grid(size_t N, int per) {
   return (int)b;
 }
 
-// Grid of a grid-stride vector kernel: whole waves (SMs x resident blocks of
-// that kernel, from the occupancy calculator, cached per kernel), at most
+// Blocks per SM of each vector kernel: its launch bound and, times the SMs, its
+// grid.  The grid sets the order of the kernel's sum, so it is fixed here: taken
+// from the occupancy calculator it moved with the register allocation, and with it
+// the last bit of a norm and then, by a rounding to binary32, an iterate of the
+// FP32 phase by 1e-7.
+template <typename T> constexpr int kDirBlocks = sizeof(T) == 4 ? 5 : 6;
+constexpr int kCurvBlocks = 6;
+constexpr int kVecBlocks = 8;
+
+// Grid of a grid-stride vector kernel: one wave of per_sm blocks an SM, at most
 // red_grid(N, per) -- a partial last wave would leave SMs idle at the end.
-int wave_grid(const void* kernel, size_t N, int per) {
-  static std::mutex mu;
-  static std::vector<std::pair<const void*, int>> cache;
+int wave_grid(int per_sm, size_t N, int per) {
   const int nsm = device_sm_count();
-  int per_sm = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (auto& kv : cache)
-      if (kv.first == kernel) per_sm = kv.second;
-    if (per_sm == 0) {
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRedThreads, 0) != cudaSuccess ||
-          per_sm <= 0) {
-        cudaGetLastError();
-        per_sm = 4;
-      }
-      cache.emplace_back(kernel, per_sm);
-    }
-  }
   const size_t cap = (size_t)red_grid(N, per);
   if (nsm <= 0) return (int)cap;  // SM count unknown: the size-based grid
   const size_t full = (size_t)nsm * per_sm;
@@ -588,7 +580,10 @@ __global__ void k_d_handover(Ctl* c, double tolE_eps, int nodes) {
 
 // What the last block of a reducing vector kernel does: the grid sums (in the
 // fixed order of finalize_sums) into out, then the control step that reads
-// them.  s is the plan's scalar block.
+// them.  s is the plan's scalar block.  The step is a template parameter, so that
+// a kernel holds the registers of its own step only (with all of them behind a
+// switch, k_lincomb<double> took 40 registers and a 40-byte stack instead of 32
+// and none: 6 blocks an SM instead of 8).
 enum Then {
   kThenNone, kThenInit, kThenNoise, kThenTop, kThenTopCheck, kThenDir, kThenReset, kThenReset2, kThenStep, kThenNorm,
   kThenAccept, kThenAcceptLoop
@@ -599,38 +594,33 @@ struct Fin {
   unsigned* cnt;
   const double* s;
   Ctl* c;
-  int then, nodes;
+  int nodes;
   cudaGraphConditionalHandle h;
 };
-__device__ __forceinline__ void run_then(const Fin& f) {
+template <int THEN> __device__ __forceinline__ void run_then(const Fin& f) {
   Ctl* c = f.c;
-  switch (f.then) {
-    case kThenInit: c_init(c, f.s); break;
-    case kThenNoise: c_noise(c, f.s); break;
-    case kThenTop:
-    case kThenTopCheck:
-      c_parts(c, f.s);
-      c_res(c, f.s);
-      if (f.then == kThenTopCheck) d_check(c, f.h, f.nodes);
-      break;
-    case kThenDir: c_dir(c, f.s); break;
-    case kThenReset: c_reset(c, f.s); break;
-    case kThenReset2: c_reset2(c, f.s); break;
-    case kThenStep: c_step(c, f.s); break;
-    case kThenNorm: c_norm(c, f.s); break;
-    case kThenAccept:
-    case kThenAcceptLoop:
-      c_accept(c, f.s);
-      if (f.then == kThenAcceptLoop) d_after_trial(c, f.h, f.nodes);
-      break;
-    default: break;
+  if constexpr (THEN == kThenInit) c_init(c, f.s);
+  if constexpr (THEN == kThenNoise) c_noise(c, f.s);
+  if constexpr (THEN == kThenTop || THEN == kThenTopCheck) {
+    c_parts(c, f.s);
+    c_res(c, f.s);
   }
+  if constexpr (THEN == kThenTopCheck) d_check(c, f.h, f.nodes);
+  if constexpr (THEN == kThenDir) c_dir(c, f.s);
+  if constexpr (THEN == kThenReset) c_reset(c, f.s);
+  if constexpr (THEN == kThenReset2) c_reset2(c, f.s);
+  if constexpr (THEN == kThenStep) c_step(c, f.s);
+  if constexpr (THEN == kThenNorm) c_norm(c, f.s);
+  if constexpr (THEN == kThenAccept || THEN == kThenAcceptLoop) c_accept(c, f.s);
+  if constexpr (THEN == kThenAcceptLoop) d_after_trial(c, f.h, f.nodes);
 }
-template <int NS> __device__ __forceinline__ void finish(const Fin& f) {
+template <int NS, int THEN> __device__ __forceinline__ void finish(const Fin& f) {
   if (!last_block(f.cnt, (threadIdx.x & 31) == 0)) return;
   finalize_sums<NS>(f.part, gridDim.x, f.out);
-  __syncthreads();
-  if (threadIdx.x == 0) run_then(f);
+  if constexpr (THEN != kThenNone) {
+    __syncthreads();
+    if (threadIdx.x == 0) run_then<THEN>(f);
+  }
 }
 // Grid maximum of the block maxima; out = its square root (the partials hold
 // squared distances).
@@ -649,7 +639,7 @@ __device__ __forceinline__ void finish_max(const Fin& f) {
 }
 
 // sum_j Re(u_j conj(v_j)) (FP64).
-__global__ void __launch_bounds__(kRedThreads) k_dot(const double2* __restrict__ u, const double2* __restrict__ v,
+__global__ void __launch_bounds__(kRedThreads, kVecBlocks) k_dot(const double2* __restrict__ u, const double2* __restrict__ v,
                                                      size_t N, Fin f) {
   pdl_trigger();
   Sums<double, 1> acc;
@@ -659,13 +649,13 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(const double2* __restrict__
     acc.mac(0, a.y, b.y);
   }
   acc.store(f.part);
-  finish<1>(f);
+  finish<1, kThenInit>(f);
 }
 
 // The seven sums of the direction step from one read of its five vectors:
 // <Pr,phi>, <r,Pr>, <r,phi>, <r_prev,Pr>, <r_prev,phi>, <p_prev,phi>, <phi,phi>.
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kRedThreads, kDirBlocks<T>)
 k_dir_dots(const double2* __restrict__ Pr, const double2* __restrict__ phi, const double2* __restrict__ r,
            const double2* __restrict__ rp, const double2* __restrict__ pp, size_t N, Fin f) {
   pdl_trigger();
@@ -682,7 +672,7 @@ k_dir_dots(const double2* __restrict__ Pr, const double2* __restrict__ phi, cons
     acc.next();
   }
   acc.store(f.part);
-  finish<7>(f);
+  finish<7, kThenDir>(f);
 }
 
 // A coefficient m * (*p) (p may be null: then m).
@@ -694,8 +684,8 @@ __device__ __forceinline__ double cval(const Coef& c) { return c.p ? c.m * *c.p 
 
 // out = c0 v0 + c1 v1 + c2 v2 (null vectors skipped); sums |out|^2 and
 // Re(w conj(out)) when w is given.  Skipped entirely when *pred == 0.
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
+template <typename T, int THEN>
+__global__ void __launch_bounds__(kRedThreads, kVecBlocks)
 k_lincomb(double2* __restrict__ out, const double2* __restrict__ v0, Coef c0, const double2* __restrict__ v1,
           Coef c1, const double2* __restrict__ v2, Coef c2, const double2* __restrict__ w, size_t N,
           Fin f, const int* __restrict__ pred) {
@@ -714,13 +704,13 @@ k_lincomb(double2* __restrict__ out, const double2* __restrict__ v0, Coef c0, co
     acc.next();
   }
   acc.store(f.part);
-  finish<2>(f);
+  finish<2, THEN>(f);
 }
 
 // phi+ *= *inv (FP64: the renormalisation); block max of |phi+ - phi|^2, the
 // difference taken in T (FP32 in the FP32 phase, where it is only logged).
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kRedThreads, kVecBlocks)
 k_scale_linf(double2* __restrict__ phin, const double2* __restrict__ phi, const double* __restrict__ invp, size_t N,
              Fin f) {
   __shared__ T sh[kRedThreads];
@@ -750,7 +740,7 @@ k_scale_linf(double2* __restrict__ phin, const double2* __restrict__ phi, const 
 // of the combination with its norm and a scaling pass (128 bytes, 141 -> 78 us
 // at 256x256x64).  The maximum is taken on the bit patterns, which order
 // nonnegative binary64 values like the values and stay off the FP64 pipe.
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kRedThreads, kVecBlocks)
 k_trial(double2* __restrict__ phin, const double2* __restrict__ phi, const double2* __restrict__ p,
         const double* __restrict__ ca, const double* __restrict__ cb, size_t N, Fin f) {
   __shared__ double sh[kRedThreads];
@@ -781,7 +771,7 @@ k_trial(double2* __restrict__ phin, const double2* __restrict__ phi, const doubl
 //   [2] sum (beta|phi|^2 + lambda Phi) Re(phi conj(p))
 //   [3] sum (beta|phi|^2 + lambda Phi) |p|^2
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kRedThreads, kCurvBlocks)
 k_curv_sums(const double2* __restrict__ Hp, const double2* __restrict__ phi, const double2* __restrict__ p,
             const double* __restrict__ Phi, const double* __restrict__ Phi1, double beta, double lambda, size_t N,
             Fin f) {
@@ -799,12 +789,12 @@ k_curv_sums(const double2* __restrict__ Hp, const double2* __restrict__ phi, con
     acc.next();
   }
   acc.store(f.part);
-  finish<4>(f);
+  finish<4, kThenStep>(f);
 }
 
 // [0] sum |phi|^4, [1] sum Phi |phi|^2
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads)
+template <typename T, int THEN>
+__global__ void __launch_bounds__(kRedThreads, kVecBlocks)
 k_quartic_sums(const double2* __restrict__ phi, const double* __restrict__ Phi, size_t N, Fin f) {
   pdl_trigger();
   Sums<T, 2> acc;
@@ -816,7 +806,7 @@ k_quartic_sums(const double2* __restrict__ phi, const double* __restrict__ Phi, 
     acc.next();
   }
   acc.store(f.part);
-  finish<2>(f);
+  finish<2, THEN>(f);
 }
 
 }  // namespace
@@ -958,28 +948,30 @@ struct Seq {
   cudaStream_t st() const { return B.st; }
   void chk(cudaError_t e) { if (err == cudaSuccess && e != cudaSuccess) err = e; }
 
-  Fin fin(int dst, int then, int nodes = 0, cudaGraphConditionalHandle h = 0) const {
-    return Fin{p->partials, p->scal + dst, p->cnt, p->scal, B.ctl, then, nodes, h};
+  Fin fin(int dst, int nodes = 0, cudaGraphConditionalHandle h = 0) const {
+    return Fin{p->partials, p->scal + dst, p->cnt, p->scal, B.ctl, nodes, h};
   }
-  void dot(const double2* u, const double2* v, int dst, int then) {
+  // <u, v> into S_N, then c_init.
+  void dot_init(const double2* u, const double2* v) {
     prof_begin(p, "vec_dots", 32.0 * B.N, 0.0, st());
-    const int g = wave_grid((const void*)k_dot, B.N, 4);
-    k_dot<<<g, kRedThreads, 0, st()>>>(u, v, B.N, fin(dst, then));
+    const int g = wave_grid(kVecBlocks, B.N, 4);
+    k_dot<<<g, kRedThreads, 0, st()>>>(u, v, B.N, fin(S_N));
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
   }
   // FP64 arithmetic unless this is the FP32 phase and `phase_type` allows it.
+  template <int THEN>
   void lincomb(double2* out, const double2* v0, Coef c0, const double2* v1, Coef c1, const double2* v2, Coef c2,
                const double2* w, const Fin& f, const int* pred = nullptr, bool phase_type = true) {
     const double nv = (v0 ? 1 : 0) + (v1 ? 1 : 0) + (v2 ? 1 : 0) + (w ? 1 : 0) + 1;
     prof_begin(p, "vec_lincomb", 16.0 * nv * B.N, 0.0, st());
     const bool fl = f32 && phase_type;
-    const int g = fl ? wave_grid((const void*)k_lincomb<float>, B.N, 4) : wave_grid((const void*)k_lincomb<double>, B.N, f32 ? 4 : 1);
+    const int g = wave_grid(kVecBlocks, B.N, f32 ? 4 : 1);
     if (fl)
-      k_lincomb<float><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
+      k_lincomb<float, THEN><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
     else
-      k_lincomb<double><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
+      k_lincomb<double, THEN><<<g, kRedThreads, 0, st()>>>(out, v0, c0, v1, c1, v2, c2, w, B.N, f, pred);
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
@@ -1008,34 +1000,37 @@ struct Seq {
     hop(B.phi[q], B.Hphi, S_H);
     // mu = hvol <H phi, phi> read from the sums themselves (c->mu is set by the
     // control step that ends this kernel)
-    lincomb(B.r[q], B.Hphi, Coef{nullptr, 1.0}, B.phi[q], Coef{s() + S_H + 8, -p->hvol}, nullptr, Coef{nullptr, 0.0},
-            nullptr, fin(S_R, loop ? kThenTopCheck : kThenTop, loop ? sofar() + 1 : 0, h));
+    const Coef c0{nullptr, 1.0}, c1{s() + S_H + 8, -p->hvol}, c2{nullptr, 0.0};
+    if (loop) lincomb<kThenTopCheck>(B.r[q], B.Hphi, c0, B.phi[q], c1, nullptr, c2, nullptr, fin(S_R, sofar() + 1, h));
+    else lincomb<kThenTop>(B.r[q], B.Hphi, c0, B.phi[q], c1, nullptr, c2, nullptr, fin(S_R));
   }
   void top() { top(false, 0, [] { return 0; }); }
+  template <int THEN> void quartic(const double2* phin, const Fin& f) {
+    const int g = wave_grid(kVecBlocks, B.N, f32 ? 4 : 1);
+    if (f32) k_quartic_sums<float, THEN><<<g, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
+    else k_quartic_sums<double, THEN><<<g, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
+  }
   // One trial of Step 4 (iii) with the current retraction coefficients.
   template <class F> void trial(bool loop, cudaGraphConditionalHandle h, F sofar) {
     double2* phin = B.phi[q ^ 1];
     if (f32) {
-      lincomb(phin, B.phi[q], Coef{&c()->cr, 1.0}, B.p[q], Coef{&c()->sr, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr,
-              fin(S_T, kThenNorm), nullptr, false);  // the retraction stays FP64
+      lincomb<kThenNorm>(phin, B.phi[q], Coef{&c()->cr, 1.0}, B.p[q], Coef{&c()->sr, 1.0}, nullptr, Coef{nullptr, 0.0},
+                         nullptr, fin(S_T), nullptr, false);  // the retraction stays FP64
       prof_begin(p, "vec_scale_linf", 48.0 * B.N, 0.0, st());
-      const int gs = wave_grid((const void*)k_scale_linf<float>, B.N, 4);
-      k_scale_linf<float><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L, kThenNone));
+      const int gs = wave_grid(kVecBlocks, B.N, 4);
+      k_scale_linf<float><<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], &c()->inv, B.N, fin(S_L));
     } else {
       prof_begin(p, "vec_trial", 48.0 * B.N, 0.0, st());
-      const int gs = wave_grid((const void*)k_trial, B.N, 1);
-      k_trial<<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], B.p[q], &c()->ca, &c()->cb, B.N, fin(S_L, kThenNone));
+      const int gs = wave_grid(kVecBlocks, B.N, 1);
+      k_trial<<<gs, kRedThreads, 0, st()>>>(phin, B.phi[q], B.p[q], &c()->ca, &c()->cb, B.N, fin(S_L));
     }
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
     atkm(SRC_PSI, reinterpret_cast<const double*>(phin), nullptr, B.Phi[q ^ 1]);
     prof_begin(p, "vec_quartic", 24.0 * B.N, 0.0, st());
-    const int gq = f32 ? wave_grid((const void*)k_quartic_sums<float>, B.N, 4)
-                       : wave_grid((const void*)k_quartic_sums<double>, B.N, 1);
-    const Fin f = fin(S_Q, loop ? kThenAcceptLoop : kThenAccept, loop ? sofar() + 1 : 0, h);
-    if (f32) k_quartic_sums<float><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
-    else k_quartic_sums<double><<<gq, kRedThreads, 0, st()>>>(phin, B.Phi[q ^ 1], B.N, f);
+    if (loop) quartic<kThenAcceptLoop>(phin, fin(S_Q, sofar() + 1, h));
+    else quartic<kThenAccept>(phin, fin(S_Q));
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
@@ -1057,9 +1052,8 @@ struct Seq {
   template <class F> void rest(bool loop, cudaGraphConditionalHandle h, F sofar) {
     chk(precond());
     prof_begin(p, "vec_dir_dots", 80.0 * B.N, 0.0, st());
-    const int gd = f32 ? wave_grid((const void*)k_dir_dots<float>, B.N, 4)
-                       : wave_grid((const void*)k_dir_dots<double>, B.N, 1);
-    const Fin fd = fin(S_D, kThenDir);
+    const int gd = f32 ? wave_grid(kDirBlocks<float>, B.N, 4) : wave_grid(kDirBlocks<double>, B.N, 1);
+    const Fin fd = fin(S_D);
     if (f32)
       k_dir_dots<float><<<gd, kRedThreads, 0, st()>>>(B.Pr, B.phi[q], B.r[q], B.r[q ^ 1], B.p[q ^ 1], B.N, fd);
     else
@@ -1067,10 +1061,10 @@ struct Seq {
     prof_end(p, st());
     count_launches(1);
     chk(cudaGetLastError());
-    lincomb(B.p[q], B.Pr, Coef{&c()->cp0, 1.0}, B.p[q ^ 1], Coef{&c()->cp1, 1.0}, B.phi[q], Coef{&c()->cp2, 1.0},
-            B.Hphi, fin(S_P, kThenReset));
-    lincomb(B.p[q], B.Pr, Coef{nullptr, -1.0}, B.phi[q], Coef{&c()->b, 1.0}, nullptr, Coef{nullptr, 0.0}, B.Hphi,
-            fin(S_P, kThenReset2), &c()->redo);
+    lincomb<kThenReset>(B.p[q], B.Pr, Coef{&c()->cp0, 1.0}, B.p[q ^ 1], Coef{&c()->cp1, 1.0}, B.phi[q],
+                        Coef{&c()->cp2, 1.0}, B.Hphi, fin(S_P));
+    lincomb<kThenReset2>(B.p[q], B.Pr, Coef{nullptr, -1.0}, B.phi[q], Coef{&c()->b, 1.0}, nullptr, Coef{nullptr, 0.0},
+                         B.Hphi, fin(S_P), &c()->redo);
     // H p and Phi' write different buffers and share no workspace (H: T1, T2,
     // ex[3], ex[4]; ATKM: W1, W2, ex[0..2])
     if (fork) {
@@ -1085,9 +1079,8 @@ struct Seq {
       chk(cudaStreamWaitEvent(st(), B.ev_join, 0));
     }
     prof_begin(p, "vec_curv_sums", 64.0 * B.N, 0.0, st());
-    const int gc = f32 ? wave_grid((const void*)k_curv_sums<float>, B.N, 4)
-                       : wave_grid((const void*)k_curv_sums<double>, B.N, 1);
-    const Fin fc = fin(S_C, kThenStep);
+    const int gc = wave_grid(kCurvBlocks, B.N, f32 ? 4 : 1);
+    const Fin fc = fin(S_C);
     if (f32)
       k_curv_sums<float><<<gc, kRedThreads, 0, st()>>>(B.Hp, B.phi[q], B.p[q], B.Phi[q], B.Phi1, ph.beta, ph.lambda,
                                                        B.N, fc);
@@ -1532,11 +1525,11 @@ struct Solver {
       q = 0;
       Seq S = seq(f32);
       const double2* p0 = reinterpret_cast<const double2*>(psi);
-      S.dot(p0, p0, S_N, kThenInit);
+      S.dot_init(p0, p0);
       // the normalisation stays FP64 in every precision form (as the
       // renormalisation after each retraction does)
-      S.lincomb(B->phi[0], p0, Coef{&B->ctl->inv0, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr, Coef{nullptr, 0.0},
-                nullptr, S.fin(S_T, kThenNone), nullptr, false);
+      S.lincomb<kThenNone>(B->phi[0], p0, Coef{&B->ctl->inv0, 1.0}, nullptr, Coef{nullptr, 0.0}, nullptr,
+                           Coef{nullptr, 0.0}, nullptr, S.fin(S_T), nullptr, false);
       S.atkm(SRC_PSI, reinterpret_cast<const double*>(B->phi[0]), nullptr, B->Phi[0]);
       S.ctl1(k_c_reset_state, B->ctl, 0, 1, 1);
       chk(S.err);
@@ -1548,8 +1541,8 @@ struct Solver {
         Z.atkm(SRC_PSI, p0d, nullptr, B->Phi1);
         chk(launch_H64(plan, false, ph, p0d, p0d, B->Phi1, reinterpret_cast<double*>(B->Hp), -1, B->st));
         chk(launch_H<float>(plan, ph, p0d, p0d, B->Phi[0], reinterpret_cast<double*>(B->Hphi), -1, B->st));
-        Z.lincomb(B->Pr, B->Hp, Coef{nullptr, 1.0}, B->Hphi, Coef{nullptr, -1.0}, nullptr, Coef{nullptr, 0.0},
-                  nullptr, Z.fin(S_Z, kThenNoise), nullptr, false);
+        Z.lincomb<kThenNoise>(B->Pr, B->Hp, Coef{nullptr, 1.0}, B->Hphi, Coef{nullptr, -1.0}, nullptr,
+                              Coef{nullptr, 0.0}, nullptr, Z.fin(S_Z), nullptr, false);
         chk(Z.err);
       }
       fetch_async();
