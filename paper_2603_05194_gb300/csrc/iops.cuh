@@ -64,6 +64,7 @@ template <int S1, bool SECOND, int NRED, bool LM, int SRC> struct IOpBase {
   static constexpr bool kHalfOut = false;   // only positions < L/2 of the output are used
   static constexpr bool kNyqTail = false;   // column pass over columns 0..Nx (see ipass_place)
   static constexpr bool kMul = false;       // the spectral step is mul_tile
+  static constexpr bool kLineExp = false;   // (kMul) every line has an exponent of its own, not the tile one
   // launched by launch_pdl, inputs read by plain loads; an op whose loads should
   // be moved ahead of its own stores reads by __ldg and is launched normally
   static constexpr bool kPdl = true;
@@ -127,14 +128,14 @@ template <class Op> __device__ __forceinline__ bool ipass_line(const Op& op, int
 
 // Scratch of the tile-wide reductions, one slot per use so that no barrier is
 // needed between a slot's readers and the next use.
-template <bool TWIN> struct TileRedT {
+struct TileRedBase {
   unsigned m[4][16];
   int nan[128];
 };
-template <> struct TileRedT<true> : TileRedT<false> {
-  c64 last[128];  // element L of each line (load_twin)
+template <class Op> struct TileRedT : TileRedBase {
+  c64 last[Op::kTwin ? 128 : 1];               // element L of each line (load_twin)
+  unsigned line[Op::kLineExp ? 3 : 1][128];    // line_max: size of the input, of the spectrum, of the products
 };
-using TileRed = TileRedT<false>;
 
 // Over a CTA of NW warps.
 template <int NW> __device__ __forceinline__ unsigned tile_or(unsigned v, unsigned* slot) {
@@ -159,6 +160,26 @@ template <int NW> __device__ __forceinline__ int tile_max_s(int v, unsigned* slo
   return (int)(tile_max<NW>((unsigned)v ^ 0x80000000u, slot) ^ 0x80000000u);
 }
 
+// The same over each line of a tile, into slot[t].  Lanes LO, 2 LO, ... HI apart
+// hold elements of the same line; lanes of the group's first LO (column tiles) or
+// first one (line-major) write.  All slots are zero on entry (init_lines) and hold
+// the maxima after the barrier.
+template <int LO, int HI> __device__ __forceinline__ void line_max(unsigned v, unsigned* slot, int t) {
+#pragma unroll
+  for (int o = HI; o >= LO; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if (HI < LO || (threadIdx.x & (2 * HI - LO)) == 0) atomicMax(slot + t, v);
+  __syncthreads();
+}
+// Lane distances of a tile's lines: LM: P consecutive threads a line (grouped
+// where P is a power of two); else T lines side by side.
+template <bool LM, int T, int P> struct LineLanes {
+  static constexpr bool pow2 = LM ? (P & (P - 1)) == 0 : (T & (T - 1)) == 0;
+  static constexpr int LO = pow2 ? (LM ? 1 : T) : 32, HI = pow2 && (LM ? P > 1 : T < 32) ? (LM ? (P < 32 ? P / 2 : 16) : 16) : 0;
+};
+template <class TR> __device__ __forceinline__ void init_lines(TR& tr) {
+  for (int i = threadIdx.x; i < 3 * 128; i += blockDim.x) tr.line[0][i] = 0u;
+}
+
 __device__ __forceinline__ unsigned dmag(double2 z) {
   return (unsigned)max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff);
 }
@@ -171,11 +192,14 @@ struct Tile {
   bool bad, anybad;
 };
 
-// Loads a thread's E elements (guarded by pos < L) as integers of the tile's
-// common exponent, components below 2^59 (2^60 when the first stage sees a
-// zero upper half, unless the post-twist needs the room).
-template <int E, bool FULL, int NW, class Op>
-__device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], TileRed& tr) {
+// The exponent that a tile or line of largest |hi word| M < 0x7ff00000 gets.
+template <int B> __device__ __forceinline__ int load_exp(unsigned M) { return max((int)(M >> 20), 64) - 1023 - (B - 1); }
+
+// Loads a thread's E elements (guarded by pos < L) as integers of the tile's (of
+// the line's with kLineExp) common exponent, components below 2^59 (2^60 when the
+// first stage sees a zero upper half, unless the post-twist needs the room).
+template <int E, bool FULL, int NW, class LL, class Op, class TR>
+__device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], TR& tr) {
   constexpr int EL = Op::kZeroUpper ? (E + 1) / 2 : E;  // elements that can lie below L/2 (P E >= L)
   const int lim = Op::kZeroUpper ? L / 2 : L;
   constexpr int B = (Op::kZeroUpper && !Op::kMirror) ? kInBits + 1 : kInBits;
@@ -188,30 +212,43 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
       d[r] = (l.ok && (FULL || pos < lim)) ? op.load(l.o, l.x, pos) : make_double2(0.0, 0.0);
       m = max(m, dmag(d[r]));
     }
-    unsigned M = tile_max<NW>(m, tr.m[0]);
+    unsigned M;
     bool bad = false, any = false;
-    if (M >= 0x7ff00000u) {  // a NaN or an infinity: the lines that hold one are left out of the tile's size
-      if (threadIdx.x < 128) tr.nan[threadIdx.x] = 0;
-      __syncthreads();
+    if constexpr (Op::kLineExp) {
+      __syncthreads();  // init_lines
+      line_max<LL::LO, LL::HI>(m, tr.line[0], l.t);
+      M = tr.line[0][l.t];
+      if (M >= 0x7ff00000u) {  // the line holds a NaN or an infinity
+        bad = true;
+        M = 0;
 #pragma unroll
-      for (int r = 0; r < EL; ++r) bad |= dmag(d[r]) >= 0x7ff00000u;
-      if (bad) tr.nan[l.t] = 1;
-      __syncthreads();
-      bad = tr.nan[l.t] != 0;
-      any = true;
-      m = 0;
-#pragma unroll
-      for (int r = 0; r < EL; ++r) {
-        if (bad) d[r] = make_double2(0.0, 0.0);
-        m = max(m, dmag(d[r]));
+        for (int r = 0; r < EL; ++r) d[r] = make_double2(0.0, 0.0);
       }
-      M = tile_max<NW>(m, tr.m[1]);
+    } else {
+      M = tile_max<NW>(m, tr.m[0]);
+      if (M >= 0x7ff00000u) {  // a NaN or an infinity: the lines that hold one are left out of the tile's size
+        if (threadIdx.x < 128) tr.nan[threadIdx.x] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < EL; ++r) bad |= dmag(d[r]) >= 0x7ff00000u;
+        if (bad) tr.nan[l.t] = 1;
+        __syncthreads();
+        bad = tr.nan[l.t] != 0;
+        any = true;
+        m = 0;
+#pragma unroll
+        for (int r = 0; r < EL; ++r) {
+          if (bad) d[r] = make_double2(0.0, 0.0);
+          m = max(m, dmag(d[r]));
+        }
+        M = tile_max<NW>(m, tr.m[1]);
+      }
     }
     const int ex = max((int)(M >> 20), 64);
     const int base = 64 - B + ex;
 #pragma unroll
     for (int r = 0; r < E; ++r) v[r] = r < EL ? c64{d2i(d[r < EL ? r : 0].x, base), d2i(d[r < EL ? r : 0].y, base)} : cz();
-    return Tile{ex - 1023 - (B - 1), bad, any};
+    return Tile{load_exp<B>(M), bad, any};
   } else {
     int ee[EL];
     int em = -0x40000000;
@@ -248,7 +285,7 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
 // the stored half spectrum (op.combine): loads the elements, and element L
 // into *last for the threads of position 0, scaled to 60 bits.
 template <int E, bool FULL, int NW, class Op>
-__device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, int L, c64 (&v)[E], c64* last, TileRed& tr) {
+__device__ __forceinline__ Tile load_twin(const Op& op, const Line& l, int P, int L, c64 (&v)[E], c64* last, TileRedBase& tr) {
   int ev[E], el = -0x40000000;
   *last = cz();
   if (l.ok && l.j == 0) {
@@ -306,6 +343,18 @@ __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int
   *e += op.midshift();
 }
 
+// mul_tile's shift up, from the largest mag of the tile or line, and what it does
+// to the exponent: an element of multiplier 2^(ex - 1023) f, f in [1, 2), is held as
+// v f 2^61 / 2^64.
+__device__ __forceinline__ int mul_shift(unsigned m) { return 62 - mag_bits(m); }
+__device__ __forceinline__ void mul_exp(Tile& tl, int sh, int M) {
+  tl.e += M - sh + 64 - 1084 - (kInBits - 32);
+  if (M >= 2040) {  // an infinite or NaN multiplier
+    tl.e = kExpNaN;
+    tl.bad = tl.anybad = true;
+  }
+}
+
 // The same for an op with real multipliers of any size (kMul; op.mult(c, k), c =
 // op.mline(o, x) the line's part, formed once a thread: left to the compiler, H x
 // formed it at every element, 3 of its 4 binary64 operations, 86 against 77 us at
@@ -313,13 +362,19 @@ __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int
 // the tile's largest one.  (With the multiplier in fixed point, nu^2 / 2 of
 // the low frequencies, 2^-18 of the largest at length 1024, would leave the
 // product 2^18 fewer units.)
-template <int E, bool FULL, int NW, class Op>
+template <int E, bool FULL, int NW, class LL, class Op, class TR>
 __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int L, c64 (&v)[E], Tile& tl,
-                                         typename Op::Acc& acc, TileRed& tr) {
+                                         typename Op::Acc& acc, TR& tr) {
   unsigned m = 0;
 #pragma unroll
   for (int r = 0; r < E; ++r) m |= mag(v[r]);
-  const int sh = 62 - mag_bits(tile_or<NW>(m, tr.m[2]));
+  int sh;
+  if constexpr (Op::kLineExp) {
+    line_max<LL::LO, LL::HI>(m, tr.line[1], l.t);
+    sh = mul_shift(tr.line[1][l.t]);
+  } else {
+    sh = mul_shift(tile_or<NW>(m, tr.m[2]));
+  }
   acc.e = tl.e - sh;
   const double c = op.mline(l.o, l.x);
   int ex[E];
@@ -339,19 +394,20 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
       eb = max(eb, 32 - __clz((int)mag(v[r])) + ex[r]);  // bits of the aligned product, less 32
     }
   }
-  const int M = tile_max_s<NW>(eb, tr.m[3]);
+  int M;
+  if constexpr (Op::kLineExp) {
+    line_max<LL::LO, LL::HI>((unsigned)eb ^ 0x80000000u, tr.line[2], l.t);
+    M = (int)(tr.line[2][l.t] ^ 0x80000000u);
+  } else {
+    M = tile_max_s<NW>(eb, tr.m[3]);
+  }
 #pragma unroll
   for (int r = 0; r < E; ++r) {
     const int s = kInBits - 32 - M + ex[r], lf = max(s, 0), rt = min(max(-s, 0), 64);
     v[r].x = shr_clamp((long long)((unsigned long long)v[r].x << lf), rt);
     v[r].y = shr_clamp((long long)((unsigned long long)v[r].y << lf), rt);
   }
-  // an element of multiplier 2^(ex - 1023) f, f in [1, 2), held v f 2^61 / 2^64
-  tl.e += M - sh + 64 - 1084 - (kInBits - 32);
-  if (M >= 2040) {  // an infinite or NaN multiplier
-    tl.e = kExpNaN;
-    tl.bad = tl.anybad = true;
-  }
+  mul_exp(tl, sh, M);
 }
 
 // Block sums of the threads' NR values through shared memory (NR NW 256 bytes,
@@ -472,13 +528,15 @@ template <int L, class Op>
 __global__ void __launch_bounds__(kThreads, 3) k_ifast(Op op, const int4* __restrict__ w) {
   using C = IFast<L>;
   extern __shared__ __align__(16) unsigned char ism[];
-  __shared__ __align__(16) TileRedT<Op::kTwin> tr;
+  __shared__ __align__(16) TileRedT<Op> tr;
   c64* b0 = reinterpret_cast<c64*>(ism);
   // [r][thread]: this thread's table entries
   long long* pre = reinterpret_cast<long long*>(ism + C::template bytes<Op::kLM>()) + threadIdx.x;
   Line l;
+  using LL = LineLanes<Op::kLM, C::T, C::TPL>;
   pdl_trigger();
   if (ipass_line(op, C::T, C::TPL, &l)) return;  // the whole CTA
+  if constexpr (Op::kLineExp) init_lines(tr);
   if constexpr (Op::kPre) {
     if (l.ok) {
 #pragma unroll
@@ -503,7 +561,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_ifast(Op op, const int4* __rest
     }
     __syncthreads();
   } else {
-    tl = load_tile<8, true, 8>(op, l, C::TPL, L, v, tr);
+    tl = load_tile<8, true, 8, LL>(op, l, C::TPL, L, v, tr);
   }
   typename Op::Acc acc{};
   constexpr bool kLo1 = Op::kHalfOut && !Op::kSecond && !Op::kMirror;
@@ -525,7 +583,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_ifast(Op op, const int4* __rest
     if constexpr (Op::kSecond) {
       if constexpr (Op::kPre) asm volatile("cp.async.wait_all;\n" ::: "memory");
       // its barrier also frees b0
-      if constexpr (Op::kMul) mul_tile<8, true, 8>(op, l, C::TPL, L, v, tl, acc, tr);
+      if constexpr (Op::kMul) mul_tile<8, true, 8, LL>(op, l, C::TPL, L, v, tl, acc, tr);
       else mid_tile<8, true, 8>(op, l, C::TPL, L, v, &tl.e, acc, tr.m[2], pre);
       ifast_fft<L, -Op::kSign1, Op::kLM, false, Op::kHalfOut>(v, b0, w, l.t, l.j);
       tl.e += C::SHIFT;
@@ -614,14 +672,16 @@ __device__ __forceinline__ void igen_fft(c64** a, c64** b, const IntLen& f, cons
 
 template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op, IntLen f, int T, int tsh) {
   extern __shared__ __align__(16) unsigned char ism[];
-  __shared__ __align__(16) TileRedT<Op::kTwin> tr;
+  __shared__ __align__(16) TileRedT<Op> tr;
   const int L = f.L, P = kThreads >> tsh;
   c64* a = reinterpret_cast<c64*>(ism);
   const GenTile g(T, tsh, L);
   c64* b = a + T * g.LP;
   Line l;
+  using LL = LineLanes<false, 32, 1>;
   pdl_trigger();
   if (ipass_line(op, T, P, &l)) return;  // the whole CTA
+  if constexpr (Op::kLineExp) init_lines(tr);
   if constexpr (Op::kPdl) pdl_wait();
   c64 v[kGenE];
   Tile tl;
@@ -641,7 +701,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
       if (pos < L) v[r] = op.combine(pos, v[r], pos == 0 ? tr.last[l.t] : b[g.template at<Op::kLM>(l.t, L - pos)]);
     }
   } else {
-    tl = load_tile<kGenE, false, 8>(op, l, P, L, v, tr);
+    tl = load_tile<kGenE, false, 8, LL>(op, l, P, L, v, tr);
   }
   typename Op::Acc acc{};
 #pragma unroll
@@ -665,7 +725,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
     }
     if constexpr (Op::kSecond) {
       // its barrier also frees the tile
-      if constexpr (Op::kMul) mul_tile<kGenE, false, 8>(op, l, P, L, v, tl, acc, tr);
+      if constexpr (Op::kMul) mul_tile<kGenE, false, 8, LL>(op, l, P, L, v, tl, acc, tr);
       else mid_tile<kGenE, false, 8>(op, l, P, L, v, &tl.e, acc, tr.m[2], nullptr);
 #pragma unroll
       for (int r = 0; r < kGenE; ++r) {
@@ -814,7 +874,7 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   using C = IMix<L>;
   constexpr bool LM = Op::kLM;
   extern __shared__ __align__(16) unsigned char ism[];
-  __shared__ __align__(16) TileRedT<Op::kTwin> tr;
+  __shared__ __align__(16) TileRedT<Op> tr;
   c64* b = reinterpret_cast<c64*>(ism);
   // la: this thread's line and elements j + M r; lb: those of the last stage, j + ML r
   Line la, lb;
@@ -826,6 +886,9 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   lb.ok = lb.ok && onb;
   if (!ona) la.t = 0, la.j = 1;
   if (!onb) lb.t = 0, lb.j = 1;
+  using LA = LineLanes<LM, C::T, C::M>;
+  using LB = LineLanes<LM, C::T, C::ML>;
+  if constexpr (Op::kLineExp) init_lines(tr);
   if constexpr (Op::kPdl) pdl_wait();
   c64 v[C::R0];
   Tile tl;
@@ -848,7 +911,7 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
     __syncthreads();
   } else {
     // positions from L / 2 on are zero for kZeroUpper: with an odd radix they begin inside an element's range
-    tl = load_tile<C::R0, !Op::kZeroUpper || C::R0 % 2 == 0, C::NW>(op, la, C::M, L, v, tr);
+    tl = load_tile<C::R0, !Op::kZeroUpper || C::R0 % 2 == 0, C::NW, LA>(op, la, C::M, L, v, tr);
   }
   typename Op::Acc acc{};
   constexpr bool kZU = Op::kZeroUpper && (C::R0 == 4 || C::R0 == 8);
@@ -860,6 +923,12 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   constexpr bool kLO = Op::kHalfOut && C::RL % 2 == 0;
   if (onb) IStage<L, Op::kSign1, LM, false, C::n - 1>::template go<kLO && !Op::kSecond && !Op::kMirror>(u, b, wf, lb.t, lb.j);
   tl.e += C::fshift();
+  Tile tb = tl;  // of the line lb
+  if constexpr (Op::kLineExp && LM) {
+    const unsigned M = tr.line[0][lb.t];
+    tb.bad = M >= 0x7ff00000u;
+    tb.e = load_exp<kInBits>(tb.bad ? 0u : M) + C::fshift();
+  }
   if constexpr (Op::kMirror) {
     __syncthreads();
     if (onb) {
@@ -880,8 +949,12 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
       for (int r = 0; r < C::RL; ++r) u[r] = cz();
     }
     // its barriers also free the tile
-    if constexpr (Op::kMul) mul_tile<C::RL, true, C::NW>(op, lb, C::ML, L, u, tl, acc, tr);
-    else mid_tile<C::RL, true, C::NW>(op, lb, C::ML, L, u, &tl.e, acc, tr.m[2], nullptr);
+    if constexpr (Op::kMul) {
+      mul_tile<C::RL, true, C::NW, LB>(op, lb, C::ML, L, u, tb, acc, tr);
+      // (the threads of la include some that lb leaves idle)
+      if constexpr (Op::kLineExp) mul_exp(tl, mul_shift(tr.line[1][la.t]), (int)(tr.line[2][la.t] ^ 0x80000000u));
+      else tl = tb;
+    } else mid_tile<C::RL, true, C::NW>(op, lb, C::ML, L, u, &tl.e, acc, tr.m[2], nullptr);
     IDft<C::RL, -Op::kSign1>::template go<false, false>(u);
     if (onb) imix_write<L, C::RL, 1, LM>(u, b, lb.t, lb.j);
     __syncthreads();
@@ -907,7 +980,7 @@ k_imix(Op op, const int4* __restrict__ wf, const int4* __restrict__ wr) {
   op.put_exp(la, tl);
   if constexpr (Op::kRed > 0) {
     double a[Op::kRed];
-    op.sums(lb, acc, tl, a);
+    op.sums(lb, acc, tb, a);
     ireduce_out<Op::kRed, C::NW>(a, reinterpret_cast<double*>(ism), op.part, op.pstride, op.sums_out, op.cnt);
   }
 }
@@ -1193,6 +1266,10 @@ struct IAtkmXI : IOpBase<1, false, 0, true, kSrcInt> {
 
 // ---- H_phi f (unpadded grid).  A line's multiplier is (nu_k^2 / 2 + c nu_k) / N
 // with c = Omega y on x lines, -Omega x on y lines, from the axis's tables.
+// H f at a point depends on its three lines only, so every line has its own
+// exponent (kLineExp): a quiet line beside a loud one keeps its 59 bits.  The
+// passes of the other operators mix all three axes, so that their error follows
+// the loudest line in any arithmetic, and one exponent a tile is enough.
 // Sums of k^2 |v|^2 and k |v|^2 over a thread's elements, exact but for the
 // last step: |v|^2 / 2^64 = A + F 2^-31 (v below 2^62 a component; the 31
 // fraction bits matter because k^2 reaches 2^18 where |v|^2 is small), each
@@ -1233,7 +1310,7 @@ template <bool RED> struct IHX : IOpBase<-1, true, RED ? 2 : 0, true, kSrcF64> {
   int Nx, Ny, nl;
   double Om, Ly, hy;
   double ck, cr;       // nu^2 / (2 N) = ck k'^2, Omega nu / N = cr k', k' the signed index
-  static constexpr bool kMul = true;
+  static constexpr bool kMul = true, kLineExp = true;
   struct Acc : KinAcc {};
   __device__ __forceinline__ bool valid(int o, int) const { return o < nl; }
   __device__ __forceinline__ double yc(int o) const { return -Ly + (double)(o % Ny) * hy; }
@@ -1265,7 +1342,7 @@ template <bool RED> struct IHY : IOpBase<-1, true, RED ? 2 : 0, false, kSrcF64> 
   int Nx, Ny;
   double Om, Lx, hx;
   double ck, cr;
-  static constexpr bool kMul = true;
+  static constexpr bool kMul = true, kLineExp = true;
   struct Acc : KinAcc {};
   __device__ __forceinline__ bool valid(int, int x) const { return x < Nx; }
   __device__ __forceinline__ double xc(int x) const { return -Lx + (double)x * hx; }
@@ -1309,7 +1386,7 @@ template <bool RED> struct IHZ : IOpBase<-1, true, RED ? 6 : 0, false, kSrcF64> 
   const double* hz2;
   double gx2, gy2, gz2, beta, lambda, ck;
   bool same;  // f == phi: phi is not read a second time
-  static constexpr bool kMul = true;
+  static constexpr bool kMul = true, kLineExp = true;
   static constexpr bool kPdl = false;
   struct Acc : KinAcc {
     double s[4];

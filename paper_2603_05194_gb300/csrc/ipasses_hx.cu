@@ -15,7 +15,7 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   const double pi = 3.14159265358979323846264338327950288, kx = pi / g.Lx;
   const double2* fin = reinterpret_cast<const double2*>(h.f);
   IHX<RED> op;
-  op.f = fin; op.A = p->T1; op.ex = exp_lines(p->ex[3], gx); op.Nx = g.Nx; op.Ny = g.Ny; op.nl = nl;
+  op.f = fin; op.A = p->T1; op.ex = exp_each_line(p->ex[3]); op.Nx = g.Nx; op.Ny = g.Ny; op.nl = nl;
   op.ck = 0.5 * kx * kx / g.Nx; op.cr = ph.Omega * kx / g.Nx;
   op.kin = iaxt(p, 0).kinN; op.nu = iaxt(p, 0).nuN; op.Om = ph.Omega; op.Ly = g.Ly; op.hy = g.hy;
   op.part = p->partials; op.pstride = gx.grid.x; op.sums_out = p->scal + red_slot; op.cnt = p->cnt;

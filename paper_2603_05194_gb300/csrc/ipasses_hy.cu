@@ -14,7 +14,7 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   const double pi = 3.14159265358979323846264338327950288, ky = pi / g.Ly;
   const double2* fin = reinterpret_cast<const double2*>(h.f);
   IHY<RED> op;
-  op.f = fin; op.A = p->T2; op.ex = exp_cols(p->ex[4], gy); op.Nx = g.Nx; op.Ny = g.Ny;
+  op.f = fin; op.A = p->T2; op.ex = exp_each_col(p->ex[4], g.Nx); op.Nx = g.Nx; op.Ny = g.Ny;
   op.ck = 0.5 * ky * ky / g.Ny; op.cr = -ph.Omega * ky / g.Ny;
   op.kin = iaxt(p, 1).kinN; op.nu = iaxt(p, 1).nuN; op.Om = ph.Omega; op.Lx = g.Lx; op.hx = g.hx;
   op.part = p->partials; op.pstride = gy.grid.x * gy.grid.y; op.sums_out = p->scal + red_slot + 2; op.cnt = p->cnt;

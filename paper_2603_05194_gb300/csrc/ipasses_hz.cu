@@ -16,7 +16,7 @@ cudaError_t run(atkm_plan* p, bool dw, const HArgs& h, int red_slot, cudaStream_
   const double2* fin = reinterpret_cast<const double2*>(h.f);
   IHZ<RED> op;
   op.f = fin; op.phi = reinterpret_cast<const double2*>(h.phi); op.Phi = h.Phi; op.AX = p->T1; op.AY = p->T2;
-  op.ix = exp_lines(p->ex[3], gx); op.iy = exp_cols(p->ex[4], gy);
+  op.ix = exp_each_line(p->ex[3]); op.iy = exp_each_col(p->ex[4], g.Nx);
   op.Hf = reinterpret_cast<double2*>(h.Hf); op.kin = iaxt(p, 2).kinN; op.Nx = g.Nx; op.Ny = g.Ny; op.Nz = g.Nz;
   op.hx2 = iaxt(p, 0).hxc2; op.hy2 = iaxt(p, 1).hxc2; op.hz2 = iaxt(p, 2).hxc2;
   op.gx2 = ph.gx2; op.gy2 = ph.gy2; op.gz2 = ph.gz2; op.beta = ph.beta; op.lambda = ph.lambda;

@@ -33,6 +33,9 @@ inline double ifftflops(double n) { return 5.0 * n * log2(n); }
 inline ExpTab exp_lines(int* e, const IPassGrid& pg) { return ExpTab{e, pg.tsh, 16, 1}; }
 // ... and of a column pass (one entry an outer index and column tile).
 inline ExpTab exp_cols(int* e, const IPassGrid& pg) { return ExpTab{e, 0, pg.tsh, (int)pg.grid.x}; }
+// The same with one entry a line (kLineExp): of an x line, of column x of X.
+inline ExpTab exp_each_line(int* e) { return ExpTab{e, 0, 16, 1}; }
+inline ExpTab exp_each_col(int* e, int X) { return ExpTab{e, 0, 0, X}; }
 
 // The plan's binary64 tables of axis a (see AxT in atkm_internal.cuh).
 inline AxT iaxt(const atkm_plan* p, int a) {

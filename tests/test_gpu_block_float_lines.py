@@ -1,0 +1,61 @@
+"""The binary64 operators' integer passes, line by line: H f of a quiet line
+beside loud ones, every line length that the composite-length engine is built
+for, and values next to the ends of the binary64 range."""
+import numpy as np
+import pytest
+import torch
+
+import atkm_workloads as W
+
+pytestmark = pytest.mark.gpu
+GAMMA, BETA, LAM, OM = (1.0, 1.3, 3.0), 30.0, 12.0, 0.4
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def host(t):
+    return t.detach().cpu().numpy()
+
+
+def rel2(a, b):
+    return float(np.linalg.norm((a - b).ravel()) / np.linalg.norm(b.ravel()))
+
+
+def mesh(N, L):
+    ax = [-L[a] + (2.0 * L[a] / N[a]) * np.arange(N[a]) for a in range(3)]
+    k = [np.fft.fftfreq(N[a], 1.0 / N[a]).round() * np.pi / L[a] for a in range(3)]
+    view = [(None, None, slice(None)), (None, slice(None), None), (slice(None), None, None)]
+    return [ax[a][view[a]] for a in range(3)], [k[a][view[a]] for a in range(3)]
+
+
+def ref_H(N, L, f, phi, Phi):
+    """H_phi f by numpy's transforms of each axis's lines."""
+    (x, y, z), (kx, ky, kz) = mesh(N, L)
+    line = lambda a, m: np.fft.ifft(m * np.fft.fft(f, axis=a), axis=a)  # noqa: E731
+    V = 0.5 * ((GAMMA[0] * x) ** 2 + (GAMMA[1] * y) ** 2 + (GAMMA[2] * z) ** 2)
+    return (line(2, 0.5 * kx ** 2 + OM * y * kx) + line(1, 0.5 * ky ** 2 - OM * x * ky) + line(0, 0.5 * kz ** 2)
+            + (V + BETA * np.abs(phi) ** 2 + LAM * Phi) * f)
+
+
+# each engine in each role: k_ifast (256; 512), k_imix (144, 36; 32, 16 on a small grid), k_igen (54, 50, 12)
+@pytest.mark.parametrize("N", [(256, 16, 64), (16, 512, 32), (144, 36, 20), (32, 16, 16), (54, 50, 12)])
+@pytest.mark.parametrize("quiet", [1e-9, 1e-30, 1e-200])
+def test_quiet_lines_beside_loud_ones(lib, N, quiet):
+    """f is of size one where all indices are odd, of size `quiet` where all are
+    even, and zero elsewhere: the three lines through an all-even point hold
+    quiet values only, and their neighbours loud ones.  H f at those points is as
+    good as their own lines allow: 4e-15 of its 2-norm (a binary64 transform
+    pair is good to a few 1e-16)."""
+    L = (6.0, 5.0, 4.0)
+    plan, prm = lib.Plan(N, L, (0.0, 0.0, 1.0)), lib.make_params(GAMMA, BETA, LAM, OM)
+    shape = (N[2], N[1], N[0])
+    g, phi = W.random_field(shape, 51), W.random_field(shape, 52)
+    Phi = W.random_field(shape, 53, complex_valued=False)
+    f = np.zeros(shape, complex)
+    f[1::2, 1::2, 1::2] = g[1::2, 1::2, 1::2]
+    f[::2, ::2, ::2] = quiet * g[::2, ::2, ::2]
+    got, ref = host(plan.apply_H(prm, dev(f), dev(phi), dev(Phi))), ref_H(N, L, f, phi, Phi)
+    for s in (slice(0, None, 2), slice(1, None, 2)):
+        assert rel2(got[s, s, s] / np.abs(f[s, s, s]).max(), ref[s, s, s] / np.abs(f[s, s, s]).max()) <= 4e-15, s.start
