@@ -403,9 +403,9 @@ __device__ __forceinline__ void mul_tile(const Op& op, const Line& l, int P, int
   }
 #pragma unroll
   for (int r = 0; r < E; ++r) {
-    const int s = kInBits - 32 - M + ex[r], lf = max(s, 0), rt = min(max(-s, 0), 64);
-    v[r].x = shr_clamp((long long)((unsigned long long)v[r].x << lf), rt);
-    v[r].y = shr_clamp((long long)((unsigned long long)v[r].y << lf), rt);
+    const int s = kInBits - 32 - M + ex[r], lf = max(s, 0), rt = min(max(-s, 0), 62);
+    v[r].x = shr_rnd((long long)((unsigned long long)v[r].x << lf), rt);
+    v[r].y = shr_rnd((long long)((unsigned long long)v[r].y << lf), rt);
   }
   mul_exp(tl, sh, M);
 }
