@@ -407,6 +407,24 @@ __global__ void k_out_to_psi(const float* __restrict__ o, double* __restrict__ p
   }
 }
 
+// The loss kernels' conversions, off the FP64 pipe that bounds them.  wide is
+// the cast for every value; narrow is it where it leaves *odd alone (a normal
+// result or zero), and the caller then casts.
+__device__ __forceinline__ double wide(float f) {
+  const unsigned e = (__float_as_uint(f) >> 23) & 0xffu;
+  const unsigned u = __float_as_uint(e == 0u ? f * 18446744073709551616.0f : f);  // a subnormal times 2^64
+  const unsigned off = e == 0u ? 0x34000000u : (e == 255u ? 0x70000000u : 0x38000000u), sg = u & 0x80000000u;
+  return __hiloint2double((int)((u << 1) == 0u ? sg : sg | (((u & 0x7fffffffu) >> 3) + off)), (int)(u << 29));
+}
+__device__ __forceinline__ float narrow(double d, bool* odd) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned a = (hi & 0x7fffffffu) - 0x38000000u;
+  const bool zero = ((hi << 1) | lo) == 0u;
+  *odd |= a - 0x00100000u >= 0x0fe00000u && !zero;
+  const unsigned lr = lo + 0x0fffffffu + ((lo >> 29) & 1u);  // the 29 dropped bits, to nearest even
+  return __uint_as_float((hi & 0x80000000u) | (zero ? 0u : __funnelshift_r(lr, a + (lr < lo ? 1u : 0u), 29)));
+}
+
 // Per-sample sums for the loss: s = <u, t> (complex), uu = |u|^2, tt = |t|^2,
 // u read from the L3 output, t from FP64 targets.  kLossChunks CTAs a sample,
 // each leaving its four sums in sums[b][chunk][4] (with one CTA a sample, 32
@@ -429,7 +447,7 @@ k_loss_sums(const float* __restrict__ o, const double* __restrict__ t, double* _
     out_pos(e / kN3, (int)(e % kN3), bb, z, y, x, ch);
     const float2 u = *reinterpret_cast<const float2*>(o + e);
     const double2 tv = *reinterpret_cast<const double2*>(t + 2 * ((((long)b * kOutZ + z) * kOutY + y) * kOutX + x));
-    const double ur = f2d_bits(u.x), ui = f2d_bits(u.y);
+    const double ur = wide(u.x), ui = wide(u.y);
     a[0] = fma(ur, tv.x, fma(ui, tv.y, a[0]));     // Re <u,t> = Re sum u conj(t)
     a[1] = fma(ui, tv.x, fma(-ur, tv.y, a[1]));    // Im
     a[2] = fma(ur, ur, fma(ui, ui, a[2]));
@@ -479,16 +497,26 @@ k_loss_grad(const float* __restrict__ o, const double* __restrict__ t, const dou
   const long base = (long)b * kOutN * 2;
   constexpr int per = kOutN / kLossChunks;
   const int i0 = blockIdx.y * per;
-#pragma unroll 4
-  for (int i = i0 + threadIdx.x; i < i0 + per; i += 256) {
+  auto point = [&](int i, bool cast) {
     const long e = base + 2 * i;
     int bb, z, y, x, ch;
     out_pos(e / kN3, (int)(e % kN3), bb, z, y, x, ch);
     const float2 u = *reinterpret_cast<const float2*>(o + e);
     const double2 tv = *reinterpret_cast<const double2*>(t + 2 * ((((long)b * kOutZ + z) * kOutY + y) * kOutX + x));
-    const double ur = f2d_bits(u.x), ui = f2d_bits(u.y);
+    const double ur = wide(u.x), ui = wide(u.y);
     const double gr = fma(ar, tv.x, fma(-ai, tv.y, -c * ur)), gi = fma(ar, tv.y, fma(ai, tv.x, -c * ui));
-    *reinterpret_cast<float2*>(dO + e) = make_float2(d2f_bits(gr), d2f_bits(gi));
+    bool odd = false;
+    float2 g = make_float2(narrow(gr, &odd), narrow(gi, &odd));
+    if (cast) g = make_float2((float)gr, (float)gi);
+    *reinterpret_cast<float2*>(dO + e) = g;
+    return odd;
+  };
+  bool odd = false;
+#pragma unroll 4
+  for (int i = i0 + threadIdx.x; i < i0 + per; i += 256) odd |= point(i, false);
+  if (odd) {
+#pragma unroll 1
+    for (int i = i0 + threadIdx.x; i < i0 + per; i += 256) point(i, true);
   }
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
     double acc = 0.0;
