@@ -298,10 +298,13 @@ __device__ __forceinline__ double i2d(long long v, int c) {
   const int sg = (int)(v >> 32) & (int)0x80000000;
   return a == 0 ? 0.0 : __hiloint2double(hi | sg, (int)t);
 }
-// The same for any exponent (overflow to infinity, gradual underflow).
+// The same, rounded alike, for any exponent (overflow to infinity, gradual underflow).
 static __device__ __noinline__ double i2d_any(long long v, int e) {
   if (e >= kExpNaN / 2) return __longlong_as_double(0x7ff8000000000000ll);
-  return scalbn(__ll2double_rn(v), e);
+  const long long a = v < 0 ? -v : v;
+  const long long h = a >> 53 ? 1ll << (10 - __clzll(a)) : 0;  // half a unit in the last of 53 bits (a < 2^63)
+  const long long r = (a + h) & -(h ? 2 * h : 1ll);
+  return scalbn(__ll2double_rn(v < 0 ? -r : r), e);
 }
 __device__ __forceinline__ bool i2d_ok(int e) { return (unsigned)(e + 1085 - 64) <= 2045u - 64u; }
 

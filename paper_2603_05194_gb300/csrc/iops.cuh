@@ -193,7 +193,7 @@ struct Tile {
 };
 
 // The exponent that a tile or line of largest |hi word| M < 0x7ff00000 gets.
-template <int B> __device__ __forceinline__ int load_exp(unsigned M) { return max((int)(M >> 20), 64) - 1023 - (B - 1); }
+template <int B> __device__ __forceinline__ int load_exp(unsigned M) { return (int)(M >> 20) - 1023 - (B - 1); }
 
 // Loads a thread's E elements (guarded by pos < L) as integers of the tile's (of
 // the line's with kLineExp) common exponent, components below 2^59 (2^60 when the
@@ -244,7 +244,15 @@ __device__ __forceinline__ Tile load_tile(const Op& op, const Line& l, int P, in
         M = tile_max<NW>(m, tr.m[1]);
       }
     }
-    const int ex = max((int)(M >> 20), 64);
+    int ex = (int)(M >> 20);
+    // d2i takes zeros and subnormals for 2^-1023: such a tile or line into its range
+    // first (with a branch of each thread the potential took 1% more)
+    if (__any_sync(0xffffffffu, ex < 64)) {
+      const double up = ex < 64 ? 0x1p512 : 1.0;
+      ex += ex < 64 ? 512 : 0;
+#pragma unroll
+      for (int r = 0; r < EL; ++r) d[r].x *= up, d[r].y *= up;
+    }
     const int base = 64 - B + ex;
 #pragma unroll
     for (int r = 0; r < E; ++r) v[r] = r < EL ? c64{d2i(d[r < EL ? r : 0].x, base), d2i(d[r < EL ? r : 0].y, base)} : cz();

@@ -87,3 +87,24 @@ def test_H_rounds_to_nearest(lib):
            + (V + 1000 * (F.real ** 2 + F.imag ** 2) + 400 * Phi.astype(LD)) * F)
     err = np.abs(got.astype(np.clongdouble) - ref)
     assert float(np.sqrt((err ** 2).sum() / (np.abs(ref) ** 2).sum())) <= 1e-15
+
+
+@pytest.mark.parametrize("N", [(32, 64, 16), (36, 20, 18), (54, 50, 12)])
+def test_inputs_next_to_the_smallest_normal(lib, N):
+    """H, P and the dipolar potential are linear: inputs scaled by 2^-980 give
+    results scaled by it bit for bit (no value of theirs is subnormal), inputs
+    scaled by 2^-1015 to 1e-13 of the 2-norm (their smallest are)."""
+    plan = lib.Plan(N, (4.0, 3.0, 2.0), (0.0, 0.0, 1.0))
+    prm = lib.make_params(GAMMA, BETA, LAM, OM)
+    shape = (N[2], N[1], N[0])
+    f, phi = W.random_field(shape, 71), dev(W.random_field(shape, 72))
+    Phi, rho = dev(W.random_field(shape, 73, complex_valued=False)), np.abs(f) + 0.125
+    ops = [lambda g: plan.apply_H(prm, dev(g), phi, Phi), lambda g: plan.apply_preconditioner(prm, 5.0, dev(g), phi, Phi)]
+    scaled = lambda a, k: np.ldexp(a.real, k) + 1j * np.ldexp(a.imag, k)  # noqa: E731
+    for op in ops:
+        one, a, b = host(op(f)), host(op(scaled(f, -980))), host(op(scaled(f, -1015)))
+        assert np.array_equal(a, scaled(one, -980))
+        assert rel2(scaled(b, 1000), scaled(one, -15)) <= 1e-13
+    one = host(plan.dipolar_potential(dev(rho)))
+    assert np.array_equal(host(plan.dipolar_potential(dev(np.ldexp(rho, -980)))), np.ldexp(one, -980))
+    assert rel2(np.ldexp(host(plan.dipolar_potential(dev(np.ldexp(rho, -1015)))), 1000), np.ldexp(one, -15)) <= 1e-13
