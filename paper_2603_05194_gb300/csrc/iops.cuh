@@ -1301,8 +1301,13 @@ struct KinAcc {
   // the sums of k^2 |v|^2 and k |v|^2 in binary64
   __device__ __forceinline__ double2 get() const {
     const double s = pow2d(2 * e + 64), q = 4.656612873077392578125e-10;  // 2^-31
-    return make_double2((fma((double)h2, 4294967296.0, (double)l2) + (double)f2 * q) * s,
-                        (fma((double)h1, 4294967296.0, (double)l1) + (double)f1 * q) * s);
+    const double a = fma((double)h2, 4294967296.0, (double)l2) + (double)f2 * q;
+    const double b = fma((double)h1, 4294967296.0, (double)l1) + (double)f1 * q;
+    if (2 * e + 64 < -1022) {  // v below 2^-480: the scale alone is no normal value, the sums may be
+      const double t = pow2d(e + 32);
+      return make_double2(a * t * t, b * t * t);
+    }
+    return make_double2(a * s, b * s);
   }
 };
 

@@ -108,3 +108,18 @@ def test_inputs_next_to_the_smallest_normal(lib, N):
     one = host(plan.dipolar_potential(dev(rho)))
     assert np.array_equal(host(plan.dipolar_potential(dev(np.ldexp(rho, -980)))), np.ldexp(one, -980))
     assert rel2(np.ldexp(host(plan.dipolar_potential(dev(np.ldexp(rho, -1015)))), 1000), np.ldexp(one, -15)) <= 1e-13
+
+
+@pytest.mark.parametrize("N", [(32, 64, 16), (36, 20, 18), (54, 50, 12)])
+@pytest.mark.parametrize("k", [-500, -300, 300])
+def test_energies_of_scaled_states(lib, N, k):
+    """E_kin and E_rot are quadratic in phi: they scale by 2^(2 k), to 1e-13 (sums
+    of positive and of mixed terms), as long as they are normal values."""
+    plan = lib.Plan(N, (4.0, 3.0, 2.0), (0.0, 0.0, 1.0))
+    prm = lib.make_params(GAMMA, 0.0, 0.0, OM)
+    shape = (N[2], N[1], N[0])
+    f, Phi = W.random_field(shape, 81), dev(np.zeros(shape))
+    one = plan.energy_parts(prm, dev(f), Phi)
+    got = plan.energy_parts(prm, dev(np.ldexp(f.real, k) + 1j * np.ldexp(f.imag, k)), Phi)
+    for key in ("E_kin", "E_rot"):
+        assert abs(np.ldexp(got[key], -2 * k) - one[key]) <= 1e-13 * one["E_kin"], (key, got[key], one[key])
