@@ -39,7 +39,7 @@ struct ExpTab {
 constexpr int kInBits = 59;  // components of a transform's input stay below 2^59
 
 // A real multiplier m 2^(ex - 1084): |m| in [2^61, 2^62), to within 2^-22 of it
-// at either end; ex = 0 stands for 0, ex >= 2040 for infinity and NaN.
+// at either end; ex = 0 stands for 0, ex = 4095 for infinity and NaN.
 struct Mult {
   long long m;
   int ex;
@@ -47,7 +47,8 @@ struct Mult {
 __device__ __forceinline__ Mult mult_of(double d) {
   const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
   const long long m = (long long)(((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | l) << 9);
-  return Mult{(int)h < 0 ? -m : m, (int)((h >> 20) & 0x7ffu)};
+  const int ex = (int)((h >> 20) & 0x7ffu);
+  return Mult{(int)h < 0 ? -m : m, ex + ((ex + 1) & 0x800)};
 }
 
 enum ISrc { kSrcF64 = 0, kSrcInt = 1 };
@@ -357,7 +358,7 @@ __device__ __forceinline__ void mid_tile(const Op& op, const Line& l, int P, int
 __device__ __forceinline__ int mul_shift(unsigned m) { return 62 - mag_bits(m); }
 __device__ __forceinline__ void mul_exp(Tile& tl, int sh, int M) {
   tl.e += M - sh + 64 - 1084 - (kInBits - 32);
-  if (M >= 2040) {  // an infinite or NaN multiplier
+  if (M >= 4095) {  // an infinite or NaN multiplier (a finite one: at most 2046 + 31)
     tl.e = kExpNaN;
     tl.bad = tl.anybad = true;
   }

@@ -123,3 +123,27 @@ def test_energies_of_scaled_states(lib, N, k):
     got = plan.energy_parts(prm, dev(np.ldexp(f.real, k) + 1j * np.ldexp(f.imag, k)), Phi)
     for key in ("E_kin", "E_rot"):
         assert abs(np.ldexp(got[key], -2 * k) - one[key]) <= 1e-13 * one["E_kin"], (key, got[key], one[key])
+
+
+@pytest.mark.parametrize("N", [(32, 64, 16), (36, 20, 18), (54, 50, 12)])
+def test_largest_finite_multipliers(lib, N):
+    """alpha = 1e-304, phi = Phi = 0: the zero frequency's multiplier is 1e304, so
+    that P r is w / alpha times the mean of w r (the rest is 1e-304 of it), w =
+    V^{-1/2} away from the centre (where r = 0, and w is as large as V's rounding
+    there allows).  Finite, and to 1e-13 of that mean's part; 1 / 1e-313 is infinite."""
+    L = (4.0, 3.0, 2.0)
+    plan, prm = lib.Plan(N, L, (0.0, 0.0, 1.0)), lib.make_params(GAMMA, BETA, LAM, OM)
+    shape = (N[2], N[1], N[0])
+    c = (N[2] // 2, N[1] // 2, N[0] // 2)
+    r, zero = W.random_field(shape, 91) + 2.0, np.zeros(shape)
+    r[c] = 0.0
+    (x, y, z), _ = mesh(N, L)
+    V = 0.5 * ((GAMMA[0] * x) ** 2 + (GAMMA[1] * y) ** 2 + (GAMMA[2] * z) ** 2)
+    V[c] = 1.0
+    w = 1.0 / np.sqrt(V)
+    got = host(plan.apply_preconditioner(prm, 1e-304, dev(r), dev(zero.astype(complex)), dev(zero)))
+    away = np.ones(shape, bool)
+    away[c] = False
+    ref = w * np.mean(w * r)
+    assert np.isfinite(got[away]).all() and rel2(got[away] * 1e-304, ref[away]) <= 1e-13
+    assert not np.isfinite(host(plan.apply_preconditioner(prm, 1e-313, dev(r), dev(zero.astype(complex)), dev(zero)))).any()
