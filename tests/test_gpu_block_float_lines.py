@@ -147,3 +147,49 @@ def test_largest_finite_multipliers(lib, N):
     ref = w * np.mean(w * r)
     assert np.isfinite(got[away]).all() and rel2(got[away] * 1e-304, ref[away]) <= 1e-13
     assert not np.isfinite(host(plan.apply_preconditioner(prm, 1e-313, dev(r), dev(zero.astype(complex)), dev(zero)))).any()
+
+
+# every length that k_imix is built for (i64.cuh, int_radices), as the x line, as
+# an unpadded and as a padded column
+IMIX = [16, 32, 64, 128, 256, 18, 20, 24, 30, 36, 40, 48, 60, 72, 80, 90, 96, 100, 108, 120, 144, 150, 160, 180, 192, 200, 216,
+        240, 288, 320, 384]
+
+
+@pytest.mark.parametrize("n", IMIX)
+def test_every_composite_length(lib, n):
+    """Every length of k_imix in each of its forms, on grids of few lines (where
+    the powers of two run on it too): n as Nx, as Ny and Nz (H, P), and n = 2 Ny,
+    2 Nz where n / 2 is a length (the potential).  Against transforms of numpy's
+    (1e-14 of the 2-norm: a few 1e-16 on either side, and H's nu^2 / 2 that raises
+    the reference's error at the low frequencies by less than ten) and the same
+    operators by the generic engine."""
+    grids = [(n, 4, 6), (6, n, 4), (4, 6, n)] + ([(4, n // 2, 6), (6, 4, n // 2)] if n % 4 == 0 else [])
+    L = (4.0, 3.0, 2.0)
+    for N in grids:
+        fixed, gen = lib.Plan(N, L, (0.6, 0.0, 0.8)), lib.Plan(N, L, (0.6, 0.0, 0.8), generic_fft=True)
+        prm = lib.make_params(GAMMA, BETA, LAM, OM)
+        shape = (N[2], N[1], N[0])
+        f, phi = W.random_field(shape, n), W.random_field(shape, n + 1)
+        Phi = W.random_field(shape, n + 2, complex_valued=False)
+        nz, ny, nx = shape
+        pad = np.zeros((2 * nz, 2 * ny, 2 * nx))
+        pad[:nz, :ny, :nx] = np.abs(f) ** 2
+        A = np.fft.ifftn(np.fft.fftn(pad) * host(fixed.multiplier())).real[:nz, :ny, :nx]
+        (x, y, z), (kx, ky, kz) = mesh(N, L)
+        V = 0.5 * ((GAMMA[0] * x) ** 2 + (GAMMA[1] * y) ** 2 + (GAMMA[2] * z) ** 2)
+        w = 1.0 / np.sqrt(7.0 + V + BETA * np.abs(phi) ** 2 + LAM * np.maximum(Phi, 0.0))
+        P = w * np.fft.ifftn(np.fft.fftn(w * f) / (7.0 + 0.5 * (kx ** 2 + ky ** 2 + kz ** 2)))
+        for plan in (fixed, gen):
+            got = (host(plan.dipolar_potential_from_psi(dev(f))), host(plan.apply_H(prm, dev(f), dev(phi), dev(Phi))),
+                   host(plan.apply_preconditioner(prm, 7.0, dev(f), dev(phi), dev(Phi))))
+            for a, b in zip(got, (A, ref_H(N, L, f, phi, Phi), P)):
+                assert rel2(a, b) <= 1e-14, (N, plan is gen)
+            # the forms with fused sums: E_kin and E_rot are sums over the lines' spectra
+            e = plan.energy_parts(prm, dev(f), dev(Phi))
+            h3 = np.prod([2.0 * L[i] / N[i] for i in range(3)])
+            s = [(np.abs(np.fft.fft(f, axis=a)) ** 2) / shape[a] for a in range(3)]
+            kin = h3 * sum(np.sum(0.5 * k ** 2 * s[2 - i]) for i, k in enumerate((kx, ky, kz)))
+            rot = h3 * np.sum(OM * y * kx * s[2] - OM * x * ky * s[1])
+            assert abs(e["E_kin"] - kin) <= 1e-13 * kin and abs(e["E_rot"] - rot) <= 1e-13 * kin, (N, plan is gen)
+        fixed.close()
+        gen.close()
