@@ -691,7 +691,8 @@ def autotune_case():
         plan = B.Plan(p.N, p.L, p.n, f32=True, df32=True, autotune=True)
         for t in plan.tuning():
             key = (names[t["precision"]], t["length"], "x" if t["line_major"] else "yz")
-            pick = "mixed-radix" if t["engine"] == 1 else f"generic/{1 << t['tile_shift']}"
+            pick = ("mixed-radix" if t["engine"] == 1 else "compiled" if t["compiled"]
+                    else f"generic/{1 << t['tile_shift']}")
             rows.setdefault(key, collections.Counter())[pick] += 1
             rows[key]["_ms_default"] += t["ms_default"]
             rows[key]["_ms_best"] += t["ms_best"]

@@ -131,9 +131,11 @@ int atkm_measure_fp64_fma(int blocks_per_sm, int iters, int repeats, double* gfl
  * (binary64; FP32 with ATKM_PLAN_F32; the DF32 form with ATKM_PLAN_DF32) and
  * per layout (line-major x pass, strided y / z pass), times the candidates --
  * in FP32 the mixed-radix register engine (lengths 3 * 2^a and 5 * 2^a <= 384;
- * not with ATKM_PLAN_GENERIC_FFT), in the others the engine that the fixed rule
- * takes, and the generic shared-memory engine
- * at its default tile width, 1/2 and 1/4 of it -- on the plan's own ATKM of
+ * not with ATKM_PLAN_GENERIC_FFT), in binary64 the shared-memory engine with
+ * the length's radices compiled in (two or three stages, up to 384; not with
+ * ATKM_PLAN_GENERIC_FFT), and the generic shared-memory engine at its default
+ * tile width, 1/2 and 1/4 of it (the DF32 form runs the binary64 passes, and
+ * its entries repeat theirs) -- on the plan's own ATKM of
  * |psi|^2, H psi and P r (CUDA events on `stream`, best of 3 after a warm-up)
  * and keeps the fastest; every later pass of that length and layout uses it.
  * Power-of-two lengths keep the power-of-two register engine.  Results change
@@ -148,9 +150,10 @@ typedef struct atkm_tune_info {
   int precision;   /* 0 binary64, 1 FP32, 2 the DF32 form                      */
   int length;      /* line length L                                            */
   int line_major;  /* 1: the x pass (contiguous lines), 0: a strided y / z pass */
-  int engine;      /* 1: mixed-radix register engine, 2: generic engine        */
+  int engine;      /* 1: mixed-radix register engine, 2: shared-memory engine  */
   int tile_shift;  /* generic engine: tile width = default >> tile_shift       */
-  int pad_;
+  int compiled;    /* shared-memory engine: 1 with the length's radices compiled
+                      in, 0 the generic engine                                 */
   double ms_default;  /* the timed operators under the fixed rule, ms          */
   double ms_best;     /* under the chosen candidate, ms                        */
 } atkm_tune_info;

@@ -68,7 +68,7 @@ class IterLog(C.Structure):
 
 class TuneInfo(C.Structure):
     _fields_ = [("precision", C.c_int), ("length", C.c_int), ("line_major", C.c_int), ("engine", C.c_int),
-                ("tile_shift", C.c_int), ("pad_", C.c_int), ("ms_default", C.c_double), ("ms_best", C.c_double)]
+                ("tile_shift", C.c_int), ("compiled", C.c_int), ("ms_default", C.c_double), ("ms_best", C.c_double)]
 
 
 class KernelStat(C.Structure):
@@ -414,7 +414,7 @@ class Plan:
         n = self._lib.atkm_plan_tuning(self._h, arr, cap)
         if n < 0:
             raise AtkmError(-n, "atkm_plan_tuning")
-        return [{k: getattr(arr[i], k) for k, _ in TuneInfo._fields_ if k != "pad_"} for i in range(min(n, cap))]
+        return [{k: getattr(arr[i], k) for k, _ in TuneInfo._fields_} for i in range(min(n, cap))]
 
     # ---- measurement support
     def set_profiling(self, on: bool):

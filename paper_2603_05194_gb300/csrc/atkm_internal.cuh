@@ -494,11 +494,12 @@ struct PcgBuffers;  // defined in pcg.cu
 struct Profiler;    // defined in plan.cu
 
 // One choice of the FFT-tile autotuner (tune.cu): for the arithmetic r (0
-// binary64, 1 FP32, 2 double-word), the line length L and the layout lm (1:
-// line-major x pass, 0: strided pass), the engine (mix = 1: the mixed-radix
-// register engine, else the generic shared-memory engine with its default
-// tile width shifted right by `shift`), with the timed operator set's
-// milliseconds under the default rule and under this choice.
+// binary64, 1 FP32, 2 the DF32 form), the line length L and the layout lm (1:
+// line-major x pass, 0: strided pass), the engine (mix = 1: in FP32 the
+// mixed-radix register engine, in binary64 and the DF32 form the engine of
+// compile-time lengths, k_imix; else the arithmetic's generic shared-memory
+// engine with its default tile width shifted right by `shift`), with the timed
+// operator set's milliseconds under the default rule and under this choice.
 struct TuneEntry {
   int r, L, lm, mix, shift;
   double ms_default, ms_best;
@@ -555,6 +556,10 @@ struct atkm_plan {
 };
 
 namespace atkm {
+
+// Lengths for which a plan's passes and its tuner may take k_imix (the powers of
+// two among them on small grids only, see ipass_grid).
+inline bool imix_ok(const atkm_plan* p, int L) { return int_radices(L).n > 0 && !(p->flags & ATKM_PLAN_GENERIC_FFT); }
 
 extern thread_local std::string g_last_error;
 

@@ -1010,13 +1010,15 @@ inline int ilog2(int v) {
 // LM passes: `lines` lines; column passes: X columns x `outer` outer indices.
 // The tiles of the generic engine are powers of two, narrowed until the pass
 // has two CTAs per SM (a column tile not below 8, which keeps its accesses in
-// whole 128-byte lines).
-inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long lines, int X, int outer, bool mix = true) {
+// whole 128-byte lines).  An autotuned plan's entry decides instead (the DF32
+// form runs these passes too, on the binary64 entries).
+inline IPassGrid ipass_grid(const atkm_plan* p, int L, bool LM, long lines, int X, int outer, bool mix = true) {
   IPassGrid pg;
   pg.fast = L >= 16 && L <= 1024 && (L & (L - 1)) == 0;
-  pg.mix = mix && !pg.fast && int_radices(L).n > 0 && !(p->flags & ATKM_PLAN_GENERIC_FFT);
+  const TuneEntry* te = nullptr;
   for (int i = 0; i < p->n_tune; ++i)
-    if (p->tune[i].r == r && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0) && p->tune[i].shift > 0) pg.mix = false;
+    if (p->tune[i].r == 0 && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0)) te = p->tune + i;
+  pg.mix = mix && !pg.fast && imix_ok(p, L) && (!te || te->mix);
   // Power-of-two lengths up to 256 where the register engine's CTAs (2048
   // elements, 8 a thread) would not give every SM one: k_imix has half the
   // elements a thread and a CTA, so twice the warps share the work.  All passes
@@ -1043,8 +1045,7 @@ inline IPassGrid ipass_grid(const atkm_plan* p, int r, int L, bool LM, long line
       while (T > 1 && T / 2 >= X) T >>= 1;
       while (T > 8 && (long)((X + T - 1) / T) * outer < want) T >>= 1;
     }
-    for (int i = 0; i < p->n_tune; ++i)
-      if (p->tune[i].r == r && p->tune[i].L == L && p->tune[i].lm == (LM ? 1 : 0)) T = std::max(T >> p->tune[i].shift, 1);
+    if (te && !te->mix) T = std::max(T >> te->shift, 1);
     pg.T = T;
   }
   pg.tsh = ilog2(pg.T);

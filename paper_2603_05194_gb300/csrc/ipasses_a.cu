@@ -6,10 +6,9 @@ namespace atkm {
 cudaError_t launch_atkm64(atkm_plan* p, bool dw, int mode, const double* a, const double* b, double* phi,
                           cudaStream_t st) {
   const Geo& g = p->g;
-  const int r = dw ? 2 : 0;
-  const IPassGrid gx = ipass_grid(p, r, g.Nx, true, (long)g.Nz * g.Ny, 0, 0);
-  const IPassGrid gy = ipass_grid(p, r, g.My, false, 0, g.Xh, g.Nz);
-  const IPassGrid gz = ipass_grid(p, r, g.Mz, false, 0, g.Xh, g.My);
+  const IPassGrid gx = ipass_grid(p, g.Nx, true, (long)g.Nz * g.Ny, 0, 0);
+  const IPassGrid gy = ipass_grid(p, g.My, false, 0, g.Xh, g.Nz);
+  const IPassGrid gz = ipass_grid(p, g.Mz, false, 0, g.Xh, g.My);
   cudaError_t e = iatkm_xf(p, dw, mode, a, b, gx, st);
   if (e == cudaSuccess) e = iatkm_yf(p, dw, gx, gy, st);
   if (e == cudaSuccess) e = iatkm_z(p, dw, gy, gz, st);

@@ -8,9 +8,8 @@ namespace atkm {
 cudaError_t launch_H64(atkm_plan* p, bool dw, const Phys& ph, const double* f, const double* phi, const double* Phi,
                        double* Hf, int red_slot, cudaStream_t st) {
   const Geo& g = p->g;
-  const int r = dw ? 2 : 0;
-  HArgs h{&ph, f, phi, Phi, Hf, ipass_grid(p, r, g.Nx, true, (long)g.Nz * g.Ny, 0, 0),
-          ipass_grid(p, r, g.Ny, false, 0, g.Nx, g.Nz), ipass_grid(p, r, g.Nz, false, 0, g.Nx, g.Ny)};
+  HArgs h{&ph, f, phi, Phi, Hf, ipass_grid(p, g.Nx, true, (long)g.Nz * g.Ny, 0, 0),
+          ipass_grid(p, g.Ny, false, 0, g.Nx, g.Nz), ipass_grid(p, g.Nz, false, 0, g.Nx, g.Ny)};
   cudaError_t e = ih_x(p, dw, h, red_slot, st);
   if (e == cudaSuccess) e = ih_y(p, dw, h, red_slot, st);
   if (e == cudaSuccess) e = ih_z(p, dw, h, red_slot, st);

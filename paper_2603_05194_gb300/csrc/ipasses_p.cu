@@ -7,9 +7,9 @@ namespace atkm {
 cudaError_t launch_precond64(atkm_plan* p, const Phys& ph, const double* alpha_dev, const double* r, const double* phi,
                              const double* Phi, double* Pr, cudaStream_t st) {
   const Geo& g = p->g;
-  const IPassGrid gx = ipass_grid(p, 0, g.Nx, true, (long)g.Nz * g.Ny, 0, 0);
-  const IPassGrid gy = ipass_grid(p, 0, g.Ny, false, 0, g.Nx, g.Nz);
-  const IPassGrid gz = ipass_grid(p, 0, g.Nz, false, 0, g.Nx, g.Ny);
+  const IPassGrid gx = ipass_grid(p, g.Nx, true, (long)g.Nz * g.Ny, 0, 0);
+  const IPassGrid gy = ipass_grid(p, g.Ny, false, 0, g.Nx, g.Nz);
+  const IPassGrid gz = ipass_grid(p, g.Nz, false, 0, g.Nx, g.Ny);
   cudaError_t e = ip_xf(p, ph, alpha_dev, r, phi, Phi, gx, st);
   if (e == cudaSuccess) e = ip_y<-1, true>(p, "P_y_f64", p->T1, exp_lines(p->ex[0], gx), 1, gy, st);
   if (e == cudaSuccess) e = ip_z(p, alpha_dev, gy, gz, st);
@@ -23,9 +23,9 @@ template <int S> cudaError_t run_cfft3(atkm_plan* p, double2* buf, cudaStream_t 
   const Geo& g = p->g;
   const int nl = g.Nz * g.Ny;
   const double N = (double)g.Nx * g.Ny * g.Nz;
-  const IPassGrid gx = ipass_grid(p, 0, g.Nx, true, nl, 0, 0, false);
-  const IPassGrid gy = ipass_grid(p, 0, g.Ny, false, 0, g.Nx, g.Nz);
-  const IPassGrid gz = ipass_grid(p, 0, g.Nz, false, 0, g.Nx, g.Ny, false);
+  const IPassGrid gx = ipass_grid(p, g.Nx, true, nl, 0, 0, false);
+  const IPassGrid gy = ipass_grid(p, g.Ny, false, 0, g.Nx, g.Nz);
+  const IPassGrid gz = ipass_grid(p, g.Nz, false, 0, g.Nx, g.Ny, false);
   {
     ICX<S> op;
     op.buf = buf; op.ex = exp_lines(p->ex[0], gx); op.Nx = g.Nx; op.nl = nl;

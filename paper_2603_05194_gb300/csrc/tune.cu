@@ -1,19 +1,20 @@
 // FFT-tile autotuner.  Without it, a pass's engine and tile width follow a
-// fixed rule (ops.cuh, pass_grid): the power-of-two register engine where the
-// line length allows it, else (FP32) the mixed-radix register engine (3 * 2^a
-// and 5 * 2^a), else the generic shared-memory engine at a tile
-// width narrowed until the pass has two CTAs per SM.  The tuner replaces the
+// fixed rule (ops.cuh, pass_grid; iops.cuh, ipass_grid): the power-of-two
+// register engine where the line length allows it, else in FP32 the mixed-radix
+// register engine (3 * 2^a and 5 * 2^a), in binary64 the engine of compile-time
+// lengths (int_radices), else the generic shared-memory engine at a tile width
+// narrowed until the pass has two CTAs per SM.  The tuner replaces the
 // rule by measurement for every line length of the plan that is not a power
 // of two, per arithmetic the plan carries (binary64, and FP32 / the
-// double-word form with ATKM_PLAN_F32 / ATKM_PLAN_DF32) and per layout (the
+// DF32 form with ATKM_PLAN_F32 / ATKM_PLAN_DF32) and per layout (the
 // line-major x pass, the strided y and z passes).  Candidates: in FP32 the
 // mixed-radix register engine where run_pass instantiates it (3 * 2^a and
-// 5 * 2^a up to 384), in the others the engine of the fixed rule (iops.cuh,
-// ipass_grid), and the generic engine of the arithmetic at its default tile
-// width, half of it and a quarter of it.
+// 5 * 2^a up to 384), in binary64 the engine of compile-time lengths (iops.cuh,
+// k_imix) where it is built for the length, and the generic engine of the
+// arithmetic at its default tile width, half of it and a quarter of it.  The
+// DF32 form runs the binary64 passes: its entries repeat theirs.
 // Each candidate is timed on the plan's own operators -- the ATKM of |psi|^2,
-// H psi and P r (no preconditioner in the double-word form) -- with CUDA events, the
-// best of three runs after a warm-up, while every other length keeps its
+// H psi and P r -- with CUDA events, the best of three runs after a warm-up, while every other length keeps its
 // current choice; lengths are tuned one after another in the order x, then
 // the padded and unpadded y and z lengths.  Timing and selection support of
 // the library; the paper has no counterpart.
@@ -49,13 +50,10 @@ cudaError_t run_ops(atkm_plan* p, int r, const Phys& ph, const Scratch& s, cudaS
     e = launch_atkm64(p, false, SRC_PSI, s.psi, nullptr, s.Phi, st);
     if (e == cudaSuccess) e = launch_H64(p, false, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
     if (e == cudaSuccess) e = launch_precond64(p, ph, s.alpha, s.psi, s.psi, s.Phi, s.out, st);
-  } else if (r == 1) {
+  } else {
     e = launch_atkm<float>(p, SRC_PSI, s.psi, nullptr, s.Phi, st);
     if (e == cudaSuccess) e = launch_H<float>(p, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
     if (e == cudaSuccess) e = launch_precond<float>(p, ph, s.alpha, s.psi, s.psi, s.Phi, s.out, st);
-  } else {
-    e = launch_atkm64(p, true, SRC_PSI, s.psi, nullptr, s.Phi, st);
-    if (e == cudaSuccess) e = launch_H64(p, true, ph, s.psi, s.psi, s.Phi, s.out, -1, st);
   }
   return e;
 }
@@ -78,8 +76,10 @@ cudaError_t time_ops(atkm_plan* p, int r, const Phys& ph, const Scratch& s, cuda
   return e;
 }
 
-bool default_mix(const atkm_plan* p, int r, int L) {
-  return !(p->flags & ATKM_PLAN_GENERIC_FFT) && r == 1 && mix_len(L);
+// Whether arithmetic r has a register / compile-time engine for the length: the
+// fixed rule's choice then.
+bool has_mix(const atkm_plan* p, int r, int L) {
+  return r == 1 ? !(p->flags & ATKM_PLAN_GENERIC_FFT) && mix_len(L) : imix_ok(p, L);
 }
 
 }  // namespace
@@ -126,14 +126,24 @@ int atkm_plan_autotune(atkm_plan* plan, void* stream) {
       for (int i = 0; i < plan->n_tune; ++i)
         seen = seen || (plan->tune[i].r == r && plan->tune[i].L == L && plan->tune[i].lm == lm);
       if (seen || plan->n_tune >= kMaxTune) continue;
+      if (r == 2) {  // as in binary64
+        for (int i = 0; i < plan->n_tune; ++i) {
+          const TuneEntry t = plan->tune[i];
+          if (t.r != 0 || t.L != L || t.lm != lm) continue;
+          plan->tune[plan->n_tune] = t;
+          plan->tune[plan->n_tune++].r = 2;
+          break;
+        }
+        continue;
+      }
       std::vector<std::pair<int, int>> cand;
-      if (!(plan->flags & ATKM_PLAN_GENERIC_FFT) && r == 1 && mix_len(L)) cand.push_back({1, 0});
+      if (has_mix(plan, r, L)) cand.push_back({1, 0});
       for (int sh = 0; sh <= 2; ++sh) cand.push_back({0, sh});
       TuneEntry& te = plan->tune[plan->n_tune++];
       te.r = r;
       te.L = L;
       te.lm = lm;
-      const int dmix = default_mix(plan, r, L) ? 1 : 0;
+      const int dmix = has_mix(plan, r, L) ? 1 : 0;
       double best = 1e300, dflt = 0.0;
       int bmix = dmix, bshift = 0;
       for (const auto& c : cand) {
@@ -173,7 +183,8 @@ int atkm_plan_tuning(const atkm_plan* plan, atkm_tune_info* out, int cap) {
     o.precision = t.r;
     o.length = t.L;
     o.line_major = t.lm;
-    o.engine = t.mix ? 1 : 2;
+    o.engine = t.mix && t.r == 1 ? 1 : 2;
+    o.compiled = t.mix && t.r != 1 ? 1 : 0;
     o.tile_shift = t.mix ? 0 : t.shift;
     o.ms_default = t.ms_default;
     o.ms_best = t.ms_best;

@@ -62,7 +62,7 @@ def to_tolerance(problems, psi0_fn, max_iter=12000, tol=1e-8, log=print, autotun
     if autotune:
         tun = [t for pl in plans for t in pl.tuning()]
         out["tuning"] = dict(entries=len(tun), changed=sum(1 for t in tun if t["ms_best"] < t["ms_default"]),
-                             mixed_radix=sum(1 for t in tun if t["engine"] == 1),
+                             mixed_radix=sum(1 for t in tun if t["engine"] == 1 or t["compiled"]),
                              narrowed_tiles=sum(1 for t in tun if t["engine"] == 2 and t["tile_shift"] > 0),
                              ms_default=sum(t["ms_default"] for t in tun), ms_best=sum(t["ms_best"] for t in tun))
     try:
@@ -106,7 +106,7 @@ def run(problems, psi0_fn, iters=40, full_iters=3000, tol=1e-8, precisions=(B.PR
     if autotune:
         tun = [t for pl in plans for t in pl.tuning()]
         out["tuning"] = dict(entries=len(tun), changed=sum(1 for t in tun if t["ms_best"] < t["ms_default"]),
-                             mixed_radix=sum(1 for t in tun if t["engine"] == 1),
+                             mixed_radix=sum(1 for t in tun if t["engine"] == 1 or t["compiled"]),
                              narrowed_tiles=sum(1 for t in tun if t["engine"] == 2 and t["tile_shift"] > 0),
                              ms_default=sum(t["ms_default"] for t in tun), ms_best=sum(t["ms_best"] for t in tun))
         log(f"autotuned {len(plans)} plans in {tune_s:.1f} s (plan creation included): {out['tuning']}")
