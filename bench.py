@@ -265,16 +265,53 @@ def aggregate_ranks(ms: float, evals: float, device: str = "cpu"):
     return float(tm.item()), float(te.item())
 
 
-def pass_table(stats, peaks):
-    """Every pass of the timed region: CUDA-event time, algorithmic bytes and
-    flops per launch, and the fraction of measured HBM bandwidth those bytes
-    reach."""
+# What bounds a pass.  The binary64 transforms run in 64-bit integers and are
+# bound by instruction issue: their share of the issue slots, from one ncu capture
+# on this workload (ISSUE_PROFILE), with the HBM figure beside it.
+ISSUE_PROFILE = "profiles/integer_passes_f64_256x256x64.md"
+ISSUE_SLOTS = {"atkm_x_fwd": 0.56, "atkm_y_fwd": 0.57, "atkm_z": 0.62, "atkm_y_inv": 0.58, "atkm_x_inv": 0.61, "H_x": 0.59,
+               "H_y": 0.60, "P_y": 0.52, "P_z": 0.55, "P_x_inv": 0.54}
+# FP64-pipe instructions and bytes a point of the kernels that this pipe bounds in a
+# binary64 solve (csrc/iops.cuh, csrc/pcg.cu); an FMA is one instruction.  H z takes
+# 7, and 11 with the energy sums: one launch of each an iteration.
+FP64_OPS = {"H_z_f64": (9, None), "P_x_fwd_f64": (7, None), "vec_dir_dots": (14, 80), "vec_curv_sums": (15, 64),
+            "vec_trial": (8, 48), "vec_quartic": (4, 24)}
+
+
+def kernel_bound(k, peaks, fp64_peak, binary64, points):
+    """{bound, achieved, peak, unit, frac, peak_source} of a kernel's record:
+    "issue" (binary64 transforms), "fp64" (kernels of a binary64 solve that the
+    binary64 pipe bounds; points: grid points) or "hbm" (FP32 passes, the vector
+    kernels of the FP32 form, the rest)."""
+    name, sec = k["name"], k["ms_total"] * 1e-3
+    base = name.rsplit("_", 1)[0]
+    if name in FP64_OPS and (binary64 or not name.startswith("vec_")):
+        ops, per = FP64_OPS[name]
+        n = k["bytes_total"] / per if per else points * k["launches"]
+        rate, peak = ops * n / sec / 1e9, fp64_peak["gflops"] / 2
+        return {"bound": "fp64", "achieved": round(rate, 1), "peak": round(peak, 1), "unit": "G FP64 instructions/s",
+                "frac": round(rate / peak, 4), "peak_source": fp64_peak["source"]}
+    if name.endswith(("_f64", "_df")) and base in ISSUE_SLOTS:
+        return {"bound": "issue", "achieved": round(100 * ISSUE_SLOTS[base], 1), "peak": 100.0,
+                "unit": "% of issue slots", "frac": ISSUE_SLOTS[base], "peak_source": "ncu, " + ISSUE_PROFILE}
+    gbs = k["bytes_total"] / sec / 1e9
+    return {"bound": "hbm", "achieved": round(gbs, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
+            "frac": round(gbs / peaks["hbm_gbs"], 4),
+            "peak_source": peaks["source"] + " (MEASURED_PEAKS.json hbm_gbs)"}
+
+
+def pass_table(stats, peaks, fp64_peak, binary64, points):
+    """Every pass of the timed region: CUDA-event time, what bounds it and the
+    fraction of that reached, algorithmic bytes per launch and the fraction of
+    measured HBM bandwidth those bytes reach."""
     out = []
     for k in sorted(stats, key=lambda k: -k["ms_total"]):
         if k["ms_total"] <= 0:
             continue
         gbs = k["bytes_total"] / (k["ms_total"] * 1e-3) / 1e9
+        b = kernel_bound(k, peaks, fp64_peak, binary64, points)
         row = {"name": k["name"], "launches": k["launches"], "ms_per_launch": round(k["ms_total"] / k["launches"], 4),
+               "bound": b["bound"], "frac": round(b["frac"], 3),
                "GB/s": round(gbs, 1), "hbm_frac": round(gbs / peaks["hbm_gbs"], 3)}
         if k["flops_total"] > 0:
             gf = k["flops_total"] / (k["ms_total"] * 1e-3) / 1e9
@@ -283,22 +320,18 @@ def pass_table(stats, peaks):
     return out
 
 
-def roofline(stats, peaks):
+def roofline(stats, peaks, fp64_peak, binary64, points):
     dom = max(stats, key=lambda s: s["ms_total"]) if stats else None
     if dom is None or dom["ms_total"] <= 0:
         return None
-    per_launch_ms = dom["ms_total"] / dom["launches"]
-    passes = pass_table(stats, peaks)
-    # No pass is bound by the FP64 pipe: the binary64 transforms run in integer
-    # arithmetic, and their 5 n log2 n count has no peak to be held against.
-    achieved = dom["bytes_total"] / (dom["ms_total"] * 1e-3) / 1e9
-    return {"kernel": dom["name"], "bound": "hbm", "achieved": round(achieved, 1), "peak": peaks["hbm_gbs"],
-            "unit": "GB/s", "frac": round(achieved / peaks["hbm_gbs"], 4),
-            "peak_source": peaks["source"] + " (MEASURED_PEAKS.json hbm_gbs)",
+    gbs = dom["bytes_total"] / (dom["ms_total"] * 1e-3) / 1e9
+    return {"kernel": dom["name"], **kernel_bound(dom, peaks, fp64_peak, binary64, points),
+            "hbm_GBs": round(gbs, 1), "hbm_frac": round(gbs / peaks["hbm_gbs"], 4),
             "traffic": NCU_TRAFFIC.get(dom["name"], {}).get("bytes"),
             "traffic_source": NCU_TRAFFIC.get(dom["name"], {}).get("profile"),
             "algorithmic_bytes_per_launch": dom["bytes_total"] / dom["launches"],
-            "launch_ms": round(per_launch_ms, 4), "launches": dom["launches"], "passes": passes}
+            "launch_ms": round(dom["ms_total"] / dom["launches"], 4), "launches": dom["launches"],
+            "passes": pass_table(stats, peaks, fp64_peak, binary64, points)}
 
 
 def fp64_peak_now(B) -> dict:
@@ -465,6 +498,7 @@ def run_ours(args, rank, world, local_rank):
     w = W.CONFIGS[WORKLOAD]
     precision = B.PRECISION_F32_F64 if args.precision == "mixed" else B.PRECISION_F64
     fp64_peak = fp64_peak_now(B)
+    points = math.prod(w.N)
     peaks = measured_peaks()
     plan = B.Plan(w.N, w.L, w.n, f32=True, df32=True)
     prm = B.make_params(w.gamma, w.beta, w.lam, w.Omega)
@@ -489,7 +523,7 @@ def run_ours(args, rank, world, local_rank):
         mms, mev = aggregate_ranks(mx["ms"], float(mx["evals"]), "cuda") if dist else (mx["ms"], float(mx["evals"]))
         pform = {"value": round(mev / (mms * 1e-3), 2), "unit": UNIT,
                  "ms_per_step": round(mms / max(mx["steps"], 1), 3), "steps": mx["steps"],
-                 "roofline": roofline(mx["stats"], peaks),
+                 "roofline": roofline(mx["stats"], peaks, fp64_peak, False, points),
                  "gpu_launches": mx["launches"], "residual_after_steps": mx["res"]["residual"],
                  "f32_iterations": mx["res"]["f32_iters"]}
 
@@ -541,7 +575,7 @@ def run_ours(args, rank, world, local_rank):
         ttt_u = time_to_tol(B, W.PAPER_WORKLOADS["ex31_caseII_256"], forms)
     return dict(ms=ms_max, evals=evals_all, steps=main["steps"], res=main["res"], standalone=standalone,
                 e2e_value=e2e_evals * world / (e2e_ms * 1e-3), nbytes=nbytes,
-                roof=roofline(main["stats"], peaks), stats=main["stats"], clocks=main["clocks"],
+                roof=roofline(main["stats"], peaks, fp64_peak, True, points), stats=main["stats"], clocks=main["clocks"],
                 launches=main["launches"], pform=pform, ttt=ttt, ttt_u=ttt_u, fp64_peak=fp64_peak)
 
 

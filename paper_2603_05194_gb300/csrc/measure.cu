@@ -1,6 +1,6 @@
 // Peak-rate measurement of the binary64 FMA pipe, the denominator of the
-// roofline of the binary64 FFT passes (which are bound by that pipe on this
-// GPU).  Every thread runs kChains independent FMA chains a = a * b + c with
+// roofline of the kernels of a binary64 solve that this pipe bounds (the vector
+// kernels, H z, P x forward; the transforms run in integers).  Every thread runs kChains independent FMA chains a = a * b + c with
 // |b| < 1, so each chain stays bounded and no chain waits on another; the
 // sums are stored so the compiler keeps every FMA.  Measurement support of
 // the library; the paper has no counterpart.
