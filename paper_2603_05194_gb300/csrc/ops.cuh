@@ -786,8 +786,8 @@ __device__ __forceinline__ R pv_rsqrt(const Cst<R>& c, const PhysR<R>& ph, R alp
   return rsq<R>(den);
 }
 
-// Binary64: the weight P_V^{-1/2} of each point is also stored in Pw for the
-// x inverse pass, which then reads it instead of forming it again.
+// The weight P_V^{-1/2} of each point is formed in the x forward and again in the
+// x inverse pass.
 template <typename R> struct OpPXF : OpBase<-1, false, 0, true> {
   const double2* r; const double2* phi; const double* Phi; cx<R>* Wk; Cst<R> c; PhysR<R> ph; const double* alpha;
   __device__ bool valid(int o, int) const { return o < c.Nz * c.Ny; }

@@ -142,8 +142,8 @@ cudaError_t launch_atkm(atkm_plan* p, int mode, const double* a, const double* b
 // One axis pass of H_phi f (a function of its own so that heavy
 // instantiations can be compiled in separate translation units).
 template <typename R>
-cudaError_t h_pass_x(atkm_plan* p, const Phys& ph, const double* f, const double* phi, const double* Phi, double* Hf,
-                    int red_slot, cudaStream_t st) {
+cudaError_t h_pass_x(atkm_plan* p, const Phys& ph, const double* f, const double*, const double*, double*, int red_slot,
+                    cudaStream_t st) {
   const Geo& g = p->g;
   cx<R>* acc = p->T1f;
   if (!acc) return cudaErrorInvalidValue;
@@ -151,11 +151,8 @@ cudaError_t h_pass_x(atkm_plan* p, const Phys& ph, const double* f, const double
   const Cst<R> c = make_cst<R>(g);
   const PhysR<R> pr = make_physr<R>(ph);
   const double2* fin = reinterpret_cast<const double2*>(f);
-  const double2* pin = reinterpret_cast<const double2*>(phi);
-  double2* out = reinterpret_cast<double2*>(Hf);
   const double N = (double)g.Nx * g.Ny * g.Nz, s = (double)sizeof(cx<R>);
   const long nl = (long)g.Nz * g.Ny;
-  (void)pin; (void)out; (void)nl; (void)pr;
   // x
   {
     const PassGrid pg = pass_grid<R>(p, g.Nx, true, nl, 0, 0);
@@ -175,8 +172,8 @@ cudaError_t h_pass_x(atkm_plan* p, const Phys& ph, const double* f, const double
 }
 
 template <typename R>
-cudaError_t h_pass_y(atkm_plan* p, const Phys& ph, const double* f, const double* phi, const double* Phi, double* Hf,
-                    int red_slot, cudaStream_t st) {
+cudaError_t h_pass_y(atkm_plan* p, const Phys& ph, const double* f, const double*, const double*, double*, int red_slot,
+                    cudaStream_t st) {
   const Geo& g = p->g;
   cx<R>* acc = p->T1f;
   if (!acc) return cudaErrorInvalidValue;
@@ -184,11 +181,7 @@ cudaError_t h_pass_y(atkm_plan* p, const Phys& ph, const double* f, const double
   const Cst<R> c = make_cst<R>(g);
   const PhysR<R> pr = make_physr<R>(ph);
   const double2* fin = reinterpret_cast<const double2*>(f);
-  const double2* pin = reinterpret_cast<const double2*>(phi);
-  double2* out = reinterpret_cast<double2*>(Hf);
   const double N = (double)g.Nx * g.Ny * g.Nz, s = (double)sizeof(cx<R>);
-  const long nl = (long)g.Nz * g.Ny;
-  (void)pin; (void)out; (void)nl; (void)pr;
   // y
   {
     const PassGrid pg = pass_grid<R>(p, g.Ny, false, 0, g.Nx, g.Nz);
@@ -220,8 +213,6 @@ cudaError_t h_pass_z(atkm_plan* p, const Phys& ph, const double* f, const double
   const double2* pin = reinterpret_cast<const double2*>(phi);
   double2* out = reinterpret_cast<double2*>(Hf);
   const double N = (double)g.Nx * g.Ny * g.Nz, s = (double)sizeof(cx<R>);
-  const long nl = (long)g.Nz * g.Ny;
-  (void)pin; (void)out; (void)nl; (void)pr;
   // z + pointwise
   {
     const PassGrid pg = pass_grid<R>(p, g.Nz, false, 0, g.Nx, g.Ny);
@@ -229,14 +220,12 @@ cudaError_t h_pass_z(atkm_plan* p, const Phys& ph, const double* f, const double
     const char* n = "H_z_f32";
     if (red) {
       OpHZ<R, true> op; op.f = fin; op.phi = pin; op.Phi = Phi; op.acc = acc; op.Hf = out; op.c = c; op.ph = pr;
-     
       op.same = fin == pin;
       op.part = p->partials; op.pstride = pg.grid.x * pg.grid.y;
       op.sums = p->scal + red_slot + 4; op.cnt = p->cnt;
       ATKM_RUN(n, (op.same ? 40 : 56) * N + N * s, fl, op, p->fN[2], pg);
     } else {
       OpHZ<R, false> op; op.f = fin; op.phi = pin; op.Phi = Phi; op.acc = acc; op.Hf = out; op.c = c; op.ph = pr;
-     
       op.same = fin == pin;
       ATKM_RUN(n, (op.same ? 40 : 56) * N + N * s, fl, op, p->fN[2], pg);
     }
@@ -270,7 +259,6 @@ cudaError_t launch_precond(atkm_plan* p, const Phys& ph, const double* alpha_dev
   {
     OpPXF<R> op; op.r = reinterpret_cast<const double2*>(r); op.phi = reinterpret_cast<const double2*>(phi);
     op.Phi = Phi; op.Wk = Wk; op.c = c; op.ph = pr; op.alpha = alpha_dev;
-   
     const double by = 40.0 * N + N * s;
     ATKM_RUN("P_x_fwd_f32", by, fx, op, p->fN[0], gx);
   }

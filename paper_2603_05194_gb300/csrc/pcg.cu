@@ -1347,9 +1347,12 @@ struct Solver {
     Seq S{plan, *B, ph, is32, qq};
     S.aux32 = (split || dwm) && !is32;
     S.dw = dwm && !is32;
-    // seq_q's kernels are captured into the solve graph; the FP32 passes fill the
-    // memory system by themselves (a second branch slowed ten iterations at
-    // 256x256x64 from 11.3 to 11.5 ms)
+    // seq_q's kernels are captured into the solve graph; the FP32 phase keeps one
+    // branch (a second one slowed ten iterations at 256x256x64 from 11.3 to 11.5 ms).
+    // The polish of the split forms, whose two operators are FP32 passes too, keeps
+    // both: 100 of its iterations 180.5 against 179.2 ms with one branch at
+    // 256x256x64, but 200 at 128x128x32 77.0 against 80.1, 400 at 64x64x16 68.9
+    // against 73.1.
     S.fork = !is32;
     return S;
   }
