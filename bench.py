@@ -71,7 +71,7 @@ def parse():
                          "binary64 PCG to residual 1e-8 at 128x128x32; one JSON line each")
     ap.add_argument("--sweep-max-iter", type=int, default=12000, help="iteration cap of each sweep instance")
     ap.add_argument("--cpu-sample", action="store_true", help=argparse.SUPPRESS)
-    ap.add_argument("--profile-case", choices=["atkm_f32", "atkm_f64", "atkm_df32", "pcg_f64", "pcg_mixed",
+    ap.add_argument("--profile-case", choices=["atkm_f32", "atkm_f64", "atkm_df32", "operators_f64", "pcg_f64", "pcg_mixed",
                                                "profiling_overhead", "polish_df32", "fp64_peak", "iterations",
                                                "virial_vs_tol", "engines", "finest_level", "basin",
                                                "f32_floor", "mg_policy", "guess_gemm", "autotune"],
@@ -269,8 +269,8 @@ def aggregate_ranks(ms: float, evals: float, device: str = "cpu"):
 # bound by instruction issue: their share of the issue slots, from one ncu capture
 # on this workload (ISSUE_PROFILE), with the HBM figure beside it.
 ISSUE_PROFILE = "profiles/integer_passes_f64_256x256x64.md"
-ISSUE_SLOTS = {"atkm_x_fwd": 0.56, "atkm_y_fwd": 0.57, "atkm_z": 0.62, "atkm_y_inv": 0.58, "atkm_x_inv": 0.61, "H_x": 0.59,
-               "H_y": 0.60, "P_y": 0.52, "P_z": 0.55, "P_x_inv": 0.54}
+ISSUE_SLOTS = {"atkm_x_fwd": 0.56, "atkm_y_fwd": 0.57, "atkm_z": 0.62, "atkm_y_inv": 0.58, "atkm_x_inv": 0.61, "H_x": 0.60,
+               "H_y": 0.60, "P_y": 0.53, "P_z": 0.59, "P_x_inv": 0.54}
 # FP64-pipe instructions and bytes a point of the kernels that this pipe bounds in a
 # binary64 solve (csrc/iops.cuh, csrc/pcg.cu); an FMA is one instruction.  H z takes
 # 7, and 11 with the energy sums: one launch of each an iteration.
@@ -964,8 +964,8 @@ def forms_case(case: str):
 
 def profile_case(case: str):
     """Small fixed workloads on the bench grid for ncu captures (about 1 GB of
-    device memory): two ATKM evaluations, or three PCG iterations; or a
-    timing quoted in the design notes; or the binary64 FMA peak (fp64_peak:
+    device memory): two ATKM evaluations, one ATKM, H and P twice over
+    (operators_f64), or three PCG iterations; or a timing quoted in the design notes; or the binary64 FMA peak (fp64_peak:
     the roofline denominator of the binary64 passes, one JSON line)."""
     if case in ("profiling_overhead", "polish_df32"):
         timing_case(case)
@@ -1002,6 +1002,13 @@ def profile_case(case: str):
             Phi = plan.dipolar_potential_from_psi(psi, f32=(case == "atkm_f32"), df32=(case == "atkm_df32"))
         torch.cuda.synchronize()
         print(case, "max|Phi|", float(Phi.abs().max()))
+    elif case == "operators_f64":
+        prm = B.make_params(w.gamma, w.beta, w.lam, w.Omega)
+        for _ in range(2):
+            Phi = plan.dipolar_potential_from_psi(psi)
+            plan.apply_H(prm, psi, psi, Phi)
+            plan.apply_preconditioner(prm, 40.0, psi, psi, Phi)
+        torch.cuda.synchronize()
     else:
         prm = B.make_params(w.gamma, w.beta, w.lam, w.Omega)
         prec = B.PRECISION_F64 if case == "pcg_f64" else B.PRECISION_F32_F64

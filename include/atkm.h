@@ -227,6 +227,10 @@ typedef struct atkm_params {
  *   phi  N complex: the state whose density enters beta |phi|^2.
  *   Phi  N doubles: the dipolar potential of |phi|^2 (from dipolar_potential).
  *   Hf   N complex output; must not alias f, phi or Phi.
+ * The kinetic and rotation part is accurate line by line: its error follows the
+ * largest values on the three grid lines through a point (64-bit integers with
+ * one exponent a line).  In the dipolar potential and the preconditioner, which
+ * mix all axes, it follows the largest values of the whole result.
  */
 int apply_H(atkm_plan* plan, const atkm_params* prm, const double* f, const double* phi,
             const double* Phi, double* Hf, void* stream);

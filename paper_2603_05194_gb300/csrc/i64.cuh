@@ -3,7 +3,7 @@
 //
 // GB300 issues 2 binary64 operations per clock and SM, 1/64 of its 32-bit
 // rate, so an FFT in binary64 is bound by that pipe (88-93% busy before this
-// form).  Here a CTA's tile of line elements shares one exponent e and each
+// form).  Here a CTA's tile of line elements (in H each line) shares one exponent e and each
 // real number is a 64-bit integer X with value X 2^e, |X| < 2^63: 58 to 62
 // significant bits of the tile's largest element against binary64's 53.  An
 // addition is two 32-bit instructions, a product with a twiddle three

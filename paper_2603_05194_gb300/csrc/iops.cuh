@@ -8,9 +8,9 @@
 //     every stage;
 //   * k_igen: every other {2,3,5}-smooth length up to 2048, radix-8/6/5/4/3/2
 //     stages between two shared-memory tiles.
-// A pass whose input is binary64 finds its tile's largest exponent and turns
-// the elements into integers; between passes the spectra stay integers in the
-// workspaces, each tile with its exponent in a small table, so only the first
+// A pass whose input is binary64 finds its tile's largest exponent (H: each
+// line's) and turns the elements into integers; between passes the spectra stay integers in the
+// workspaces, each tile (line) with its exponent in a small table, so only the first
 // and the last pass of an operator convert.  Between a forward and an inverse
 // transform the tile is scaled up again to its actual size.
 #pragma once
@@ -446,8 +446,9 @@ __device__ __forceinline__ void ireduce_out(double (&acc)[NR], double* sh, doubl
 // cost 10-15% (H 318 against 276 us at 256x256x64), four, at 64, gained 2% in the
 // forward passes and lost 7% in the inverse ones.  At 256x256x64, against radix-8
 // transforms in FP64 instructions (FP64 pipe 88-93% busy): ATKM x, y, z, y, x 246,
-// 336, 1063, 357, 238 -> 51, 72, 231, 76, 59 us; H x, y, z 351, 369, 344 -> 77, 80,
-// 110; P x, y, z, y, x 298, 168, 336, 168, 183 -> 107, 43, 70, 43, 61.
+// 336, 1063, 357, 238 -> 51, 71, 231, 76, 60 us; H x, y, z 351, 369, 344 -> 84, 85,
+// 115 (77, 80, 110 with one exponent a tile); P x, y, z, y, x 298, 168, 336, 168,
+// 183 -> 108, 42, 70, 42, 61.
 constexpr int kIElems = 2048;  // elements per CTA (256 threads x 8)
 
 template <int L> struct IFast {
@@ -775,7 +776,7 @@ template <class Op> __global__ void __launch_bounds__(kThreads, 2) k_igen(Op op,
 // in registers, and the inverse transform takes the radices in the opposite
 // order, so that its first stage finds its inputs in the registers where the
 // forward transform left them.  All passes of an ATKM, an H and a P against
-// k_igen: 550 -> 348 us at 144x144x36, 648 -> 475 at 160x160x40, 231 -> 152 at
+// k_igen: 561 -> 351 us at 144x144x36, 656 -> 473 at 160x160x40, 234 -> 151 at
 // 96x96x24.  Bound by instruction issue, as k_ifast.
 template <int L> struct IMix {
   static constexpr RadList R = int_radices(L);
