@@ -536,7 +536,7 @@ struct atkm_plan {
   atkm::c64* W1;       // [Nz][Ny][XS] half spectrum in x
   atkm::c64* W2;       // [Nz][My][XS]
   atkm::c64* T1;       // [Nz][Ny][Nx]
-  atkm::c64* T2;       // [Nz][Ny][Nx], the y part of H
+  atkm::c64* T2;       // [Nz][Ny][Nx], the y part of H; W2 itself where memory is short (share_T2)
   int* ex[5];          // tile exponents of the integer arrays (ATKM and P: 0..2, H: 3, 4)
   float2* W1f;
   float2* W2f;
@@ -556,6 +556,13 @@ struct atkm_plan {
 };
 
 namespace atkm {
+
+// H's y part has a workspace of its own so that H p and the ATKM of Re(conj(phi) p)
+// can run side by side.  Where the device has no room for it (16 bytes a point of
+// about 130 for a plan, 300 with a solve's vectors) it lies in W2, and the two run
+// one after the other.
+inline bool T2_shared(const atkm_plan* p) { return p->T2 == p->W2; }
+void share_T2(atkm_plan* p);
 
 // Lengths for which a plan's passes and its tuner may take k_imix (the powers of
 // two among them on small grids only, see ipass_grid).

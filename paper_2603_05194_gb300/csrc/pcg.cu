@@ -895,7 +895,7 @@ void pcg_free(atkm_plan* p) {
   p->pcg = nullptr;
 }
 
-static cudaError_t pcg_alloc(atkm_plan* p) {
+static cudaError_t pcg_alloc_once(atkm_plan* p) {
   if (p->pcg) return cudaSuccess;
   PcgBuffers* b = new PcgBuffers();
   p->pcg = b;
@@ -923,6 +923,16 @@ static cudaError_t pcg_alloc(atkm_plan* p) {
   }
   if (e == cudaSuccess) e = cudaMemset(b->ctl, 0, sizeof(Ctl));
   if (e != cudaSuccess) pcg_free(p);
+  return e;
+}
+static cudaError_t pcg_alloc(atkm_plan* p) {
+  const unsigned long long before = p->bytes;
+  cudaError_t e = pcg_alloc_once(p);
+  if (e != cudaSuccess) p->bytes = before;
+  if (e == cudaErrorMemoryAllocation && !T2_shared(p)) {
+    share_T2(p);
+    return pcg_alloc(p);
+  }
   return e;
 }
 
@@ -1353,7 +1363,7 @@ struct Solver {
     // both: 100 of its iterations 180.5 against 179.2 ms with one branch at
     // 256x256x64, but 200 at 128x128x32 77.0 against 80.1, 400 at 64x64x16 68.9
     // against 73.1.
-    S.fork = !is32;
+    S.fork = !is32 && !T2_shared(plan);
     return S;
   }
   int log_room() const { return (logbuf && opts->log_capacity > logc) ? opts->log_capacity - logc : 0; }

@@ -58,6 +58,15 @@ cudaError_t dev_alloc(atkm_plan* p, void** ptr, size_t bytes) {
   return e;
 }
 
+void share_T2(atkm_plan* p) {
+  if (p->T2) {
+    cudaFree(p->T2);
+    p->bytes -= (size_t)p->g.Nx * p->g.Ny * p->g.Nz * sizeof(c64);
+  }
+  p->T2 = p->W2;
+  cudaGetLastError();  // of the allocation that failed
+}
+
 Phys make_phys(const atkm_params* prm) {
   Phys ph;
   ph.gx2 = prm->gamma[0] * prm->gamma[0];
@@ -433,6 +442,7 @@ bool make_int_len(int L, IntLen& f) {
 }
 
 void free_plan_memory(atkm_plan* p) {
+  if (T2_shared(p)) p->T2 = nullptr;
   void* ptrs[] = {p->tw32, p->twi, p->axtab, p->Pw, p->U0, p->U0f, p->Kz, p->W1, p->W2, p->T1, p->T2,
                   p->W1f, p->W2f, p->T1f, p->ex[0], p->ex[1], p->ex[2], p->ex[3], p->ex[4], p->partials, p->scal, p->cnt};
   for (void* q : ptrs)
@@ -771,7 +781,6 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   if ((e = dev_alloc(p, (void**)&p->W1, n_w1 * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = dev_alloc(p, (void**)&p->W2, n_w2 * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = dev_alloc(p, (void**)&p->T1, Nt * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
-  if ((e = dev_alloc(p, (void**)&p->T2, Nt * sizeof(c64))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   // tile exponents: at most one per x line, or one per outer index and column
   const size_t n_ex = std::max((size_t)g.Nz * g.Ny, (size_t)std::max(g.My, std::max(g.Nz, g.Ny)) * g.Xh);
   for (int*& q : p->ex)
@@ -795,6 +804,9 @@ int atkm_plan_create(atkm_plan** out, const int N[3], const double L[3], const d
   if ((e = dev_alloc(p, (void**)&p->scal, SC_COUNT * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = cudaMallocHost((void**)&p->scal_host, SC_COUNT * sizeof(double))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = dev_alloc(p, (void**)&p->cnt, sizeof(unsigned))) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
+  e = dev_alloc(p, (void**)&p->T2, Nt * sizeof(c64));  // the last one: the plan can do without
+  if (e == cudaErrorMemoryAllocation) share_T2(p);
+  else if (e != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan workspace"));
   if ((e = cudaMemsetAsync(p->cnt, 0, sizeof(unsigned), st)) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = cudaMemsetAsync(p->scal, 0, SC_COUNT * sizeof(double), st)) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan scalars"));
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(cuda_fail(nullptr, e, "plan create"));
